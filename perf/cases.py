@@ -288,3 +288,103 @@ def tolerance(case):
         # `hidden` elements of its gradient by its whole size: counted once there is a chance of it
         return {"rel": 1e-5, "max": 4e-5} if hidden < 100000 else {"rel": 1e-5 + 2.0 * hidden ** -0.5, "max": 0.5}
     return {"rel": 1e-2, "max": 0.5 if relu else 0.1}
+
+
+def _attention_exact(x, p, heads_out, causal, scale):
+    q, k, v = (torch.einsum("bld,dhk->blhk", x, p[n]) for n in ("wq", "wk", "wv"))
+    s = torch.einsum("blhk,bmhk->bhlm", q, k).mul_(scale)
+    if causal:
+        s.masked_fill_(torch.ones(s.shape[-2:], dtype=torch.bool, device=s.device).triu(1), float("-inf"))
+    w = torch.softmax(s, -1)
+    o = torch.einsum("bhlm,bmhk->blhk", w, v)
+    heads_out.update(q=q, kk=k, vv=v, weights=w, o=o)
+    return torch.einsum("blhk,hkd->bld", o, p["wo"])
+
+
+def _attention_grads(x, p, r, dy, scale):
+    do = torch.einsum("bld,hkd->blhk", dy, p["wo"])
+    r["dwo"] = torch.einsum("blhk,bld->hkd", r["o"], dy)
+    dw = torch.einsum("blhk,bmhk->bhlm", do, r["vv"])
+    dv = torch.einsum("bhlm,blhk->bmhk", r["weights"], do)
+    ds = r["weights"] * (dw - (dw * r["weights"]).sum(-1, keepdim=True))
+    dq, dk = (torch.einsum(e, ds, r[n]).mul_(scale) for e, n in (("bhlm,bmhk->blhk", "kk"), ("bhlm,blhk->bmhk", "q")))
+    dx = 0.0
+    for n, d in (("wq", dq), ("wk", dk), ("wv", dv)):
+        r["d" + n] = torch.einsum("bld,blhk->dhk", x, d)
+        dx = dx + torch.einsum("blhk,dhk->bld", d, p[n])
+    return dx
+
+
+def _ffn_exact(x, p, r):
+    r["h"] = torch.relu(x @ p["w"] + p["bias"])
+    return r["h"] @ p["v"]
+
+
+def _ffn_grads(x, p, r, dy):
+    dh = (dy @ p["v"].T) * (r["h"] > 0)
+    r["dv"], r["dw"], r["dbias"] = r["h"].flatten(0, 1).T @ dy.flatten(0, 1), x.flatten(0, 1).T @ dh.flatten(0, 1), dh.sum((0, 1))
+    return dh @ p["w"].T
+
+
+def _norm_exact(x, gamma, beta):
+    mu = x.mean(-1, keepdim=True)
+    rstd = ((x - mu) ** 2).mean(-1, keepdim=True).add(1e-6).rsqrt()
+    return gamma * (x - mu) * rstd + beta, torch.cat([mu, rstd], -1)
+
+
+def _norm_grads(x, stats, gamma, dy):
+    xh = (x - stats[..., :1]) * stats[..., 1:]
+    g = dy * gamma
+    dx = stats[..., 1:] * (g - g.mean(-1, keepdim=True) - xh * (g * xh).mean(-1, keepdim=True))
+    return dx, (dy * xh).sum((0, 1)), dy.sum((0, 1))
+
+
+def exact(case, seed):
+    """What `run` returns, in 64 bits with nothing rounded in between, in plain torch."""
+    s, kind, back = prepare(case, seed), case["kind"], case.get("backward", True)
+    p = {n: t.double() if t.is_floating_point() else t.long() for n, t in s.t.items() if n not in s.out or kind == "vocab"}
+    names = list(s.out)
+    del s
+    torch.cuda.empty_cache()
+    r = {}
+    if kind == "vocab":
+        B, L = case["batch"], case["length"]
+        x = p["table"][p["ids"]]
+        z = x @ p["wout"]
+        r["lse"] = torch.logsumexp(z, -1)
+        r["loss"] = r["lse"] - z.gather(1, p["targets"][:, None])[:, 0]
+        g = z.sub_(r["lse"][:, None]).exp_()
+        g[torch.arange(B * L, device=g.device), p["targets"]] -= 1.0
+        g.mul_(p["dloss"].view(-1, 1))
+        r["logits"], r["x"], r["dx"], r["dwout"] = g, x, g @ p["wout"].T, x.T @ g
+        r["dtable"] = torch.zeros_like(p["table"]).index_add_(0, p["ids"], r["dx"])
+        for w in ("table", "wout"):
+            r[w + "_momentum"] = 0.9 * p[w + "_momentum"] + r["d" + w]
+            r[w + "_master"] = p[w + "_master"] - 0.01 * (r[w + "_momentum"] + 1e-4 * p[w + "_master"])
+            r[w] = r[w + "_master"]
+        for n in ("x", "dx", "logits", "lse", "loss"):
+            r[n] = r[n].view(B, L, *r[n].shape[1:])
+        return {n: r.get(n) for n in names}
+    x, dy = p["x"], p.get("dy")
+    if kind == "ffn":
+        r["y"] = _ffn_exact(x, p, r)
+        if back:
+            r["dx"] = _ffn_grads(x, p, r, dy)
+        return {n: r.get(n) for n in names}
+    scale = case["d_k"] ** -0.5
+    y = _attention_exact(x, p, r, case["causal"], scale)
+    if kind == "attention":
+        r["y"] = y
+        if back:
+            r["dx"] = _attention_grads(x, p, r, dy, scale)
+        return {n: r.get(n) for n in names}
+    r["s1"] = x + y
+    r["a"], r["stats1"] = _norm_exact(r["s1"], p["ln1_gamma"], p["ln1_beta"])
+    r["s2"] = r["a"] + _ffn_exact(r["a"], p, r)
+    r["y"], r["stats2"] = _norm_exact(r["s2"], p["ln2_gamma"], p["ln2_beta"])
+    if back:
+        ds2, r["dln2_gamma"], r["dln2_beta"] = _norm_grads(r["s2"], r["stats2"], p["ln2_gamma"], dy)
+        da = ds2 + _ffn_grads(r["a"], p, r, ds2)
+        ds1, r["dln1_gamma"], r["dln1_beta"] = _norm_grads(r["s1"], r["stats1"], p["ln1_gamma"], da)
+        r["dx"] = ds1 + _attention_grads(x, p, r, ds1, scale)
+    return {n: r.get(n) for n in names}
