@@ -5,8 +5,8 @@
 // partials are then added in that order (the Allreduce, realised on the device).  Component-wise
 // work (Section 6, Section 7 broadcasting) is applied to the sum before the store.
 //
-// This family is the fp32 path and the fallback for shapes the tensor-core family does not take;
-// it is plain FFMA code and makes no attempt at tiling.
+// This is the fallback for structures that neither the tensor-core kernels nor the f32 matrix-product kernel
+// (einsum_f32.cu) take; it is plain FFMA code and makes no attempt at tiling.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 

@@ -98,6 +98,20 @@ struct TcParams {
   int bias_along_m = 0;                      // bias varies with m (after a swap) instead of n
 };
 
+// ---- parameters of the f32 matrix-product kernel -------------------------------------------------------
+// The same canonical form with element strides for every index; the layout's slices need no trace here, since every
+// output element is one sum over all of K whoever owns its parts.
+struct F32Params {
+  int64_t M = 1, N = 1, K = 1;
+  int64_t sAm = 0, sAk = 0, sBn = 0, sBk = 0;
+  int64_t ldc = 0;                           // element stride of M in C (N is contiguous)
+  int n_outer = 0;
+  int64_t outer_size[mtf::kMaxOuter] = {1, 1, 1};
+  int64_t outer_sA[mtf::kMaxOuter] = {0, 0, 0}, outer_sB[mtf::kMaxOuter] = {0, 0, 0}, outer_sC[mtf::kMaxOuter] = {0, 0, 0};
+  int swapped = 0;                           // in[0] and in[1] exchanged so that N is contiguous in C
+  int bias_along_m = 0;
+};
+
 struct EpilogueDesc {
   bool on = false;
   float scale = 1.f;
@@ -133,6 +147,8 @@ struct mtf_plan_s {
   int n_reduce_mesh_dims = 0;
   // kernel parameters (pointers filled in at exec time)
   SimtParams simt;
+  bool f32_ok = false;      // generic family: the f32 matrix-product kernel takes this einsum
+  F32Params f32;
   TcParams tc;
   std::string key;
 };
@@ -175,6 +191,8 @@ mtf_status rank_wait(const mtf_layout_t* L, void* stream);
 
 // launchers (defined in the .cu files)
 mtf_status launch_simt(const SimtParams& p, int64_t rsum_elems, void* stream);
+mtf_status launch_f32(const F32Params& p, const void* A, const void* B, void* C, int dtC, const void* bias, int dtBias, const void* mask, int dtMask,
+                      const void* resid, int dtRes, float scale, int relu, float* rsum, void* stream);
 mtf_status launch_tc(const mtf_plan_t& plan, const void* A, const void* B, void* C, const void* bias, int dtBias,
                      const void* mask, int dtMask, const void* resid, int dtRes, float scale, int relu, float* rsum,
                      void* workspace, size_t workspace_bytes, void* stream, int n_terms = 1,

@@ -287,6 +287,52 @@ static bool plan_tc(mtf_plan_t* P, std::string* why, int force_single_cta) {
   return true;
 }
 
+// The f32 matrix-product form of an einsum (see F32Params); false: the generic kernel runs it.
+static bool plan_f32(mtf_plan_t* P) {
+  if (!P->has_B || P->dtA != MTF_F32 || P->dtB != MTF_F32) return false;
+  std::vector<IterDim> it = P->iter;
+  for (auto& d : it) { d.nsplit = 1; d.mesh_dim = -1; }       // where a dimension is cut does not matter here
+  std::vector<int> cb, cm, cn, ck;
+  for (int i = 0; i < (int)it.size(); ++i) {
+    const IterDim& d = it[i];
+    if (d.inA && d.inB) (d.inC ? cb : ck).push_back(i);
+    else if (d.inC) (d.inA ? cm : cn).push_back(i);
+    else return false;
+  }
+  if (cm.empty() || cn.empty() || ck.empty() || (int)cb.size() > kMaxOuter) return false;
+  const Merged mm = merge_category(it, cm, true, false, true), mn = merge_category(it, cn, false, true, true), mk = merge_category(it, ck, true, true, false);
+  if (!mm.ok || !mn.ok || !mk.ok || (mn.sC != 1 && mm.sC != 1)) return false;
+  const bool swap = mn.sC != 1;
+  F32Params t;
+  t.swapped = swap ? 1 : 0;
+  t.M = swap ? mn.size : mm.size; t.N = swap ? mm.size : mn.size; t.K = mk.size;
+  if (t.M > 0x7fffffffLL || t.N > 0x7fffffffLL || t.K > 0x7fffffffLL) return false;
+  t.sAm = swap ? mn.sB : mm.sA; t.sAk = swap ? mk.sB : mk.sA;
+  t.sBn = swap ? mm.sA : mn.sB; t.sBk = swap ? mk.sA : mk.sB;
+  t.ldc = swap ? mn.sC : mm.sC;
+  t.n_outer = (int)cb.size();
+  for (int j = 0; j < t.n_outer; ++j) {
+    const IterDim& d = it[cb[j]];
+    t.outer_size[j] = d.size;
+    t.outer_sA[j] = swap ? d.sB : d.sA; t.outer_sB[j] = swap ? d.sA : d.sB; t.outer_sC[j] = d.sC;
+  }
+  // bias: exactly the kernel's N (or M) group; fused reduce_sum: exactly its N group - both in storage order
+  auto covers = [&](const std::vector<Dim>& dims, std::vector<int> grp) {
+    std::sort(grp.begin(), grp.end(), [&](int a, int b) { return it[a].sC > it[b].sC; });
+    bool same = dims.size() == grp.size();
+    for (size_t j = 0; same && j < grp.size(); ++j) same = dims[j].name == it[grp[j]].name;
+    return same;
+  };
+  const std::vector<int>&gm = swap ? cn : cm, &gn = swap ? cm : cn;
+  if (P->epi.has_bias) {
+    if (covers(P->epi.bias_dims, gm)) t.bias_along_m = 1;
+    else if (!covers(P->epi.bias_dims, gn)) return false;
+  }
+  if (P->epi.has_rsum && !covers(P->epi.rsum_dims, gn)) return false;
+  P->f32 = t;
+  return true;
+}
+
 mtf_status make_plan(const mtf_layout_t* L, int n_in, const mtf_tensor* in, const mtf_tensor* out,
                      const mtf_epilogue* epi, int force_kernel, int force_reduce, std::unique_ptr<mtf_plan_t>* result) {
   if (!L || !in || !out) return fail(MTF_ERR_INVALID_ARG, "einsum: NULL argument");
@@ -487,6 +533,7 @@ mtf_status make_plan(const mtf_layout_t* L, int n_in, const mtf_tensor* in, cons
   s.relu = P->epi.relu ? 1 : 0;
 
   // ---- kernel family and reduce mode ----
+  P->f32_ok = force_kernel != MTF_KERNEL_SIMT && plan_f32(P.get());      // (forcing the generic kernel means that kernel)
   std::string why;
   const int force_single_cta = force_kernel == 2 ? 1 : 0;     // testing hook: tensor cores without CTA pairs
   const int wide_pref = force_kernel == 3 ? 1 : (force_kernel == 4 ? 0 : -1);   // testing hook: wide pair tiles always / never
