@@ -25,6 +25,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <cstdio>
 #include <atomic>
 #include <mutex>
@@ -1480,6 +1481,8 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   }
 }
 
+#include "gemm_cluster.cuh"
+
 // ---- host side -----------------------------------------------------------------------------------------
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                                   const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -1740,6 +1743,128 @@ size_t tc_workspace_bytes(const TcParams& t) {
   return (size_t)tiles * t.sk * tc_tile_rows(t) * t.block_n * sizeof(float) + (size_t)tiles * (tc_tile_rows(t) / 32) * 4 * sizeof(unsigned) + 256;
 }
 
+// Which contractions run on 128-row tiles with K over a cluster, and how: the shorter of two estimates of a launch's time,
+// whose constants (microseconds) are fits to launches of 24 shapes from 128 x 1024 x 1024 to 4096 x 8192 x 1024 on each of
+// the eight variants and on gemm_tcgen05_kernel (B200, replayed back to back).  Both sides at some of them, us:
+//   128 x 1024 x 4096  35.6 there,  8.0 here (BN 64, split 8);    512 x 1024 x 1024  12.3 and 6.3 (64, 2);
+//   1024 x 1024 x 8192 60.8 and 23.6 (128, 4);   2048 x 1024 x 4096 30.8 and 19.9 (128, 2);
+//   24 x [200 x 64 x 200] 6.5 and 3.9 (64, 1);   8192 x 1024 x 1024 20.9 and 21.3 (128, 1);   4096 x 4096 x 1024 35.2 and 39.7.
+// There the persistent kernel pays a fixed part and a wave of tiles costs its k-blocks at the rate one SM takes operands in;
+// here a round of two CTAs an SM costs the same k-blocks (at half the reuse), the epilogue, and the exchange between the
+// CTAs of a cluster, which is what keeps the split small.
+static ClusterPick cluster_pick(const TcParams& t, int n_terms, int n_groups) {
+  ClusterPick best = {0, 0};
+  if (!t.cluster_ok) return best;
+  const double sms = sm_count();
+  const double kb = (double)((t.K + BK - 1) / BK) * n_terms;
+  double outer = n_groups;
+  for (int j = 0; j < t.n_outer; ++j) outer *= (double)t.outer_size[j];
+  const int64_t rows = t.cta_pair ? 2 * BM : BM;
+  const double tiles = (double)((t.M / t.sm + rows - 1) / rows * t.sm) * (double)((t.N / t.sn + t.block_n - 1) / t.block_n * t.sn) * outer;
+  const double per_kb = t.cta_pair ? (t.block_n == 256 ? 0.36 : 0.24) : (t.block_n == 256 ? 0.45 : t.block_n == 128 ? 0.33 : 0.27);
+  double best_us = 0.95 * (7.0 + std::ceil(tiles / std::floor(sms / (t.cta_pair ? 2 : 1))) * kb * per_kb);
+  for (int bn = 64; bn <= 128; bn += 64) {
+    const double ctas1 = (double)((t.M + BM - 1) / BM) * (double)((t.N + bn - 1) / bn) * outer;
+    for (int split = 1; split <= 8 && split <= kb; split *= 2) {
+      const double ctas = ctas1 * split, part = std::ceil(kb / split);
+      const bool two = ctas > sms;
+      const double exchange = split == 1 ? 0.0 : (split == 2 ? 1.2 : split == 4 ? 1.8 : 2.8) + (two ? 1.0 : 0.0);
+      const double per = bn == 64 ? (two ? 0.34 : 0.27) : (two ? 0.44 : 0.34);
+      const double us = 2.2 + std::ceil(ctas / (2.0 * sms)) * (part * per + (bn == 64 ? 0.8 : 1.8) + exchange);
+      if (us < best_us) { best_us = us; best = {bn, split}; }
+    }
+  }
+  return best;
+}
+
+template <int BN, int kSplit, bool kEpi>
+static mtf_status launch_cluster_variant(const CUtensorMap& map_a, const CUtensorMap& map_b, const ExtraMaps& extra, const ClusterArgs& a, long long ctas, cudaStream_t st) {
+  static std::once_flag once[kMaxDevices];           // the shared-memory opt-in is a property of a device
+  static cudaError_t attr[kMaxDevices];
+  const int dev = current_device();
+  std::call_once(once[dev], [dev] { attr[dev] = cudaFuncSetAttribute(gemm_cluster_kernel<BN, kSplit, kEpi>, cudaFuncAttributeMaxDynamicSharedMemorySize, kClSmemBytes); });
+  if (attr[dev] != cudaSuccess) return fail(MTF_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(attr[dev]));
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = kSplit; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)ctas, 1, 1); cfg.blockDim = dim3(kClThreads, 1, 1);
+  cfg.dynamicSmemBytes = kClSmemBytes; cfg.stream = st; cfg.attrs = at; cfg.numAttrs = 2;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_cluster_kernel<BN, kSplit, kEpi>, map_a, map_b, extra, a);
+  if (e != cudaSuccess) return fail(MTF_ERR_CUDA, "gemm_cluster_kernel: %s", cudaGetErrorString(e));
+  count_launch();
+  return MTF_OK;
+}
+
+// The arguments have passed launch_tc's checks; A and B are in the kernel's order (extra and group operands in the caller's).
+static mtf_status launch_cluster(const mtf_plan_t& plan, ClusterPick pick, const void* A, const void* B, void* C, const void* bias, int dtBias, const void* mask,
+                                 int dtMask, const void* resid, int dtRes, float scale, int relu, float* rsum, void* workspace, size_t workspace_bytes, void* stream,
+                                 int n_terms, const void* const* extra_operands, int n_groups, const void* const* group_operands) {
+  const TcParams& t = plan.tc;
+  cudaStream_t st = (cudaStream_t)stream;
+  ClusterArgs a;
+  a.M = (int)t.M; a.N = (int)t.N;
+  a.n_outer = t.n_outer;
+  long long outer = 1;
+  for (int j = 0; j < 3; ++j) { a.outer_size[j] = (int)t.outer_size[j]; a.outer_sC[j] = t.outer_sC[j]; if (j < t.n_outer) outer *= t.outer_size[j]; }
+  a.a_mn_major = t.a_mn_major; a.b_mn_major = t.b_mn_major; a.ldc = t.ldc;
+  a.m_tiles = (a.M + BM - 1) / BM; a.n_tiles = (a.N + pick.bn - 1) / pick.bn;
+  const long long row_blocks = outer * a.m_tiles, tiles = row_blocks * a.n_tiles, ctas = tiles * n_groups * pick.split;
+  if (ctas > 0x7fffffffLL) return fail(MTF_ERR_UNSUPPORTED, "more than 2^31 tiles");
+  a.tiles_group = (int)tiles;
+  a.kb_term = (int)((t.K + BK - 1) / BK); a.kb_total = a.kb_term * n_terms;
+  a.grouped = n_groups > 1;
+  a.C[0] = a.C[1] = a.C[2] = C;
+  a.c_bf16 = plan.dtC == MTF_BF16;
+  a.bias = bias; a.bias_bf16 = dtBias == MTF_BF16; a.bias_along_m = t.bias_along_m;
+  a.mask = mask; a.mask_bf16 = dtMask == MTF_BF16;
+  a.resid = resid; a.resid_bf16 = dtRes == MTF_BF16;
+  a.scale = scale; a.relu = relu;
+  a.rsum = rsum; a.rsum_store = 0; a.rsum_partial = nullptr;
+  a.late_wait = (take_independent_hint() && !rsum) ? 1 : 0;
+  (void)sched_for_launch(st, false, &a.late_wait);                   // (counts consecutive late launches of the stream)
+  const long long groups = row_blocks * pick.split;
+  if (rsum) {
+    if (groups == 1) a.rsum_store = 1;
+    else if (workspace && !(reinterpret_cast<uintptr_t>(workspace) & 15) && workspace_bytes >= (size_t)groups * t.N * sizeof(float)) a.rsum_partial = reinterpret_cast<float*>(workspace);
+    else {
+      mtf_status zs = zero_words(rsum, t.N, st);
+      if (zs != MTF_OK) return zs;
+    }
+  }
+  CUtensorMap map_a, map_b;
+  ExtraMaps extra;
+  auto maps = [&](const void* Ap, const void* Bp, CUtensorMap* ma, CUtensorMap* mb) {
+    mtf_status s = t.a_mn_major ? make_map(ma, Ap, 2, t.M, t.K, t.a_ld, 64, BK, t, t.outer_sA) : make_map(ma, Ap, 2, t.K, t.M, t.a_ld, 64, BM, t, t.outer_sA);
+    if (s != MTF_OK) return s;
+    return t.b_mn_major ? make_map(mb, Bp, 2, t.N, t.K, t.b_ld, 64, BK, t, t.outer_sB) : make_map(mb, Bp, 2, t.K, t.N, t.b_ld, 64, pick.bn, t, t.outer_sB);
+  };
+  mtf_status s = maps(A, B, &map_a, &map_b);
+  if (s != MTF_OK) return s;
+  for (int i = 0; i < 4; ++i) extra.m[i] = i % 2 == 0 ? map_a : map_b;
+  extra.c[0] = extra.c[1] = map_a;
+  for (int i = 1; i < std::max(n_terms, n_groups); ++i) {
+    const void* Ai = n_terms > 1 ? extra_operands[2 * (i - 1)] : group_operands[3 * (i - 1)];
+    const void* Bi = n_terms > 1 ? extra_operands[2 * (i - 1) + 1] : group_operands[3 * (i - 1) + 1];
+    if (t.swapped) std::swap(Ai, Bi);
+    if (!Ai || !Bi) return fail(MTF_ERR_INVALID_ARG, "contraction: NULL operand");
+    if ((s = maps(Ai, Bi, &extra.m[2 * (i - 1)], &extra.m[2 * (i - 1) + 1])) != MTF_OK) return s;
+    if (n_groups > 1) {
+      a.C[i] = const_cast<void*>(group_operands[3 * (i - 1) + 2]);
+      if (!a.C[i] || (reinterpret_cast<uintptr_t>(a.C[i]) & 15)) return fail(MTF_ERR_INVALID_ARG, "grouped launch: NULL or misaligned output");
+    }
+  }
+  const bool stages = bias || relu || mask || resid || rsum;
+#define MTF_CL(BN, S) (stages ? launch_cluster_variant<BN, S, true>(map_a, map_b, extra, a, ctas, st) : launch_cluster_variant<BN, S, false>(map_a, map_b, extra, a, ctas, st))
+  if (pick.bn == 64) s = pick.split == 8 ? MTF_CL(64, 8) : pick.split == 4 ? MTF_CL(64, 4) : pick.split == 2 ? MTF_CL(64, 2) : MTF_CL(64, 1);
+  else s = pick.split == 8 ? MTF_CL(128, 8) : pick.split == 4 ? MTF_CL(128, 4) : pick.split == 2 ? MTF_CL(128, 2) : MTF_CL(128, 1);
+#undef MTF_CL
+  if (s != MTF_OK || !a.rsum_partial) return s;
+  return launch_colsum_finalize(a.rsum_partial, (int)groups, 1, (int)t.N, rsum, nullptr, stream);
+}
+
 mtf_status launch_tc(const mtf_plan_t& plan, const void* A, const void* B, void* C, const void* bias, int dtBias,
                      const void* mask, int dtMask, const void* resid, int dtRes, float scale, int relu, float* rsum,
                      void* workspace, size_t workspace_bytes, void* stream, int n_terms, const void* const* extra_operands,
@@ -1755,6 +1880,17 @@ mtf_status launch_tc(const mtf_plan_t& plan, const void* A, const void* B, void*
   if (bias && !t.bias_along_m && (reinterpret_cast<uintptr_t>(bias) & 15)) return fail(MTF_ERR_INVALID_ARG, "tensor-core path needs a 16-byte aligned bias");
   if ((mask && (reinterpret_cast<uintptr_t>(mask) & 15)) || (resid && (reinterpret_cast<uintptr_t>(resid) & 15)))
     return fail(MTF_ERR_INVALID_ARG, "tensor-core path needs 16-byte aligned epilogue operands");
+  if (t.reduce_mode == MTF_REDUCE_WORKSPACE && n_groups == 1) {
+    const size_t need = tc_workspace_bytes(t);
+    if (!workspace || workspace_bytes < need) return fail(MTF_ERR_WORKSPACE_TOO_SMALL, "einsum needs %zu workspace bytes, got %zu", need, workspace_bytes);
+    if (reinterpret_cast<uintptr_t>(workspace) & 255) return fail(MTF_ERR_INVALID_ARG, "workspace must be 256-byte aligned");
+  }
+  if (!row_softmax) {
+    const ClusterPick pick = cluster_pick(t, n_terms, n_groups);
+    if (pick.split)
+      return launch_cluster(plan, pick, A, B, C, bias, dtBias, mask, dtMask, resid, dtRes, scale, relu, rsum, workspace, workspace_bytes, stream, n_terms,
+                            extra_operands, n_groups, group_operands);
+  }
 
   TcArgs a;
   a.M = (int)t.M; a.N = (int)t.N; a.K = (int)t.K;
@@ -1898,9 +2034,6 @@ mtf_status launch_tc(const mtf_plan_t& plan, const void* A, const void* B, void*
     }
   }
   if (a.reduce_mode == MTF_REDUCE_WORKSPACE) {
-    const size_t need = tc_workspace_bytes(t);
-    if (!workspace || workspace_bytes < need) return fail(MTF_ERR_WORKSPACE_TOO_SMALL, "einsum needs %zu workspace bytes, got %zu", need, workspace_bytes);
-    if (reinterpret_cast<uintptr_t>(workspace) & 255) return fail(MTF_ERR_INVALID_ARG, "workspace must be 256-byte aligned");
     const size_t part_bytes = (size_t)a.total_tiles * a.sk * tile_rows * a.block_n * sizeof(float);
     a.ws_partials = reinterpret_cast<float*>(workspace);
     a.ws_counters = reinterpret_cast<unsigned*>(reinterpret_cast<uint8_t*>(workspace) + ((part_bytes + 255) / 256) * 256);

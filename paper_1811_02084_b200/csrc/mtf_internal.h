@@ -93,6 +93,7 @@ struct TcParams {
   int wide_pref = -1;                        // 256 x 512 pair tiles: -1 = launcher's wave heuristic, 0 = never, 1 = wherever the shape allows
   int balance = 0;                           // tiles leave a partly filled last wave: balanced k-range schedule (needs workspace)
   int cta_pair = 0;                          // two CTAs (a cluster) own a 256-row tile, tcgen05 cta_group::2
+  int cluster_ok = 0;                        // no kernel or reduce mode was asked for: the launcher may take 128-row tiles with K over a cluster
   int swapped = 0;                           // in[0] and in[1] exchanged so that N is contiguous in C
   int reduce_mode = MTF_REDUCE_NONE;
   int bias_along_m = 0;                      // bias varies with m (after a swap) instead of n

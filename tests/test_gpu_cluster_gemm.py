@@ -1,0 +1,72 @@
+"""bf16 contractions on 128-row tiles with K over a cluster, against the fp64 oracle: every operand order, edges of the
+tiles, every split (few tiles and a longer and longer K), both tile widths, the fused stages and column sums."""
+import numpy as np
+import pytest
+
+import seeded_inputs as si
+from helpers import TOL, from_torch, parity_error, to_torch
+from test_gpu_einsum import layout, mtf, run_einsum  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+ONE = ([("all", 1)], [])
+
+
+@pytest.mark.parametrize("m,n,k", [(8, 8, 8), (128, 64, 64), (136, 72, 640), (40, 200, 1024), (264, 56, 1096), (24, 72, 4096)])
+@pytest.mark.parametrize("order", ["ik,kj", "ik,jk", "ki,kj", "ki,jk"])
+def test_orders_edges_and_splits(mtf, order, m, n, k):
+    size = {"i": m, "j": n, "k": k}
+    a, b = [[(c, size[c]) for c in t] for t in order.split(",")]
+    for out, dt in ((["i", "j"], "bf16"), (["i", "j"], "f32"), (["j", "i"], "bf16")):
+        got, ref, info = run_einsum(mtf, layout(mtf, *ONE), [a, b], [(c, size[c]) for c in out], "bf16", dt)
+        assert info["kernel_kind"] == mtf.MTF_KERNEL_TCGEN05
+        assert parity_error(got, ref) <= TOL["bf16"]
+
+
+def test_wider_tiles(mtf):
+    a, b = [("b", 200), ("i", 41), ("k", 72)], [("b", 200), ("k", 72), ("j", 136)]
+    got, ref, _ = run_einsum(mtf, layout(mtf, *ONE), [a, b], [("b", 200), ("i", 41), ("j", 136)], "bf16")
+    assert parity_error(got, ref) <= TOL["bf16"]
+    a, b = [("k", 4096), ("i", 1000)], [("k", 4096), ("j", 1032)]
+    got, ref, _ = run_einsum(mtf, layout(mtf, *ONE), [a, b], [("i", 1000), ("j", 1032)], "bf16", "f32")
+    assert parity_error(got, ref) <= TOL["bf16"]
+
+
+@pytest.mark.parametrize("mesh,rules", [ONE, ([("r", 5), ("c", 4)], [("b", "r"), ("k", "c")])], ids=["whole", "split"])
+def test_batch_dims_and_slices(mtf, mesh, rules):
+    a, b = [("b", 5), ("l", 37), ("h", 3), ("k", 64)], [("b", 5), ("m", 40), ("h", 3), ("k", 64)]
+    got, ref, _ = run_einsum(mtf, layout(mtf, mesh, rules), [a, b], [("b", 5), ("h", 3), ("l", 37), ("m", 40)], "bf16", "f32")
+    assert parity_error(got, ref) <= TOL["bf16"]
+    a, b = [("b", 5), ("l", 37), ("k", 256)], [("k", 256), ("j", 104)]
+    got, ref, _ = run_einsum(mtf, layout(mtf, mesh, rules), [a, b], [("b", 5), ("l", 37), ("j", 104)], "bf16")
+    assert parity_error(got, ref) <= TOL["bf16"]
+
+
+@pytest.mark.parametrize("m,n,k", [(136, 72, 64), (100, 136, 640), (264, 64, 1024), (24, 72, 4096)])
+@pytest.mark.parametrize("out_dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("out", [["i", "j"], ["j", "i"]], ids=["in-order", "exchanged"])
+def test_stages(mtf, out, out_dtype, m, n, k):
+    size = {"i": m, "j": n, "k": k}
+    if out[1] == "i":
+        size["i"] = (m + 7) // 8 * 8                  # (the contiguous output dimension holds whole store pieces)
+    dims = [[(c, size[c]) for c in t] for t in ("ik", "kj")]
+    for bias in ("i", "j"):
+        ep = {"scale": -0.5, "bias": [(bias, size[bias])], "relu": True, "relu_mask": True, "residual": True}
+        got, ref, _ = run_einsum(mtf, layout(mtf, *ONE), dims, [(c, size[c]) for c in out], "bf16", out_dtype, epilogue=ep)
+        assert parity_error(got, ref) <= TOL["bf16"]
+
+
+@pytest.mark.parametrize("m,n,k", [(8, 72, 64), (300, 136, 640), (136, 64, 4096)])
+@pytest.mark.parametrize("scratch", [0, 1 << 22])
+def test_column_sums(mtf, scratch, m, n, k):
+    import torch
+    x, y = si.normal(3, "x", [m, k], "bf16"), si.normal(3, "y", [k, n], "bf16", k ** -0.5)
+    mask = si.normal(3, "mask", [m, n], "bf16")
+    out, col = torch.full((m, n), float("nan"), dtype=torch.bfloat16, device="cuda"), torch.full((n,), float("nan"), device="cuda")
+    ep = mtf.Epilogue(relu_mask=mtf.named(to_torch(mask), ["i", "j"]), reduce_sum_out=mtf.named(col, ["j"]))
+    ws = torch.empty(scratch, dtype=torch.uint8, device="cuda") if scratch else None
+    mtf.mtf_einsum(layout(mtf, *ONE), None, [mtf.named(to_torch(x), ["i", "k"]), mtf.named(to_torch(y), ["k", "j"])], mtf.named(out, ["i", "j"]), ep, ws)
+    mtf.mtf_device_status()
+    ref = (x.f64 @ y.f64) * (mask.f64 > 0)
+    assert parity_error(from_torch(out), ref) <= TOL["bf16"]
+    assert parity_error(from_torch(col), ref.sum(0)) <= TOL["f32"]
