@@ -1752,9 +1752,13 @@ size_t tc_workspace_bytes(const TcParams& t) {
 // There the persistent kernel pays a fixed part and a wave of tiles costs its k-blocks at the rate one SM takes operands in;
 // here a round of two CTAs an SM costs the same k-blocks (at half the reuse), the epilogue, and the exchange between the
 // CTAs of a cluster, which is what keeps the split small.
+static thread_local bool g_whole_sums = false;
+bool swap_whole_sums(bool on) { const bool was = g_whole_sums; g_whole_sums = on; return was; }
+
 static ClusterPick cluster_pick(const TcParams& t, int n_terms, int n_groups) {
   ClusterPick best = {0, 0};
-  if (!t.cluster_ok) return best;
+  if (!t.cluster_ok || (g_whole_sums && t.reduce_mode == MTF_REDUCE_WORKSPACE)) return best;
+  const int most = g_whole_sums ? 1 : 8;
   const double sms = sm_count();
   const double kb = (double)((t.K + BK - 1) / BK) * n_terms;
   double outer = n_groups;
@@ -1765,7 +1769,7 @@ static ClusterPick cluster_pick(const TcParams& t, int n_terms, int n_groups) {
   double best_us = 0.95 * (7.0 + std::ceil(tiles / std::floor(sms / (t.cta_pair ? 2 : 1))) * kb * per_kb);
   for (int bn = 64; bn <= 128; bn += 64) {
     const double ctas1 = (double)((t.M + BM - 1) / BM) * (double)((t.N + bn - 1) / bn) * outer;
-    for (int split = 1; split <= 8 && split <= kb; split *= 2) {
+    for (int split = 1; split <= most && split <= kb; split *= 2) {
       const double ctas = ctas1 * split, part = std::ceil(kb / split);
       const bool two = ctas > sms;
       const double exchange = split == 1 ? 0.0 : (split == 2 ? 1.2 : split == 4 ? 1.8 : 2.8) + (two ? 1.0 : 0.0);

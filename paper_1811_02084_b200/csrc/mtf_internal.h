@@ -208,6 +208,9 @@ void hint_next_launch_independent();
 // Sets the reduce mode that plans made on this thread are forced to (-1: the planner's choice); returns the old one.
 int swap_force_reduce(int mode);
 bool take_independent_hint();
+// While on (this thread): contractions of few tiles add up K in one accumulator as large ones do, so that a value does not
+// depend on how many rows stand beside it.  Returns the old state.
+bool swap_whole_sums(bool on);
 // n_groups (1..3) independent einsums with the dims of group 0 (names may differ, sizes and types may
 // not) in one launch, so that contractions with few output tiles fill the GPU together.
 // MTF_ERR_UNSUPPORTED when the plan cannot (generic kernel): the caller then runs them one by one.
