@@ -20,6 +20,7 @@ mtf_status debug_wait_test(long long limit_cycles, int skip_first_commit);
 mtf_status read_attention_status(int* code);
 mtf_status launch_permute_copy(const void* src, void* dst, int elem_bytes, int ndim, const int64_t* sizes, const int64_t* sstr, const int64_t* dstr, void* stream);
 mtf_status read_attention_bwd_status(int* code);
+mtf_status read_attention_rows_status(int* code);
 }  // namespace mtf
 
 using mtf::Dim;
@@ -523,6 +524,7 @@ mtf_status mtf::einsum_terms(const mtf_layout_t* layout, int n_terms, const mtf_
 
 void mtf::hint_next_launch_independent() { g_next_independent = true; }
 int mtf::swap_force_reduce(int mode) { const int was = g_force_reduce; g_force_reduce = mode; return was; }
+bool mtf::plan_forced() { return g_force_kernel >= 0 || g_force_reduce >= 0; }
 bool mtf::take_independent_hint() {
   const bool v = g_next_independent;
   g_next_independent = false;
@@ -549,6 +551,22 @@ mtf_status mtf::einsum_group(const mtf_layout_t* layout, int n_groups, const mtf
     }
   }
   return exec_plan(P, ins[0], outs[0], nullptr, workspace, workspace_bytes, stream, 1, nullptr, 0, n_groups, ops);
+}
+
+mtf_status mtf::attention_kv(const mtf_layout_t* layout, const mtf_tensor* ds, const mtf_tensor* q, mtf_tensor* dkk, float scale, const mtf_tensor* weights,
+                             const mtf_tensor* dout, mtf_tensor* dvv, int causal, void* stream) {
+  const mtf_tensor in[2] = {*ds, *q};
+  const mtf_plan_t* P = nullptr;
+  mtf_status st = cached_plan(layout, 2, in, dkk, nullptr, &P);
+  if (st != MTF_OK) return st;
+  if (P->kernel_kind != MTF_KERNEL_TCGEN05 || P->rank_sum) return fail(MTF_ERR_UNSUPPORTED, "attention key / value gradients: not on this plan");
+  const mtf_tensor* const pairs[3][2] = {{ds, weights}, {q, dout}, {dkk, dvv}};
+  for (auto& p : pairs) {
+    bool same = p[0]->ndim == p[1]->ndim && p[0]->dtype == MTF_BF16 && p[1]->dtype == MTF_BF16;
+    for (int i = 0; same && i < p[0]->ndim; ++i) same = p[0]->dims[i].size == p[1]->dims[i].size;
+    if (!same) return fail(MTF_ERR_UNSUPPORTED, "attention key / value gradients: the two sums differ in shape or type");
+  }
+  return mtf::launch_attention_kv(*P, ds->data, q->data, dkk->data, scale, weights->data, dout->data, dvv->data, causal, stream);
 }
 
 mtf_status mtf::einsum_row_softmax(const mtf_layout_t* layout, const mtf_tensor* a, const mtf_tensor* b, mtf_tensor* weights, float scale,
@@ -668,6 +686,7 @@ mtf_status mtf_device_status(int32_t* code) {
   int rc = 0;
   if ((st = mtf::read_attention_status(&rc)) != MTF_OK) return st;
   if (!rc && (st = mtf::read_attention_bwd_status(&rc)) != MTF_OK) return st;
+  if (!rc && (st = mtf::read_attention_rows_status(&rc)) != MTF_OK) return st;
   if (!rc && (st = mtf::read_row_status(&rc)) != MTF_OK) return st;
   if (rc) {
     if (code) *code = rc;

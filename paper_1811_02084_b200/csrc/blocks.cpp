@@ -22,6 +22,9 @@ bool attention_fused_supported(int64_t L, int64_t d_k, int64_t d_v);
 bool attention_bwd_fused_supported(int64_t L, int64_t d_k, int64_t d_v);
 mtf_status launch_attention_bwd_fused(const void* q, const void* kk, const void* vv, const void* weights, const void* dout, void* dq, void* dkk, void* dvv,
                                       void* dlogits_dump, int64_t B, int64_t H, int64_t L, float scale, int causal, void* stream);
+bool attention_rows_supported(int64_t B, int64_t H, int64_t L, int64_t d_k, int64_t d_v);
+mtf_status launch_attention_rows(bool backward, const void* own, const void* kk, const void* vv, const void* weights, void* ds, void* out, int64_t B, int64_t H,
+                                 int64_t L, int64_t D, float scale, int causal, int zeros, void* stream);
 bool tap_is_open();
 mtf_status launch_attention_fwd_fused(const void* q, const void* kk, const void* vv, void* weights, void* o, int64_t B, int64_t H, int64_t L, float scale,
                                       int causal, void* stream);
@@ -130,6 +133,12 @@ mtf_status attention_shapes(const mtf_tensor* x, const mtf_tensor* wq, const mtf
     return fail(MTF_ERR_SIZE_MISMATCH, "attention: projection shapes do not fit x / each other");
   s->scale = 1.0 / std::sqrt((double)s->k.size);
   return MTF_OK;
+}
+
+// The core by rows (attention_rows.cu), for shapes the one-pair-per-CTA cores do not take.  Its key / value half needs the
+// tensor-core plan that nothing was forced on.
+bool rows_core_wanted(const AttShapes& s) {
+  return !mtf::plan_forced() && mtf::attention_rows_supported(s.b.size, s.h.size, s.l.size, s.k.size, s.v.size);
 }
 
 mtf_epilogue epi_none() {
@@ -303,10 +312,13 @@ mtf_status mtf_attention_forward(const mtf_layout_t* layout, const mtf_tensor* x
     const bool canonical = order(q, {s.b, s.l, s.h, s.k}) && order(kk, {s.b, s.m, s.h, s.k}) && order(vv, {s.b, s.m, s.h, s.v}) &&
                            order(weights, {s.b, s.h, s.l, s.m}) && order(o, {s.b, s.l, s.h, s.v});
     // (legality and divisibility of the batch and heads splits were checked by the projections' plans above)
-    if (canonical && mtf::attention_fused_supported(s.l.size, s.k.size, s.v.size) && unsplit(s.l) && unsplit(s.m) && unsplit(s.k) && unsplit(s.v)) {
-      if ((st = mtf::launch_attention_fwd_fused(q->data, kk->data, vv->data, weights->data, o->data, s.b.size, s.h.size, s.l.size, (float)s.scale, causal ? 1 : 0,
-                                                stream)) != MTF_OK)
-        return st;
+    const bool whole = canonical && unsplit(s.l) && unsplit(s.m) && unsplit(s.k) && unsplit(s.v);
+    const bool core = whole && mtf::attention_fused_supported(s.l.size, s.k.size, s.v.size);
+    if (core || (whole && rows_core_wanted(s))) {
+      st = core ? mtf::launch_attention_fwd_fused(q->data, kk->data, vv->data, weights->data, o->data, s.b.size, s.h.size, s.l.size, (float)s.scale, causal ? 1 : 0, stream)
+                : mtf::launch_attention_rows(false, q->data, kk->data, vv->data, weights->data, nullptr, o->data, s.b.size, s.h.size, s.l.size, s.k.size, (float)s.scale,
+                                             causal ? 1 : 0, 1, stream);
+      if (st != MTF_OK) return st;
       mtf_epilogue er2 = epi_none();
       er2.residual = residual;
       if ((st = ein(layout, *o, *wo, y, residual ? &er2 : nullptr, rest, rest_bytes, stream)) != MTF_OK) return st;
@@ -358,7 +370,7 @@ mtf_status mtf_attention_backward(const mtf_layout_t* layout, const mtf_tensor* 
   // The whole core - dP, the softmax backward, dvv, dq, dkk - in one launch under the conditions of the forward core
   // (d_k = d_v = 64, rows of at most 512, only batch and heads split, canonical dimension orders): the weights are read
   // once and the gradient of the logits never leaves the chip.
-  bool core_ok = false;
+  bool core_ok = false, rows_ok = false;
   {
     auto unsplit = [&](const mtf_dim& d) { const int j = layout->mesh_dim_of(d.name); return j < 0 || layout->mesh[j].size == 1; };
     auto order = [](const mtf_tensor* t, std::initializer_list<mtf_dim> want) {
@@ -369,7 +381,9 @@ mtf_status mtf_attention_backward(const mtf_layout_t* layout, const mtf_tensor* 
     };
     const bool canonical = order(q, {s.b, s.l, s.h, s.k}) && order(kk, {s.b, s.m, s.h, s.k}) && order(vv, {s.b, s.m, s.h, s.v}) &&
                            order(weights, {s.b, s.h, s.l, s.m}) && order(o, {s.b, s.l, s.h, s.v});
-    core_ok = canonical && mtf::attention_bwd_fused_supported(s.l.size, s.k.size, s.v.size) && unsplit(s.l) && unsplit(s.m) && unsplit(s.k) && unsplit(s.v);
+    const bool whole = canonical && unsplit(s.l) && unsplit(s.m) && unsplit(s.k) && unsplit(s.v);
+    core_ok = whole && mtf::attention_bwd_fused_supported(s.l.size, s.k.size, s.v.size);
+    rows_ok = whole && !core_ok && rows_core_wanted(s);
   }
   // dWo reads o and dy and nothing the core touches.  Behind the one-launch core it is issued as an independent launch
   // with the group sum chained in its accumulators (no cleared counters in front of it), so its tiles start on the SMs
@@ -396,6 +410,16 @@ mtf_status mtf_attention_backward(const mtf_layout_t* layout, const mtf_tensor* 
         if (st != MTF_OK) return st;
       }
     }
+  }
+  if (rows_ok) {
+    // by rows of queries: dq and the gradient of the logits (written once, as the contractions over queries consume it), then
+    // dkk and dvv in one grouped launch; the blocks right of the diagonal are neither written nor read (nor, with the stage tap
+    // closed, are their zeros)
+    st = mtf::launch_attention_rows(true, dob.t.data, kk->data, vv->data, weights->data, dlg.t.data, dq.t.data, s.b.size, s.h.size, s.l.size, s.k.size, (float)s.scale,
+                                    causal ? 1 : 0, mtf::tap_is_open() ? 1 : 0, stream);
+    if (st != MTF_OK || (st = mtf::tap("dlogits", dlg.t, stream)) != MTF_OK) return st;
+    if ((st = mtf::attention_kv(layout, &dlg.t, q, &dkk.t, (float)s.scale, weights, &dob.t, &dvv.t, causal ? 1 : 0, stream)) != MTF_OK) return st;
+    core_done = true;
   }
   if (!core_done) {
   // dP and the softmax backward in one launch where a row fits a tile (dP then stays in tensor

@@ -34,8 +34,9 @@ struct ClusterArgs {
   int mask_bf16;
   const void* resid;
   int resid_bf16;
-  float scale;
+  float scale[3];            // per problem of a grouped launch
   int relu;
+  int k_from_row;            // the terms with k below the tile's first row are zero and are left out (one batch dimension's causal sums)
   float* rsum;               // column sums: one row group in all -> stored, else added to the zeroed output
   int rsum_store;
   float* rsum_partial;       // not NULL: [row group][N], finished in order by a launch behind this one
@@ -74,9 +75,9 @@ __device__ __forceinline__ uint32_t tile_at(int row, int piece) {
 
 // The component-wise stages on eight consecutive columns of one row, and the store.
 template <bool kEpi>
-__device__ __forceinline__ void finish_eight(const ClusterArgs& a, void* C, float* v, long long off, int m, bool second, const float* bias8, float* cs) {
+__device__ __forceinline__ void finish_eight(const ClusterArgs& a, void* C, float scale, float* v, long long off, int m, bool second, const float* bias8, float* cs) {
 #pragma unroll
-  for (int j = 0; j < 8; ++j) v[j] *= a.scale;
+  for (int j = 0; j < 8; ++j) v[j] *= scale;
   if (kEpi) {
     if (a.bias) {
       if (a.bias_along_m) {
@@ -150,7 +151,8 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     row_block = t * a.m_tiles + mt;
   }
   const int m0 = mt * BM, n0 = nt * BN;
-  const int kb0 = (int)((long long)a.kb_total * part / kSplit), kb1 = (int)((long long)a.kb_total * (part + 1) / kSplit);
+  const int kb_first = a.k_from_row ? min(m0 / BK, a.kb_total - 1) : 0, kb_count = a.kb_total - kb_first;
+  const int kb0 = kb_first + (int)((long long)kb_count * part / kSplit), kb1 = kb_first + (int)((long long)kb_count * (part + 1) / kSplit);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
@@ -232,6 +234,10 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       uint32_t v[32];
       tmem_ld32(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)col, v);
       tmem_ld_wait();
+      if (kb0 == kb1) {              // (k_from_row: the last rows' few k-blocks may not reach every part)
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] = 0u;
+      }
 #pragma unroll
       for (int j = 0; j < 8; ++j) st_shared_v4(ring + tile_at<BN>(row, col / 4 + j), v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
     }
@@ -248,6 +254,7 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   const int row0 = part * (BM / kSplit) + warp * kRowsWarp + lane / kLanesRow;
   const bool on = lane_on && n < a.N, second = n + 4 < a.N;
   void* const C = a.C[group];
+  const float scale = a.scale[group];
   float bias8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, cs[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   if (kEpi && a.bias && !a.bias_along_m && on) {
     const float4 x = ld_quad(a.bias, a.bias_bf16, n), y = second ? ld_quad(a.bias, a.bias_bf16, n + 4) : x;
@@ -276,7 +283,7 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < kPasses; ++i, off += kRowsPass * a.ldc)
-      if (on && m0 + row0 + i * kRowsPass < a.M) finish_eight<kEpi>(a, C, s[i], off, m0 + row0 + i * kRowsPass, second, bias8, cs);
+      if (on && m0 + row0 + i * kRowsPass < a.M) finish_eight<kEpi>(a, C, scale, s[i], off, m0 + row0 + i * kRowsPass, second, bias8, cs);
   } else {
 #pragma unroll 2
     for (int i = 0; i < kPasses; ++i, off += kRowsPass * a.ldc) {
@@ -285,7 +292,7 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       const uint4 x = ld_shared_v4(ring + tile_at<BN>(r, piece)), y = ld_shared_v4(ring + tile_at<BN>(r, piece + 1));
       float v[8] = {__uint_as_float(x.x), __uint_as_float(x.y), __uint_as_float(x.z), __uint_as_float(x.w),
                     __uint_as_float(y.x), __uint_as_float(y.y), __uint_as_float(y.z), __uint_as_float(y.w)};
-      finish_eight<kEpi>(a, C, v, off, m0 + r, second, bias8, cs);
+      finish_eight<kEpi>(a, C, scale, v, off, m0 + r, second, bias8, cs);
     }
   }
   if (kEpi && a.rsum) {              // fused reduce_sum over this CTA's rows, in a fixed order

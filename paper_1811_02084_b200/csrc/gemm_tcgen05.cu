@@ -1805,7 +1805,8 @@ static mtf_status launch_cluster_variant(const CUtensorMap& map_a, const CUtenso
 // The arguments have passed launch_tc's checks; A and B are in the kernel's order (extra and group operands in the caller's).
 static mtf_status launch_cluster(const mtf_plan_t& plan, ClusterPick pick, const void* A, const void* B, void* C, const void* bias, int dtBias, const void* mask,
                                  int dtMask, const void* resid, int dtRes, float scale, int relu, float* rsum, void* workspace, size_t workspace_bytes, void* stream,
-                                 int n_terms, const void* const* extra_operands, int n_groups, const void* const* group_operands) {
+                                 int n_terms, const void* const* extra_operands, int n_groups, const void* const* group_operands, int k_from_row = 0,
+                                 const float* group_scale = nullptr) {
   const TcParams& t = plan.tc;
   cudaStream_t st = (cudaStream_t)stream;
   ClusterArgs a;
@@ -1825,7 +1826,8 @@ static mtf_status launch_cluster(const mtf_plan_t& plan, ClusterPick pick, const
   a.bias = bias; a.bias_bf16 = dtBias == MTF_BF16; a.bias_along_m = t.bias_along_m;
   a.mask = mask; a.mask_bf16 = dtMask == MTF_BF16;
   a.resid = resid; a.resid_bf16 = dtRes == MTF_BF16;
-  a.scale = scale; a.relu = relu;
+  for (int g = 0; g < 3; ++g) a.scale[g] = group_scale && g < n_groups ? group_scale[g] : scale;
+  a.relu = relu; a.k_from_row = k_from_row;
   a.rsum = rsum; a.rsum_store = 0; a.rsum_partial = nullptr;
   a.late_wait = (take_independent_hint() && !rsum) ? 1 : 0;
   (void)sched_for_launch(st, false, &a.late_wait);                   // (counts consecutive late launches of the stream)
@@ -1867,6 +1869,26 @@ static mtf_status launch_cluster(const mtf_plan_t& plan, ClusterPick pick, const
 #undef MTF_CL
   if (s != MTF_OK || !a.rsum_partial) return s;
   return launch_colsum_finalize(a.rsum_partial, (int)groups, 1, (int)t.N, rsum, nullptr, stream);
+}
+
+// Two independent sums over queries of one shape, each with a scale of its own: dkk = s dS^T q and dvv = P^T do (the plan is
+// dkk's).  causal: both left operands are zero where the query comes before the key, so those k-blocks are left out.
+mtf_status launch_attention_kv(const mtf_plan_t& plan, const void* ds, const void* q, void* dkk, float scale, const void* weights, const void* dout, void* dvv,
+                               int causal, void* stream) {
+  const TcParams& t = plan.tc;
+  if (!t.cluster_ok || t.swapped || t.K != t.M) return fail(MTF_ERR_UNSUPPORTED, "attention key / value gradients: not on this plan");
+  for (const void* p : {ds, q, (const void*)dkk, weights, dout, (const void*)dvv})
+    if (!p || (reinterpret_cast<uintptr_t>(p) & 15)) return fail(MTF_ERR_INVALID_ARG, "attention key / value gradients: NULL or misaligned tensor");
+  // one 128-key tile per CTA over all its queries; split where that leaves half of the chip's slots empty
+  const int bn = t.N > 64 ? 128 : 64;
+  double ctas = 2.0 * (double)((t.M + BM - 1) / BM) * (double)((t.N + bn - 1) / bn);
+  for (int j = 0; j < t.n_outer; ++j) ctas *= (double)t.outer_size[j];
+  int split = 1;
+  while (split < 4 && ctas * split <= sm_count() && (t.K + BK - 1) / BK >= 8 * split) split *= 2;
+  const void* const group[3] = {weights, dout, dvv};
+  const float scales[2] = {scale, 1.f};
+  (void)take_independent_hint();
+  return launch_cluster(plan, {bn, split}, ds, q, dkk, nullptr, 0, nullptr, 0, nullptr, 0, 1.f, 0, nullptr, nullptr, 0, stream, 1, nullptr, 2, group, causal ? 1 : 0, scales);
 }
 
 mtf_status launch_tc(const mtf_plan_t& plan, const void* A, const void* B, void* C, const void* bias, int dtBias,

@@ -211,6 +211,8 @@ bool take_independent_hint();
 // While on (this thread): contractions of few tiles add up K in one accumulator as large ones do, so that a value does not
 // depend on how many rows stand beside it.  Returns the old state.
 bool swap_whole_sums(bool on);
+// Is a kernel family or reduce mode forced on this thread (mtf_plan_force)?
+bool plan_forced();
 // n_groups (1..3) independent einsums with the dims of group 0 (names may differ, sizes and types may
 // not) in one launch, so that contractions with few output tiles fill the GPU together.
 // MTF_ERR_UNSUPPORTED when the plan cannot (generic kernel): the caller then runs them one by one.
@@ -237,6 +239,12 @@ mtf_status einsum_row_softmax(const mtf_layout_t* layout, const mtf_tensor* a, c
 // (generic kernel, workspace reduce mode): the caller then chains einsums through the residual stage.
 mtf_status einsum_terms(const mtf_layout_t* layout, int n_terms, const mtf_tensor (*terms)[2], mtf_tensor* out,
                         const mtf_epilogue* epilogue, void* workspace, size_t workspace_bytes, void* stream);
+// dkk = scale * sum_l ds q and dvv = sum_l weights do in one launch (grouped, causal blocks left out).
+// MTF_ERR_UNSUPPORTED when the plan cannot (generic kernel, a kernel or reduce mode was asked for): the caller runs two einsums.
+mtf_status attention_kv(const mtf_layout_t* layout, const mtf_tensor* ds, const mtf_tensor* q, mtf_tensor* dkk, float scale, const mtf_tensor* weights,
+                        const mtf_tensor* dout, mtf_tensor* dvv, int causal, void* stream);
+mtf_status launch_attention_kv(const mtf_plan_t& plan, const void* ds, const void* q, void* dkk, float scale, const void* weights, const void* dout, void* dvv,
+                               int causal, void* stream);
 size_t tc_workspace_bytes(const TcParams& t);
 size_t tc_rsum_partial_bytes(const TcParams& t);
 // out0[c] (and out1[c] when planes = 2) = sum over g = 0 .. groups-1, in that order, of partial[g][plane][c]
