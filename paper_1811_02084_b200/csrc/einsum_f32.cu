@@ -9,8 +9,10 @@
 // they do not, up to 8 blocks of a cluster share one tile's K and add their parts through distributed shared memory.
 // The split of K over groups and blocks also shortens every chain of additions, so the sums are no less exact than one
 // thread's sequential loop over K (all of K is walked in ascending order inside each part, parts are added in ascending
-// order).  Measured against one thread per output element (the generic kernel): the feed-forward block forward and
-// backward on 1024 tokens, 256 x 1024 hidden, 4804 -> 156 us (20 of 75 TFLOP/s); on 8 tokens, 64 x 256 hidden, 179 ->
+// order).  Two thirds of the instructions are not multiply-adds (the doubling of A's values, the staging): staging A doubled
+// takes six shared loads a step instead of four and measured 210 us where this takes 149, plain multiply-adds 169.
+// Measured against one thread per output element (the generic kernel): the feed-forward block forward and
+// backward on 1024 tokens, 256 x 1024 hidden, 4804 -> 149 us (22 of 75 TFLOP/s); on 8 tokens, 64 x 256 hidden, 179 ->
 // 33 us (six launches); its error against 64 bits there 5.3e-7 -> 2.0e-7.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -57,52 +59,58 @@ __device__ __forceinline__ unsigned long long twice(float x) {
   return r;
 }
 
-// Column c of row k of a staged tile lives at k * 64 + (c ^ 4 ((k / 4) mod 8)): the exchange keeps 16-byte pieces whole
-// and makes the transposing stores of a K-contiguous operand free of bank conflicts.
-__device__ __forceinline__ int at(int k, int c) { return k * kTile + (c ^ (((k >> 2) & 7) << 2)); }
+// Column c of row k of a staged tile lives at column c ^ 4 ((k / 4) mod 8): the exchange keeps 16-byte pieces whole and
+// spreads the transposing stores of a K-contiguous operand over the banks.
+__device__ __forceinline__ int swz(int k, int c) { return c ^ (((k >> 2) & 7) << 2); }
+__device__ __forceinline__ int at(int k, int c) { return k * kTile + swz(k, c); }
 
-// This thread's two 16-byte pieces of a 64 x 32 operand tile, global -> registers.  s_k == 1: pieces run along k
-// (piece f: row f / 8, k 4 (f mod 8)); otherwise along m|n (piece f: k f / 16, column 4 (f mod 16)).
-__device__ __forceinline__ void load_pieces(const float* base, long long s_mn, long long s_k, bool along_k, int vec, int mn0, int mn_end, int k0, int k_end,
-                                            float4* r) {
+// This thread's two 16-byte pieces of a 64 x 32 operand tile.  Along k (s_k == 1): piece f is row f / 8, k 4 (f mod 8);
+// otherwise along m|n: piece f is k f / 16, column 4 (f mod 16).
+struct Pieces {
+  const float* base;
+  int off[2];                  // element offset of the piece in the first k-block
+  int step;                    // ... and what a k-block adds
+  int s_mn, k_at[2], mn_left[2];      // first k of the piece inside a k-block, columns of it inside the tensor
+  bool along_k, vec;
+  __device__ __forceinline__ void init(const float* b, int smn, int sk, int v, int mn0, int mn_end) {
+    base = b; s_mn = smn; along_k = sk == 1; vec = v != 0; step = kBK * sk;
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int f = threadIdx.x + i * kThreads;
-    float v[4] = {0.f, 0.f, 0.f, 0.f};
-    if (along_k) {
-      const int mn = mn0 + (f >> 3), k = k0 + 4 * (f & 7);
-      if (mn < mn_end && k < k_end) {
-        const float* q = base + mn * s_mn + k;
-        if (vec && k + 4 <= k_end) { r[i] = __ldg(reinterpret_cast<const float4*>(q)); continue; }
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-          if (k + e < k_end) v[e] = __ldg(q + e);
-      }
-    } else {
-      const int k = k0 + (f >> 4), mn = mn0 + 4 * (f & 15);
-      if (k < k_end && mn < mn_end) {
-        const float* q = base + k * s_k + mn * s_mn;
-        if (vec && mn + 4 <= mn_end) { r[i] = __ldg(reinterpret_cast<const float4*>(q)); continue; }
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-          if (mn + e < mn_end) v[e] = __ldg(q + e * s_mn);
-      }
-    }
-    r[i] = make_float4(v[0], v[1], v[2], v[3]);
-  }
-}
-__device__ __forceinline__ void store_pieces(float* tile, bool along_k, const float4* r) {
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int f = threadIdx.x + i * kThreads;
-    if (along_k) {
-      const int mn = f >> 3, k = 4 * (f & 7);
-      tile[at(k, mn)] = r[i].x; tile[at(k + 1, mn)] = r[i].y; tile[at(k + 2, mn)] = r[i].z; tile[at(k + 3, mn)] = r[i].w;
-    } else {
-      *reinterpret_cast<float4*>(tile + at(f >> 4, 4 * (f & 15))) = r[i];
+    for (int i = 0; i < 2; ++i) {
+      const int f = threadIdx.x + i * kThreads;
+      const int mn = mn0 + (along_k ? f >> 3 : 4 * (f & 15));
+      k_at[i] = along_k ? 4 * (f & 7) : f >> 4;
+      mn_left[i] = mn_end - mn;
+      off[i] = mn * smn + k_at[i] * sk;
     }
   }
-}
+  __device__ __forceinline__ void load(int kb, int K, float4* r) const {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      r[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      const int left = K - (kb * kBK + k_at[i]);
+      if (left <= 0 || mn_left[i] <= 0) continue;
+      const float* const q = base + (off[i] + kb * step);
+      const int in = along_k ? left : mn_left[i], s = along_k ? 1 : s_mn;
+      if (vec && in >= 4) { r[i] = __ldg(reinterpret_cast<const float4*>(q)); continue; }
+      r[i].x = __ldg(q);
+      if (in > 1) r[i].y = __ldg(q + s);
+      if (in > 2) r[i].z = __ldg(q + 2 * s);
+      if (in > 3) r[i].w = __ldg(q + 3 * s);
+    }
+  }
+  __device__ __forceinline__ void store(float* tile, const float4* r) const {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int f = threadIdx.x + i * kThreads;
+      if (along_k) {
+        const int mn = f >> 3, k = 4 * (f & 7);
+        tile[at(k, mn)] = r[i].x; tile[at(k + 1, mn)] = r[i].y; tile[at(k + 2, mn)] = r[i].z; tile[at(k + 3, mn)] = r[i].w;
+      } else {
+        *reinterpret_cast<float4*>(tile + at(f >> 4, 4 * (f & 15))) = r[i];
+      }
+    }
+  }
+};
 
 __device__ __forceinline__ float4 ld_peer(uint32_t addr, uint32_t rank) {
   float4 v;
@@ -150,38 +158,47 @@ __global__ void __launch_bounds__(kThreads, 2) einsum_f32_kernel(const __grid_co
   for (int i = 0; i < 8; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+  Pieces pa, pb;
+  pa.init(A, (int)p.sAm, (int)p.sAk, a.vecA, m0, M);
+  pb.init(B, (int)p.sBn, (int)p.sBk, a.vecB, n0, N);
   float4 ra[2], rb[2];
   if (kb0 < kb1) {
-    load_pieces(A, p.sAm, p.sAk, alongA, a.vecA, m0, M, kb0 * kBK, K, ra);
-    load_pieces(B, p.sBn, p.sBk, alongB, a.vecB, n0, N, kb0 * kBK, K, rb);
-    store_pieces(smem, alongA, ra);
-    store_pieces(smem + kBK * kTile, alongB, rb);
+    pa.load(kb0, K, ra);
+    pb.load(kb0, K, rb);
+    pa.store(smem, ra);
+    pb.store(smem + kBK * kTile, rb);
   }
   __syncthreads();
+#pragma unroll 1
   for (int kb = kb0; kb < kb1; ++kb) {
     const float* const sa = smem + ((kb - kb0) & 1) * kBufFloats;
     const float* const sb = sa + kBK * kTile;
     const bool more = kb + 1 < kb1;
     if (more) {
-      load_pieces(A, p.sAm, p.sAk, alongA, a.vecA, m0, M, (kb + 1) * kBK, K, ra);
-      load_pieces(B, p.sBn, p.sBk, alongB, a.vecB, n0, N, (kb + 1) * kBK, K, rb);
+      pa.load(kb + 1, K, ra);
+      pb.load(kb + 1, K, rb);
     }
-#pragma unroll 4                                    // (all 8 at once: 148 bytes of spills)
-    for (int kk = 0; kk < kBK / kGroups; ++kk) {
-      const int k = g * (kBK / kGroups) + kk;
-      const float4 a0 = *reinterpret_cast<const float4*>(sa + at(k, 4 * ty)), a1 = *reinterpret_cast<const float4*>(sa + at(k, 32 + 4 * ty));
-      const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(sb + at(k, 4 * tx)), b1 = *reinterpret_cast<const ulonglong2*>(sb + at(k, 32 + 4 * tx));
-      const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+#pragma unroll 1
+    for (int k4 = 0; k4 < kBK / kGroups; k4 += 4) {
+      const int k0 = g * (kBK / kGroups) + k4;
+      const float* const ka = sa + at(k0, 4 * ty);                 // (columns 32 further on lie 32 floats on, the next k 64 floats on)
+      const float* const kbp = sb + at(k0, 4 * tx);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const unsigned long long d = twice(av[i]);
-        fma2(acc[i][0], d, b0.x); fma2(acc[i][1], d, b0.y); fma2(acc[i][2], d, b1.x); fma2(acc[i][3], d, b1.y);
+      for (int kk = 0; kk < 4; ++kk) {
+        const float4 a0 = *reinterpret_cast<const float4*>(ka + kk * kTile), a1 = *reinterpret_cast<const float4*>(ka + kk * kTile + 32);
+        const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(kbp + kk * kTile), b1 = *reinterpret_cast<const ulonglong2*>(kbp + kk * kTile + 32);
+        const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const unsigned long long d = twice(av[i]);
+          fma2(acc[i][0], d, b0.x); fma2(acc[i][1], d, b0.y); fma2(acc[i][2], d, b1.x); fma2(acc[i][3], d, b1.y);
+        }
       }
     }
     if (more) {                                     // (the other stage: its last readers passed the barrier at the end of the round before)
       float* const nsa = smem + ((kb + 1 - kb0) & 1) * kBufFloats;
-      store_pieces(nsa, alongA, ra);
-      store_pieces(nsa + kBK * kTile, alongB, rb);
+      pa.store(nsa, ra);
+      pb.store(nsa + kBK * kTile, rb);
     }
     __syncthreads();
   }

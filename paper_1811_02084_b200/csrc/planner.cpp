@@ -310,6 +310,8 @@ static bool plan_f32(mtf_plan_t* P) {
   t.sAm = swap ? mn.sB : mm.sA; t.sAk = swap ? mk.sB : mk.sA;
   t.sBn = swap ? mm.sA : mn.sB; t.sBk = swap ? mk.sA : mk.sB;
   t.ldc = swap ? mn.sC : mm.sC;
+  // (a batch entry of an operand is addressed with 32-bit offsets, up to a tile and a k-block past its ends)
+  if ((t.M + 64) * t.sAm + (t.K + 64) * t.sAk > 0x7fffffffLL || (t.N + 64) * t.sBn + (t.K + 64) * t.sBk > 0x7fffffffLL) return false;
   t.n_outer = (int)cb.size();
   for (int j = 0; j < t.n_outer; ++j) {
     const IterDim& d = it[cb[j]];
