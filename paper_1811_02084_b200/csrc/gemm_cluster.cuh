@@ -37,8 +37,9 @@ struct ClusterArgs {
   float scale[3];            // per problem of a grouped launch
   int relu;
   int k_from_row;            // the terms with k below the tile's first row are zero and are left out (one batch dimension's causal sums)
-  float* rsum;               // column sums: one row group in all -> stored, else added to the zeroed output
-  int rsum_store;
+  float* rsum;               // column sums: added to the zeroed output, unless
+  int rsum_store;            // ... one CTA has all rows: it stores them
+  int rsum_gather;           // ... one cluster has all rows: its first CTA adds them up in order
   float* rsum_partial;       // not NULL: [row group][N], finished in order by a launch behind this one
 };
 
@@ -54,6 +55,11 @@ __device__ __forceinline__ uint32_t peer_addr(uint32_t addr, uint32_t rank) {
 __device__ __forceinline__ float4 ld_cluster(uint32_t addr) {
   float4 v;
   asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
+  return v;
+}
+__device__ __forceinline__ float ld_cluster1(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr));
   return v;
 }
 
@@ -262,7 +268,6 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   }
   long long off = c_off + (long long)(m0 + row0) * a.ldc + n;
   if (kSplit > 1) {
-    // every part is read before the first store, so that the rest of the cluster need not wait for this CTA's stores
     float s[kPasses][8];
 #pragma unroll
     for (int i = 0; i < kPasses; ++i) {
@@ -279,11 +284,13 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         }
       }
     }
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < kPasses; ++i, off += kRowsPass * a.ldc)
       if (on && m0 + row0 + i * kRowsPass < a.M) finish_eight<kEpi>(a, C, scale, s[i], off, m0 + row0 + i * kRowsPass, second, bias8, cs);
+    // The parts are in registers (the stores have taken them): the rest of the cluster may end.  Nothing is published here,
+    // and a releasing arrive would wait for the stores (0.5 us).
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   } else {
 #pragma unroll 2
     for (int i = 0; i < kPasses; ++i, off += kRowsPass * a.ldc) {
@@ -311,9 +318,22 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       float x = 0.f;
 #pragma unroll
       for (int w = 0; w < 8; ++w) x += col_part[w][c];
-      if (a.rsum_partial) a.rsum_partial[(size_t)(row_block * kSplit + part) * a.N + n0 + c] = x;
+      if (a.rsum_gather) col_part[0][c] = x;
+      else if (a.rsum_partial) a.rsum_partial[(size_t)(row_block * kSplit + part) * a.N + n0 + c] = x;
       else if (a.rsum_store) a.rsum[n0 + c] = x;
       else atomicAdd(a.rsum + n0 + c, x);
+    }
+    if (kSplit > 1 && a.rsum_gather) {
+      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+      cluster_sync();
+      if (part == 0 && c < BN && n0 + c < a.N) {
+        float x = 0.f;
+#pragma unroll
+        for (int q = 0; q < kSplit; ++q) x += ld_cluster1(peer_addr(smem_u32(&col_part[0][c]), q));
+        a.rsum[n0 + c] = x;
+      }
+      __syncwarp();
+      asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     }
   }
   if (*abort_flag)

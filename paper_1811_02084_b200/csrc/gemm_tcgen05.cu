@@ -1828,12 +1828,12 @@ static mtf_status launch_cluster(const mtf_plan_t& plan, ClusterPick pick, const
   a.resid = resid; a.resid_bf16 = dtRes == MTF_BF16;
   for (int g = 0; g < 3; ++g) a.scale[g] = group_scale && g < n_groups ? group_scale[g] : scale;
   a.relu = relu; a.k_from_row = k_from_row;
-  a.rsum = rsum; a.rsum_store = 0; a.rsum_partial = nullptr;
+  a.rsum = rsum; a.rsum_store = a.rsum_gather = 0; a.rsum_partial = nullptr;
   a.late_wait = (take_independent_hint() && !rsum) ? 1 : 0;
   (void)sched_for_launch(st, false, &a.late_wait);                   // (counts consecutive late launches of the stream)
   const long long groups = row_blocks * pick.split;
   if (rsum) {
-    if (groups == 1) a.rsum_store = 1;
+    if (row_blocks == 1) (pick.split == 1 ? a.rsum_store : a.rsum_gather) = 1;
     else if (workspace && !(reinterpret_cast<uintptr_t>(workspace) & 15) && workspace_bytes >= (size_t)groups * t.N * sizeof(float)) a.rsum_partial = reinterpret_cast<float*>(workspace);
     else {
       mtf_status zs = zero_words(rsum, t.N, st);

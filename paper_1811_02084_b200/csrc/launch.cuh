@@ -1,0 +1,27 @@
+// Launches chained on their stream: a kernel launched with launch_chained may be set up while the launch before it still
+// drains, calls chain_wait() before it touches memory, and from there on lets the launch behind it do the same.  (About 1.5
+// us a launch on a stream of short ones.)
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace mtf {
+
+__device__ __forceinline__ void chain_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// The error is left for the caller's cudaGetLastError.
+template <typename... P, typename... A>
+void launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3(grid, 1, 1); cfg.blockDim = dim3(block, 1, 1); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+}  // namespace mtf

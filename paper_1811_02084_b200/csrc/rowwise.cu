@@ -12,6 +12,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "launch.cuh"
 #include "mtf_internal.h"
 
 namespace {
@@ -50,6 +51,7 @@ __device__ __forceinline__ uint4 float_to_bf16x8(const float* f) {
 // logits fp32, weights bf16, n a multiple of 8.
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 softmax_fwd_kernel(const float* __restrict__ logits, __nv_bfloat16* __restrict__ weights, int64_t rows, int n, int L, int causal) {
+  mtf::chain_wait();
   const int64_t row = (int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
   if (row >= rows) return;
   const int lane = threadIdx.x & 31;
@@ -89,6 +91,7 @@ softmax_fwd_kernel(const float* __restrict__ logits, __nv_bfloat16* __restrict__
 // dlogits[row, :] = P * (dP - sum_j dP_j P_j);  P bf16, dP fp32, dlogits bf16.
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 softmax_bwd_kernel(const __nv_bfloat16* __restrict__ P, const float* __restrict__ dP, __nv_bfloat16* __restrict__ dlg, int64_t rows, int n) {
+  mtf::chain_wait();
   const int64_t row = (int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
   if (row >= rows) return;
   const int lane = threadIdx.x & 31;
@@ -121,6 +124,7 @@ softmax_bwd_kernel(const __nv_bfloat16* __restrict__ P, const float* __restrict_
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 layernorm_fwd_kernel(const __nv_bfloat16* __restrict__ x, const float* __restrict__ gamma, const float* __restrict__ beta,
                      __nv_bfloat16* __restrict__ y, float* __restrict__ stats, int64_t rows, int n, float eps) {
+  mtf::chain_wait();
   const int64_t row = (int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
   if (row >= rows) return;
   const int lane = threadIdx.x & 31;
@@ -161,6 +165,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 layernorm_bwd_dx_kernel(const __nv_bfloat16* __restrict__ dy, const __nv_bfloat16* __restrict__ x, const float* __restrict__ stats,
                         const float* __restrict__ gamma, const __nv_bfloat16* __restrict__ residual, __nv_bfloat16* __restrict__ dx,
                         int64_t rows, int n) {
+  mtf::chain_wait();
   const int64_t row = (int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
   if (row >= rows) return;
   const int lane = threadIdx.x & 31;
@@ -204,6 +209,7 @@ template <int NCH>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 layernorm_fwd_rows_kernel(const __nv_bfloat16* __restrict__ x, const float* __restrict__ gamma, const float* __restrict__ beta,
                           __nv_bfloat16* __restrict__ y, float* __restrict__ stats, int64_t rows, float eps) {
+  mtf::chain_wait();
   constexpr int n = NCH * 256;
   const int64_t row = (int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
   if (row >= rows) return;
@@ -258,6 +264,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 1)
 layernorm_bwd_rows_kernel(const __nv_bfloat16* __restrict__ dy, const __nv_bfloat16* __restrict__ x, const float* __restrict__ stats,
                           const float* __restrict__ gamma, const __nv_bfloat16* __restrict__ residual, __nv_bfloat16* __restrict__ dx,
                           float* __restrict__ dgamma, float* __restrict__ dbeta, float* __restrict__ partial, int64_t rows) {
+  mtf::chain_wait();
   constexpr int n = NCH * 256;
   constexpr int kAccRegs = kSmemAcc ? 1 : NCH;
   extern __shared__ float4 sh_dyn[];
@@ -375,6 +382,7 @@ layernorm_bwd_rows_kernel(const __nv_bfloat16* __restrict__ dy, const __nv_bfloa
 // timing, so the result repeats bit for bit.  planes = 2: out0 from plane 0, out1 from plane 1.
 __global__ void __launch_bounds__(256) colsum_finalize_kernel(const float* __restrict__ partial, int groups, int planes, int n, float* __restrict__ out0,
                                                               float* __restrict__ out1) {
+  mtf::chain_wait();
   __shared__ float sh[2][8][32];
   const int tx = threadIdx.x & 31, seg = threadIdx.x >> 5;
   const int c = blockIdx.x * 32 + tx;
@@ -464,7 +472,7 @@ mtf_status launch_softmax_fwd(const float* logits, void* weights, int64_t rows, 
   if (rows <= 0) return MTF_OK;
   const int64_t blocks = (rows + kWarpsPerBlock - 1) / kWarpsPerBlock;
   if (blocks > 0x7fffffffLL) return fail(MTF_ERR_UNSUPPORTED, "softmax: too many rows");
-  softmax_fwd_kernel<<<(unsigned)blocks, kWarpsPerBlock * 32, 0, (cudaStream_t)stream>>>(logits, reinterpret_cast<__nv_bfloat16*>(weights), rows, n, L, causal);
+  launch_chained(softmax_fwd_kernel, (unsigned)blocks, kWarpsPerBlock * 32, 0, (cudaStream_t)stream, logits, reinterpret_cast<__nv_bfloat16*>(weights), rows, n, L, causal);
   count_launch();
   return check("softmax_fwd_kernel");
 }
@@ -474,7 +482,7 @@ mtf_status launch_softmax_bwd(const void* P, const float* dP, void* dlg, int64_t
   if (rows <= 0) return MTF_OK;
   const int64_t blocks = (rows + kWarpsPerBlock - 1) / kWarpsPerBlock;
   if (blocks > 0x7fffffffLL) return fail(MTF_ERR_UNSUPPORTED, "softmax backward: too many rows");
-  softmax_bwd_kernel<<<(unsigned)blocks, kWarpsPerBlock * 32, 0, (cudaStream_t)stream>>>(reinterpret_cast<const __nv_bfloat16*>(P), dP, reinterpret_cast<__nv_bfloat16*>(dlg), rows, n);
+  launch_chained(softmax_bwd_kernel, (unsigned)blocks, kWarpsPerBlock * 32, 0, (cudaStream_t)stream, reinterpret_cast<const __nv_bfloat16*>(P), dP, reinterpret_cast<__nv_bfloat16*>(dlg), rows, n);
   count_launch();
   return check("softmax_bwd_kernel");
 }
@@ -489,11 +497,11 @@ mtf_status launch_layernorm_fwd(const void* x, const float* gamma, const float* 
   cudaStream_t st = (cudaStream_t)stream;
   // rows of 256, 512, 1024 or 2048 columns stay in registers; other lengths re-read the row per pass
   switch (n) {
-    case 256: layernorm_fwd_rows_kernel<1><<<(unsigned)blocks, kWarpsPerBlock * 32, 0, st>>>(xb, gamma, beta, yb, stats, rows, eps); break;
-    case 512: layernorm_fwd_rows_kernel<2><<<(unsigned)blocks, kWarpsPerBlock * 32, 0, st>>>(xb, gamma, beta, yb, stats, rows, eps); break;
-    case 1024: layernorm_fwd_rows_kernel<4><<<(unsigned)blocks, kWarpsPerBlock * 32, 0, st>>>(xb, gamma, beta, yb, stats, rows, eps); break;
-    case 2048: layernorm_fwd_rows_kernel<8><<<(unsigned)blocks, kWarpsPerBlock * 32, 0, st>>>(xb, gamma, beta, yb, stats, rows, eps); break;
-    default: layernorm_fwd_kernel<<<(unsigned)blocks, kWarpsPerBlock * 32, 0, st>>>(xb, gamma, beta, yb, stats, rows, n, eps);
+    case 256: launch_chained(layernorm_fwd_rows_kernel<1>, (unsigned)blocks, kWarpsPerBlock * 32, 0, st, xb, gamma, beta, yb, stats, rows, eps); break;
+    case 512: launch_chained(layernorm_fwd_rows_kernel<2>, (unsigned)blocks, kWarpsPerBlock * 32, 0, st, xb, gamma, beta, yb, stats, rows, eps); break;
+    case 1024: launch_chained(layernorm_fwd_rows_kernel<4>, (unsigned)blocks, kWarpsPerBlock * 32, 0, st, xb, gamma, beta, yb, stats, rows, eps); break;
+    case 2048: launch_chained(layernorm_fwd_rows_kernel<8>, (unsigned)blocks, kWarpsPerBlock * 32, 0, st, xb, gamma, beta, yb, stats, rows, eps); break;
+    default: launch_chained(layernorm_fwd_kernel, (unsigned)blocks, kWarpsPerBlock * 32, 0, st, xb, gamma, beta, yb, stats, rows, n, eps);
   }
   count_launch();
   return check("layernorm_fwd_kernel");
@@ -506,7 +514,7 @@ size_t layernorm_bwd_scratch_bytes(int n) {
 }
 
 mtf_status launch_colsum_finalize(const float* partial, int groups, int planes, int n, float* out0, float* out1, void* stream) {
-  colsum_finalize_kernel<<<(unsigned)((n + 31) / 32), 256, 0, (cudaStream_t)stream>>>(partial, groups, planes, n, out0, out1);
+  launch_chained(colsum_finalize_kernel, (unsigned)((n + 31) / 32), 256, 0, (cudaStream_t)stream, partial, groups, planes, n, out0, out1);
   count_launch();
   return check("colsum_finalize_kernel");
 }
@@ -538,13 +546,13 @@ mtf_status launch_layernorm_bwd(const void* dy, const void* x, const float* stat
     float* dbp = want ? dbeta : nullptr;
     const size_t sm_small = 2 * (size_t)n * sizeof(float), sm_big = sm_small * (1 + kWarpsPerBlock);       // 144 KB for 2048 columns
     switch (n) {
-      case 256: layernorm_bwd_rows_kernel<1, false><<<grid, kWarpsPerBlock * 32, sm_small, st>>>(db, xb, stats, gamma, rb, ob, dg, dbp, partial, rows); break;
-      case 512: layernorm_bwd_rows_kernel<2, false><<<grid, kWarpsPerBlock * 32, sm_small, st>>>(db, xb, stats, gamma, rb, ob, dg, dbp, partial, rows); break;
-      case 1024: layernorm_bwd_rows_kernel<4, false><<<grid, kWarpsPerBlock * 32, sm_small, st>>>(db, xb, stats, gamma, rb, ob, dg, dbp, partial, rows); break;
+      case 256: launch_chained(layernorm_bwd_rows_kernel<1, false>, grid, kWarpsPerBlock * 32, sm_small, st, db, xb, stats, gamma, rb, ob, dg, dbp, partial, rows); break;
+      case 512: launch_chained(layernorm_bwd_rows_kernel<2, false>, grid, kWarpsPerBlock * 32, sm_small, st, db, xb, stats, gamma, rb, ob, dg, dbp, partial, rows); break;
+      case 1024: launch_chained(layernorm_bwd_rows_kernel<4, false>, grid, kWarpsPerBlock * 32, sm_small, st, db, xb, stats, gamma, rb, ob, dg, dbp, partial, rows); break;
       default: {
         static cudaError_t attr = cudaFuncSetAttribute(layernorm_bwd_rows_kernel<8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * 2048 * sizeof(float) * (1 + kWarpsPerBlock)));
         if (attr != cudaSuccess) return fail(MTF_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(attr));
-        layernorm_bwd_rows_kernel<8, true><<<grid, kWarpsPerBlock * 32, sm_big, st>>>(db, xb, stats, gamma, rb, ob, dg, dbp, partial, rows);
+        launch_chained(layernorm_bwd_rows_kernel<8, true>, grid, kWarpsPerBlock * 32, sm_big, st, db, xb, stats, gamma, rb, ob, dg, dbp, partial, rows);
       }
     }
     count_launch();
@@ -554,7 +562,7 @@ mtf_status launch_layernorm_bwd(const void* dy, const void* x, const float* stat
   }
   const int64_t blocks = (rows + kWarpsPerBlock - 1) / kWarpsPerBlock;
   if (blocks > 0x7fffffffLL) return fail(MTF_ERR_UNSUPPORTED, "layernorm backward: too many rows");
-  layernorm_bwd_dx_kernel<<<(unsigned)blocks, kWarpsPerBlock * 32, 0, st>>>(reinterpret_cast<const __nv_bfloat16*>(dy), reinterpret_cast<const __nv_bfloat16*>(x), stats, gamma,
+  launch_chained(layernorm_bwd_dx_kernel, (unsigned)blocks, kWarpsPerBlock * 32, 0, st, reinterpret_cast<const __nv_bfloat16*>(dy), reinterpret_cast<const __nv_bfloat16*>(x), stats, gamma,
                                                                           reinterpret_cast<const __nv_bfloat16*>(residual), reinterpret_cast<__nv_bfloat16*>(dx), rows, n);
   count_launch();
   mtf_status s = check("layernorm_bwd_dx_kernel");

@@ -10,6 +10,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "launch.cuh"
 #include "mtf_internal.h"
 
 namespace {
@@ -17,6 +18,7 @@ namespace {
 template <bool kMom, bool kGradBf16, bool kParam>
 __global__ void __launch_bounds__(256) sgd_update_kernel(float* __restrict__ master, __nv_bfloat16* __restrict__ param, const void* __restrict__ grad,
                                                          float* __restrict__ mom, long long n, float lr, float mu, float wd) {
+  mtf::chain_wait();
   const long long n4 = n / 4;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (long long)gridDim.x * blockDim.x) {
     float4 w = reinterpret_cast<const float4*>(master)[i];
@@ -66,7 +68,7 @@ mtf_status launch_sgd_update(float* master, void* param, const void* grad, int g
   const long long blocks = std::min<long long>((n / 4 + 255) / 256 + 1, (long long)device_sm_count() * 8);
   cudaStream_t st = (cudaStream_t)stream;
   __nv_bfloat16* pb = reinterpret_cast<__nv_bfloat16*>(param);
-#define MTF_UPD(M, G, P) sgd_update_kernel<M, G, P><<<(unsigned)blocks, 256, 0, st>>>(master, pb, grad, mom, n, lr, mu, wd)
+#define MTF_UPD(M, G, P) launch_chained(sgd_update_kernel<M, G, P>, (unsigned)blocks, 256, 0, st, master, pb, grad, mom, n, lr, mu, wd)
   if (mom) {
     if (grad_bf16) { if (param) MTF_UPD(true, true, true); else MTF_UPD(true, true, false); }
     else { if (param) MTF_UPD(true, false, true); else MTF_UPD(true, false, false); }

@@ -17,6 +17,7 @@
 
 #include <algorithm>
 
+#include "launch.cuh"
 #include "mtf_internal.h"
 
 namespace {
@@ -32,6 +33,7 @@ __device__ __forceinline__ void bf16x8(const uint4& u, float* f) {
 
 __global__ void __launch_bounds__(256) embedding_gather_kernel(const int32_t* __restrict__ ids, const uint4* __restrict__ table, uint4* __restrict__ x,
                                                                long long n_tokens, int pieces, int vocab, int* __restrict__ bad) {
+  mtf::chain_wait();
   const long long total = n_tokens * pieces;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
     const long long t = i / pieces;
@@ -80,6 +82,7 @@ __device__ __forceinline__ void lse_combine(float& m, float& s, float m2, float 
 
 __global__ void __launch_bounds__(256) xent_rows_kernel(const __nv_bfloat16* __restrict__ logits, const int32_t* __restrict__ targets, float* __restrict__ lse,
                                                         float* __restrict__ loss, int vocab, int* __restrict__ bad) {
+  mtf::chain_wait();
   __shared__ float red_m[8], red_s[8];
   const long long row = blockIdx.x;
   const uint4* r = reinterpret_cast<const uint4*>(logits + row * vocab);
@@ -120,6 +123,7 @@ __global__ void __launch_bounds__(256) xent_rows_kernel(const __nv_bfloat16* __r
 __global__ void __launch_bounds__(256) xent_combine_kernel(const float2* __restrict__ partial, int parts, const __nv_bfloat16* __restrict__ logits,
                                                            const int32_t* __restrict__ targets, float* __restrict__ lse, float* __restrict__ loss,
                                                            long long n_rows, int vocab, int* __restrict__ bad) {
+  mtf::chain_wait();
   const long long row = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
   if (row >= n_rows) return;
   const int lane = threadIdx.x & 31;
@@ -145,6 +149,7 @@ __global__ void __launch_bounds__(256) xent_combine_kernel(const float2* __restr
 // dlogits[t, v] = (exp(logits[t, v] - lse[t]) - [v == target[t]]) * dloss[t], written over the logits
 __global__ void __launch_bounds__(256) xent_backward_kernel(__nv_bfloat16* __restrict__ logits, const int32_t* __restrict__ targets, const float* __restrict__ lse,
                                                             const float* __restrict__ dloss, long long n_rows, int vocab) {
+  mtf::chain_wait();
   const int pieces = vocab / 8;
   const long long total = n_rows * pieces;
   uint4* lg = reinterpret_cast<uint4*>(logits);
@@ -192,7 +197,7 @@ mtf_status launch_embedding_gather(const int32_t* ids, const void* table, void* 
     return fail(MTF_ERR_UNSUPPORTED, "embedding: rows must be multiples of 16 bytes and 16-byte aligned");
   const int pieces = (int)(d * elem_bytes / 16);
   const long long blocks = std::min<long long>((n_tokens * pieces + 255) / 256, (long long)device_sm_count() * 16);
-  embedding_gather_kernel<<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(ids, reinterpret_cast<const uint4*>(table), reinterpret_cast<uint4*>(x), n_tokens, pieces, (int)vocab, bad_flag());
+  launch_chained(embedding_gather_kernel, (unsigned)blocks, 256, 0, (cudaStream_t)stream, ids, reinterpret_cast<const uint4*>(table), reinterpret_cast<uint4*>(x), n_tokens, pieces, (int)vocab, bad_flag());
   return after("embedding_gather_kernel");
 }
 
@@ -210,7 +215,7 @@ mtf_status launch_xent_rows(const void* logits, const int32_t* targets, float* l
   if (n_rows <= 0) return MTF_OK;
   if (vocab % 8 || (reinterpret_cast<uintptr_t>(logits) & 15)) return fail(MTF_ERR_UNSUPPORTED, "cross-entropy: vocab must be a multiple of 8 and the logits 16-byte aligned");
   if (n_rows > 0x7fffffffLL) return fail(MTF_ERR_UNSUPPORTED, "cross-entropy: too many rows");
-  xent_rows_kernel<<<(unsigned)n_rows, 256, 0, (cudaStream_t)stream>>>(reinterpret_cast<const __nv_bfloat16*>(logits), targets, lse, loss, (int)vocab, bad_flag());
+  launch_chained(xent_rows_kernel, (unsigned)n_rows, 256, 0, (cudaStream_t)stream, reinterpret_cast<const __nv_bfloat16*>(logits), targets, lse, loss, (int)vocab, bad_flag());
   return after("xent_rows_kernel");
 }
 
@@ -218,7 +223,7 @@ mtf_status launch_xent_combine(const void* partial, int parts, const void* logit
                                void* stream) {
   if (n_rows <= 0) return MTF_OK;
   if (parts <= 0 || n_rows > 0x7fffffffLL) return fail(MTF_ERR_UNSUPPORTED, "cross-entropy combine: bad sizes");
-  xent_combine_kernel<<<(unsigned)((n_rows + 7) / 8), 256, 0, (cudaStream_t)stream>>>(reinterpret_cast<const float2*>(partial), parts,
+  launch_chained(xent_combine_kernel, (unsigned)((n_rows + 7) / 8), 256, 0, (cudaStream_t)stream, reinterpret_cast<const float2*>(partial), parts,
                                                                                    reinterpret_cast<const __nv_bfloat16*>(logits), targets, lse, loss, n_rows, (int)vocab,
                                                                                    bad_flag());
   return after("xent_combine_kernel");
@@ -227,7 +232,7 @@ mtf_status launch_xent_combine(const void* partial, int parts, const void* logit
 mtf_status launch_xent_backward(void* logits, const int32_t* targets, const float* lse, const float* dloss, int64_t n_rows, int64_t vocab, void* stream) {
   if (n_rows <= 0) return MTF_OK;
   const long long blocks = std::min<long long>((n_rows * (vocab / 8) + 255) / 256, (long long)device_sm_count() * 16);
-  xent_backward_kernel<<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(reinterpret_cast<__nv_bfloat16*>(logits), targets, lse, dloss, n_rows, (int)vocab);
+  launch_chained(xent_backward_kernel, (unsigned)blocks, 256, 0, (cudaStream_t)stream, reinterpret_cast<__nv_bfloat16*>(logits), targets, lse, dloss, n_rows, (int)vocab);
   return after("xent_backward_kernel");
 }
 
