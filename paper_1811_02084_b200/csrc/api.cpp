@@ -136,14 +136,14 @@ mtf_status cached_plan(const mtf_layout_t* L, int n_in, const mtf_tensor* in, co
     if (in[q].ndim < 0 || in[q].ndim > mtf::kMaxTensorDims || (in[q].ndim && !in[q].dims)) return fail(MTF_ERR_INVALID_ARG, "einsum: bad input descriptor");
   if (out->ndim < 0 || out->ndim > mtf::kMaxTensorDims || (out->ndim && !out->dims)) return fail(MTF_ERR_INVALID_ARG, "einsum: bad output descriptor");
   mtf_layout_t* Lm = const_cast<mtf_layout_t*>(L);
-  const std::string key = mtf::plan_key(n_in, in, out, epi, g_force_kernel, g_force_reduce);
+  static thread_local std::string key;
+  mtf::plan_key(n_in, in, out, epi, g_force_kernel, g_force_reduce, &key);
   std::lock_guard<std::mutex> lock(Lm->mu);
   auto it = Lm->cache.find(key);
   if (it == Lm->cache.end()) {
     std::unique_ptr<mtf_plan_t> P;
     mtf_status st = mtf::make_plan(L, n_in, in, out, epi, g_force_kernel, g_force_reduce, &P);
     if (st != MTF_OK) return st;
-    P->key = key;
     it = Lm->cache.emplace(key, std::move(P)).first;
   }
   *plan = it->second.get();

@@ -151,7 +151,6 @@ struct mtf_plan_s {
   bool f32_ok = false;      // generic family: the f32 matrix-product kernel takes this einsum
   F32Params f32;
   TcParams tc;
-  std::string key;
 };
 
 struct mtf_layout_s {
@@ -181,7 +180,7 @@ mtf_status check_tensor(const mtf_layout_t* L, const std::vector<Dim>& dims);
 mtf_status slice_box(const mtf_layout_t* L, const std::vector<Dim>& dims, int64_t p, int64_t* offs, int64_t* sizes);
 mtf_status make_plan(const mtf_layout_t* L, int n_in, const mtf_tensor* in, const mtf_tensor* out,
                      const mtf_epilogue* epi, int force_kernel, int force_reduce, std::unique_ptr<mtf_plan_t>* plan);
-std::string plan_key(int n_in, const mtf_tensor* in, const mtf_tensor* out, const mtf_epilogue* epi, int fk, int fr);
+void plan_key(int n_in, const mtf_tensor* in, const mtf_tensor* out, const mtf_epilogue* epi, int fk, int fr, std::string* key);
 
 // rank binding (ranks.cpp): does summing out `reduced` (dimension names) leave a sum across ranks to do?
 bool rank_sum_needed(const mtf_layout_t* L, const std::vector<std::string>& reduced);

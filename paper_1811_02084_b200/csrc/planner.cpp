@@ -105,35 +105,32 @@ mtf_status slice_box(const mtf_layout_t* L, const std::vector<Dim>& dims, int64_
   return MTF_OK;
 }
 
-static const char* dt_name(int dt) { return dt == MTF_BF16 ? "bf16" : "f32"; }
-
-std::string plan_key(int n_in, const mtf_tensor* in, const mtf_tensor* out, const mtf_epilogue* epi, int fk, int fr) {
-  std::string k;
+// What a plan depends on, as bytes: it is built on every call (no decimal text and no allocation once `k` has its size).
+void plan_key(int n_in, const mtf_tensor* in, const mtf_tensor* out, const mtf_epilogue* epi, int fk, int fr, std::string* key) {
+  std::string& k = *key;
+  k.clear();
   auto add_t = [&](const mtf_tensor* t) {
-    k += dt_name(t->dtype);
-    k += '[';
+    k += (char)t->dtype;
+    k += (char)t->ndim;
     for (int i = 0; i < t->ndim; ++i) {
       k += t->dims[i].name ? t->dims[i].name : "?";
-      k += ':';
-      k += std::to_string((long long)t->dims[i].size);
-      k += ',';
+      k += '\0';
+      k.append(reinterpret_cast<const char*>(&t->dims[i].size), sizeof(t->dims[i].size));
     }
-    k += ']';
   };
+  k += (char)fk;
+  k += (char)fr;
+  k += (char)n_in;
   for (int q = 0; q < n_in; ++q) add_t(&in[q]);
-  k += "->";
   add_t(out);
   if (epi) {
-    k += "|e";
     k += epi->relu ? 'r' : '-';
     k += (epi->scale != 1.f) ? 's' : '-';
     if (epi->bias) { k += 'b'; add_t(epi->bias); }
-    if (epi->relu_mask) { k += 'm'; k += dt_name(epi->relu_mask->dtype); }
-    if (epi->residual) { k += 'a'; k += dt_name(epi->residual->dtype); }
+    if (epi->relu_mask) { k += 'm'; k += (char)epi->relu_mask->dtype; }
+    if (epi->residual) { k += 'a'; k += (char)epi->residual->dtype; }
     if (epi->reduce_sum_out) { k += 'S'; add_t(epi->reduce_sum_out); }
   }
-  k += "|f" + std::to_string(fk) + "," + std::to_string(fr);
-  return k;
 }
 
 static bool same_dims(const std::vector<Dim>& a, const std::vector<Dim>& b) {
