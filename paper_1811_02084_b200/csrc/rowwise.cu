@@ -203,21 +203,24 @@ layernorm_bwd_dx_kernel(const __nv_bfloat16* __restrict__ dy, const __nv_bfloat1
   }
 }
 
-// Rows of exactly NCH * 256 columns: a lane keeps its NCH pieces of 8 columns in registers, so the row
-// is read from memory once and all its loads are in flight together.
-template <int NCH>
+// Rows of NCH * 256 columns, or with kTail of up to that many (a multiple of 8): a lane keeps its NCH pieces of 8 columns in
+// registers, so the row is read from memory once and all its loads are in flight together.  (Lengths that are no multiple
+// of 256 re-read the row per pass before, and their backward pass read it again for the parameter gradients and added those
+// up with atomics: together 830 -> 690 us of a decoder layer forward and backward, most of it this.)
+template <int NCH, bool kTail>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 layernorm_fwd_rows_kernel(const __nv_bfloat16* __restrict__ x, const float* __restrict__ gamma, const float* __restrict__ beta,
-                          __nv_bfloat16* __restrict__ y, float* __restrict__ stats, int64_t rows, float eps) {
+                          __nv_bfloat16* __restrict__ y, float* __restrict__ stats, int64_t rows, int n_cols, float eps) {
   mtf::chain_wait();
-  constexpr int n = NCH * 256;
+  const int n = kTail ? n_cols : NCH * 256;
   const int64_t row = (int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
   if (row >= rows) return;
   const int lane = threadIdx.x & 31;
+  auto in = [&](int i) { return !kTail || i < NCH - 1 || i * 256 + lane * 8 < n; };      // (only the last piece may lie past the row)
   const __nv_bfloat16* xr = x + row * n + lane * 8;
   uint4 xv[NCH];
 #pragma unroll
-  for (int i = 0; i < NCH; ++i) xv[i] = *reinterpret_cast<const uint4*>(xr + i * 256);
+  for (int i = 0; i < NCH; ++i) xv[i] = in(i) ? *reinterpret_cast<const uint4*>(xr + i * 256) : make_uint4(0u, 0u, 0u, 0u);
   float s = 0.f;
 #pragma unroll
   for (int i = 0; i < NCH; ++i) {
@@ -230,6 +233,7 @@ layernorm_fwd_rows_kernel(const __nv_bfloat16* __restrict__ x, const float* __re
   float q = 0.f;
 #pragma unroll
   for (int i = 0; i < NCH; ++i) {
+    if (!in(i)) continue;
     float f[8];
     bf16x8_to_float(xv[i], f);
 #pragma unroll
@@ -241,6 +245,7 @@ layernorm_fwd_rows_kernel(const __nv_bfloat16* __restrict__ x, const float* __re
 #pragma unroll
   for (int i = 0; i < NCH; ++i) {
     const int c = i * 256 + lane * 8;
+    if (!in(i)) continue;
     float f[8], o[8];
     bf16x8_to_float(xv[i], f);
     const float4 g0 = *reinterpret_cast<const float4*>(gamma + c), g1 = *reinterpret_cast<const float4*>(gamma + c + 4);
@@ -253,19 +258,19 @@ layernorm_fwd_rows_kernel(const __nv_bfloat16* __restrict__ x, const float* __re
   }
 }
 
-// Backward for rows of NCH * 256 columns, dx and the parameter gradients in one pass over dy and x:
+// Backward for rows of NCH * 256 columns (kTail: of up to that many), dx and the parameter gradients in one pass over dy and x:
 // a persistent grid of 8-warp blocks, every warp walks rows with both rows in registers and keeps
 // its lanes' partial dgamma / dbeta sums in registers; at the end the block adds them up in shared
 // memory and issues one fp32 atomic per column and block.
-// kSmemAcc (the 2048-column case, whose 128 partial sums per lane do not fit the registers next to
+// kSmemAcc (more than 1024 columns, whose up to 128 partial sums per lane do not fit the registers next to
 // the two rows): every warp keeps its partial sums in a shared-memory strip of its own instead.
-template <int NCH, bool kSmemAcc>
+template <int NCH, bool kTail, bool kSmemAcc>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32, 1)
 layernorm_bwd_rows_kernel(const __nv_bfloat16* __restrict__ dy, const __nv_bfloat16* __restrict__ x, const float* __restrict__ stats,
                           const float* __restrict__ gamma, const __nv_bfloat16* __restrict__ residual, __nv_bfloat16* __restrict__ dx,
-                          float* __restrict__ dgamma, float* __restrict__ dbeta, float* __restrict__ partial, int64_t rows) {
+                          float* __restrict__ dgamma, float* __restrict__ dbeta, float* __restrict__ partial, int64_t rows, int n_cols) {
   mtf::chain_wait();
-  constexpr int n = NCH * 256;
+  const int n = kTail ? n_cols : NCH * 256;
   constexpr int kAccRegs = kSmemAcc ? 1 : NCH;
   extern __shared__ float4 sh_dyn[];
   float* const sh = reinterpret_cast<float*>(sh_dyn);                 // [2][n] block sums, then (kSmemAcc) [warps][2][n] strips
@@ -273,6 +278,7 @@ layernorm_bwd_rows_kernel(const __nv_bfloat16* __restrict__ dy, const __nv_bfloa
   for (int i = threadIdx.x; i < n_sh; i += kWarpsPerBlock * 32) sh[i] = 0.f;
   __syncthreads();
   const int lane = threadIdx.x & 31;
+  auto in = [&](int i) { return !kTail || i < NCH - 1 || i * 256 + lane * 8 < n; };
   float* const strip = sh + 2 * n * (1 + (threadIdx.x >> 5));           // this warp's strip: [2][n]
   const int64_t wid = (int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5), nw = (int64_t)gridDim.x * kWarpsPerBlock;
   float ag[kAccRegs][8], ab[kAccRegs][8];
@@ -285,12 +291,16 @@ layernorm_bwd_rows_kernel(const __nv_bfloat16* __restrict__ dy, const __nv_bfloa
     const __nv_bfloat16* dr = dy + row * n + lane * 8;
     uint4 xv[NCH], dv[NCH];
 #pragma unroll
-    for (int i = 0; i < NCH; ++i) { xv[i] = *reinterpret_cast<const uint4*>(xr + i * 256); dv[i] = *reinterpret_cast<const uint4*>(dr + i * 256); }
+    for (int i = 0; i < NCH; ++i) {
+      xv[i] = in(i) ? *reinterpret_cast<const uint4*>(xr + i * 256) : make_uint4(0u, 0u, 0u, 0u);
+      dv[i] = in(i) ? *reinterpret_cast<const uint4*>(dr + i * 256) : make_uint4(0u, 0u, 0u, 0u);
+    }
     const float mu = stats[2 * row], rstd = stats[2 * row + 1];
     float s1 = 0.f, s2 = 0.f;
 #pragma unroll
     for (int i = 0; i < NCH; ++i) {
       const int c = i * 256 + lane * 8;
+      if (!in(i)) continue;
       float xf[8], df[8];
       bf16x8_to_float(xv[i], xf);
       bf16x8_to_float(dv[i], df);
@@ -328,6 +338,7 @@ layernorm_bwd_rows_kernel(const __nv_bfloat16* __restrict__ dy, const __nv_bfloa
 #pragma unroll
     for (int i = 0; i < NCH; ++i) {
       const int c = i * 256 + lane * 8;
+      if (!in(i)) continue;
       float xf[8], df[8], o[8], rf[8];
       bf16x8_to_float(xv[i], xf);
       bf16x8_to_float(dv[i], df);
@@ -361,7 +372,7 @@ layernorm_bwd_rows_kernel(const __nv_bfloat16* __restrict__ dy, const __nv_bfloa
 #pragma unroll
           for (int i = 0; i < kAccRegs; ++i)
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
+            for (int e = 0; e < 8 && in(i); ++e) {
               sh[i * 256 + lane * 8 + e] += ag[i][e];
               sh[n + i * 256 + lane * 8 + e] += ab[i][e];
             }
@@ -495,14 +506,20 @@ mtf_status launch_layernorm_fwd(const void* x, const float* gamma, const float* 
   const __nv_bfloat16* xb = reinterpret_cast<const __nv_bfloat16*>(x);
   __nv_bfloat16* yb = reinterpret_cast<__nv_bfloat16*>(y);
   cudaStream_t st = (cudaStream_t)stream;
-  // rows of 256, 512, 1024 or 2048 columns stay in registers; other lengths re-read the row per pass
-  switch (n) {
-    case 256: launch_chained(layernorm_fwd_rows_kernel<1>, (unsigned)blocks, kWarpsPerBlock * 32, 0, st, xb, gamma, beta, yb, stats, rows, eps); break;
-    case 512: launch_chained(layernorm_fwd_rows_kernel<2>, (unsigned)blocks, kWarpsPerBlock * 32, 0, st, xb, gamma, beta, yb, stats, rows, eps); break;
-    case 1024: launch_chained(layernorm_fwd_rows_kernel<4>, (unsigned)blocks, kWarpsPerBlock * 32, 0, st, xb, gamma, beta, yb, stats, rows, eps); break;
-    case 2048: launch_chained(layernorm_fwd_rows_kernel<8>, (unsigned)blocks, kWarpsPerBlock * 32, 0, st, xb, gamma, beta, yb, stats, rows, eps); break;
+  // rows of at most 2048 columns stay in registers; longer ones are re-read per pass
+#define MTF_LN(NCH, TAIL) launch_chained(layernorm_fwd_rows_kernel<NCH, TAIL>, (unsigned)blocks, kWarpsPerBlock * 32, 0, st, xb, gamma, beta, yb, stats, rows, n, eps)
+  switch (n > 2048 ? 0 : (n + 255) / 256) {
+    case 1: n == 256 ? MTF_LN(1, false) : MTF_LN(1, true); break;
+    case 2: n == 512 ? MTF_LN(2, false) : MTF_LN(2, true); break;
+    case 3: MTF_LN(3, true); break;
+    case 4: n == 1024 ? MTF_LN(4, false) : MTF_LN(4, true); break;
+    case 5: MTF_LN(5, true); break;
+    case 6: MTF_LN(6, true); break;
+    case 7: MTF_LN(7, true); break;
+    case 8: n == 2048 ? MTF_LN(8, false) : MTF_LN(8, true); break;
     default: launch_chained(layernorm_fwd_kernel, (unsigned)blocks, kWarpsPerBlock * 32, 0, st, xb, gamma, beta, yb, stats, rows, n, eps);
   }
+#undef MTF_LN
   count_launch();
   return check("layernorm_fwd_kernel");
 }
@@ -519,17 +536,28 @@ mtf_status launch_colsum_finalize(const float* partial, int groups, int planes, 
   return check("colsum_finalize_kernel");
 }
 
+template <int NCH, bool kTail, bool kSmemAcc>
+static mtf_status launch_ln_bwd(unsigned grid, size_t smem, cudaStream_t st, const __nv_bfloat16* dy, const __nv_bfloat16* x, const float* stats, const float* gamma,
+                                const __nv_bfloat16* residual, __nv_bfloat16* dx, float* dgamma, float* dbeta, float* partial, int64_t rows, int n) {
+  if (kSmemAcc) {
+    const cudaError_t e = cudaFuncSetAttribute(layernorm_bwd_rows_kernel<NCH, kTail, kSmemAcc>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * NCH * 256 * sizeof(float) * (1 + kWarpsPerBlock)));
+    if (e != cudaSuccess) return fail(MTF_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
+  }
+  launch_chained(layernorm_bwd_rows_kernel<NCH, kTail, kSmemAcc>, grid, kWarpsPerBlock * 32, smem, st, dy, x, stats, gamma, residual, dx, dgamma, dbeta, partial, rows, n);
+  return MTF_OK;
+}
+
 mtf_status launch_layernorm_bwd(const void* dy, const void* x, const float* stats, const float* gamma, const void* residual, void* dx,
                                 float* dgamma, float* dbeta, int64_t rows, int n, void* scratch, size_t scratch_bytes, void* stream) {
   if (n % 8 || !aligned16(x) || !aligned16(dy) || !aligned16(dx) || !aligned16(gamma) || (residual && !aligned16(residual)))
     return fail(MTF_ERR_UNSUPPORTED, "layernorm backward: row length must be a multiple of 8 and pointers 16-byte aligned");
   if (rows <= 0) return MTF_OK;
   cudaStream_t st = (cudaStream_t)stream;
-  if (n == 256 || n == 512 || n == 1024 || n == 2048) {
+  if (n <= 2048) {
     // one pass over dy and x for dx and the parameter gradients (persistent grid)
     const int sms = device_sm_count();
     unsigned grid = (unsigned)std::min<int64_t>((rows + kWarpsPerBlock - 1) / kWarpsPerBlock, 2 * (int64_t)sms);
-    if (n == 2048) grid = std::min(grid, (unsigned)sms);
+    if (n > 1024) grid = std::min(grid, (unsigned)sms);
     const bool want = dgamma && dbeta;
     float* partial = nullptr;
     if (want && scratch && !(reinterpret_cast<uintptr_t>(scratch) & 15) && scratch_bytes >= (size_t)grid * 2 * n * sizeof(float)) partial = reinterpret_cast<float*>(scratch);
@@ -545,16 +573,20 @@ mtf_status launch_layernorm_bwd(const void* dy, const void* x, const float* stat
     float* dg = want ? dgamma : nullptr;
     float* dbp = want ? dbeta : nullptr;
     const size_t sm_small = 2 * (size_t)n * sizeof(float), sm_big = sm_small * (1 + kWarpsPerBlock);       // 144 KB for 2048 columns
-    switch (n) {
-      case 256: launch_chained(layernorm_bwd_rows_kernel<1, false>, grid, kWarpsPerBlock * 32, sm_small, st, db, xb, stats, gamma, rb, ob, dg, dbp, partial, rows); break;
-      case 512: launch_chained(layernorm_bwd_rows_kernel<2, false>, grid, kWarpsPerBlock * 32, sm_small, st, db, xb, stats, gamma, rb, ob, dg, dbp, partial, rows); break;
-      case 1024: launch_chained(layernorm_bwd_rows_kernel<4, false>, grid, kWarpsPerBlock * 32, sm_small, st, db, xb, stats, gamma, rb, ob, dg, dbp, partial, rows); break;
-      default: {
-        static cudaError_t attr = cudaFuncSetAttribute(layernorm_bwd_rows_kernel<8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * 2048 * sizeof(float) * (1 + kWarpsPerBlock)));
-        if (attr != cudaSuccess) return fail(MTF_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(attr));
-        launch_chained(layernorm_bwd_rows_kernel<8, true>, grid, kWarpsPerBlock * 32, sm_big, st, db, xb, stats, gamma, rb, ob, dg, dbp, partial, rows);
-      }
+    mtf_status as = MTF_OK;
+#define MTF_LNB(NCH, TAIL, SM) (as = launch_ln_bwd<NCH, TAIL, SM>(grid, SM ? sm_big : sm_small, st, db, xb, stats, gamma, rb, ob, dg, dbp, partial, rows, n))
+    switch ((n + 255) / 256) {
+      case 1: n == 256 ? MTF_LNB(1, false, false) : MTF_LNB(1, true, false); break;
+      case 2: n == 512 ? MTF_LNB(2, false, false) : MTF_LNB(2, true, false); break;
+      case 3: MTF_LNB(3, true, false); break;
+      case 4: n == 1024 ? MTF_LNB(4, false, false) : MTF_LNB(4, true, false); break;
+      case 5: MTF_LNB(5, true, true); break;
+      case 6: MTF_LNB(6, true, true); break;
+      case 7: MTF_LNB(7, true, true); break;
+      default: n == 2048 ? MTF_LNB(8, false, true) : MTF_LNB(8, true, true); break;
     }
+#undef MTF_LNB
+    if (as != MTF_OK) return as;
     count_launch();
     mtf_status s2 = check("layernorm_bwd_rows_kernel");
     if (s2 != MTF_OK || !partial) return s2;
