@@ -272,7 +272,7 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 #pragma unroll
     for (int i = 0; i < kPasses; ++i) {
       const uint32_t at0 = ring + tile_at<BN>(row0 + i * kRowsPass, piece), at1 = ring + tile_at<BN>(row0 + i * kRowsPass, piece + 1);
-      if (on) {
+      if (on && m0 + row0 + i * kRowsPass < a.M) {
         float4 x[kSplit], y[kSplit];
 #pragma unroll
         for (int q = 0; q < kSplit; ++q) { x[q] = ld_cluster(peer_addr(at0, q)); y[q] = ld_cluster(peer_addr(at1, q)); }
@@ -284,13 +284,13 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         }
       }
     }
+    // With its reads done a CTA lets the rest of the cluster end (a peer's shared memory is gone once it has).  The releasing
+    // arrive waits for those reads, used or not, and stands in front of the stores, which it would wait for as well (0.5 us).
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < kPasses; ++i, off += kRowsPass * a.ldc)
       if (on && m0 + row0 + i * kRowsPass < a.M) finish_eight<kEpi>(a, C, scale, s[i], off, m0 + row0 + i * kRowsPass, second, bias8, cs);
-    // The parts are in registers (the stores have taken them): the rest of the cluster may end.  Nothing is published here,
-    // and a releasing arrive would wait for the stores (0.5 us).
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   } else {
 #pragma unroll 2
     for (int i = 0; i < kPasses; ++i, off += kRowsPass * a.ldc) {
@@ -326,14 +326,15 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     if (kSplit > 1 && a.rsum_gather) {
       asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
       cluster_sync();
-      if (part == 0 && c < BN && n0 + c < a.N) {
-        float x = 0.f;
+      const bool mine = part == 0 && c < BN && n0 + c < a.N;
+      float x = 0.f;
+      if (mine) {
 #pragma unroll
         for (int q = 0; q < kSplit; ++q) x += ld_cluster1(peer_addr(smem_u32(&col_part[0][c]), q));
-        a.rsum[n0 + c] = x;
       }
       __syncwarp();
-      asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");      // (the reads are done: see above)
+      if (mine) a.rsum[n0 + c] = x;
     }
   }
   if (*abort_flag)

@@ -70,3 +70,20 @@ def test_column_sums(mtf, scratch, m, n, k):
     ref = (x.f64 @ y.f64) * (mask.f64 > 0)
     assert parity_error(from_torch(out), ref) <= TOL["bf16"]
     assert parity_error(from_torch(col), ref.sum(0)) <= TOL["f32"]
+
+
+@pytest.mark.parametrize("m", [8, 24, 136, 200])
+@pytest.mark.parametrize("k", [256, 640, 4096])
+def test_tiles_with_few_rows_leave_the_cluster_together(mtf, m, k):
+    """Most CTAs of a cluster own no row of such a tile (or of the last one): launches back to back, more than fill the chip,
+    all give the first one's bits."""
+    import torch
+    n = 1032
+    x, y = si.normal(7, "x", [m, k], "bf16"), si.normal(7, "y", [k, n], "bf16", k ** -0.5)
+    tx, ty, lay = to_torch(x), to_torch(y), layout(mtf, *ONE)
+    outs = [torch.full((m, n), float("nan"), device="cuda") for _ in range(40)]
+    for out in outs:
+        mtf.mtf_einsum(lay, None, [mtf.named(tx, ["i", "k"]), mtf.named(ty, ["k", "j"])], mtf.named(out, ["i", "j"]))
+    mtf.mtf_device_status()
+    assert parity_error(from_torch(outs[0]), x.f64 @ y.f64) <= TOL["bf16"]
+    assert all(torch.equal(outs[0], o) for o in outs[1:])
