@@ -476,13 +476,19 @@ const char* mtf_last_error(void);
 mtf_status mtf_device_status(int32_t* code);
 /* Testing hook for the failure path of the bounded device-side waits.  limit_cycles > 0 sets how many SM
  * cycles a wait may take before it gives up (<= 0 restores the default of about two seconds);
- * withhold_one_signal != 0 makes every tensor-core launch leave out the "accumulator complete" signal
- * of its first tile, so that the wait for it runs out: the kernel records a code, all its roles
+ * withhold_one_signal != 0 makes every launch of the persistent tensor-core kernel leave out the "accumulator complete"
+ * signal of its first tile, so that the wait for it runs out: the kernel records a code, all its roles
  * leave through the common teardown (copies and MMAs in flight are given time to land, tensor memory
  * is freed), the launch ends normally, its output is unspecified, and the next mtf_device_status
  * returns MTF_ERR_TIMEOUT.  Nothing traps or faults and the context stays usable.  Affects the current
  * device until changed back; not for production use. */
 mtf_status mtf_debug_wait_test(int64_t limit_cycles, int32_t withhold_one_signal);
+/* Testing hook: tensor-core contractions launched afterwards by this thread, where they may run on 128-row tiles with K
+ * over a cluster of CTAs (nothing forced through mtf_plan_force, no row softmax), run on tiles of `columns` (64 or 128)
+ * columns with K over `split` (1, 2, 4 or 8) CTAs, provided K has that many 64-deep blocks; 0, 0 gives the choice back to
+ * the library.  ran_columns, ran_split (may be NULL): what this thread's last contraction before the call ran on; 0, 0 if
+ * on the persistent kernel. */
+mtf_status mtf_debug_contraction(int32_t columns, int32_t split, int32_t* ran_columns, int32_t* ran_split);
 /* Number of kernels this library has launched from this process (all threads). */
 int64_t mtf_launch_count(void);
 

@@ -156,6 +156,7 @@ def _load():
         "mtf_xent_backward": [vp, POINTER(mtf_tensor), POINTER(mtf_tensor), vp, POINTER(mtf_tensor), POINTER(mtf_tensor), POINTER(mtf_tensor), POINTER(mtf_tensor),
                               POINTER(mtf_tensor), vp, c_size_t, vp],
         "mtf_debug_wait_test": [c_int64, c_int32],
+        "mtf_debug_contraction": [c_int32, c_int32, POINTER(c_int32), POINTER(c_int32)],
         "mtf_stage_tap_begin": [vp, c_size_t],
         "mtf_stage_tap_end": [POINTER(c_int32)],
         "mtf_stage_tap_entry": [c_int32, POINTER(c_char_p), POINTER(c_size_t), POINTER(c_size_t)],
@@ -653,6 +654,13 @@ def mtf_stage_tap_entry(index: int):
     name, off, size = c_char_p(), c_size_t(), c_size_t()
     _check(_lib.mtf_stage_tap_entry(index, byref(name), byref(off), byref(size)))
     return name.value.decode(), off.value, size.value
+
+
+def mtf_debug_contraction(columns: int = 0, split: int = 0) -> tuple[int, int]:
+    """Testing hook: see mtf_debug_contraction in include/mtf.h.  Returns what the last contraction ran on."""
+    bn, sp = c_int32(), c_int32()
+    _check(_lib.mtf_debug_contraction(int(columns), int(split), byref(bn), byref(sp)))
+    return bn.value, sp.value
 
 
 def mtf_debug_wait_test(limit_cycles: int = 0, withhold_one_signal: bool = False) -> None:

@@ -1754,6 +1754,20 @@ size_t tc_workspace_bytes(const TcParams& t) {
   return (size_t)tiles * t.sk * tc_tile_rows(t) * t.block_n * sizeof(float) + (size_t)tiles * (tc_tile_rows(t) / 32) * 4 * sizeof(unsigned) + 256;
 }
 
+static thread_local bool g_whole_sums = false;
+bool swap_whole_sums(bool on) { const bool was = g_whole_sums; g_whole_sums = on; return was; }
+
+// Testing hook (mtf_debug_contraction): the tiles and split asked for on this thread, and what its last contraction ran on.
+static thread_local ClusterPick g_asked_pick = {0, 0}, g_last_pick = {0, 0};
+mtf_status debug_contraction(int bn, int split, int* ran_bn, int* ran_split) {
+  if (!(bn == 0 && split == 0) && ((bn != 64 && bn != 128) || (split != 1 && split != 2 && split != 4 && split != 8)))
+    return fail(MTF_ERR_INVALID_ARG, "debug_contraction: tiles of 64 or 128 columns with K over 1, 2, 4 or 8 CTAs (0, 0: the library's choice)");
+  g_asked_pick = {bn, split};
+  if (ran_bn) *ran_bn = g_last_pick.bn;
+  if (ran_split) *ran_split = g_last_pick.split;
+  return MTF_OK;
+}
+
 // Which contractions run on 128-row tiles with K over a cluster, and how: the shorter of two estimates of a launch's time,
 // whose constants (microseconds) are fits to launches of 24 shapes from 128 x 1024 x 1024 to 4096 x 8192 x 1024 on each of
 // the eight variants and on gemm_tcgen05_kernel (B200, replayed back to back).  Both sides at some of them, us:
@@ -1763,12 +1777,10 @@ size_t tc_workspace_bytes(const TcParams& t) {
 // There the persistent kernel pays a fixed part and a wave of tiles costs its k-blocks at the rate one SM takes operands in;
 // here a round of two CTAs an SM costs the same k-blocks (at half the reuse), the epilogue, and the exchange between the
 // CTAs of a cluster, which is what keeps the split small.
-static thread_local bool g_whole_sums = false;
-bool swap_whole_sums(bool on) { const bool was = g_whole_sums; g_whole_sums = on; return was; }
-
 static ClusterPick cluster_pick(const TcParams& t, int n_terms, int n_groups) {
   ClusterPick best = {0, 0};
   if (!t.cluster_ok || (g_whole_sums && t.reduce_mode == MTF_REDUCE_WORKSPACE)) return best;
+  if (g_asked_pick.split) return g_asked_pick.split <= (t.K + BK - 1) / BK * n_terms ? g_asked_pick : best;
   const int most = g_whole_sums ? 1 : 8;
   const double sms = sm_count();
   const double kb = (double)((t.K + BK - 1) / BK) * n_terms;
@@ -1922,8 +1934,9 @@ mtf_status launch_tc(const mtf_plan_t& plan, const void* A, const void* B, void*
     if (!workspace || workspace_bytes < need) return fail(MTF_ERR_WORKSPACE_TOO_SMALL, "einsum needs %zu workspace bytes, got %zu", need, workspace_bytes);
     if (reinterpret_cast<uintptr_t>(workspace) & 255) return fail(MTF_ERR_INVALID_ARG, "workspace must be 256-byte aligned");
   }
+  g_last_pick = {0, 0};
   if (!row_softmax) {
-    const ClusterPick pick = cluster_pick(t, n_terms, n_groups);
+    const ClusterPick pick = g_last_pick = cluster_pick(t, n_terms, n_groups);
     if (pick.split)
       return launch_cluster(plan, pick, A, B, C, bias, dtBias, mask, dtMask, resid, dtRes, scale, relu, rsum, workspace, workspace_bytes, stream, n_terms,
                             extra_operands, n_groups, group_operands);

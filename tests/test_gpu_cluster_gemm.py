@@ -1,5 +1,8 @@
-"""bf16 contractions on 128-row tiles with K over a cluster, against the fp64 oracle: every operand order, edges of the
-tiles, every split (few tiles and a longer and longer K), both tile widths, the fused stages and column sums."""
+"""bf16 contractions on 128-row tiles with K over a cluster, against the fp64 oracle.  The tests that ask for a variant run
+every one (tiles of 64 and 128 columns, K over 1, 2, 4 and 8 CTAs) with operand orders, fused stages and column sums, and
+check that it is the one that ran; the others take what the library chooses for few tiles and a longer and longer K."""
+import contextlib
+
 import numpy as np
 import pytest
 
@@ -10,6 +13,67 @@ from test_gpu_einsum import layout, mtf, run_einsum  # noqa: F401
 pytestmark = pytest.mark.gpu
 
 ONE = ([("all", 1)], [])
+VARIANTS = [(columns, split) for columns in (64, 128) for split in (1, 2, 4, 8)]
+
+
+@contextlib.contextmanager
+def asked(mtf, variant):
+    """Contractions inside run on this variant; the last of them is checked."""
+    mtf.mtf_debug_contraction(*variant)
+    try:
+        yield
+    finally:
+        ran = mtf.mtf_debug_contraction(0, 0)
+    assert ran == variant
+
+
+@pytest.mark.parametrize("variant", VARIANTS, ids=str)
+@pytest.mark.parametrize("order", ["ik,kj", "ik,jk", "ki,kj", "ki,jk"])
+def test_every_variant(mtf, variant, order):
+    for m, n, k in ((8, 8, 520), (136, 200, 1032), (264, 72, 512)):
+        size = {"i": m, "j": n, "k": k}
+        a, b = [[(c, size[c]) for c in t] for t in order.split(",")]
+        for dt in ("bf16", "f32"):
+            with asked(mtf, variant):
+                got, ref, _ = run_einsum(mtf, layout(mtf, *ONE), [a, b], [("i", m), ("j", n)], "bf16", dt)
+            assert parity_error(got, ref) <= TOL["bf16"]
+
+
+@pytest.mark.parametrize("variant", VARIANTS, ids=str)
+@pytest.mark.parametrize("out_dtype", ["bf16", "f32"])
+def test_every_variant_with_stages(mtf, variant, out_dtype):
+    size = {"i": 264, "j": 136, "k": 1032}
+    dims = [[(c, size[c]) for c in t] for t in ("ik", "kj")]
+    for out in ("ij", "ji"):
+        for bias in "ij":
+            ep = {"scale": -0.5, "bias": [(bias, size[bias])], "relu": True, "relu_mask": True, "residual": True}
+            with asked(mtf, variant):
+                got, ref, _ = run_einsum(mtf, layout(mtf, *ONE), dims, [(c, size[c]) for c in out], "bf16", out_dtype, epilogue=ep)
+            assert parity_error(got, ref) <= TOL["bf16"]
+
+
+@pytest.mark.parametrize("variant", VARIANTS, ids=str)
+@pytest.mark.parametrize("m", [8, 100, 300])
+def test_every_variant_with_column_sums(mtf, variant, m):
+    """One block of rows: stored by its CTA or gathered inside the cluster; several: partial rows in the workspace, or atomics
+    without one.  All but the last repeat bit for bit."""
+    import torch
+    n, k = 136, 1032
+    x, y, mask = si.normal(3, "x", [m, k], "bf16"), si.normal(3, "y", [k, n], "bf16", k ** -0.5), si.normal(3, "mask", [m, n], "bf16")
+    tx, ty, tm, lay = to_torch(x), to_torch(y), to_torch(mask), layout(mtf, *ONE)
+    ref = ((x.f64 @ y.f64) * (mask.f64 > 0)).sum(0)
+    for scratch in (0, 1 << 20):
+        ws = torch.empty(scratch, dtype=torch.uint8, device="cuda") if scratch else None
+        cols = [torch.full((n,), float("nan"), device="cuda") for _ in range(5)]
+        for col in cols:
+            out = torch.empty(m, n, dtype=torch.bfloat16, device="cuda")
+            ep = mtf.Epilogue(relu_mask=mtf.named(tm, ["i", "j"]), reduce_sum_out=mtf.named(col, ["j"]))
+            with asked(mtf, variant):
+                mtf.mtf_einsum(lay, None, [mtf.named(tx, ["i", "k"]), mtf.named(ty, ["k", "j"])], mtf.named(out, ["i", "j"]), ep, ws)
+        mtf.mtf_device_status()
+        assert parity_error(from_torch(cols[0]), ref) <= TOL["f32"]
+        if scratch or m <= 128:
+            assert all(torch.equal(cols[0], c) for c in cols[1:])
 
 
 @pytest.mark.parametrize("m,n,k", [(8, 8, 8), (128, 64, 64), (136, 72, 640), (40, 200, 1024), (264, 56, 1096), (24, 72, 4096)])
