@@ -159,43 +159,31 @@ __global__ void __launch_bounds__(256) xent_combine_kernel(const float2* __restr
   }
 }
 
-// dlogits[t, v] = (exp(logits[t, v] - lse[t]) - [v == target[t]]) * dloss[t], written over the logits.  kGroup threads own a
-// row (a warp where a row has fewer than 256 pieces of 16 bytes, else the block), so that no index is divided, and keep four
-// pieces in flight each: 188 -> 175 us for 8192 rows of 32768 (6.1 TB/s; one piece in flight and a 64-bit division a piece
-// before).
-template <int kGroup>
+// dlogits[t, v] = (exp(logits[t, v] - lse[t]) - [v == target[t]]) * dloss[t], written over the logits.  Bound by memory: a
+// thread takes single pieces of 16 bytes, a grid of threads apart, in whatever rows they lie.  I: 32-bit indices where they
+// suffice: 8192 rows of 32768 184 -> 176 us (6.1 TB/s) against a 64-bit division a piece, 100 rows 4.6 -> 3.4, 1000 rows of
+// 32768 21.5 -> 18.8.  Two pieces in flight a thread take 192 us and four 211 (the rows a wave of threads works on lie
+// further apart); a block to a row takes 190, and 4 to 6 us for single rows of 32768 and 50000 where this takes 1.5.
+template <typename I>
 __global__ void __launch_bounds__(256) xent_backward_kernel(__nv_bfloat16* __restrict__ logits, const int32_t* __restrict__ targets, const float* __restrict__ lse,
-                                                            const float* __restrict__ dloss, long long n_rows, int vocab) {
+                                                            const float* __restrict__ dloss, I total, I pieces) {
   mtf::chain_wait();
-  constexpr int kRows = 256 / kGroup;
-  const int pieces = vocab / 8, first = threadIdx.x % kGroup;
-  for (long long t = (long long)blockIdx.x * kRows + threadIdx.x / kGroup; t < n_rows; t += (long long)gridDim.x * kRows) {
-    uint4* const row = reinterpret_cast<uint4*>(logits + t * vocab);
+  uint4* const lg = reinterpret_cast<uint4*>(logits);
+  for (I i = (I)blockIdx.x * 256 + threadIdx.x; i < total; i += (I)gridDim.x * 256) {
+    const I t = i / pieces;
     const float l = lse[t], g = dloss[t];
-    const int target = targets[t];
-    for (int p0 = first; p0 < pieces; p0 += 4 * kGroup) {
-      uint4 u[4];
+    const int tg = targets[t] - (int)(i - t * pieces) * 8;
+    float f[8];
+    bf16x8(lg[i], f);
+    uint32_t w[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (p0 + i * kGroup < pieces) u[i] = row[p0 + i * kGroup];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int p = p0 + i * kGroup;
-        if (p >= pieces) break;
-        const int tg = target - p * 8;
-        float f[8];
-        bf16x8(u[i], f);
-        uint32_t w[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float a = (__expf(f[2 * e] - l) - (tg == 2 * e ? 1.f : 0.f)) * g;
-          const float b = (__expf(f[2 * e + 1] - l) - (tg == 2 * e + 1 ? 1.f : 0.f)) * g;
-          __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-          w[e] = *reinterpret_cast<uint32_t*>(&h);
-        }
-        row[p] = make_uint4(w[0], w[1], w[2], w[3]);
-      }
+    for (int e = 0; e < 4; ++e) {
+      const float a = (__expf(f[2 * e] - l) - (tg == 2 * e ? 1.f : 0.f)) * g;
+      const float b = (__expf(f[2 * e + 1] - l) - (tg == 2 * e + 1 ? 1.f : 0.f)) * g;
+      __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+      w[e] = *reinterpret_cast<uint32_t*>(&h);
     }
+    lg[i] = make_uint4(w[0], w[1], w[2], w[3]);
   }
 }
 
@@ -262,10 +250,11 @@ mtf_status launch_xent_combine(const void* partial, int parts, const void* logit
 
 mtf_status launch_xent_backward(void* logits, const int32_t* targets, const float* lse, const float* dloss, int64_t n_rows, int64_t vocab, void* stream) {
   if (n_rows <= 0) return MTF_OK;
-  const bool wide = vocab / 8 >= 256;
-  const long long blocks = std::min<long long>(wide ? n_rows : (n_rows + 7) / 8, (long long)device_sm_count() * 8);
-  if (wide) launch_chained(xent_backward_kernel<256>, (unsigned)blocks, 256, 0, (cudaStream_t)stream, reinterpret_cast<__nv_bfloat16*>(logits), targets, lse, dloss, n_rows, (int)vocab);
-  else launch_chained(xent_backward_kernel<32>, (unsigned)blocks, 256, 0, (cudaStream_t)stream, reinterpret_cast<__nv_bfloat16*>(logits), targets, lse, dloss, n_rows, (int)vocab);
+  const long long pieces = vocab / 8, total = n_rows * pieces, blocks = std::min<long long>((total + 255) / 256, (long long)device_sm_count() * 16);
+  cudaStream_t st = (cudaStream_t)stream;
+  __nv_bfloat16* const lg = reinterpret_cast<__nv_bfloat16*>(logits);
+  if (total < (1LL << 31)) launch_chained(xent_backward_kernel<uint32_t>, (unsigned)blocks, 256, 0, st, lg, targets, lse, dloss, (uint32_t)total, (uint32_t)pieces);
+  else launch_chained(xent_backward_kernel<uint64_t>, (unsigned)blocks, 256, 0, st, lg, targets, lse, dloss, (uint64_t)total, (uint64_t)pieces);
   return after("xent_backward_kernel");
 }
 

@@ -1,5 +1,5 @@
 """Row kernels at lengths between their register sizes: layer norm forward and backward at row lengths around multiples of
-256 (and beyond the lengths that stay in registers), the cross-entropy's gradient for rows of a warp and of a block, and
+256 (and beyond the lengths that stay in registers), the cross-entropy's gradient for few and many, short and long rows, and
 the table gradient for row lengths with and without whole 16-byte pieces; against fp64 arithmetic on the same inputs."""
 import numpy as np
 import pytest
@@ -39,7 +39,7 @@ def test_layernorm_lengths(mtf, n, rows, scratch):
     assert parity_error(from_torch(db), dy.f64.sum(0)) <= TOL["f32"]
 
 
-@pytest.mark.parametrize("vocab", [8, 264, 2040, 2048, 5000, 9000])
+@pytest.mark.parametrize("vocab", [8, 264, 2040, 2048, 5000, 9000, 50000])
 @pytest.mark.parametrize("rows", [1, 9, 1500])
 def test_cross_entropy_gradient(mtf, vocab, rows):
     import torch
