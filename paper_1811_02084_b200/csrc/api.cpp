@@ -96,17 +96,18 @@ mtf_status exec_plan(const mtf_plan_t* P, const mtf_tensor* in, mtf_tensor* out,
                         P->epi.dtRes, scale, relu, rsum, workspace, workspace_bytes, stream, n_terms, extra_operands, row_softmax, n_groups, group_operands);
   } else {
     if (n_terms != 1 || row_softmax || n_groups != 1) return fail(MTF_ERR_UNSUPPORTED, "multi-term, grouped or fused-softmax contraction on the generic kernel");
-    if (P->f32_ok) {
+    if (P->f32_ok && (P->f32_tiled || mtf::contraction_asked())) {
       st = mtf::launch_f32(P->f32, in[0].data, in[1].data, out->data, P->dtC, bias, P->epi.dtBias, mask, P->epi.dtMask, resid, P->epi.dtRes, scale, relu, rsum, stream);
     } else {
       SimtParams s = P->simt;
-    s.A = in[0].data;
-    s.B = P->has_B ? in[1].data : nullptr;
-    s.C = out->data;
-    s.bias = bias; s.mask = mask; s.resid = resid;
-    s.scale = scale; s.relu = relu;
-    s.rsum = rsum;
-    st = mtf::launch_simt(s, rsum_elems, stream);
+      s.A = in[0].data;
+      s.B = P->has_B ? in[1].data : nullptr;
+      s.C = out->data;
+      s.bias = bias; s.mask = mask; s.resid = resid;
+      s.scale = scale; s.relu = relu;
+      s.rsum = rsum;
+      mtf::note_contraction(0, 0);
+      st = mtf::launch_simt(s, rsum_elems, stream);
     }
   }
   if (st != MTF_OK) return st;

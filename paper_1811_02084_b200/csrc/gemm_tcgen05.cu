@@ -1768,6 +1768,9 @@ mtf_status debug_contraction(int bn, int split, int* ran_bn, int* ran_split) {
   return MTF_OK;
 }
 
+bool contraction_asked() { return g_asked_pick.split != 0; }
+void note_contraction(int columns, int split) { g_last_pick = {columns, split}; }
+
 // Which contractions run on 128-row tiles with K over a cluster, and how: the shorter of two estimates of a launch's time,
 // whose constants (microseconds) are fits to launches of 24 shapes from 128 x 1024 x 1024 to 4096 x 8192 x 1024 on each of
 // the eight variants and on gemm_tcgen05_kernel (B200, replayed back to back).  Both sides at some of them, us:

@@ -148,7 +148,8 @@ struct mtf_plan_s {
   int n_reduce_mesh_dims = 0;
   // kernel parameters (pointers filled in at exec time)
   SimtParams simt;
-  bool f32_ok = false;      // generic family: the f32 matrix-product kernel takes this einsum
+  bool f32_ok = false;      // generic family: the f32 matrix-product kernel can take this einsum
+  bool f32_tiled = false;   // ... and is the shorter one
   F32Params f32;
   TcParams tc;
 };
@@ -191,6 +192,7 @@ mtf_status rank_wait(const mtf_layout_t* L, void* stream);
 
 // launchers (defined in the .cu files)
 mtf_status launch_simt(const SimtParams& p, int64_t rsum_elems, void* stream);
+bool f32_tiles_pay(const F32Params& p);
 mtf_status launch_f32(const F32Params& p, const void* A, const void* B, void* C, int dtC, const void* bias, int dtBias, const void* mask, int dtMask,
                       const void* resid, int dtRes, float scale, int relu, float* rsum, void* stream);
 mtf_status launch_tc(const mtf_plan_t& plan, const void* A, const void* B, void* C, const void* bias, int dtBias,
@@ -210,6 +212,9 @@ bool take_independent_hint();
 // While on (this thread): contractions of few tiles add up K in one accumulator as large ones do, so that a value does not
 // depend on how many rows stand beside it.  Returns the old state.
 bool swap_whole_sums(bool on);
+// mtf_debug_contraction: was a tiled kernel asked for on this thread; what its last contraction ran on.
+bool contraction_asked();
+void note_contraction(int columns, int split);
 // Is a kernel family or reduce mode forced on this thread (mtf_plan_force)?
 bool plan_forced();
 // n_groups (1..3) independent einsums with the dims of group 0 (names may differ, sizes and types may

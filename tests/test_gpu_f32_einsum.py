@@ -10,6 +10,32 @@ from test_gpu_einsum import layout, mtf, run_einsum  # noqa: F401
 pytestmark = pytest.mark.gpu
 
 
+@pytest.fixture(autouse=True, params=["asked", "chosen"])
+def tiled(request, mtf):  # noqa: F811
+    """Every test twice: on the tiles, however small the product, and on what the library takes for its size."""
+    asked = request.param == "asked"
+    mtf.mtf_debug_contraction(*((64, 1) if asked else (0, 0)))
+    yield asked
+    ran = mtf.mtf_debug_contraction(0, 0)
+    assert not asked or ran[0] == 64
+
+
+# Batches of small products, single rows and columns, short K: one thread per output is many times faster there
+SMALL = [(100000, 1, 1, 1), (65536, 2, 2, 8), (4096, 4, 4, 4), (20000, 1, 16, 4), (1000, 8, 8, 8), (1, 1, 200000, 1), (1, 200000, 2, 8), (1, 45, 2, 1)]
+
+
+@pytest.mark.parametrize("b,m,n,k", SMALL + [(1, 8, 256, 64), (1, 64, 64, 32), (1, 1000, 520, 40), (64, 40, 40, 200)])
+def test_small_products_stay_with_one_thread_per_output(mtf, tiled, b, m, n, k):
+    import torch
+    x, y = torch.randn(b, m, k, device="cuda"), torch.randn(b, k, n, device="cuda")
+    out = torch.full((b, m, n), float("nan"), device="cuda")
+    mtf.mtf_einsum(layout(mtf, [("all", 1)], []), None, [mtf.named(x, ["b", "i", "k"]), mtf.named(y, ["b", "k", "j"])], mtf.named(out, ["b", "i", "j"]))
+    mtf.mtf_device_status()
+    assert parity_error(from_torch(out), torch.bmm(x.double(), y.double()).cpu().numpy()) <= TOL["f32"]
+    if not tiled:
+        assert (mtf.mtf_debug_contraction() == (0, 0)) == ((b, m, n, k) in SMALL)
+
+
 @pytest.mark.parametrize("m,n,k", [(1, 1, 1), (8, 256, 64), (64, 64, 32), (65, 63, 33), (130, 68, 127), (7, 200, 1023), (300, 36, 256), (1000, 520, 40)])
 @pytest.mark.parametrize("order", ["ik,kj", "ik,jk", "ki,kj", "ki,jk"])
 def test_f32_orders_and_edges(mtf, order, m, n, k):
