@@ -151,3 +151,20 @@ def test_tiles_with_few_rows_leave_the_cluster_together(mtf, m, k):
     mtf.mtf_device_status()
     assert parity_error(from_torch(outs[0]), x.f64 @ y.f64) <= TOL["bf16"]
     assert all(torch.equal(outs[0], o) for o in outs[1:])
+
+
+# which side of the rule a product lies on: few tiles on the cluster kernel; a chip full of 128-row tiles, where rows off
+# 128-byte lines and f32 outputs measured 1.15 to 1.5 times their time on the persistent kernel, there
+@pytest.mark.parametrize("a,b,out,dtype,cluster", [
+    ([128, 4096], [4096, 1024], [128, 1024], "bf16", True), ([512, 1024], [1024, 1024], [512, 1024], "bf16", True),
+    ([2664, 200], [2992, 200], [2664, 2992], "f32", False), ([264, 3032], [264, 1792], [3032, 1792], "bf16", False),
+    ([2160, 264], [3176, 264], [2160, 3176], "f32", False), ([6208, 112], [112, 944], [6208, 944], "f32", False)])
+def test_which_products_it_takes(mtf, a, b, out, dtype, cluster):
+    import torch
+    k = (set(a) & set(b)).pop()
+    sizes = [dict(zip(("i", "k") if a[1] == k else ("k", "i"), a)), dict(zip(("k", "j") if b[0] == k else ("j", "k"), b))]
+    t = [torch.randn(list(s.values()), device="cuda").to(torch.bfloat16) for s in sizes]
+    c = torch.empty(out, dtype=torch.float32 if dtype == "f32" else torch.bfloat16, device="cuda")
+    mtf.mtf_einsum(layout(mtf, *ONE), None, [mtf.named(x, list(s)) for x, s in zip(t, sizes)], mtf.named(c, ["i", "j"]))
+    mtf.mtf_device_status()
+    assert (mtf.mtf_debug_contraction()[1] > 0) == cluster
