@@ -1734,14 +1734,6 @@ static int64_t tc_total_tiles(const TcParams& t) {
   return tiles;
 }
 
-// Scratch for a fused reduce_sum whose column sums are finished in a fixed order: one fp32 row of N per 32-row group
-size_t tc_rsum_partial_bytes(const TcParams& t) {
-  const int rows = tc_tile_rows(t);
-  int64_t groups = ((t.M / t.sm + rows - 1) / rows) * (rows / 32) * t.sm;
-  for (int j = 0; j < t.n_outer; ++j) groups *= t.outer_size[j];
-  return (size_t)groups * t.N * sizeof(float);
-}
-
 size_t tc_workspace_bytes(const TcParams& t) {
   if (t.reduce_mode != MTF_REDUCE_WORKSPACE) {
     if (!t.balance) return 0;
@@ -1785,11 +1777,9 @@ void note_contraction(int columns, int split) { g_last_pick = {columns, split}; 
 // count 1.2 times their estimate, more than one round 1.3 times, and the persistent kernel 0.9 times its own.  Of 4400 drawn
 // products (rows of any multiple of 16 bytes) 4 then take more than 1.03 times their time there (at most 1.15 times; 88, up to
 // 1.5, without the factors), and the mean gain is the same: exp(0.54).
-static ClusterPick cluster_pick(const TcParams& t, int n_terms, int n_groups) {
+static ClusterPick cluster_rule(const TcParams& t, int n_terms, int n_groups, int most) {
   ClusterPick best = {0, 0};
-  if (!t.cluster_ok || (g_whole_sums && t.reduce_mode == MTF_REDUCE_WORKSPACE)) return best;
-  if (g_asked_pick.split) return g_asked_pick.split <= (t.K + BK - 1) / BK * n_terms ? g_asked_pick : best;
-  const int most = g_whole_sums ? 1 : 8;
+  if (!t.cluster_ok) return best;
   const double sms = sm_count();
   const double kb = (double)((t.K + BK - 1) / BK) * n_terms;
   double outer = n_groups;
@@ -1811,6 +1801,22 @@ static ClusterPick cluster_pick(const TcParams& t, int n_terms, int n_groups) {
     }
   }
   return best;
+}
+
+static ClusterPick cluster_pick(const TcParams& t, int n_terms, int n_groups) {
+  if (!t.cluster_ok || (g_whole_sums && t.reduce_mode == MTF_REDUCE_WORKSPACE)) return {0, 0};
+  if (g_asked_pick.split) return g_asked_pick.split <= (t.K + BK - 1) / BK * n_terms ? g_asked_pick : ClusterPick{0, 0};
+  return cluster_rule(t, n_terms, n_groups, g_whole_sums ? 1 : 8);
+}
+
+// Scratch for a fused reduce_sum whose column sums are finished in a fixed order: one fp32 row of N per 32-row group of the
+// persistent kernel's tiles, or per CTA of the cluster kernel (128 / split rows), whichever of the two is more
+size_t tc_rsum_partial_bytes(const TcParams& t) {
+  const int rows = tc_tile_rows(t);
+  int64_t outer = 1;
+  for (int j = 0; j < t.n_outer; ++j) outer *= t.outer_size[j];
+  const int64_t groups = std::max(((t.M / t.sm + rows - 1) / rows) * (rows / 32) * t.sm, (t.M + BM - 1) / BM * cluster_rule(t, 1, 1, 8).split) * outer;
+  return (size_t)groups * t.N * sizeof(float);
 }
 
 template <int BN, int kSplit, bool kEpi>
@@ -1841,6 +1847,18 @@ static mtf_status launch_cluster(const mtf_plan_t& plan, ClusterPick pick, const
                                  const float* group_scale = nullptr) {
   const TcParams& t = plan.tc;
   cudaStream_t st = (cudaStream_t)stream;
+  const bool room = workspace && !(reinterpret_cast<uintptr_t>(workspace) & 15);
+  if (rsum && room) {
+    // column sums: a smaller split where the workspace holds its partial rows (one per CTA) and not the larger one's, so that
+    // they are still finished in a fixed order (a workspace of the size the persistent kernel wants always holds a split of 4)
+    long long blocks = (t.M + BM - 1) / BM;
+    for (int j = 0; j < t.n_outer; ++j) blocks *= t.outer_size[j];
+    const auto need = [&](int split) { return (size_t)blocks * split * t.N * sizeof(float); };
+    int split = pick.split;
+    while (split > 1 && workspace_bytes < need(split)) split /= 2;
+    if (blocks > 1 && workspace_bytes >= need(split)) pick.split = split;
+    note_contraction(pick.bn, pick.split);
+  }
   ClusterArgs a;
   a.M = (int)t.M; a.N = (int)t.N;
   a.n_outer = t.n_outer;
@@ -1866,7 +1884,7 @@ static mtf_status launch_cluster(const mtf_plan_t& plan, ClusterPick pick, const
   const long long groups = row_blocks * pick.split;
   if (rsum) {
     if (row_blocks == 1) (pick.split == 1 ? a.rsum_store : a.rsum_gather) = 1;
-    else if (workspace && !(reinterpret_cast<uintptr_t>(workspace) & 15) && workspace_bytes >= (size_t)groups * t.N * sizeof(float)) a.rsum_partial = reinterpret_cast<float*>(workspace);
+    else if (room && workspace_bytes >= (size_t)groups * t.N * sizeof(float)) a.rsum_partial = reinterpret_cast<float*>(workspace);
     else {
       mtf_status zs = zero_words(rsum, t.N, st);
       if (zs != MTF_OK) return zs;

@@ -153,6 +153,28 @@ def test_tiles_with_few_rows_leave_the_cluster_together(mtf, m, k):
     assert all(torch.equal(outs[0], o) for o in outs[1:])
 
 
+@pytest.mark.parametrize("m,n,k,split", [(200, 512, 2048, 8), (136, 64, 4096, 8), (300, 136, 640, 2)])
+@pytest.mark.parametrize("room", ["reported", "a row per 32 rows"])
+def test_column_sums_repeat_with_the_reported_workspace(mtf, m, n, k, split, room):
+    """... and with one of a partial row per 32 rows, the persistent kernel's, which holds those of a split of 4."""
+    import torch
+    x, y = si.normal(3, "x", [m, k], "bf16"), si.normal(3, "y", [k, n], "bf16", k ** -0.5)
+    tx, ty, lay = to_torch(x), to_torch(y), layout(mtf, *ONE)
+    nx, ny = mtf.named(tx, ["i", "k"]), mtf.named(ty, ["k", "j"])
+    cols = [torch.full((n,), float("nan"), device="cuda") for _ in range(20)]
+    for col in cols:
+        out = mtf.named(torch.empty(m, n, dtype=torch.bfloat16, device="cuda"), ["i", "j"])
+        ep = mtf.Epilogue(relu=True, reduce_sum_out=mtf.named(col, ["j"]))
+        size = mtf.mtf_einsum_workspace_bytes(lay, [nx, ny], out, ep)
+        if room != "reported":
+            size = (m + 127) // 128 * 4 * n * 4
+        mtf.mtf_einsum(lay, None, [nx, ny], out, ep, torch.empty(size, dtype=torch.uint8, device="cuda"))
+    mtf.mtf_device_status()
+    assert mtf.mtf_debug_contraction()[1] == (split if room == "reported" else min(split, 4))
+    assert parity_error(from_torch(cols[0]), np.maximum(x.f64 @ y.f64, 0).sum(0)) <= TOL["f32"]
+    assert all(torch.equal(cols[0], c) for c in cols[1:])
+
+
 # which side of the rule a product lies on: few tiles on the cluster kernel; a chip full of 128-row tiles, where rows off
 # 128-byte lines and f32 outputs measured 1.15 to 1.5 times their time on the persistent kernel, there
 @pytest.mark.parametrize("a,b,out,dtype,cluster", [
