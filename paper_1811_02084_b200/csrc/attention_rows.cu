@@ -365,7 +365,13 @@ attention_rows_kernel(const __grid_constant__ CUtensorMap map_own, const __grid_
 #pragma unroll
         for (int i = 0; i < 32; ++i) m4[i & 3] = fmaxf(m4[i & 3], __uint_as_float(v[i]));
         const float m2 = fmaxf(mx, fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])));
-        if (m2 == -INFINITY) continue;                     // no live column of this row yet
+        if (m2 == -INFINITY) {                             // no column above -inf yet; a NaN among them (fmaxf drops it) stays in the sum
+          float t = 0.f;
+#pragma unroll
+          for (int i = 0; i < 32; ++i) t += __uint_as_float(v[i]);
+          if (t != t) sum = t;
+          continue;
+        }
         const float off = m2 * sl2;
         float s4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -379,7 +385,7 @@ attention_rows_kernel(const __grid_constant__ CUtensorMap map_own, const __grid_
       const float top = fmaxf(fmaxf(ms[0], ms[1]), fmaxf(ms[2], ms[3])), off = top * sl2;
       float total = 0.f;
 #pragma unroll
-      for (int p = 0; p < 4; ++p) total += ms[p] == -INFINITY ? 0.f : ss[p] * ex2(fmaf(ms[p], sl2, -off));
+      for (int p = 0; p < 4; ++p) total += ms[p] == -INFINITY ? ss[p] : ss[p] * ex2(fmaf(ms[p], sl2, -off));
       const float inv = 1.f / total;
       for (int j = 0; j < nk; ++j) {
         const int c0 = j * 128 + part * 32, n = twice ? nk + j : j;
