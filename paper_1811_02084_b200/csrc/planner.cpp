@@ -109,9 +109,10 @@ mtf_status slice_box(const mtf_layout_t* L, const std::vector<Dim>& dims, int64_
 void plan_key(int n_in, const mtf_tensor* in, const mtf_tensor* out, const mtf_epilogue* epi, int fk, int fr, std::string* key) {
   std::string& k = *key;
   k.clear();
+  auto add_i = [&](int v) { k.append(reinterpret_cast<const char*>(&v), sizeof(v)); };      // (whole: a type that does not exist is no other's)
   auto add_t = [&](const mtf_tensor* t) {
-    k += (char)t->dtype;
-    k += (char)t->ndim;
+    add_i((int)t->dtype);
+    add_i(t->ndim);
     for (int i = 0; i < t->ndim; ++i) {
       k += t->dims[i].name ? t->dims[i].name : "?";
       k += '\0';
@@ -127,8 +128,8 @@ void plan_key(int n_in, const mtf_tensor* in, const mtf_tensor* out, const mtf_e
     k += epi->relu ? 'r' : '-';
     k += (epi->scale != 1.f) ? 's' : '-';
     if (epi->bias) { k += 'b'; add_t(epi->bias); }
-    if (epi->relu_mask) { k += 'm'; k += (char)epi->relu_mask->dtype; }
-    if (epi->residual) { k += 'a'; k += (char)epi->residual->dtype; }
+    if (epi->relu_mask) { k += 'm'; add_i((int)epi->relu_mask->dtype); }
+    if (epi->residual) { k += 'a'; add_i((int)epi->residual->dtype); }
     if (epi->reduce_sum_out) { k += 'S'; add_t(epi->reduce_sum_out); }
   }
 }

@@ -255,6 +255,19 @@ def test_kernel_family_and_reduce_groups_of_the_benchmark_shapes():
     assert info["kernel_kind"] == mtf.MTF_KERNEL_SIMT and info["n_slices"] == 4
 
 
+def test_a_cached_plan_serves_no_unknown_type():
+    L = mtf.mtf_layout(mtf.mtf_mesh_create([("all", 1)]), [])
+    for dtype in ("bf16", "f32"):
+        a, b, c = mtf.desc([("i", 64), ("k", 64)], dtype), mtf.desc([("k", 64), ("j", 64)], dtype), mtf.desc([("i", 64), ("j", 64)], dtype)
+        mtf.mtf_einsum_workspace_bytes(L, [a, b], c)
+        for t in (a, b, c):
+            good, t.c.dtype = t.c.dtype, t.c.dtype + 256
+            with pytest.raises(mtf.MtfError) as e:
+                mtf.mtf_einsum_workspace_bytes(L, [a, b], c)
+            assert e.value.code == "MTF_ERR_INVALID_ARG"
+            t.c.dtype = good
+
+
 def test_forced_choices_are_validated():
     L, _ = both([("all", 2)], [("k", "all")])
     a, b, c = mtf.desc([("i", 128), ("k", 256)], "f32"), mtf.desc([("k", 256), ("j", 128)], "f32"), mtf.desc([("i", 128), ("j", 128)], "f32")
