@@ -243,8 +243,8 @@ mtf_status einsum_row_softmax(const mtf_layout_t* layout, const mtf_tensor* a, c
 // (generic kernel, workspace reduce mode): the caller then chains einsums through the residual stage.
 mtf_status einsum_terms(const mtf_layout_t* layout, int n_terms, const mtf_tensor (*terms)[2], mtf_tensor* out,
                         const mtf_epilogue* epilogue, void* workspace, size_t workspace_bytes, void* stream);
-// dkk = scale * sum_l ds q and dvv = sum_l weights do in one launch (grouped, causal blocks left out).
-// MTF_ERR_UNSUPPORTED when the plan cannot (generic kernel, a kernel or reduce mode was asked for): the caller runs two einsums.
+// dkk = scale * sum_l ds q and dvv = sum_l weights do in one launch (grouped, causal blocks left out).  Every shape and layout
+// that the core by rows takes has the tensor-core plan this needs; MTF_ERR_UNSUPPORTED otherwise (there is no fallback).
 mtf_status attention_kv(const mtf_layout_t* layout, const mtf_tensor* ds, const mtf_tensor* q, mtf_tensor* dkk, float scale, const mtf_tensor* weights,
                         const mtf_tensor* dout, mtf_tensor* dvv, int causal, void* stream);
 mtf_status launch_attention_kv(const mtf_plan_t& plan, const void* ds, const void* q, void* dkk, float scale, const void* weights, const void* dout, void* dvv,

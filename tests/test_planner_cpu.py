@@ -268,6 +268,18 @@ def test_a_cached_plan_serves_no_unknown_type():
             t.c.dtype = good
 
 
+@pytest.mark.parametrize("mesh,rules", [([("all", 1)], []), ([("r", 2), ("c", 4)], [("batch", "r"), ("heads", "c")])])
+@pytest.mark.parametrize("L,D", [(8, 64), (8, 128), (40, 64), (200, 128), (640, 64), (1000, 128)])
+def test_key_and_value_gradients_of_the_rows_core_have_a_tensor_core_plan(mesh, rules, L, D):
+    """The attention core by rows leaves dkk and dvv to one grouped contraction, for which it has no other way."""
+    lay = mtf.mtf_layout(mtf.mtf_mesh_create(mesh), rules)
+    ds = mtf.desc([("batch", 2), ("heads", 4), ("length", L), ("memory_length", L)], "bf16")
+    q = mtf.desc([("batch", 2), ("length", L), ("heads", 4), ("d_k", D)], "bf16")
+    plan = mtf.mtf_einsum_plan(lay, [ds, q], mtf.desc([("batch", 2), ("memory_length", L), ("heads", 4), ("d_k", D)], "bf16"))
+    info = mtf.mtf_plan_info(plan)
+    assert info["kernel_kind"] == mtf.MTF_KERNEL_TCGEN05 and info["group_size"] == 1
+
+
 def test_forced_choices_are_validated():
     L, _ = both([("all", 2)], [("k", "all")])
     a, b, c = mtf.desc([("i", 128), ("k", 256)], "f32"), mtf.desc([("k", 256), ("j", 128)], "f32"), mtf.desc([("i", 128), ("j", 128)], "f32")
