@@ -1772,10 +1772,10 @@ void note_contraction(int columns, int split) { g_last_pick = {columns, split}; 
 // There the persistent kernel pays a fixed part and a wave of tiles costs its k-blocks at the rate one SM takes operands in;
 // here a round of two CTAs an SM costs the same k-blocks (at half the reuse), the epilogue, and the exchange between the
 // CTAs of a cluster, which is what keeps the split small.
-// The fits are to rows on 128-byte lines, and a full chip misses them where rows are not, where the output is f32 and where
-// the last tile of a row is mostly empty (2664 x 2992 x 200: 13.9 us there, 19.7 here, estimated 13.1).  So two CTAs on an SM
-// count 1.2 times their estimate, more than one round 1.3 times, and the persistent kernel 0.9 times its own.  Of 4400 drawn
-// products (rows of any multiple of 16 bytes) 4 then take more than 1.03 times their time there (at most 1.15 times; 88, up to
+// Products that fill the chip with 128-row tiles stray from the fits, those whose operands' rows do not lie on 128-byte lines
+// most (2664 x 2992 x 200: 13.9 us there, 19.7 here, estimated 13.1).  So more than one round counts 1.1 times its estimate; with
+// rows off the lines a round of two CTAs an SM counts 1.2 times, more than one 1.3 times, and the persistent kernel 0.9 instead of
+// 0.95 times its own.  Of 4400 drawn products 6 then take more than 1.03 times their time there (at most 1.15 times; 88, up to
 // 1.5, without the factors), and the mean gain is the same: exp(0.54).
 static ClusterPick cluster_rule(const TcParams& t, int n_terms, int n_groups, int most) {
   ClusterPick best = {0, 0};
@@ -1787,7 +1787,8 @@ static ClusterPick cluster_rule(const TcParams& t, int n_terms, int n_groups, in
   const int64_t rows = t.cta_pair ? 2 * BM : BM;
   const double tiles = (double)((t.M / t.sm + rows - 1) / rows * t.sm) * (double)((t.N / t.sn + t.block_n - 1) / t.block_n * t.sn) * outer;
   const double per_kb = t.cta_pair ? (t.block_n == 256 ? 0.36 : 0.24) : (t.block_n == 256 ? 0.45 : t.block_n == 128 ? 0.33 : 0.27);
-  double best_us = 0.9 * (7.0 + std::ceil(tiles / std::floor(sms / (t.cta_pair ? 2 : 1))) * kb * per_kb);
+  const bool on_lines = t.a_ld % 64 == 0 && t.b_ld % 64 == 0;
+  double best_us = (on_lines ? 0.95 : 0.9) * (7.0 + std::ceil(tiles / std::floor(sms / (t.cta_pair ? 2 : 1))) * kb * per_kb);
   for (int bn = 64; bn <= 128; bn += 64) {
     const double ctas1 = (double)((t.M + BM - 1) / BM) * (double)((t.N + bn - 1) / bn) * outer;
     for (int split = 1; split <= most && split <= kb; split *= 2) {
@@ -1795,7 +1796,7 @@ static ClusterPick cluster_rule(const TcParams& t, int n_terms, int n_groups, in
       const bool two = ctas > sms;
       const double exchange = split == 1 ? 0.0 : (split == 2 ? 1.2 : split == 4 ? 1.8 : 2.8) + (two ? 1.0 : 0.0);
       const double per = bn == 64 ? (two ? 0.34 : 0.27) : (two ? 0.44 : 0.34);
-      const double rounds = std::ceil(ctas / (2.0 * sms)), surer = rounds > 1.0 ? 1.3 : two ? 1.2 : 1.0;
+      const double rounds = std::ceil(ctas / (2.0 * sms)), surer = rounds > 1.0 ? (on_lines ? 1.1 : 1.3) : two && !on_lines ? 1.2 : 1.0;
       const double us = surer * (2.2 + rounds * (part * per + (bn == 64 ? 0.8 : 1.8) + exchange));
       if (us < best_us) { best_us = us; best = {bn, split}; }
     }
