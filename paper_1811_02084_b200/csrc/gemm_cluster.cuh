@@ -325,6 +325,7 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       else atomicAdd(a.rsum + n0 + c, x);
     }
     if (kSplit > 1 && a.rsum_gather) {
+      __syncwarp();                  // (the aligned barriers take whole warps)
       asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
       cluster_sync();
       if (part == 0 && c < BN && n0 + c < a.N) {
@@ -339,6 +340,7 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   }
   if (*abort_flag)
     for (int i = 0; i < 2000; ++i) __nanosleep(1000);      // failure path: copies and MMAs in flight land before the resources go away
+  __syncwarp();
   if (kSplit > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");      // the cluster has read this CTA's part
   __syncthreads();
   if (a.late_wait) asm volatile("griddepcontrol.wait;" ::: "memory");
