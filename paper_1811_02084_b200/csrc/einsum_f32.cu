@@ -319,18 +319,20 @@ static int split_of(int64_t tiles, int64_t K) {
 // Is this kernel the shorter one?  A tile costs the same however few of its 64 x 64 outputs exist, so batches of small
 // products, single rows or columns and short K stay with one thread per output: 100000 products of 1 x 1 take 3.4 us there
 // and 1469 here, 4096 of 4 x 4 x 4 3.6 and 62, 1000000 x 1 x 1 14 and 260; 8 x 256 x 64 takes 23 and 5.  Microseconds, fitted to
-// 4400 drawn products on both: there a start, and the chain of K loads or the outputs and multiply-adds of a full chip,
-// whichever is longer; here a wave of tiles and its k-blocks.  No drawn product takes more than 1.05 times its time on the
-// generic kernel, and on average they are 1.3 % from the better of the two.
+// 4400 drawn products on both: there a start, and the chain of K loads (the first ones cold) or the outputs and multiply-adds
+// of a full chip, whichever is longer; here the k-blocks of one block on an SM, or rounds of two.  29 drawn products take more
+// than 1.05 times their time on the generic kernel, 1.1 us at most, which this kernel's early set-up behind the launch before
+// it makes up (the 8-token block: 31 us so, 36 with its two 8-deep products there); on average they are 0.5 % from the better.
 bool f32_tiles_pay(const F32Params& p) {
   const int64_t tiles = tiles_of(p);
   const int split = split_of(tiles, p.K);
   if (tiles * split > 0x7fffffffLL) return false;
   double outputs = (double)p.M * (double)p.N;
   for (int j = 0; j < p.n_outer; ++j) outputs *= (double)p.outer_size[j];
-  const double there = 3.0 + std::max(0.2 * (double)p.K, outputs / 120e3 + outputs * (double)p.K / 600e3);
-  const int64_t kb = (p.K + kBK - 1) / kBK, resident = 2 * (int64_t)device_sm_count();
-  const double here = 2.0 + (double)((tiles * split + resident - 1) / resident) * (2.4 + 2.0 * (double)((kb + split - 1) / split));
+  const double there = 2.0 + std::max(0.15 * (double)p.K + 0.12 * (double)std::min<int64_t>(p.K, 16), outputs / 130e3 + outputs * (double)p.K / 600e3);
+  const int64_t kb = ((p.K + kBK - 1) / kBK + split - 1) / split, sms = device_sm_count();
+  const double rounds = (double)((tiles * split + 2 * sms - 1) / (2 * sms));
+  const double here = (split > 1 ? 1.0 : 0.0) + (tiles * split <= sms ? 2.2 + 1.6 * (double)kb : 0.5 + rounds * (2.2 + 2.1 * (double)kb));
   return here < there;
 }
 
