@@ -122,6 +122,7 @@ __device__ __forceinline__ float4 ld_peer(uint32_t addr, uint32_t rank) {
   return v;
 }
 __device__ __forceinline__ void cluster_sync() {
+  __syncwarp();                      // (the aligned barrier takes whole warps; lanes leave the loops before it one by one)
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
