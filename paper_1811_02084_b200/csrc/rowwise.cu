@@ -204,9 +204,9 @@ layernorm_bwd_dx_kernel(const __nv_bfloat16* __restrict__ dy, const __nv_bfloat1
 }
 
 // Rows of NCH * 256 columns, or with kTail of up to that many (a multiple of 8): a lane keeps its NCH pieces of 8 columns in
-// registers, so the row is read from memory once and all its loads are in flight together.  (Lengths that are no multiple
-// of 256 re-read the row per pass before, and their backward pass read it again for the parameter gradients and added those
-// up with atomics: together 830 -> 690 us of a decoder layer forward and backward, most of it this.)
+// registers, so the row is read from memory once and all its loads are in flight together.  (Against a kernel that re-reads
+// the row per pass, whose backward pass reads it again for the parameter gradients: 16384 rows of 1000 forward 17.9 -> 14.2 us,
+// backward 47 -> 34.)
 template <int NCH, bool kTail>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 layernorm_fwd_rows_kernel(const __nv_bfloat16* __restrict__ x, const float* __restrict__ gamma, const float* __restrict__ beta,
@@ -369,12 +369,21 @@ layernorm_bwd_rows_kernel(const __nv_bfloat16* __restrict__ dy, const __nv_bfloa
     } else {
       for (int w = 0; w < kWarpsPerBlock; ++w) {
         if ((int)(threadIdx.x >> 5) == w) {
+          // 16 bytes at a time (of single floats, eight lanes would share a bank), all loads before the first store: with n known
+          // only at run time the two planes may overlap for all the compiler knows, and load and store would alternate
+          float4 was[kAccRegs][4];
+          auto at = [&](int i, int q) { return reinterpret_cast<float4*>(sh + (q < 2 ? 0 : n) + i * 256 + lane * 8) + (q & 1); };
 #pragma unroll
           for (int i = 0; i < kAccRegs; ++i)
 #pragma unroll
-            for (int e = 0; e < 8 && in(i); ++e) {
-              sh[i * 256 + lane * 8 + e] += ag[i][e];
-              sh[n + i * 256 + lane * 8 + e] += ab[i][e];
+            for (int q = 0; q < 4; ++q)
+              if (in(i)) was[i][q] = *at(i, q);
+#pragma unroll
+          for (int i = 0; i < kAccRegs; ++i)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const float* const add = (q < 2 ? ag[i] : ab[i]) + 4 * (q & 1);
+              if (in(i)) *at(i, q) = make_float4(was[i][q].x + add[0], was[i][q].y + add[1], was[i][q].z + add[2], was[i][q].w + add[3]);
             }
         }
         __syncthreads();
