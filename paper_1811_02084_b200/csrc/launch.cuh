@@ -3,9 +3,20 @@
 // us a launch on a stream of short ones.)
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 namespace mtf {
+
+// A driver call that wants a current context, which a thread has only once a runtime call that needs the device was made on it
+// (cuTensorMapEncodeTiled as a thread's first call: CUDA_ERROR_INVALID_CONTEXT).
+template <typename F>
+CUresult in_context(F call) {
+  CUresult r = call();
+  int dev = 0;
+  if (r == CUDA_ERROR_INVALID_CONTEXT && cudaGetDevice(&dev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess) r = call();
+  return r;
+}
 
 __device__ __forceinline__ void chain_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
