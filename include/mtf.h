@@ -308,7 +308,7 @@ mtf_status mtf_layernorm_forward(const mtf_layout_t* layout, const mtf_tensor* x
  * workspace (device, 16-byte aligned; may be NULL): with at least mtf_layernorm_workspace_bytes(row
  * length) bytes the two column sums are added up in a fixed order (per-block partial sums, then one
  * pass in block order) and repeat bit for bit from run to run; with less, or for row lengths that
- * report 0 bytes, they are accumulated with fp32 atomics into the zeroed outputs (order not fixed). */
+ * report 0 bytes (more than 2048 columns), they are accumulated with fp32 atomics into the zeroed outputs (order not fixed). */
 mtf_status mtf_layernorm_backward(const mtf_layout_t* layout, const mtf_tensor* dy, const mtf_tensor* x, const mtf_tensor* stats, const mtf_tensor* gamma,
                                   const mtf_tensor* residual, mtf_tensor* dx, mtf_tensor* dgamma, mtf_tensor* dbeta, void* workspace,
                                   size_t workspace_bytes, void* stream);

@@ -6,8 +6,9 @@
 // memory_length, reduce_sum over d_model) with component-wise work around it.  A row is handled by
 // one warp and never leaves the GPU, so the group sum over a split reduced dimension is the warp's
 // own shuffle reduction over the whole row.  The column sums (reduce out the token dims, i.e. the
-// gradient Allreduce of Algorithm 1 under a batch split) accumulate per block and finish with fp32
-// atomics.  All loads and stores are 16-byte vectors, coalesced along the row.
+// gradient Allreduce of Algorithm 1 under a batch split) accumulate per block and finish in block order
+// where the caller gives scratch for them, with fp32 atomics otherwise and for rows of more than 2048
+// columns.  All loads and stores are 16-byte vectors, coalesced along the row.
 #include <algorithm>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -261,7 +262,7 @@ layernorm_fwd_rows_kernel(const __nv_bfloat16* __restrict__ x, const float* __re
 // Backward for rows of NCH * 256 columns (kTail: of up to that many), dx and the parameter gradients in one pass over dy and x:
 // a persistent grid of 8-warp blocks, every warp walks rows with both rows in registers and keeps
 // its lanes' partial dgamma / dbeta sums in registers; at the end the block adds them up in shared
-// memory and issues one fp32 atomic per column and block.
+// memory and leaves one partial row (or, without scratch, issues one fp32 atomic per column).
 // kSmemAcc (more than 1024 columns, whose up to 128 partial sums per lane do not fit the registers next to
 // the two rows): every warp keeps its partial sums in a shared-memory strip of its own instead.
 template <int NCH, bool kTail, bool kSmemAcc>
@@ -533,9 +534,10 @@ mtf_status launch_layernorm_fwd(const void* x, const float* gamma, const float* 
   return check("layernorm_fwd_kernel");
 }
 
-// Bytes of scratch with which the parameter gradients are summed in a fixed order (0: this row length always uses atomics)
+// Bytes of scratch with which the parameter gradients are summed in a fixed order (0: rows of this length are not kept in
+// registers, or not taken at all, and the sums always use atomics)
 size_t layernorm_bwd_scratch_bytes(int n) {
-  if (n != 256 && n != 512 && n != 1024 && n != 2048) return 0;
+  if (n > 2048 || n % 8) return 0;
   return (size_t)device_sm_count() * 2 * 2 * n * sizeof(float);
 }
 
