@@ -75,8 +75,10 @@ typedef struct { void* data; mtf_dtype dtype; int32_t ndim; const mtf_dim* dims;
  * reduce_sum_out : optional second output (Section 6 "Reduction" fused into the einsum): an f32
  *             tensor whose dims are a subset of the output dims; it receives the sum of t (taken
  *             after the relu_mask stage, before the residual and the cast) over the other output
- *             dims.  The library zeroes it on the stream before the launch and accumulates with
- *             fp32 atomics (order not fixed).  Used for dbias = sum over tokens of dhp.
+ *             dims.  On the tensor-core path, with the workspace that the plan reports, it is added
+ *             up in a fixed order and repeats bit for bit; otherwise it is zeroed on the stream
+ *             before the launch and accumulated with fp32 atomics (order not fixed).  Used for
+ *             dbias = sum over tokens of dhp.
  * NULL pointers / relu = 0 / scale = 1 switch a stage off.  The struct is read during planning
  * only for which stages are on and their descriptors; data pointers are read at exec time. */
 typedef struct {
@@ -177,7 +179,8 @@ mtf_status mtf_rank_wait(const mtf_layout_t* bound_layout, void* stream);
 mtf_status mtf_einsum_plan(const mtf_layout_t* layout, int32_t n_in, const mtf_tensor* in_desc,
                            const mtf_tensor* out_desc, const mtf_epilogue* epilogue, mtf_plan_t** out);
 mtf_status mtf_plan_destroy(mtf_plan_t* plan);
-/* Scratch bytes mtf_einsum_exec needs (0 unless the reduce mode is WORKSPACE). */
+/* Scratch bytes mtf_einsum_exec needs (reduce mode WORKSPACE) or, for a fused reduce_sum_out, wants: with less its sums are
+ * accumulated with atomics.  Else 0. */
 mtf_status mtf_plan_workspace_bytes(const mtf_plan_t* plan, size_t* bytes);
 /* Per-processor cost counts (Table 1; Appendix B): multiply-adds of the local einsum, values
  * entering the Allreduce (one output slice when a split dimension is reduced out, else 0), local
@@ -354,6 +357,9 @@ typedef struct {
 typedef struct {
   mtf_tensor *dwq, *dwk, *dwv, *dwo, *dln1_gamma, *dln1_beta, *dw, *dbias /* may be NULL */, *dv, *dln2_gamma, *dln2_beta;
 } mtf_decoder_grads;
+/* The attention half adds up every contraction in one accumulator for any number of tokens; mtf_attention_forward called
+ * by itself may cut a sum into parts where there are few tokens.  There the layer and its composition from the calls above
+ * can differ in where a sum is rounded to bf16, and in what follows from it. */
 mtf_status mtf_decoder_layer_forward(const mtf_layout_t* layout, const mtf_tensor* x, const mtf_decoder_params* params,
                                      int32_t causal, float eps, const mtf_decoder_saved* saved, mtf_tensor* out,
                                      void* workspace, size_t workspace_bytes, void* stream);

@@ -504,7 +504,7 @@ mtf_status mtf_decoder_layer_forward(const mtf_layout_t* layout, const mtf_tenso
   // s1 = x + Attention(x) (the residual rides in the output projection's epilogue); a = LN1(s1)
   // What the attention half computes decides the signs of the hidden units through the layer norm: a sum in another order
   // moves one value in 10^4 to its bf16 neighbour, that moves every row a little, and 1 to 3 % of `a` with it (measured on 480,
-  // 768 and 248 tokens), so its contractions keep one order of additions for every number of tokens.
+  // 768 and 248 tokens), so its contractions add up in one accumulator for every number of tokens (the core differs by length).
   const bool was = mtf::swap_whole_sums(true);
   st = mtf_attention_forward(layout, x, p->wq, p->wk, p->wv, p->wo, causal, x, sv->q, sv->kk, sv->vv, sv->weights, sv->o, sv->s1, workspace, workspace_bytes, stream);
   mtf::swap_whole_sums(was);
