@@ -336,3 +336,11 @@ def test_decoder_layer(mtf, mesh_dims, rules):
     _, res = run_decoder_stagewise(mtf, layout(mtf, mesh_dims, rules), inp)
     ref, _ = run_decoder_oracle(inp, None)
     end_to_end_report({k: from_torch(res[k]) for k in ref}, ref, "decoder layer", rms_gate=None)
+
+
+def test_decoder_layer_with_the_attention_core_by_rows(mtf):
+    """Heads of 128 and 200 positions: the layer's attention half runs on the core by rows, its contractions unsplit."""
+    inp = decoder_case(16, 2, 200, 256, 2, 128, 320)
+    _, res = run_decoder_stagewise(mtf, layout(mtf, [("all", 1)], []), inp)
+    ref, _ = run_decoder_oracle(inp, None)
+    end_to_end_report({k: from_torch(res[k]) for k in ref}, ref, "decoder layer, core by rows", rms_gate=None)
