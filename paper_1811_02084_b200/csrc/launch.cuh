@@ -23,6 +23,10 @@ __device__ __forceinline__ void chain_wait() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// The wait alone, for a kernel of one short block per row: a launch let in at the start takes the free block slots of whichever
+// SM has them, and when that launch is another such kernel its blocks then lie unevenly.  This way it is let in as the blocks end.
+__device__ __forceinline__ void chain_wait_only() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // The error is left for the caller's cudaGetLastError.
 template <typename... P, typename... A>
 void launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... args) {
