@@ -492,8 +492,9 @@ mtf_status mtf_debug_wait_test(int64_t limit_cycles, int32_t withhold_one_signal
 /* Testing hook: tensor-core contractions launched afterwards by this thread, where they may run on 128-row tiles with K
  * over a cluster of CTAs (nothing forced through mtf_plan_force, no row softmax), run on tiles of `columns` (64 or 128)
  * columns with K over `split` (1, 2, 4 or 8) CTAs, provided K has that many 64-deep blocks; 0, 0 gives the choice back to
- * the library.  While something is asked for, f32 contractions of matrix-product form run on their 64 x 64 tiles (the split
- * is the library's) where they might be left to one thread per output.  ran_columns, ran_split (may be NULL): what this
+ * the library.  While something is asked for, f32 contractions of matrix-product form run on tiles (the split is the
+ * library's) where they might be left to one thread per output: with 64 columns on the 64 x 64 tiles of plain FP32 arithmetic, with 128 on
+ * the tensor cores, in bf16 pieces of the values (128 rows a tile).  ran_columns, ran_split (may be NULL): what this
  * thread's last contraction before the call ran on; 0, 0 if on the persistent or the generic kernel. */
 mtf_status mtf_debug_contraction(int32_t columns, int32_t split, int32_t* ran_columns, int32_t* ran_split);
 /* Number of kernels this library has launched from this process (all threads). */

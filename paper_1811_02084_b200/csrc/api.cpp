@@ -22,6 +22,7 @@ mtf_status read_attention_status(int* code);
 mtf_status launch_permute_copy(const void* src, void* dst, int elem_bytes, int ndim, const int64_t* sizes, const int64_t* sstr, const int64_t* dstr, void* stream);
 mtf_status read_attention_bwd_status(int* code);
 mtf_status read_attention_rows_status(int* code);
+mtf_status read_f32_status(int* code);
 }  // namespace mtf
 
 using mtf::Dim;
@@ -96,8 +97,9 @@ mtf_status exec_plan(const mtf_plan_t* P, const mtf_tensor* in, mtf_tensor* out,
                         P->epi.dtRes, scale, relu, rsum, workspace, workspace_bytes, stream, n_terms, extra_operands, row_softmax, n_groups, group_operands);
   } else {
     if (n_terms != 1 || row_softmax || n_groups != 1) return fail(MTF_ERR_UNSUPPORTED, "multi-term, grouped or fused-softmax contraction on the generic kernel");
-    if (P->f32_ok && (P->f32_tiled || mtf::contraction_asked())) {
-      st = mtf::launch_f32(P->f32, in[0].data, in[1].data, out->data, P->dtC, bias, P->epi.dtBias, mask, P->epi.dtMask, resid, P->epi.dtRes, scale, relu, rsum, stream);
+    const int asked = mtf::contraction_asked();
+    if (P->f32_ok && (P->f32_tiled || asked)) {
+      st = ((asked ? asked == 128 : P->f32_tensor_cores) ? mtf::launch_f32_tc : mtf::launch_f32)(P->f32, in[0].data, in[1].data, out->data, P->dtC, bias, P->epi.dtBias, mask, P->epi.dtMask, resid, P->epi.dtRes, scale, relu, rsum, stream);
     } else {
       SimtParams s = P->simt;
       s.A = in[0].data;
@@ -689,6 +691,7 @@ mtf_status mtf_device_status(int32_t* code) {
   if ((st = mtf::read_attention_status(&rc)) != MTF_OK) return st;
   if (!rc && (st = mtf::read_attention_bwd_status(&rc)) != MTF_OK) return st;
   if (!rc && (st = mtf::read_attention_rows_status(&rc)) != MTF_OK) return st;
+  if (!rc && (st = mtf::read_f32_status(&rc)) != MTF_OK) return st;
   if (!rc && (st = mtf::read_row_status(&rc)) != MTF_OK) return st;
   if (rc) {
     if (code) *code = rc;

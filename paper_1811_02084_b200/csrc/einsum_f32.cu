@@ -1,6 +1,6 @@
 // f32 einsums with the structure of a (batched) matrix product: C[o..][m][n] = sum_k A[o..][m][k] B[o..][k][n], each of
-// M, N, K one merged strided dimension, up to three batch dimensions.  Plain FP32 arithmetic throughout (no tensor
-// cores, whose 32-bit formats carry fewer bits): the path on which a layout's numbers are checked.  Component-wise
+// M, N, K one merged strided dimension, up to three batch dimensions.  Plain FP32 arithmetic, for products of short K and
+// batches of a few rows; the others run on the tensor cores in pieces (einsum_f32_tc.cu).  Component-wise
 // stages of Section 6 / Section 7 run on the sum before the store, as in the generic kernel.
 //
 // Bound: the FP32 pipe at large sizes, launch and load latency at small ones.  A block of 256 threads owns a 64 x 64
@@ -324,17 +324,20 @@ static int split_of(int64_t tiles, int64_t K) {
 // of a full chip, whichever is longer; here the k-blocks of one block on an SM, or rounds of two.  29 drawn products take more
 // than 1.05 times their time on the generic kernel, 1.1 us at most, which this kernel's early set-up behind the launch before
 // it makes up (the 8-token block: 31 us so, 36 with its two 8-deep products there); on average they are 0.5 % from the better.
+double f32_tile_us(const F32Params& p) {
+  const int64_t tiles = tiles_of(p), sms = device_sm_count();
+  const int split = split_of(tiles, p.K);
+  const int64_t kb = ((p.K + kBK - 1) / kBK + split - 1) / split;
+  const double rounds = (double)((tiles * split + 2 * sms - 1) / (2 * sms));
+  return (split > 1 ? 1.0 : 0.0) + (tiles * split <= sms ? 2.2 + 1.6 * (double)kb : 0.5 + rounds * (2.2 + 2.1 * (double)kb));
+}
 bool f32_tiles_pay(const F32Params& p) {
   const int64_t tiles = tiles_of(p);
-  const int split = split_of(tiles, p.K);
-  if (tiles * split > 0x7fffffffLL) return false;
+  if (tiles * split_of(tiles, p.K) > 0x7fffffffLL) return false;
   double outputs = (double)p.M * (double)p.N;
   for (int j = 0; j < p.n_outer; ++j) outputs *= (double)p.outer_size[j];
   const double there = 2.0 + std::max(0.15 * (double)p.K + 0.12 * (double)std::min<int64_t>(p.K, 16), outputs / 130e3 + outputs * (double)p.K / 600e3);
-  const int64_t kb = ((p.K + kBK - 1) / kBK + split - 1) / split, sms = device_sm_count();
-  const double rounds = (double)((tiles * split + 2 * sms - 1) / (2 * sms));
-  const double here = (split > 1 ? 1.0 : 0.0) + (tiles * split <= sms ? 2.2 + 1.6 * (double)kb : 0.5 + rounds * (2.2 + 2.1 * (double)kb));
-  return here < there;
+  return f32_tile_us(p) < there;
 }
 
 mtf_status launch_f32(const F32Params& p, const void* A, const void* B, void* C, int dtC, const void* bias, int dtBias, const void* mask, int dtMask,

@@ -1761,7 +1761,7 @@ mtf_status debug_contraction(int bn, int split, int* ran_bn, int* ran_split) {
   return MTF_OK;
 }
 
-bool contraction_asked() { return g_asked_pick.split != 0; }
+int contraction_asked() { return g_asked_pick.split ? g_asked_pick.bn : 0; }
 void note_contraction(int columns, int split) { g_last_pick = {columns, split}; }
 
 // Which contractions run on 128-row tiles with K over a cluster, and how: the shorter of two estimates of a launch's time,

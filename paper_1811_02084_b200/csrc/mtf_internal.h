@@ -150,6 +150,7 @@ struct mtf_plan_s {
   SimtParams simt;
   bool f32_ok = false;      // generic family: the f32 matrix-product kernel can take this einsum
   bool f32_tiled = false;   // ... and is the shorter one
+  bool f32_tensor_cores = false;   // ... on the tensor cores
   F32Params f32;
   TcParams tc;
 };
@@ -193,8 +194,12 @@ mtf_status rank_wait(const mtf_layout_t* L, void* stream);
 // launchers (defined in the .cu files)
 mtf_status launch_simt(const SimtParams& p, int64_t rsum_elems, void* stream);
 bool f32_tiles_pay(const F32Params& p);
+double f32_tile_us(const F32Params& p);
+bool f32_tensor_cores_pay(const F32Params& p);
 mtf_status launch_f32(const F32Params& p, const void* A, const void* B, void* C, int dtC, const void* bias, int dtBias, const void* mask, int dtMask,
                       const void* resid, int dtRes, float scale, int relu, float* rsum, void* stream);
+mtf_status launch_f32_tc(const F32Params& p, const void* A, const void* B, void* C, int dtC, const void* bias, int dtBias, const void* mask, int dtMask,
+                         const void* resid, int dtRes, float scale, int relu, float* rsum, void* stream);
 mtf_status launch_tc(const mtf_plan_t& plan, const void* A, const void* B, void* C, const void* bias, int dtBias,
                      const void* mask, int dtMask, const void* resid, int dtRes, float scale, int relu, float* rsum,
                      void* workspace, size_t workspace_bytes, void* stream, int n_terms = 1,
@@ -212,8 +217,8 @@ bool take_independent_hint();
 // While on (this thread): contractions of few tiles add up K in one accumulator as large ones do, so that a value does not
 // depend on how many rows stand beside it.  Returns the old state.
 bool swap_whole_sums(bool on);
-// mtf_debug_contraction: was a tiled kernel asked for on this thread; what its last contraction ran on.
-bool contraction_asked();
+// mtf_debug_contraction: columns of the tiles asked for on this thread (0: none); what its last contraction ran on.
+int contraction_asked();
 void note_contraction(int columns, int split);
 // Is a kernel family or reduce mode forced on this thread (mtf_plan_force)?
 bool plan_forced();

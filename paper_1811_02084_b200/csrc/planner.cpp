@@ -535,6 +535,7 @@ mtf_status make_plan(const mtf_layout_t* L, int n_in, const mtf_tensor* in, cons
   // ---- kernel family and reduce mode ----
   P->f32_ok = force_kernel != MTF_KERNEL_SIMT && plan_f32(P.get());      // (forcing the generic kernel means that kernel)
   P->f32_tiled = P->f32_ok && f32_tiles_pay(P->f32);
+  P->f32_tensor_cores = P->f32_tiled && f32_tensor_cores_pay(P->f32);
   std::string why;
   const int asked_kernel = force_kernel;
   const int force_single_cta = force_kernel == 2 ? 1 : 0;     // testing hook: tensor cores without CTA pairs

@@ -1,0 +1,104 @@
+"""The f32 products that run on the tensor cores in bf16 pieces: edges of the 128 x 64 tile, of the 64-deep stage and its 16-deep
+steps, every split of K, operand orders, the fused stages, values whose pieces leave bf16's range, and the error
+against 64 bits beside that of plain FP32 arithmetic."""
+import numpy as np
+import pytest
+
+from helpers import TOL, from_torch, parity_error
+from test_gpu_einsum import layout, mtf, run_einsum  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+ONE = ([("all", 1)], [])
+
+
+@pytest.fixture
+def asked(mtf):  # noqa: F811
+    mtf.mtf_debug_contraction(128, 1)
+    yield
+    assert mtf.mtf_debug_contraction(0, 0)[0] == 128
+
+
+@pytest.mark.parametrize("m,n,k", [(1, 1, 1), (128, 64, 64), (129, 65, 65), (127, 63, 16), (5, 200, 17), (260, 36, 1000), (8, 64, 33), (1000, 520, 130)])
+@pytest.mark.parametrize("order", ["ik,kj", "ik,jk", "ki,kj", "ki,jk"])
+def test_orders_and_edges(mtf, asked, order, m, n, k):  # noqa: F811
+    size = {"i": m, "j": n, "k": k}
+    a, b = [[(c, size[c]) for c in t] for t in order.split(",")]
+    for out, dt in ((["i", "j"], "f32"), (["j", "i"], "f32"), (["i", "j"], "bf16")):
+        got, ref, _ = run_einsum(mtf, layout(mtf, *ONE), [a, b], [(c, size[c]) for c in out], "f32", dt)
+        assert parity_error(got, ref) <= TOL[dt]
+
+
+@pytest.mark.parametrize("m,n,k", [(8, 256, 64), (77, 101, 300), (520, 130, 64)])
+def test_stages_and_column_sums(mtf, asked, m, n, k):  # noqa: F811
+    import torch
+    size = {"i": m, "j": n, "k": k}
+    dims = [[(c, size[c]) for c in t] for t in ("ik", "kj")]
+    for out in ("ij", "ji"):
+        for bias in "ij":
+            ep = {"scale": -0.5, "bias": [(bias, size[bias])], "relu": True, "relu_mask": True, "residual": True}
+            got, ref, _ = run_einsum(mtf, layout(mtf, *ONE), dims, [(c, size[c]) for c in out], "f32", epilogue=ep)
+            assert parity_error(got, ref) <= TOL["f32"]
+    x, y = torch.randn(m, k, device="cuda"), torch.randn(k, n, device="cuda")
+    o, col = torch.empty(m, n, device="cuda"), torch.full((n,), float("nan"), device="cuda")
+    mtf.mtf_einsum(layout(mtf, *ONE), None, [mtf.named(x, ["i", "k"]), mtf.named(y, ["k", "j"])], mtf.named(o, ["i", "j"]),
+                   mtf.Epilogue(relu=True, reduce_sum_out=mtf.named(col, ["j"])))
+    assert parity_error(from_torch(col), (x.double() @ y.double()).relu().sum(0).cpu().numpy()) <= TOL["f32"]
+
+
+def product(mtf, x, y, columns):  # noqa: F811
+    import torch
+    o = torch.full((x.shape[0], y.shape[1]), float("nan"), device="cuda")
+    mtf.mtf_debug_contraction(columns, 1)
+    mtf.mtf_einsum(layout(mtf, *ONE), None, [mtf.named(x, ["i", "k"]), mtf.named(y, ["k", "j"])], mtf.named(o, ["i", "j"]))
+    assert mtf.mtf_debug_contraction(0, 0)[0] == columns
+    mtf.mtf_device_status()
+    return o
+
+
+@pytest.mark.parametrize("k", [16, 64, 256, 1000, 4096])
+def test_error_is_no_larger_than_plain_arithmetic(mtf, k):  # noqa: F811
+    """Both within a few roundings of the sum; the pieces' rounding is below that of one chain of f32 additions."""
+    import torch
+    torch.manual_seed(k)
+    x, y = torch.randn(384, k, device="cuda"), torch.randn(k, 192, device="cuda")
+    ref = x.double() @ y.double()
+    err = [((product(mtf, x, y, c).double() - ref).norm() / ref.norm()).item() for c in (64, 128)]
+    assert err[1] <= err[0]
+
+
+@pytest.mark.parametrize("k", [40, 520])
+def test_values_outside_the_pieces_range(mtf, k):  # noqa: F811
+    """Infinities, NaN, the type's largest values and values whose last piece is below bf16's smallest come out as plain f32 arithmetic has them."""
+    import torch
+    torch.manual_seed(1)
+    x, y = torch.randn(200, k, device="cuda"), torch.randn(k, 100, device="cuda")
+    x[3, 5], x[17, 0], x[40, k - 1], x[41, 7] = float("inf"), float("nan"), -float("inf"), float("inf")
+    x[60] = torch.where(torch.arange(k, device="cuda") % 2 == 0, 3.4e38, 0.0)      # rounds to infinity as a bf16
+    y[:, 9] = 0.0                                                                       # infinity times zero
+    y[:, 10] = torch.where(torch.arange(k, device="cuda") == 0, 0.5, 0.0)
+    x[90] = float(np.finfo(np.float32).min)
+    y[:, 11] = 0.0
+    y[2, 11] = 1.0
+    x[100] *= 1e-36
+    y[:, 20] *= 1e-37
+    got = product(mtf, x, y, 128).cpu().numpy()
+    ref = (x.cpu().double().numpy() @ y.cpu().double().numpy())
+    f32 = np.where(np.abs(ref) > 3.4028235e38, np.sign(ref) * np.inf, ref)
+    same = np.isnan(ref) == np.isnan(got)
+    same &= np.isinf(f32) == np.isinf(got)
+    same[[60, 90]] |= np.isin(np.arange(100), [9, 10, 11], invert=True)      # (sums of many huge terms pass through infinities in any f32 order; single terms don't)
+    assert same.all()
+    ok = np.isfinite(f32) & np.isfinite(got) & (np.abs(f32) > 1e-30)
+    scale = np.abs(x.cpu().double().numpy()) @ np.abs(y.cpu().double().numpy())
+    assert (np.abs(got - f32)[ok] <= k * 6e-8 * scale[ok]).all()
+    tiny = got[100], ref[100]
+    assert (np.abs(tiny[0] - tiny[1]) <= k * 6e-8 * scale[100] + 1e-44 * k).all()
+
+
+def test_pieces_are_chosen_by_size(mtf):  # noqa: F811
+    import torch
+    mtf.mtf_debug_contraction(0, 0)
+    for m, n, k, ran in ((1024, 1024, 256, 128), (1024, 256, 1024, 128), (8, 256, 64, 128), (256, 64, 16, 64), (1000, 500, 32, 64)):
+        x, y, o = torch.randn(m, k, device="cuda"), torch.randn(k, n, device="cuda"), torch.empty(m, n, device="cuda")
+        mtf.mtf_einsum(layout(mtf, *ONE), None, [mtf.named(x, ["i", "k"]), mtf.named(y, ["k", "j"])], mtf.named(o, ["i", "j"]))
+        assert mtf.mtf_debug_contraction()[0] == ran, (m, n, k)
