@@ -249,7 +249,7 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
 
   if (warp == 0) {
     // ------------------------------- TMA producer -------------------------------
-    if (lane == 0) {
+    if (mtf::elect_one()) {
       StepIter it, pf;
       it.init(blockIdx.x, gridDim.x, a.units, nb, a.causal);
       // the tiles of P are asked into L2 kPrefetch steps before their load into shared memory is issued: the rings hold
@@ -294,7 +294,7 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     }
   } else if (warp == 1) {
     // ------------------------------- MMA issuer ---------------------------------
-    if (lane == 0) {
+    if (mtf::elect_one()) {
       StepIter cur, nxt;
       cur.init(blockIdx.x, gridDim.x, a.units, nb, a.causal);
       nxt = cur;

@@ -197,7 +197,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
 
   if (warp == 0) {
     // ------------------------------- TMA producer -------------------------------
-    if (lane == 0) {
+    if (mtf::elect_one()) {
       long long tile_seq = 0, unit_seq = -1;
       bool ok = true;
       for (long long g = g0; ok && g < g1; ++g, ++tile_seq) {
@@ -225,7 +225,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     }
   } else if (warp == 1) {
     // ------------------------------- MMA issuer ---------------------------------
-    if (lane == 0) {
+    if (mtf::elect_one()) {
       long long tile_seq = 0, unit_seq = -1;
       uint32_t pu[kPBufs] = {0u, 0u, 0u, 0u};          // uses of every chunk buffer so far
       const uint64_t dP0 = smem_desc(sP, 0), dV0 = smem_desc(sV, 1), dQ0 = smem_desc(sQ, 0), dK0 = smem_desc(sK, 0);

@@ -206,7 +206,7 @@ attention_rows_kernel(const __grid_constant__ CUtensorMap map_own, const __grid_
 
   if (warp == 0) {
     // ------------------------------- TMA loads ----------------------------------
-    if (lane == 0) {
+    if (mtf::elect_one()) {
       bool ok = true;
       int seq = 0, tiles = 0;
       auto block = [&](const CUtensorMap* map, int j) {
@@ -242,7 +242,7 @@ attention_rows_kernel(const __grid_constant__ CUtensorMap map_own, const __grid_
     }
   } else if (warp == 1) {
     // ------------------------------- MMA issue ----------------------------------
-    if (lane == 0) {
+    if (mtf::elect_one()) {
       const uint32_t id_s = idesc_of(0, 128), id_acc = idesc_of(1, D);
       const uint64_t d_own = smem_desc(base + S::own, 0);
       int seq = 0, sbuf = 0;                       // key-side blocks taken, logits (dP) blocks issued
@@ -299,7 +299,7 @@ attention_rows_kernel(const __grid_constant__ CUtensorMap map_own, const __grid_
     }
   } else if (warp == 2) {
     // ------------------------------- TMA stores ---------------------------------
-    if (lane == 0) {
+    if (mtf::elect_one()) {
       const CUtensorMap* const map = kBwd ? &map_ds : &map_p;
       if (a.zeros)
         for (int j = nk; j < n_blocks; ++j)

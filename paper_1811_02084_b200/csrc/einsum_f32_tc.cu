@@ -25,6 +25,7 @@
 #include <cmath>
 #include <mutex>
 
+#include "launch.cuh"
 #include "mtf_internal.h"
 
 namespace {
@@ -95,11 +96,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* v) {
       : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
         "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
       : "r"(taddr) : "memory");
-}
-__device__ __forceinline__ bool elect_one() {
-  uint32_t p;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
-  return p != 0;
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // 128B-swizzled boxes: K-major (a row of 128 bytes holds 64 k of one m|n), or MN-major (64 m|n of one k; the next 64 m|n 8 KB on)
@@ -362,7 +358,7 @@ __global__ void __launch_bounds__(kThreads, 1) einsum_f32_tc_kernel(const __grid
       __syncthreads();
       if (warp == 0) {
         fence_after();
-        if (elect_one()) issue(c, u);
+        if (mtf::elect_one()) issue(c, u);
         __syncwarp();
       }
     }

@@ -180,7 +180,7 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (mtf::elect_one()) {
       int stage = 0;
       uint32_t phase = 0;
       for (int kb = kb0; kb < kb1; ++kb) {
@@ -208,7 +208,7 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (mtf::elect_one()) {
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a.a_mn_major << 15) | ((uint32_t)a.b_mn_major << 16) |
                              ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
       const uint32_t a_step = a.a_mn_major ? 2048u : 32u, b_step = a.b_mn_major ? 2048u : 32u;
@@ -219,9 +219,9 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         if (!(ok = mbar_wait(full_bar(stage), phase, 0xA10 + stage, abort_flag))) break;
         tcgen05_fence_after();
         const uint32_t sa = ring + stage * kStage, sb = sa + kAStageBytes;
+        const uint64_t da = make_smem_desc(sa, a.a_mn_major), db = make_smem_desc(sb, a.b_mn_major);
 #pragma unroll
-        for (int k = 0; k < BK / 16; ++k)
-          umma_bf16<false>(tmem, make_smem_desc(sa + k * a_step, a.a_mn_major), make_smem_desc(sb + k * b_step, a.b_mn_major), idesc, (kb > kb0 || k) ? 1u : 0u);
+        for (int k = 0; k < BK / 16; ++k) umma_bf16<false>(tmem, da + k * (a_step >> 4), db + k * (b_step >> 4), idesc, (kb > kb0 || k) ? 1u : 0u);
         umma_commit<false>(empty_bar(stage), 0);
         if (++stage == kStages) { stage = 0; phase ^= 1u; }
       }

@@ -797,7 +797,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 
   if (warp == 0) {
     // ------------------------------- TMA producer -------------------------------
-    if (lane == 0) {
+    if (mtf::elect_one()) {
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
@@ -885,7 +885,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     }
   } else if (warp == 1) {
     // ------------------------------- MMA issuer (even CTA of a pair only) -------
-    if (lane == 0 && leader) {
+    if (leader && mtf::elect_one()) {
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a.a_mn_major << 15) |
                              ((uint32_t)a.b_mn_major << 16) | ((uint32_t)((kWide ? 256 : a.block_n) >> 3) << 17) | ((uint32_t)(kPairRows >> 4) << 24);
       // completion signals: this pair's two CTAs, and every CTA whose loads land in this pair's tiles
