@@ -72,7 +72,7 @@ struct BwdArgs {
   __nv_bfloat16* dq;             // [B, L, H, 64]
   __nv_bfloat16* dk;
   __nv_bfloat16* dv;
-  long long units;               // B * H
+  int units;                     // B * H
 };
 
 __device__ __forceinline__ uint32_t s_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -168,21 +168,29 @@ __device__ __forceinline__ void sts_v4(uint32_t addr, uint32_t x, uint32_t y, ui
 // gradients); per pass key blocks j, per key block query blocks i (under the causal limit from j on).  Every role walks
 // the same sequence.
 struct StepIter {
-  long long u, units, stride;
+  int u, units, stride, H;
+  int b, h;                          // the pair's batch entry and head
   int nb, causal;
   int pass, j, i;
-  long long step_seq, s1_seq, kv_seq, k_seq, unit_seq;      // counts of steps / steps of pass 1 / key blocks (both passes) / key blocks of pass 1 / pairs before this one
-  long long dpu0;                    // dP tiles before this step (one per step of pass 1)
+  // Where this step's tiles stand in the rings of three and how often its slot was used before (parity): all steps, and steps
+  // of pass 1.  32-bit counters that advance with the step: every role works these out once a step, on the path between its
+  // hand-overs.  With 64-bit counts, their remainders and divisions there and elected issue missing, 256 pairs of 512 positions took
+  // 158 us, now 114; the elected threads alone brought about 130.
+  int slot, s1slot;
+  uint32_t par, s1par;
+  uint32_t s1_seq, kv_seq, k_seq, unit_seq;      // counts of steps of pass 1 / key blocks (both passes) / key blocks of pass 1 / pairs before this one
+  uint32_t dpu0;                     // dP tiles before this step (one per step of pass 1)
   // Rows of at most 256 leave tensor-memory columns [128, 256) free (dq takes 64 per query block): dP then alternates
   // between two buffers, so the next step's dP is computed while the warps still read this one.
   __device__ int dp_buf() const { return nb <= 2 ? (int)(dpu0 & 1) : 0; }
-  __device__ long long dp_use() const { return nb <= 2 ? (dpu0 >> 1) : dpu0; }      // earlier uses of this step's buffer
+  __device__ uint32_t dp_use() const { return nb <= 2 ? (dpu0 >> 1) : dpu0; }      // earlier uses of this step's buffer
   __device__ uint32_t dp_col() const { return dp_buf() ? 128u : 384u; }
   bool valid;
-  __device__ void init(long long first, long long stride_, long long units_, int nb_, int causal_) {
-    u = first; stride = stride_; units = units_; nb = nb_; causal = causal_;
-    pass = 0; j = 0; i = 0; step_seq = 0; s1_seq = 0; kv_seq = 0; k_seq = 0; unit_seq = 0; dpu0 = 0;
+  __device__ void init(int first, int stride_, int units_, int H_, int nb_, int causal_) {
+    u = first; stride = stride_; units = units_; H = H_; nb = nb_; causal = causal_;
+    pass = 0; j = 0; i = 0; slot = 0; s1slot = 0; par = 0; s1par = 0; s1_seq = 0; kv_seq = 0; k_seq = 0; unit_seq = 0; dpu0 = 0;
     valid = u < units;
+    b = u / H; h = u - b * H;
   }
   // dP exists in pass 1 only, in one buffer
   __device__ bool last_of_pass0() const { return pass == 0 && j == nb - 1 && i == nb - 1; }
@@ -191,9 +199,12 @@ struct StepIter {
   __device__ bool first_of_unit() const { return pass == 0 && j == 0 && first_i(); }
   __device__ bool last_of_unit() const { return pass == 1 && j == nb - 1 && i == nb - 1; }
   __device__ void advance() {
-    if (pass == 1) ++dpu0;
-    ++step_seq;
-    if (pass == 1) ++s1_seq;
+    if (++slot == kRing) { slot = 0; par ^= 1u; }
+    if (pass == 1) {
+      ++dpu0;
+      ++s1_seq;
+      if (++s1slot == kRing) { s1slot = 0; s1par ^= 1u; }
+    }
     if (i + 1 < nb) { ++i; return; }
     ++kv_seq;
     if (pass == 1) ++k_seq;
@@ -204,6 +215,7 @@ struct StepIter {
     ++unit_seq;
     u += stride;
     valid = u < units;
+    b = u / H; h = u - b * H;
   }
 };
 
@@ -251,23 +263,22 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     // ------------------------------- TMA producer -------------------------------
     if (mtf::elect_one()) {
       StepIter it, pf;
-      it.init(blockIdx.x, gridDim.x, a.units, nb, a.causal);
+      it.init((int)blockIdx.x, (int)gridDim.x, a.units, a.H, nb, a.causal);
       // the tiles of P are asked into L2 kPrefetch steps before their load into shared memory is issued: the rings hold
       // two steps' worth of loads in flight, which alone does not cover the latency of HBM
       constexpr int kPrefetch = 6;
       pf = it;
       auto prefetch_p = [&](const StepIter& t) {
-        const int pb = (int)(t.u / a.H), ph = (int)(t.u % a.H);
-        tma_prefetch_4d(&map_p, t.j * 128, t.i * 128, ph, pb);
-        tma_prefetch_4d(&map_p, t.j * 128 + 64, t.i * 128, ph, pb);
+        tma_prefetch_4d(&map_p, t.j * 128, t.i * 128, t.h, t.b);
+        tma_prefetch_4d(&map_p, t.j * 128 + 64, t.i * 128, t.h, t.b);
       };
       for (int n = 0; n < kPrefetch && pf.valid; ++n) { prefetch_p(pf); pf.advance(); }
       bool ok = true;
       while (ok && it.valid) {
-        const int b = (int)(it.u / a.H), h = (int)(it.u % a.H);
+        const int b = it.b, h = it.h;
         if (pf.valid) { prefetch_p(pf); pf.advance(); }
-        const int slot = (int)(it.step_seq % kRing);
-        const uint32_t par = (uint32_t)(it.step_seq / kRing) & 1u;
+        const int slot = it.slot;
+        const uint32_t par = it.par;
         const uint32_t kvpar = (uint32_t)it.kv_seq & 1u;
         if (it.first_i()) {      // a new key block: V first (the next step's dP wants it), K after this step's tiles
           if (!(ok = mb_wait(bar(B_V_EMPTY), kvpar ^ 1u, 0xA01, abort_flag))) break;
@@ -296,18 +307,18 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     // ------------------------------- MMA issuer ---------------------------------
     if (mtf::elect_one()) {
       StepIter cur, nxt;
-      cur.init(blockIdx.x, gridDim.x, a.units, nb, a.causal);
+      cur.init((int)blockIdx.x, (int)gridDim.x, a.units, a.H, nb, a.causal);
       nxt = cur;
       if (nxt.valid) nxt.advance();
-      long long n_dp = 0;                      // dP tiles issued so far (one per step of pass 1)
-      long long n_dv = 0;                      // dvv contributions issued so far (one per step of pass 1)
+      uint32_t n_dp = 0;                      // dP tiles issued so far (one per step of pass 1)
+      uint32_t n_dv = 0;                      // dvv contributions issued so far (one per step of pass 1)
       bool ok = true;
       const uint32_t id_dp = idesc_of(0, 0, 128), id_kv = idesc_of(1, 1, 64), id_dq = idesc_of(0, 1, 64);
       // pass 0, one step: O_i += P_ij vv_j (M = queries, N = d_v, k = keys; A K-major over two 64-key boxes, B MN-major) into the
       // columns where dq_i will accumulate in pass 1.  Nothing of it concerns the warps until the pass ends.
       auto issue_o = [&](const StepIter& t) -> bool {
-        const int slot = (int)(t.step_seq % kRing);
-        const uint32_t par = (uint32_t)(t.step_seq / kRing) & 1u;
+        const int slot = t.slot;
+        const uint32_t par = t.par;
         if (t.first_of_unit() && !mb_wait(bar(B_DQ_EMPTY), ((uint32_t)t.unit_seq & 1u) ^ 1u, 0xB08, abort_flag)) return false;   // the previous pair's dq has been read out
         if (t.first_i() && !mb_wait(bar(B_V_FULL), (uint32_t)t.kv_seq & 1u, 0xB01, abort_flag)) return false;
         if (!mb_wait(bar(B_QDO_FULL + slot), par, 0xB02, abort_flag)) return false;      // (an empty phase in pass 0: keeps the ring's phases in step)
@@ -326,8 +337,8 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       };
       // dP of a step of pass 1: wants do of the step, V of its key block and the dP columns read out by the warps
       auto issue_dp = [&](const StepIter& t) -> bool {
-        const int slot = (int)(t.step_seq % kRing);
-        const uint32_t par = (uint32_t)(t.step_seq / kRing) & 1u;
+        const int slot = t.slot;
+        const uint32_t par = t.par;
         if (t.first_i() && !mb_wait(bar(B_V_FULL), (uint32_t)t.kv_seq & 1u, 0xB01, abort_flag)) return false;
         if (!mb_wait(bar(B_QDO_FULL + slot), par, 0xB02, abort_flag)) return false;
         if (!mb_wait(bar(B_DP_EMPTY + t.dp_buf()), ((uint32_t)t.dp_use() & 1u) ^ 1u, 0xB03, abort_flag)) return false;      // the buffer's previous dP has been read out
@@ -343,8 +354,8 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       // dvv_j += P^T do_i of a step of pass 1 (M = keys, N = d_v, k = queries; both operands MN-major).  It needs nothing
       // from the warps, and once it has run they may overwrite the tile of P with dS.
       auto issue_dv = [&](const StepIter& t) -> bool {
-        const int slot = (int)(t.step_seq % kRing);
-        const uint32_t par = (uint32_t)(t.step_seq / kRing) & 1u;
+        const int slot = t.slot;
+        const uint32_t par = t.par;
         if (!mb_wait(bar(B_P_FULL + slot), par, 0xB04, abort_flag)) return false;
         if (t.first_i() && !mb_wait(bar(B_DKV_EMPTY), ((uint32_t)t.k_seq & 1u) ^ 1u, 0xB06, abort_flag)) return false;   // the previous key block's dkk, dvv have been read out
         fence_after();
@@ -352,7 +363,7 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         const uint32_t acc = t.first_i() ? 0u : 1u;
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks) umma(tmem + kColDV, da + (uint64_t)(ks * (2048 >> 4)), db + (uint64_t)(ks * (2048 >> 4)), id_kv, acc | (uint32_t)ks);
-        umma_commit(bar(B_PV_DONE + (int)(t.s1_seq % kRing)));
+        umma_commit(bar(B_PV_DONE + t.s1slot));
         ++n_dv;
         return true;
       };
@@ -363,7 +374,7 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
           if (nxt.valid) nxt.advance();
           continue;
         }
-        const int slot = (int)(cur.step_seq % kRing);
+        const int slot = cur.slot;
         if (n_dp == cur.s1_seq && !(ok = issue_dp(cur))) break;
         if (n_dv == cur.s1_seq && !(ok = issue_dv(cur))) break;
         // ahead of this step's remaining MMAs: the next step's dP (as soon as the warps have this step's dP in registers)
@@ -372,8 +383,8 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
           if (!(ok = issue_dp(nxt))) break;
           if (!nxt.first_i() && !(ok = issue_dv(nxt))) break;
         }
-        const int s1slot = (int)(cur.s1_seq % kRing);
-        if (!(ok = mb_wait(bar(B_DS_FULL + s1slot), (uint32_t)(cur.s1_seq / kRing) & 1u, 0xB05, abort_flag))) break;      // dS stands where P stood
+        const int s1slot = cur.s1slot;
+        if (!(ok = mb_wait(bar(B_DS_FULL + s1slot), cur.s1par, 0xB05, abort_flag))) break;      // dS stands where P stood
         if (cur.first_i() && !(ok = mb_wait(bar(B_K_FULL), (uint32_t)cur.k_seq & 1u, 0xB07, abort_flag))) break;
         fence_after();
         const uint32_t acc_kv = cur.first_i() ? 0u : 1u;
@@ -405,13 +416,8 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     const int row_l = q * 32 + lane;               // row inside a 128-row block
     const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16);
     const uint32_t sw = (uint32_t)(row_l & 7);
-    auto wait_all = [&](int b, uint32_t parity, int code) -> bool {      // all lanes wait (lane 0 polls first)
-      int w_ok = 1;
-      if (lane == 0) w_ok = mb_wait(bar(b), parity, code, abort_flag) ? 1 : 0;
-      w_ok = __shfl_sync(0xffffffffu, w_ok, 0);
-      if (!w_ok) return false;
-      bool mine_ok = lane == 0 ? true : mb_wait(bar(b), parity, code, abort_flag);
-      return __all_sync(0xffffffffu, mine_ok);
+    auto wait_all = [&](int b, uint32_t parity, int code) -> bool {      // all lanes wait
+      return __all_sync(0xffffffffu, mb_wait(bar(b), parity, code, abort_flag));
     };
     auto store_row = [&](__nv_bfloat16* dst, const uint32_t* r0, const uint32_t* r1, float s) {      // 64 fp32 -> one 128-byte row
       uint4* d4 = reinterpret_cast<uint4*>(dst);
@@ -425,13 +431,13 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                                pack2(__uint_as_float(r1[g * 8 + 4]) * s, __uint_as_float(r1[g * 8 + 5]) * s), pack2(__uint_as_float(r1[g * 8 + 6]) * s, __uint_as_float(r1[g * 8 + 7]) * s));
     };
     StepIter it;
-    it.init(blockIdx.x, gridDim.x, a.units, nb, a.causal);
+    it.init((int)blockIdx.x, (int)gridDim.x, a.units, a.H, nb, a.causal);
     float D0 = 0.f, D1 = 0.f, D2 = 0.f, D3 = 0.f;      // D of this thread's row in each of the pair's query blocks
     bool ok = true;
     while (ok && it.valid) {
-      const int b = (int)(it.u / a.H), h = (int)(it.u % a.H);
-      const int slot = (int)(it.step_seq % kRing);
-      const uint32_t par = (uint32_t)(it.step_seq / kRing) & 1u;
+      const int b = it.b, h = it.h;
+      const int slot = it.slot;
+      const uint32_t par = it.par;
       uint32_t r0[32], r1[32];
       if (it.pass == 0) {
         // pass 0 belongs to the MMA thread (O_i = sum_j P_ij vv_j in fp32, in the columns of dq_i).  When it ends, every warp
@@ -485,13 +491,9 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                              pack2(bf_lo(pv.z) * (__uint_as_float(rr[4]) - Dr), bf_hi(pv.z) * (__uint_as_float(rr[5]) - Dr)),
                              pack2(bf_lo(pv.w) * (__uint_as_float(rr[6]) - Dr), bf_hi(pv.w) * (__uint_as_float(rr[7]) - Dr)));
       }
-      const int s1slot = (int)(it.s1_seq % kRing);
-      {   // dS goes where this tile of P stands: its last reader, the dvv MMAs of this step, must have run
-        int w_ok = 1;
-        if (lane == 0) w_ok = mb_wait(bar(B_PV_DONE + s1slot), (uint32_t)(it.s1_seq / kRing) & 1u, 0xC03, abort_flag) ? 1 : 0;
-        w_ok = __shfl_sync(0xffffffffu, w_ok, 0);
-        if (!w_ok) { ok = false; break; }
-      }
+      const int s1slot = it.s1slot;
+      // dS goes where this tile of P stands: its last reader, the dvv MMAs of this step, must have run
+      if (!(ok = wait_all(B_PV_DONE + s1slot, it.s1par, 0xC03))) break;
       if (a.ds_dump) {      // (testing: the bf16 values the two contractions below consume)
         uint4* dd = reinterpret_cast<uint4*>(a.ds_dump + ((((long long)b * a.H + h) * L + it.i * 128 + row_l) * L + it.j * 128 + half * 64));
 #pragma unroll
@@ -589,6 +591,7 @@ mtf_status launch_attention_bwd_fused(const void* q, const void* kk, const void*
   for (const void* p : {q, kk, vv, weights, dout, (const void*)dq, (const void*)dkk, (const void*)dvv})
     if (!p || (reinterpret_cast<uintptr_t>(p) & 15)) return fail(MTF_ERR_INVALID_ARG, "fused attention backward: NULL or misaligned tensor");
   if (B * H <= 0) return MTF_OK;
+  if (B * H > 0x3fffffff) return fail(MTF_ERR_UNSUPPORTED, "fused attention backward: %lld pairs", (long long)(B * H));
   CUtensorMap mq, mk, mv, md, mp;
   const int64_t qd[4] = {64, L, H, B}, qs[3] = {H * 64, 64, L * H * 64};
   const int64_t pd[4] = {L, L, H, B}, ps[3] = {L, L * L, H * L * L};
@@ -603,7 +606,7 @@ mtf_status launch_attention_bwd_fused(const void* q, const void* kk, const void*
   a.dq = reinterpret_cast<__nv_bfloat16*>(dq);
   a.dk = reinterpret_cast<__nv_bfloat16*>(dkk);
   a.dv = reinterpret_cast<__nv_bfloat16*>(dvv);
-  a.units = B * H;
+  a.units = (int)(B * H);
   if (dlogits_dump && causal) {      // the blocks the kernel skips under the hint hold zeros
     cudaError_t ze = cudaMemsetAsync(dlogits_dump, 0, (size_t)B * H * L * L * 2, (cudaStream_t)stream);
     if (ze != cudaSuccess) return fail(MTF_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(ze));

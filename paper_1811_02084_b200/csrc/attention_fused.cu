@@ -305,13 +305,8 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       }
       return r;
     };
-    auto wait_all = [&](int b, uint32_t parity, int code) -> bool {      // all lanes wait (lane 0 polls first)
-      int w_ok = 1;
-      if (lane == 0) w_ok = mb_wait(bar(b), parity, code, abort_flag) ? 1 : 0;
-      w_ok = __shfl_sync(0xffffffffu, w_ok, 0);
-      if (!w_ok) return false;
-      bool mine_ok = lane == 0 ? true : mb_wait(bar(b), parity, code, abort_flag);
-      return __all_sync(0xffffffffu, mine_ok);
+    auto wait_all = [&](int b, uint32_t parity, int code) -> bool {      // all lanes wait
+      return __all_sync(0xffffffffu, mb_wait(bar(b), parity, code, abort_flag));
     };
     // The trip counts below depend on the arguments alone: after a failed wait a warp keeps going through the tiles (waits
     // then return at once, work is skipped) so that its peers never wait for it at a named barrier.
