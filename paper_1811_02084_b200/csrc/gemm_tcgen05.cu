@@ -10,9 +10,9 @@
 // also sum up to three operand pairs into one accumulator, or run up to three independent problems
 // of one shape.
 //
-// Structure of a CTA (320 threads, one CTA per SM, persistent over work items; by default two CTAs
+// Structure of a CTA (352 threads, one CTA per SM, persistent over work items; by default two CTAs
 // form a pair that owns a 256-row tile through tcgen05 cta_group::2):
-//   warp 0   : TMA producer   - cp.async.bulk.tensor loads (128B swizzle) into a shared-memory ring
+//   warps 0, 10: TMA producers - cp.async.bulk.tensor loads (128B swizzle) into a shared-memory ring
 //                               (16 KB of A plus this CTA's part of B per stage, as many stages as fit)
 //   warp 1   : MMA issuer     - tcgen05.mma kind::f16 (bf16 x bf16 -> fp32), accumulators in TMEM,
 //                               two 128 x 256 accumulators so the epilogue of tile i overlaps tile i+1
@@ -50,7 +50,8 @@ constexpr int kStagingBytes = kEpilogueWarps * 2 * 4096;   // per epilogue warp:
 constexpr int kMaxStages = 8;                      // ring slots with barriers; a launch uses as many as fit its stage size
 constexpr int kSchedSlots = 4;                      // ring of drawn tile numbers that a CTA's roles read in turn
 constexpr int kSmemBytes = kRingBytes + kStagingBytes + 1024 /*alignment slack*/ + 320 /*barriers*/ + 96 /*drawn tiles: 2 x 4 barriers, 4 numbers*/;
-constexpr int kThreads = 64 + 32 * kEpilogueWarps;
+constexpr int kProducers = 2;                      // threads that load, taking turns (see the producer role)
+constexpr int kThreads = 64 + 32 * kEpilogueWarps + 32 * (kProducers - 1);
 constexpr int kTmemCols = 512;
 constexpr long long kTimeoutCycles = 4000000000LL;
 
@@ -758,7 +759,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     for (int s = 0; s < kStages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), CM + CN - 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(tfull_bar(i), 1); mbar_init(tempty_bar(i), (kPair ? 2 : 1) * kEpilogueWarps); }
     for (int i = 0; i < 2 * kEpilogueWarps; ++i) mbar_init(bar_base + 8u * (2 * kMaxStages + 4 + i), 1);
-    for (int i = 0; i < kSchedSlots; ++i) { mbar_init(sched_ring + 8u * i, 1); mbar_init(sched_ring + 32u + 8u * i, (kPair ? 2 : 1) * (1 + kEpilogueWarps)); }
+    for (int i = 0; i < kSchedSlots; ++i) { mbar_init(sched_ring + 8u * i, 1); mbar_init(sched_ring + 32u + 8u * i, (kPair ? 2 : 1) * (kProducers + kEpilogueWarps)); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_a) : "memory");
@@ -795,10 +796,14 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   const int n_local = kPair ? a.block_n / 2 : a.block_n;       // N columns of B this CTA stages (wide: two runs of 128)
   const uint32_t b_bytes = (uint32_t)n_local * BK * 2;
 
-  if (warp == 0) {
-    // ------------------------------- TMA producer -------------------------------
+  if (warp == 0 || warp >= 2 + kEpilogueWarps) {
+    // ------------------------------- TMA producers ------------------------------
+    // A wait, the barrier's byte count and the copies of a k-block take one thread 560 - 680 cycles, however many stages the ring has; the
+    // MMAs of a 256 x 256 tile's k-block take 512.  So two threads take turns: 8192 x 8192 x 1024 103.5 -> 97.5 us, 8192 x 32768 x 1024 415 -> 390,
+    // 16384 x 2048 x 2048 101 -> 97.6 (launches apart; less where a stream of them runs into the power limit).
+    const int producer = warp == 0 ? 0 : warp - 1 - kEpilogueWarps;
     if (mtf::elect_one()) {
-      int stage = 0;
+      int stage = 0, turn = 0;
       uint32_t phase = 0;
       bool ok = true;
       SegIter it(a, work_first, work_step);
@@ -809,11 +814,12 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       uint32_t dseq = 0;
       unsigned pending = 0;
       bool have_pending = false;
-      if (drawn && leader) { pending = (unsigned)work_first; have_pending = true; }      // (the first tile needs no ticket: worker w starts with tile w, ticket n is tile W + n)
+      const bool drawer = leader && producer == 0;
+      if (drawn && drawer) { pending = (unsigned)work_first; have_pending = true; }      // (the first tile needs no ticket: worker w starts with tile w, ticket n is tile W + n)
       auto next_tile = [&]() -> bool {
         if (!drawn) return it.next(sg);
         unsigned t;
-        if (leader) {
+        if (drawer) {
           if (!have_pending) pending = (unsigned)work_step + atomicAdd(a.sched, 1u);
           have_pending = false;
           t = pending;
@@ -832,7 +838,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         const int n0 = tl.n0 + pn * a.block_n + cta_rank * n_local;
         int term = kb_first / a.kb_term, kt = kb_first - term * a.kb_term;
         for (int kb = 0; kb < kb_count; ++kb) {
-          if (drawn && leader && !have_pending && kb == (kb_count > 4 ? kb_count - 4 : 0)) { pending = (unsigned)work_step + atomicAdd(a.sched, 1u); have_pending = true; }
+          if (drawn && drawer && !have_pending && kb == (kb_count > 4 ? kb_count - 4 : 0)) { pending = (unsigned)work_step + atomicAdd(a.sched, 1u); have_pending = true; }
           // slices of the reduce group are walked in ascending order: k0 runs through slice 0's
           // block of K, then slice 1's, ... (the blocks are contiguous in the global tensor); a
           // multi-term launch then goes on with the next product's operands
@@ -841,12 +847,18 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
           const CUtensorMap* const pa = sel == 0 ? &map_a : &extra.m[2 * (sel - 1)];
           const CUtensorMap* const pb = sel == 0 ? &map_b : &extra.m[2 * (sel - 1) + 1];
           if (++kt == a.kb_term) { kt = 0; ++term; }
-          if (!(ok = mbar_wait(empty_bar(stage), phase ^ 1u, 0x100 + stage, abort_flag))) break;
+          const bool mine = turn == producer;
+          if (++turn == kProducers) turn = 0;
+          const int at = stage;
+          const uint32_t at_phase = phase;
+          if (++stage == kStages) { stage = 0; phase ^= 1u; }
+          if (!mine) continue;
+          if (!(ok = mbar_wait(empty_bar(at), at_phase ^ 1u, 0x100 + at, abort_flag))) break;
           // a pair's loads all count on the even CTA's barrier, which expects both CTAs' bytes
-          if (!kPair) mbar_expect_tx(full_bar(stage), kAStageBytes + b_bytes);
-          else if (leader) mbar_expect_tx(full_bar(stage), 2u * (kAStageBytes + b_bytes));
-          const uint32_t fb = kPair ? (full_bar(stage) & 0xFEFFFFFFu) : full_bar(stage);
-          const uint32_t sa = tiles_base + stage * kStageBytes;
+          if (!kPair) mbar_expect_tx(full_bar(at), kAStageBytes + b_bytes);
+          else if (leader) mbar_expect_tx(full_bar(at), 2u * (kAStageBytes + b_bytes));
+          const uint32_t fb = kPair ? (full_bar(at) & 0xFEFFFFFFu) : full_bar(at);
+          const uint32_t sa = tiles_base + at * kStageBytes;
           const uint32_t sb = sa + kAStageBytes;
 #if defined(MTF_CLUSTER_SHARE)
           if (CN > 1) cluster_share_load_a(sa, pa, fb, pm, pn, CN, cta_rank, a.a_mn_major, BM / CN, m0, k0, tl.o[2], tl.o[1], tl.o[0]);
@@ -879,7 +891,6 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
           } else {
             tma_load_5d<kPair>(sb, pb, fb, k0, n0, tl.o[2], tl.o[1], tl.o[0]);
           }
-          if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
       }
     }
@@ -1474,7 +1485,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     }
   }
 
-  if (warp >= 2 && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // staged output stores have landed
+  if (warp >= 2 && warp < 2 + kEpilogueWarps && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // staged output stores have landed
 
   // ------------------------------- teardown --------------------------------------
   if (*abort_flag) {
