@@ -7,11 +7,11 @@
 //
 // The slices that a layout cuts M, N and the batch dimensions into do not appear here: every output element is one sum
 // over all of K whoever owns it, so tiles run across slice boundaries and no slice edge is padded to a tile.
-// Bound: at these sizes a fixed part (set-up, first loads, exchange, stores: 3 - 6 us) and 0.27 us (BN 64) or 0.34 us
-// (BN 128) per 64-deep k-block of a CTA's part, which is the latency of the loads its ring keeps in flight.  Measured
-// against 256-row tiles with the whole of K on one pair: the feed-forward block (forward and backward) on 128 tokens,
-// 1024 x 4096, 116 -> 56 us; the decoder layer's forward pass on 512 tokens 103 -> 65 us; the attention block on
-// 3 x 200 tokens 118 -> 71 us.
+// Bound: at these sizes a fixed part (set-up, first loads, exchange, stores: 2.5 - 5 us) and 0.19 us (BN 64) or 0.21 us (BN 128) per
+// 64-deep k-block of a CTA alone on its SM, which is what two loading threads in turn need for one (330 - 390 cycles).
+// Measured against 256-row tiles with the whole of K on one pair: the feed-forward block (forward and backward) on 128 tokens,
+// 1024 x 4096, 116 -> 45 us; the decoder layer's forward pass on 512 tokens 103 -> 51 us; the attention block on
+// 3 x 200 tokens 118 -> 48 us (its core included).
 // Included by gemm_tcgen05.cu, whose wrappers, bounded waits and status word it uses.
 
 struct ClusterArgs {
