@@ -1,12 +1,15 @@
-// f32 einsums of matrix-product form (see F32Params) on the bf16 tensor cores, without giving up bits: every f32 value is the
-// exact sum of three bf16 values, a = a1 + a2 + a3 (a1 = bf16(a), a2 = bf16(a - a1), a3 = a - a1 - a2), and
-//   a b  =  a1 b1  +  (a1 b2 + a2 b1)  +  (a1 b3 + a2 b2 + a3 b1)  +  terms below 2^-25 |a b|,
-// six exact products.  What limits the sums is the accumulator in tensor memory, which rounds towards zero on every addition.  So
+// f32 einsums of matrix-product form (see F32Params) on the bf16 tensor cores, without giving up bits: 2^16 times an f32 value below
+// 2^111 is the exact sum of three bf16 values, 2^16 a = a1 + a2 + a3 (a1 = bf16(2^16 a), a2 = bf16(2^16 a - a1), a3 = 2^16 a - a1 - a2), and
+//   2^32 a b  =  a1 b1  +  (a1 b2 + a2 b1)  +  (a1 b3 + a2 b2 + a3 b1)  +  terms below 2^-25 |2^32 a b|,
+// six exact products (the splitting of Henry, Tang and Heinecke, "Leveraging the bfloat16 Artificial Intelligence Datatype For
+// Higher-Precision Computations", 2019).  The 2^16 puts the last bit of f32's smallest values, 2^-149, on bf16's, 2^-133: without it values below
+// 2^-110 would lose bits, and a product below 2^-126 would too; what now leaves the range below is under 2^-155 a term, less than one f32
+// addition drops there.  A value or a sum that leaves it above comes out infinite or NaN.  What limits the sums is the accumulator in tensor memory, which rounds towards zero on every addition.  So
 // the large products never meet there: each 16-deep step of a1 b1 has an accumulator block of its own (one instruction, nothing added
 // to it), the threads add the four blocks of a 64-deep stage pairwise and then to a running f32 sum, rounding to nearest; the small products stay
 // in two more blocks (their rounding is 2^-8 of the large ones') and are added once at the end.
-// Outputs that come out infinite, NaN or below 2^-90 (an operand whose pieces leave bf16's range: infinities, values within
-// 2^-9 of the largest, values below 2^-110) are computed again by the thread that owns them, in plain f32 over the same part of K.
+// Outputs that come out infinite or NaN (an infinity or NaN among their operands, a value from 2^111 or a sum from 2^96 on) are computed
+// again by the thread that owns them, in plain f32 over the same part of K.
 //
 // A block of 512 threads owns a 128 x 64 tile: all threads load f32 (two stages ahead, in registers), split, and write the pieces into
 // 128-byte-swizzled K- or MN-major boxes, whichever way the operand lies in memory; one thread issues a stage's 16 MMAs and they
@@ -38,7 +41,7 @@ constexpr uint32_t kPieceA = kTM * kBK * 2, kPieceB = kTN * kBK * 2, kStage = 3 
 constexpr uint32_t kSmemBytes = kRing * kStage + 1024;
 constexpr int kTmemCols = 512;          // four blocks of a1 b1, two of the small products, 64 columns each (allocations are powers of two)
 constexpr long long kWaitCycles = 4000000000LL;
-constexpr float kSmall = 8.0779356694631608874e-28f;      // 2^-90
+constexpr float kUp = 65536.f, kDown = 2.3283064365386962891e-10f;      // 2^16 on every operand, 2^-32 on the sums
 
 __device__ int g_f32_status = 0;
 
@@ -168,6 +171,11 @@ __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
 
 // This thread's 16-byte pieces of a kRows x 64 operand tile.  Along k (s_k == 1): piece i is row tid / 16 + 32 i, k 4 (tid mod 16);
 // otherwise along m|n: row 4 (tid mod (kRows / 4)), k tid / (kRows / 4) + (2048 / kRows) i.  Either way a thread's pieces lie at one
@@ -216,12 +224,12 @@ struct Pieces {
       if (in > 3) r[i].w = __ldg(q + 3 * s);
     }
   }
-  // the three bf16 pieces of every value into three tiles, `piece_bytes` apart
+  // the three bf16 pieces of every value, times 2^16, into three tiles, `piece_bytes` apart
   template <uint32_t kPieceBytes>
   __device__ __forceinline__ void store(uint8_t* tile, const float4* r) const {
 #pragma unroll
     for (int i = 0; i < kN; ++i) {
-      f32x2 xy = pair(r[i].x, r[i].y), zw = pair(r[i].z, r[i].w);
+      f32x2 xy = mul2(pair(r[i].x, r[i].y), pair(kUp, kUp)), zw = mul2(pair(r[i].z, r[i].w), pair(kUp, kUp));
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
         float x, y, z, w;
@@ -373,14 +381,12 @@ __global__ void __launch_bounds__(kThreads, 1) einsum_f32_tc_kernel(const __grid
     uint32_t odd = 0u;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      sum2[j] = add2(sum2[j], add2(pair_bits(x[2 * j], x[2 * j + 1]), pair_bits(y[2 * j], y[2 * j + 1])));
+      sum2[j] = mul2(add2(sum2[j], add2(pair_bits(x[2 * j], x[2 * j + 1]), pair_bits(y[2 * j], y[2 * j + 1]))), pair(kDown, kDown));
       unpair(sum2[j], sum[2 * j], sum[2 * j + 1]);
     }
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const float v = fabsf(sum[j]);
-      if (!(v <= 3.402823466e38f) || (v < kSmall && v != 0.f)) odd |= 1u << j;
-    }
+    for (int j = 0; j < 16; ++j)
+      if (!(fabsf(sum[j]) <= 3.402823466e38f)) odd |= 1u << j;
     if (odd && m0 + row < M) {
       const float* const pr = A + (long long)(m0 + row) * p.sAm;
 #pragma unroll 1

@@ -68,7 +68,7 @@ def test_error_is_no_larger_than_plain_arithmetic(mtf, k):  # noqa: F811
 
 @pytest.mark.parametrize("k", [40, 520])
 def test_values_outside_the_pieces_range(mtf, k):  # noqa: F811
-    """Infinities, NaN, the type's largest values and values whose last piece is below bf16's smallest come out as plain f32 arithmetic has them."""
+    """Infinities, NaN and the type's largest values come out as plain f32 arithmetic has them, and so do small values beside ordinary and small ones."""
     import torch
     torch.manual_seed(1)
     x, y = torch.randn(200, k, device="cuda"), torch.randn(k, 100, device="cuda")
@@ -88,11 +88,36 @@ def test_values_outside_the_pieces_range(mtf, k):  # noqa: F811
     same &= np.isinf(f32) == np.isinf(got)
     same[[60, 90]] |= np.isin(np.arange(100), [9, 10, 11], invert=True)      # (sums of many huge terms pass through infinities in any f32 order; single terms don't)
     assert same.all()
-    ok = np.isfinite(f32) & np.isfinite(got) & (np.abs(f32) > 1e-30)
+    ok = np.isfinite(f32) & np.isfinite(got)
     scale = np.abs(x.cpu().double().numpy()) @ np.abs(y.cpu().double().numpy())
-    assert (np.abs(got - f32)[ok] <= k * 6e-8 * scale[ok]).all()
-    tiny = got[100], ref[100]
-    assert (np.abs(tiny[0] - tiny[1]) <= k * 6e-8 * scale[100] + 1e-44 * k).all()
+    assert (np.abs(got - f32)[ok] <= (k * 6e-8 * scale + k * 2.0 ** -149)[ok]).all()
+
+
+@pytest.mark.parametrize("k", [40, 520])
+@pytest.mark.parametrize("small,large", [(1e-35, 1e12), (1e-36, 1e20), (1e-38, 1e25), (1e-40, 1e30), (1e-42, 1e30), (1e-44, 1e30), (1e-25, 1e-15), (1e-28, 1.0), (1e-33, 2e33), (1e-6, 1e31)])
+@pytest.mark.parametrize("flip", [False, True])
+def test_small_operands_beside_large_ones(mtf, k, small, large, flip):  # noqa: F811
+    """Rows of small, ordinary and single small values (whose pieces would lose bits or vanish unscaled) times columns of large, ordinary and small ones: one chain of
+    k f32 additions errs by about 2^-24 sqrt(k / 12) of the result, and by half of 2^-149 a term below f32's normal range; twice and more is allowed."""
+    import torch
+    torch.manual_seed(k)
+    dev = {"device": "cuda", "dtype": torch.float64}
+    rows, cols = torch.randn(200, k, **dev), torch.randn(k, 100, **dev)
+    rows[:60] *= small
+    cols[:, :30] *= large
+    cols[:, 30:40] *= small
+    rows[60:90] = 0.0
+    rows[torch.arange(60, 90), torch.arange(60, 90) % k] = small      # one value in a row of zeros
+    rows[90:100, 3] = small                                             # ... and beside ordinary ones
+    cols[:, 95:] = 0.0
+    x, y = rows.float(), cols.float()
+    got = product(mtf, y.T.contiguous(), x.T.contiguous(), 128).T if flip else product(mtf, x, y, 128)
+    ref, got = x.double() @ y.double(), got.double()
+    assert got.isfinite().all()
+    for r in (slice(0, 60), slice(60, 90), slice(90, 100), slice(100, 200)):
+        for c in (slice(0, 30), slice(30, 40), slice(40, 95), slice(95, 100)):
+            e, f = (got - ref)[r, c], ref[r, c]
+            assert e.norm() <= 2 ** -24 * k ** 0.5 * f.norm() + k * 2 ** -149 * f.numel() ** 0.5, (r, c)
 
 
 def test_pieces_are_chosen_by_size(mtf):  # noqa: F811
