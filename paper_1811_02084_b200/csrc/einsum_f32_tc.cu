@@ -9,17 +9,17 @@
 // to it), the threads add the four blocks of a 64-deep stage pairwise and then to a running f32 sum, rounding to nearest; the small products stay
 // in two more blocks (their rounding is 2^-8 of the large ones') and are added once at the end.
 // Outputs that come out infinite or NaN (an infinity or NaN among their operands, a value from 2^111 or a sum from 2^96 on) are computed
-// again by the thread that owns them, in plain f32 over the same part of K.
+// again by the warp that owns them, in plain f32 over the same part of K.
 //
 // A block of 512 threads owns a 128 x 64 tile: all threads load f32 (two stages ahead, in registers), split, and write the pieces into
 // 128-byte-swizzled K- or MN-major boxes, whichever way the operand lies in memory; one thread issues a stage's 16 MMAs and they
 // run while the block splits the next one.  Few tiles: K over up to 8 blocks of a cluster, whose parts are added in ascending order
-// through distributed shared memory.  (Warps of their own for splitting, adding and issuing: 228 us where this takes 175, below, and 1 us
+// through distributed shared memory.  (Warps of their own for splitting, adding and issuing: 228 us where this took 175, 2048^3 below, and 1 us
 // more for a small product: every stage goes through shared memory's one port, 72 KB of pieces written, 112 KB read by the MMAs,
 // 48 KB through L1, and that port is what they all wait for.)
 // Bound: that port, 1.35 us a stage; a small product's chain of launch, first loads, one stage and stores (4.5 us).
-// Measured against plain FP32 arithmetic on the 64 x 64 tiles of einsum_f32.cu: 1024 x 1024 x 256 22.3 -> 10.1 us, 1024 x 256 x 1024 23.3 ->
-// 11.5, 2048^3 504 -> 174, 128^3 6.3 -> 5.6, 8 x 256 x 64 4.8 -> 4.5; error against 64 bits (2-norm, normal values) 1.5e-7 -> 6.4e-8 at K = 256,
+// Measured against plain FP32 arithmetic on the 64 x 64 tiles of einsum_f32.cu: 1024 x 1024 x 256 22.2 -> 9.7 us, 1024 x 256 x 1024 23.3 ->
+// 11.5, 2048^3 503 -> 170, 128^3 6.2 -> 5.4, 8 x 256 x 64 4.8 -> 4.5; error against 64 bits (2-norm, normal values) 1.5e-7 -> 6.4e-8 at K = 256,
 // 4.1e-7 -> 1.2e-7 at K = 2048, 6.0e-8 -> 4.8e-8 or less at K = 16.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -39,8 +39,10 @@ constexpr int kThreads = 512;
 constexpr int kRing = 2;
 constexpr uint32_t kPieceA = kTM * kBK * 2, kPieceB = kTN * kBK * 2, kStage = 3 * (kPieceA + kPieceB);
 constexpr uint32_t kSmemBytes = kRing * kStage + 1024;
+static_assert(32768 + kThreads / 32 * 32 * 53 * 4 <= kRing * kStage, "a stage per warp past the tile");
 constexpr int kTmemCols = 512;          // four blocks of a1 b1, two of the small products, 64 columns each (allocations are powers of two)
 constexpr long long kWaitCycles = 4000000000LL;
+constexpr float kMost = 3.402823466e38f;                  // the largest f32
 constexpr float kUp = 65536.f, kDown = 2.3283064365386962891e-10f;      // 2^16 on every operand, 2^-32 on the sums
 
 __device__ int g_f32_status = 0;
@@ -242,6 +244,62 @@ struct Pieces {
   }
 };
 
+// Plain f32 for the outputs of one warp's 32 rows x 16 columns that came out infinite or NaN: k from k0 to k1 in order, 32 at a time through the
+// warp's own `stage`, loaded by lanes that lie side by side in memory.  `out`: this lane's row of the tile; piece q of its columns at 16 (q ^ sw).
+// Bound: issue, about half of it multiply-adds.  All NaN, beside ordinary values and beside einsum_f32.cu (which takes the same time for either): 1024 x 1024 x 256
+// 42.8, 9.7 and 22.2 us; 2048^3 1132, 170 and 503.  One NaN, which costs the warps of its row: 33 and 279.
+constexpr int kStageA = 33, kStageB = 20, kStageFloats = 32 * (kStageA + kStageB);      // rows of A 33 words apart: no bank conflicts; of B 20: 16-byte pieces
+__device__ __noinline__ void redo_plain(uint8_t* out, uint32_t sw, uint32_t q0, float* stage, const float* A, const float* B, int sAm, int sAk, int sBn, int sBk, int rows, int cols, int k0,
+                                        int k1) {
+  const int lane = threadIdx.x & 31, hi = lane >> 4, lo = lane & 15;
+  const bool along_a = sAk == 1, along_b = sBk == 1;
+  // this lane's values: along k, row (column) i at k = lane; otherwise row lane at k = i, column lo at k = 2 i + hi
+  const float* pa = A + (along_a ? lane : lane * sAm);
+  const float* pb = B + (along_b ? lane : lo * sBn + hi * sBk);
+  const int step_a = along_a ? sAm : sAk, step_b = along_b ? sBn : 2 * sBk;
+  float* const sa = stage + (along_a ? lane * kStageA : lane);
+  float* const sb = stage + 32 * kStageA;
+  float* const sb0 = sb + (along_b ? lane * kStageB : hi * kStageB + lo);
+  const int put_a = along_a ? 1 : kStageA, put_b = along_b ? 1 : 2 * kStageB;
+  float sum[16];
+#pragma unroll
+  for (int j = 0; j < 16; ++j) sum[j] = 0.f;
+  pa += (long long)k0 * sAk;
+  pb += (long long)k0 * sBk;
+#pragma unroll 1
+  for (int left = k1 - k0; left > 0; left -= 32, pa += 32 * sAk, pb += 32 * sBk) {
+    const int na = along_a ? (lane < left ? rows : 0) : (lane < rows ? left : 0), nb = along_b ? (lane < left ? cols : 0) : (lo < cols ? (left - hi + 1) / 2 : 0);
+    float x[32], y[16];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) x[i] = i < na ? __ldg(pa + i * step_a) : 0.f;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) y[i] = i < nb ? __ldg(pb + i * step_b) : 0.f;
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 32; ++i) sa[i * put_a] = x[i];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) sb0[i * put_b] = y[i];
+    __syncwarp();
+#pragma unroll 4
+    for (int k = 0; k < min(left, 32); ++k) {
+      const float v = stage[k * kStageA + lane];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 b = *reinterpret_cast<const float4*>(sb + k * kStageB + 4 * q);
+        sum[4 * q] = fmaf(v, b.x, sum[4 * q]);
+        sum[4 * q + 1] = fmaf(v, b.y, sum[4 * q + 1]);
+        sum[4 * q + 2] = fmaf(v, b.z, sum[4 * q + 2]);
+        sum[4 * q + 3] = fmaf(v, b.w, sum[4 * q + 3]);
+      }
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    float* const o = reinterpret_cast<float*>(out + (((q0 + j / 4) ^ sw) << 4)) + (j & 3);
+    if (!(fabsf(*o) <= kMost)) *o = sum[j];
+  }
+}
+
 template <bool kAlongA, bool kAlongB>
 __global__ void __launch_bounds__(kThreads, 1) einsum_f32_tc_kernel(const __grid_constant__ F32TcArgs a) {
   extern __shared__ uint8_t smem_raw[];
@@ -377,39 +435,25 @@ __global__ void __launch_bounds__(kThreads, 1) einsum_f32_tc_kernel(const __grid
     tmem_ld16(mine + 256u, x);
     tmem_ld16(mine + 320u, y);
     tmem_ld_wait();
-    float sum[16];
-    uint32_t odd = 0u;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
+    for (int j = 0; j < 8; ++j)
       sum2[j] = mul2(add2(sum2[j], add2(pair_bits(x[2 * j], x[2 * j + 1]), pair_bits(y[2 * j], y[2 * j + 1]))), pair(kDown, kDown));
-      unpair(sum2[j], sum[2 * j], sum[2 * j + 1]);
-    }
-#pragma unroll
-    for (int j = 0; j < 16; ++j)
-      if (!(fabsf(sum[j]) <= 3.402823466e38f)) odd |= 1u << j;
-    if (odd && m0 + row < M) {
-      const float* const pr = A + (long long)(m0 + row) * p.sAm;
-#pragma unroll 1
-      for (int j = 0; j < 16; ++j) {
-        const int n = n0 + col + j;
-        if (!(odd >> j & 1u) || n >= N) continue;
-        const float* const pc = B + (long long)n * p.sBn;
-        float v = 0.f;
-        for (int k = s0 * kBK; k < min(K, s1 * kBK); ++k) v = fmaf(__ldg(pr + (long long)k * p.sAk), __ldg(pc + (long long)k * p.sBk), v);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) sum[i] = i == j ? v : sum[i];
-      }
-#pragma unroll
-      for (int j = 0; j < 8; ++j) sum2[j] = pair(sum[2 * j], sum[2 * j + 1]);
-    }
   }
   // this block's part of the tile: 16-byte piece q of row r at r * 256 + ((q ^ (r mod 8)) * 16); every MMA has read the ring
+  bool odd = false;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     float v[4];
     unpair(sum2[2 * q], v[0], v[1]);
     unpair(sum2[2 * q + 1], v[2], v[3]);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) odd = odd || (!(fabsf(v[j]) <= kMost) && n0 + col + 4 * q + j < N);
     *reinterpret_cast<float4*>(ring + row * 256 + (((col / 4 + q) ^ (row & 7)) << 4)) = make_float4(v[0], v[1], v[2], v[3]);
+  }
+  if (__any_sync(0xffffffffu, ok && odd && m0 + row < M)) {      // (past the tile there is room for every warp's stage)
+    const int m = m0 + row - lane, n = n0 + col;
+    redo_plain(ring + row * 256, (uint32_t)(row & 7), (uint32_t)col / 4, reinterpret_cast<float*>(ring + 32768) + warp * kStageFloats, A + (long long)m * p.sAm,
+               B + (long long)n * p.sBn, (int)p.sAm, (int)p.sAk, (int)p.sBn, (int)p.sBk, M - m, N - n, s0 * kBK, min(K, s1 * kBK));
   }
   fence_before();
   if (a.split > 1) cluster_sync();

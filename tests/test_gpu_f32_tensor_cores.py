@@ -120,6 +120,29 @@ def test_small_operands_beside_large_ones(mtf, k, small, large, flip):  # noqa: 
             assert e.norm() <= 2 ** -24 * k ** 0.5 * f.norm() + k * 2 ** -149 * f.numel() ** 0.5, (r, c)
 
 
+@pytest.mark.parametrize("order", ["ik,kj", "ki,jk"])
+def test_results_out_of_range_cost_what_plain_arithmetic_costs(mtf, order):  # noqa: F811
+    """A product of nothing but NaN is computed twice; measured, 4.4 times the time of ordinary values (with each thread computing its own outputs again: 112 times)."""
+    import torch
+    m, n, k = 1024, 1024, 256
+    size = {"i": m, "j": n, "k": k}
+    x, y = [torch.randn([size[c] for c in t], device="cuda") for t in order.split(",")]
+    o = torch.empty(m, n, device="cuda")
+    nan = torch.full_like(x, float("nan"))
+    at = [torch.cuda.Event(enable_timing=True) for _ in range(4)]
+    mtf.mtf_debug_contraction(128, 1)
+    for _ in range(2):
+        for t, pair in ((x, at[:2]), (nan, at[2:])):
+            pair[0].record()
+            for _ in range(20):
+                mtf.mtf_einsum(layout(mtf, *ONE), None, [mtf.named(t, list(order[:2])), mtf.named(y, list(order[3:]))], mtf.named(o, ["i", "j"]))
+            pair[1].record()
+    torch.cuda.synchronize()
+    assert mtf.mtf_debug_contraction(0, 0)[0] == 128
+    assert o.isnan().all()
+    assert at[2].elapsed_time(at[3]) <= 9 * at[0].elapsed_time(at[1])
+
+
 def test_pieces_are_chosen_by_size(mtf):  # noqa: F811
     import torch
     mtf.mtf_debug_contraction(0, 0)
