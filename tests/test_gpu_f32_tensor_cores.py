@@ -45,6 +45,34 @@ def test_stages_and_column_sums(mtf, asked, m, n, k):  # noqa: F811
     assert parity_error(from_torch(col), (x.double() @ y.double()).relu().sum(0).cpu().numpy()) <= TOL["f32"]
 
 
+@pytest.mark.parametrize("m,n,k", [(130, 70, 70), (33, 65, 300), (128, 64, 256)])
+@pytest.mark.parametrize("dims", ["bihk,bjhk,bhij", "bihk,bhkj,bihj", "bhki,bkhj,bhji", "hbik,bhkj,bihj", "bik,bkj,bji", "kbi,jbk,bij"])
+def test_batches(mtf, asked, dims, m, n, k):  # noqa: F811
+    """One and two batch dimensions beside and between the others, row lengths and batch strides on and off 16 bytes, operands exchanged."""
+    size = {"b": 2, "h": 3, "i": m, "j": n, "k": k}
+    a, b, out = [[(c, size[c]) for c in t] for t in dims.split(",")]
+    for dt in ("f32", "bf16"):
+        got, ref, _ = run_einsum(mtf, layout(mtf, *ONE), [a, b], out, "f32", dt)
+        assert parity_error(got, ref) <= TOL[dt]
+    ep = {"scale": 2.0, "bias": [("j", n)], "relu": True, "residual": True}
+    got, ref, _ = run_einsum(mtf, layout(mtf, *ONE), [a, b], out, "f32", epilogue=ep)
+    assert parity_error(got, ref) <= TOL["f32"]
+
+
+@pytest.mark.parametrize("batch,m,n,k,split", [(1, 300, 70, 70, 2), (1, 2100, 70, 20, 1), (3, 40, 70, 300, 4), (1, 40, 70, 300, 4)])
+def test_column_sums_over_tiles_and_batches(mtf, asked, batch, m, n, k, split):  # noqa: F811
+    """Sums over every row of every batch entry: several row tiles add to the zeroed output, one row tile stores it, a cluster gathers it."""
+    import torch
+    x, y = torch.randn(batch, m, k, device="cuda"), torch.randn(batch, k, n, device="cuda")
+    o, col = torch.empty(batch, m, n, device="cuda"), torch.full((n,), float("nan"), device="cuda")
+    mtf.mtf_einsum(layout(mtf, *ONE), None, [mtf.named(x, ["b", "i", "k"]), mtf.named(y, ["b", "k", "j"])], mtf.named(o, ["b", "i", "j"]),
+                   mtf.Epilogue(reduce_sum_out=mtf.named(col, ["j"])))
+    assert mtf.mtf_debug_contraction(128, 1) == (128, split)
+    ref = x.double() @ y.double()
+    assert parity_error(from_torch(o), ref.cpu().numpy()) <= TOL["f32"]
+    assert parity_error(from_torch(col), ref.sum((0, 1)).cpu().numpy()) <= TOL["f32"]
+
+
 def product(mtf, x, y, columns):  # noqa: F811
     import torch
     o = torch.full((x.shape[0], y.shape[1]), float("nan"), device="cuda")
