@@ -173,6 +173,11 @@ __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
 __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
   f32x2 r;
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
@@ -440,17 +445,18 @@ __global__ void __launch_bounds__(kThreads, 1) einsum_f32_tc_kernel(const __grid
       sum2[j] = mul2(add2(sum2[j], add2(pair_bits(x[2 * j], x[2 * j + 1]), pair_bits(y[2 * j], y[2 * j + 1]))), pair(kDown, kDown));
   }
   // this block's part of the tile: 16-byte piece q of row r at r * 256 + ((q ^ (r mod 8)) * 16); every MMA has read the ring
-  bool odd = false;
+  f32x2 odd2 = 0ull;                 // zero times every value: NaN if one is infinite or NaN
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     float v[4];
     unpair(sum2[2 * q], v[0], v[1]);
     unpair(sum2[2 * q + 1], v[2], v[3]);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) odd = odd || (!(fabsf(v[j]) <= kMost) && n0 + col + 4 * q + j < N);
+    odd2 = fma2(sum2[2 * q], 0ull, fma2(sum2[2 * q + 1], 0ull, odd2));
     *reinterpret_cast<float4*>(ring + row * 256 + (((col / 4 + q) ^ (row & 7)) << 4)) = make_float4(v[0], v[1], v[2], v[3]);
   }
-  if (__any_sync(0xffffffffu, ok && odd && m0 + row < M)) {      // (past the tile there is room for every warp's stage)
+  float odd_x, odd_y;
+  unpair(odd2, odd_x, odd_y);
+  if (__builtin_expect(__any_sync(0xffffffffu, ok && !(odd_x + odd_y == 0.f) && m0 + row < M && n0 + col < N), 0)) {      // (past the tile there is room for every warp's stage)
     const int m = m0 + row - lane, n = n0 + col;
     redo_plain(ring + row * 256, (uint32_t)(row & 7), (uint32_t)col / 4, reinterpret_cast<float*>(ring + 32768) + warp * kStageFloats, A + (long long)m * p.sAm,
                B + (long long)n * p.sBn, (int)p.sAm, (int)p.sAk, (int)p.sBn, (int)p.sBk, M - m, N - n, s0 * kBK, min(K, s1 * kBK));
