@@ -175,7 +175,9 @@ mtf_status mtf_rank_wait(const mtf_layout_t* bound_layout, void* stream);
  * an N slice that is not a multiple of 8, a reduced dimension that only one operand has, more than
  * three batch dimensions) runs on the generic one-thread-per-element kernel only up to 2^30
  * multiply-adds; above that the plan is refused with MTF_ERR_UNSUPPORTED and the reason in
- * mtf_last_error(), unless mtf_plan_force(MTF_KERNEL_SIMT, ..) asked for the generic kernel. */
+ * mtf_last_error(), unless mtf_plan_force(MTF_KERNEL_SIMT, ..) asked for the generic kernel.
+ * f32 x f32 products have f32 accuracy over the type's whole range, subnormal numbers included, on every kernel; those that run on the tensor
+ * cores (as exact bf16 pieces) take longer where results are infinite or NaN, operands 2^111 or sums 2^96 and more. */
 mtf_status mtf_einsum_plan(const mtf_layout_t* layout, int32_t n_in, const mtf_tensor* in_desc,
                            const mtf_tensor* out_desc, const mtf_epilogue* epilogue, mtf_plan_t** out);
 mtf_status mtf_plan_destroy(mtf_plan_t* plan);

@@ -14,12 +14,14 @@
 // A block of 512 threads owns a 128 x 64 tile: all threads load f32 (two stages ahead, in registers), split, and write the pieces into
 // 128-byte-swizzled K- or MN-major boxes, whichever way the operand lies in memory; one thread issues a stage's 16 MMAs and they
 // run while the block splits the next one.  Few tiles: K over up to 8 blocks of a cluster, whose parts are added in ascending order
-// through distributed shared memory.  (Warps of their own for splitting, adding and issuing: 228 us where this took 175, 2048^3 below, and 1 us
-// more for a small product: every stage goes through shared memory's one port, 72 KB of pieces written, 112 KB read by the MMAs,
-// 48 KB through L1, and that port is what they all wait for.)
-// Bound: that port, 1.35 us a stage; a small product's chain of launch, first loads, one stage and stores (4.5 us).
-// Measured against plain FP32 arithmetic on the 64 x 64 tiles of einsum_f32.cu: 1024 x 1024 x 256 22.2 -> 9.7 us, 1024 x 256 x 1024 23.3 ->
-// 11.5, 2048^3 503 -> 170, 128^3 6.2 -> 5.4, 8 x 256 x 64 4.8 -> 4.5; error against 64 bits (2-norm, normal values) 1.5e-7 -> 6.4e-8 at K = 256,
+// through distributed shared memory.  (Warps of their own for splitting, adding and issuing: 2048^3 228 us where this took 175, and 1 us
+// more for a small product.)
+// Bound: a stage takes 1.3 us (2500 cycles) and no unit is full in it: issue slots 53 %, shared memory's wavefronts 41 %, tensor pipe 28 % of the
+// active cycles (2048 x 2048 x 1024).  Its steps follow one another: split and store, wait for the stage before, read its accumulators, barrier, issue; the
+// tensor core idles from that wait to the issue, since a second set of a1 b1 blocks would need 640 of 512 columns.  A small product is the chain of
+// launch, first loads, one stage and stores (4.5 us).
+// Measured against plain FP32 arithmetic on the 64 x 64 tiles of einsum_f32.cu: 1024 x 1024 x 256 22.2 -> 9.5 us, 1024 x 256 x 1024 23.3 ->
+// 11.2, 2048^3 503 -> 170, 128^3 6.1 -> 5.2, 8 x 256 x 64 4.8 -> 4.5; error against 64 bits (2-norm, normal values) 1.5e-7 -> 6.4e-8 at K = 256,
 // 4.1e-7 -> 1.2e-7 at K = 2048, 6.0e-8 -> 4.8e-8 or less at K = 16.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -252,7 +254,7 @@ struct Pieces {
 // Plain f32 for the outputs of one warp's 32 rows x 16 columns that came out infinite or NaN: k from k0 to k1 in order, 32 at a time through the
 // warp's own `stage`, loaded by lanes that lie side by side in memory.  `out`: this lane's row of the tile; piece q of its columns at 16 (q ^ sw).
 // Bound: issue, about half of it multiply-adds.  All NaN, beside ordinary values and beside einsum_f32.cu (which takes the same time for either): 1024 x 1024 x 256
-// 42.8, 9.7 and 22.2 us; 2048^3 1132, 170 and 503.  One NaN, which costs the warps of its row: 33 and 279.
+// 42.6, 9.5 and 22.2 us; 2048^3 1132, 170 and 503.  One NaN, which costs the warps of its row: 33 and 278.
 constexpr int kStageA = 33, kStageB = 20, kStageFloats = 32 * (kStageA + kStageB);      // rows of A 33 words apart: no bank conflicts; of B 20: 16-byte pieces
 __device__ __noinline__ void redo_plain(uint8_t* out, uint32_t sw, uint32_t q0, float* stage, const float* A, const float* B, int sAm, int sAk, int sBn, int sBk, int rows, int cols, int k0,
                                         int k1) {
@@ -581,8 +583,8 @@ static int split_of(int64_t tiles, int64_t K) {
 }
 
 // Is this kernel the shorter one for a product that einsum_f32.cu's tiles would take?  Microseconds, fitted to 900 drawn products on both
-// (f32_tile_us is that kernel's estimate; a batch counts 0.2 more a round: its tiles are mostly padding when they are cheap; of the 900 none then takes over 1.03 times its time there).  It stays there for K up to about 32, where three pieces of a mostly empty stage are no gain (256 x 64 x 8: 4.1 us there,
-// 4.8 here), and for batches of a few rows, where a 128-row tile is mostly padding (250 x [16 x 50 x 393]: 44 and 72).
+// (f32_tile_us is that kernel's estimate; a batch counts 0.2 more a round: its tiles are mostly padding when they are cheap; of the 900 none then takes over 1.03 times its time there).  It stays there for K up to about 32, where three pieces of a mostly empty stage are no gain (256 x 64 x 8: 3.9 us there,
+// 4.7 here), and for batches of a few rows, where a 128-row tile is mostly padding (250 x [16 x 50 x 393]: 44 and 72).
 bool f32_tensor_cores_pay(const F32Params& p) {
   const int64_t tiles = tiles_of(p);
   const int split = split_of(tiles, p.K);

@@ -7,11 +7,12 @@
 //
 // The slices that a layout cuts M, N and the batch dimensions into do not appear here: every output element is one sum
 // over all of K whoever owns it, so tiles run across slice boundaries and no slice edge is padded to a tile.
-// Bound: at these sizes a fixed part (set-up, first loads, exchange, stores: 2.5 - 5 us) and 0.19 us (BN 64) or 0.21 us (BN 128) per
+// Bound: at these sizes a fixed part (set-up, first loads, exchange, stores: 2.5 - 5 us) and 0.18 us (BN 64) or 0.20 us (BN 128) per
 // 64-deep k-block of a CTA alone on its SM, which is what two loading threads in turn need for one (330 - 390 cycles).
 // Measured against 256-row tiles with the whole of K on one pair: the feed-forward block (forward and backward) on 128 tokens,
-// 1024 x 4096, 116 -> 45 us; the decoder layer's forward pass on 512 tokens 103 -> 51 us; the attention block on
-// 3 x 200 tokens 118 -> 48 us (its core included).
+// 1024 x 4096, 116 -> 48.6 us; the decoder layer's forward pass on 512 tokens 103 -> 57.4 us; the attention block on
+// 3 x 200 tokens 118 -> 48.2 us (its core included).  These are passes over tensors that change from one to the next; over the same ones, which then lie in
+// L2, 44.7, 51.6 and 47.6, and replayed from a graph 42.7, 49.0 and 44.3.
 // Included by gemm_tcgen05.cu, whose wrappers, bounded waits and status word it uses.
 
 struct ClusterArgs {

@@ -710,8 +710,8 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                     const __grid_constant__ CUtensorMap map_w, const __grid_constant__ ExtraMaps extra, const TcArgs a) {
   // kWide (pairs only): the pair owns a 256 x 512 tile, which fills the tensor memory: one accumulator,
   // so a tile's epilogue is not overlapped with the next tile's MMAs, but a CTA pulls 48 KB per
-  // k-block through L2 for twice the flops (24 KB per 256 x 256 x 64 instead of 32 KB).  For long K,
-  // where the contraction is bound by the L2-to-SM traffic and the exposed epilogue is small.
+  // k-block through L2 for twice the flops (24 KB per 256 x 256 x 64 instead of 32 KB), and its k-blocks are half as
+  // many for the threads that load.  For long K, where the exposed epilogue is small.
   static_assert(!kWide || (kPair && CM == 1 && CN == 1), "wide tiles: plain CTA pairs only");
   // The ring has a.n_stages stages of a.stage_bytes (32 KB for a pair with 256-column tiles: 5 stages;
   // 48 KB for wide and single-CTA 256-column tiles: 3 stages; narrower tiles get deeper rings).  The
@@ -1777,18 +1777,21 @@ void note_contraction(int columns, int split) { g_last_pick = {columns, split}; 
 
 // Which contractions run on 128-row tiles with K over a cluster, and how: the shorter of two estimates of a launch's time,
 // whose constants (microseconds) are fits to launches of 24 shapes from 128 x 1024 x 1024 to 4096 x 8192 x 1024 on each of
-// the eight variants and on gemm_tcgen05_kernel (B200, replayed back to back).  Both sides at some of them, us:
-//   128 x 1024 x 4096  35.6 there,  8.0 here (BN 64, split 8);    512 x 1024 x 1024  12.3 and 6.3 (64, 2);
-//   1024 x 1024 x 8192 60.8 and 23.6 (128, 4);   2048 x 1024 x 4096 30.8 and 19.9 (128, 2);
-//   24 x [200 x 64 x 200] 6.5 and 3.9 (64, 1);   8192 x 1024 x 1024 20.9 and 21.3 (128, 1);   4096 x 4096 x 1024 35.2 and 39.7.
-// There the persistent kernel pays a fixed part and a wave of tiles costs its k-blocks at the rate one SM takes operands in;
+// the eight variants and on gemm_tcgen05_kernel (B200, replayed back to back) when one thread loaded in either kernel.  Two load now, and a k-block costs
+// less on both sides than what stands here (0.18 us for 0.27, 0.20 for 0.34).  Both sides at some of the shapes as they are now, us:
+//   128 x 1024 x 4096  23.6 there,  7.0 here (BN 64, split 8);    512 x 1024 x 1024  11.1 and 5.3 (64, 2);
+//   1024 x 1024 x 8192 42.7 and 20.7 (128, 4);   2048 x 1024 x 4096 25.4 and 18.8 (128, 2);
+//   24 x [200 x 64 x 200] 5.7 and 3.7 (64, 1);   8192 x 1024 x 1024 19.1 and 20.7 (128, 1);   4096 x 4096 x 1024 30.6 and 39.0.
+// There the persistent kernel pays a fixed part and a wave of tiles costs its k-blocks;
 // here a round of two CTAs an SM costs the same k-blocks (at half the reuse), the epilogue, and the exchange between the
 // CTAs of a cluster, which is what keeps the split small.
+// 1451 drawn products on all nine: the choice is 2.3 % from the best on average, 9 % at the 90th percentile, 28 % at the 99th; the worst are long K cut too
+// finely (256 x 4608 x 3136: 19.4 us with K over 4, 12.4 over 2).  12 take more than 1.03 times their time on the persistent kernel, at most 1.23 times.
 // Products that fill the chip with 128-row tiles stray from the fits, those whose operands' rows do not lie on 128-byte lines
 // most (2664 x 2992 x 200: 13.9 us there, 19.7 here, estimated 13.1).  So more than one round counts 1.1 times its estimate; with
 // rows off the lines a round of two CTAs an SM counts 1.2 times, more than one 1.3 times, and the persistent kernel 0.9 instead of
-// 0.95 times its own.  Of 4400 drawn products 6 then take more than 1.03 times their time there (at most 1.15 times; 88, up to
-// 1.5, without the factors), and the mean gain is the same: exp(0.54).
+// 0.95 times its own.  (When the factors came, 6 of 4400 drawn products then took more than 1.03 times their time there, at most 1.15 times; 88, up to
+// 1.5, without them; the mean gain was the same.)
 static ClusterPick cluster_rule(const TcParams& t, int n_terms, int n_groups, int most) {
   ClusterPick best = {0, 0};
   if (!t.cluster_ok) return best;
@@ -2024,6 +2027,9 @@ mtf_status launch_tc(const mtf_plan_t& plan, const void* A, const void* B, void*
   const bool wide_legal = t.cta_pair && t.block_n == 256 && t.reduce_mode != MTF_REDUCE_WORKSPACE && (plain_epi || resid_only_epi) && !row_lse && a.Ns % 512 == 0;
   if (t.wide_pref == 1 && !wide_legal)
     return fail(MTF_ERR_UNSUPPORTED, "wide tiles need CTA pairs, a plain or residual-only epilogue, no workspace reduction and an N slice that is a multiple of 512");
+  // Wide tiles where they take less than two thirds of the waves and K hides their epilogue.  474 drawn products that may run on either: 0.5 % from the better
+  // on average; of the 114 that run wide 32 take more than 1.03 times their time on narrow tiles (7936 x 2560 x 5120 worst: 191 us and 164), of the 360 others 6
+  // (at most 1.09 times).  Always narrow: 0.7 %, 46 products, at most 1.15 times.
   if (wide_legal && t.wide_pref != 0) {
     long long tiles = (long long)((a.Ms + 2 * BM - 1) / (2 * BM)) * (a.Ns / 256) * a.sm * a.sn;
     for (int j = 0; j < t.n_outer; ++j) tiles *= t.outer_size[j];
