@@ -148,6 +148,29 @@ def test_small_operands_beside_large_ones(mtf, k, small, large, flip):  # noqa: 
             assert e.norm() <= 2 ** -24 * k ** 0.5 * f.norm() + k * 2 ** -149 * f.numel() ** 0.5, (r, c)
 
 
+@pytest.mark.parametrize("m,n,k", [(1, 1, 1), (130, 70, 70), (33, 65, 300), (300, 17, 33)])
+@pytest.mark.parametrize("order", ["bik,bkj", "bik,bjk", "bki,bkj", "bki,bjk", "ibk,kbj"])
+def test_large_operands(mtf, asked, order, m, n, k):  # noqa: F811
+    """Values from 2^111 on, in whole rows and columns and alone in one part of K: the second computation, whichever way the operands lie and wherever a
+    tile or a run of 32 k ends.  A sum of k products in any order of f32 additions is within k + 1 roundings, 2^-24 of the sum of magnitudes each."""
+    import torch
+    torch.manual_seed(m)
+    size = {"b": 2, "i": m, "j": n, "k": k}
+    dev = {"device": "cuda", "dtype": torch.float64}
+    x, y = torch.randn(2, m, k, **dev), torch.randn(2, k, n, **dev) * 1e-20
+    x[:, : m // 3] *= 2.0 ** 112
+    x[1, m - 1, k // 2] = 2.0 ** 120
+    y[0, :, n // 2] *= 2.0 ** 60
+    a, b = order.split(",")
+    tensors = [torch.einsum("%s->%s" % (full, t), v).contiguous().float() for full, t, v in (("bik", a, x), ("bkj", b, y))]
+    o = torch.full((2, m, n), float("nan"), device="cuda")
+    mtf.mtf_einsum(layout(mtf, *ONE), None, [mtf.named(t, list(names)) for t, names in zip(tensors, (a, b))], mtf.named(o, ["b", "i", "j"]))
+    mtf.mtf_device_status()
+    ref = torch.einsum("%s,%s->bij" % (a, b), *[t.double() for t in tensors])
+    scale = torch.einsum("%s,%s->bij" % (a, b), *[t.double().abs() for t in tensors])
+    assert ((o.double() - ref).abs() <= (k + 1) * 2 ** -24 * scale).all()
+
+
 @pytest.mark.parametrize("order", ["ik,kj", "ki,jk"])
 def test_results_out_of_range_cost_what_plain_arithmetic_costs(mtf, order):  # noqa: F811
     """A product of nothing but NaN is computed twice; measured, 4.4 times the time of ordinary values (with each thread computing its own outputs again: 112 times)."""
