@@ -385,10 +385,11 @@ mtf_status mtf_attention_backward(const mtf_layout_t* layout, const mtf_tensor* 
     core_ok = whole && mtf::attention_bwd_fused_supported(s.l.size, s.k.size, s.v.size);
     rows_ok = whole && !core_ok && rows_core_wanted(s);
   }
-  // dWo reads o and dy and nothing the core touches.  Behind the one-launch core it is issued as an independent launch
-  // with the group sum chained in its accumulators (no cleared counters in front of it), so its tiles start on the SMs
-  // that the core's last round of (batch, head) pairs leaves idle; otherwise it goes first.
-  const bool dwo_late = core_ok;
+  // dWo reads o and dy and nothing the core touches.  Behind either core it is issued as an independent launch, so its tiles
+  // start on the SMs that the core's last round leaves idle (behind the one-launch core with the group sum chained in its
+  // accumulators: no cleared counters in front of it); otherwise it goes first.  Behind the core by rows, 3 x 200 positions, 8 heads of
+  // 64: the block 48.1 -> 43.8 us; 4 x 1024, 8 heads of 128, whose core fills the chip: 205.7 and 206.4.
+  const bool dwo_late = core_ok || rows_ok;
   if (!dwo_late && (st = ein(layout, *o, *dy, dwo, nullptr, rest, rest_bytes, stream)) != MTF_OK) return st;
   if ((st = ein(layout, *dy, *wo, &dob.t, nullptr, rest, rest_bytes, stream)) != MTF_OK) return st;
   if ((st = mtf::tap("do", dob.t, stream)) != MTF_OK) return st;
@@ -418,6 +419,8 @@ mtf_status mtf_attention_backward(const mtf_layout_t* layout, const mtf_tensor* 
     st = mtf::launch_attention_rows(true, dob.t.data, kk->data, vv->data, weights->data, dlg.t.data, dq.t.data, s.b.size, s.h.size, s.l.size, s.k.size, (float)s.scale,
                                     causal ? 1 : 0, mtf::tap_is_open() ? 1 : 0, stream);
     if (st != MTF_OK || (st = mtf::tap("dlogits", dlg.t, stream)) != MTF_OK) return st;
+    mtf::hint_next_launch_independent();
+    if ((st = ein(layout, *o, *dy, dwo, nullptr, rest, rest_bytes, stream)) != MTF_OK) return st;
     if ((st = mtf::attention_kv(layout, &dlg.t, q, &dkk.t, (float)s.scale, weights, &dob.t, &dvv.t, causal ? 1 : 0, stream)) != MTF_OK) return st;
     core_done = true;
   }
