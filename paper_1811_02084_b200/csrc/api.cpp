@@ -2,6 +2,7 @@
 // numerical step runs in the CUDA kernels; this file only validates, plans and launches.
 #include <algorithm>
 #include <cstring>
+#include <initializer_list>
 
 #include "mtf_internal.h"
 
@@ -23,6 +24,12 @@ mtf_status launch_permute_copy(const void* src, void* dst, int elem_bytes, int n
 mtf_status read_attention_bwd_status(int* code);
 mtf_status read_attention_rows_status(int* code);
 mtf_status read_f32_status(int* code);
+bool tap_is_open();
+bool ffn_small_pays(int64_t T, int64_t D, int64_t F, int64_t E, bool backward);
+mtf_status launch_ffn_small_forward(int64_t T, int64_t D, int64_t F, int64_t E, const float* x, const float* w, const float* bias, const float* v, float* h, float* y,
+                                    void* stream);
+mtf_status launch_ffn_small_backward(int64_t T, int64_t D, int64_t F, int64_t E, const float* x, const float* w, const float* v, const float* h, const float* dy,
+                                     float* dx, float* dw, float* dbias, float* dv, float* dhp, void* stream);
 }  // namespace mtf
 
 using mtf::Dim;
@@ -178,9 +185,12 @@ mtf_status check_equation(const char* eq, int n_in, const mtf_tensor* in, const 
 
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
-struct FfnShapes {
-  std::vector<mtf_dim> tok_hidden, hidden_only;
-};
+bool same_dims(const mtf_tensor& a, const mtf_tensor& b) {
+  if (a.ndim != b.ndim || !a.dims || !b.dims) return false;
+  for (int i = 0; i < a.ndim; ++i)
+    if (!a.dims[i].name || !b.dims[i].name || a.dims[i].size != b.dims[i].size || strcmp(a.dims[i].name, b.dims[i].name) != 0) return false;
+  return true;
+}
 
 mtf_status ffn_check(const mtf_tensor* x, const mtf_tensor* w, const mtf_tensor* v) {
   if (!x || !w || !v) return fail(MTF_ERR_INVALID_ARG, "ffn: NULL tensor");
@@ -426,6 +436,37 @@ mtf_status mtf_ffn_forward(const mtf_layout_t* layout, const mtf_tensor* x, cons
 
 }  // extern "C"
 
+// The f32 block on a few tokens in one launch (ffn_f32_small.cu): tensors dense in the order tokens, then width; nothing forced or asked for, no
+// ranks, no output that lies over an operand or another output (launch by launch that is well defined).  `t`: operands, then outputs from `first_out`.
+static bool ffn_small_shape(const mtf_layout_t* layout, const mtf_tensor* x, const mtf_tensor* w, const mtf_tensor* v, const mtf_tensor* h, const mtf_tensor* y,
+                            const mtf_tensor* bias, std::initializer_list<const mtf_tensor*> t, int first_out, bool backward, int64_t* size) {
+  if (!layout || layout->bound_dim >= 0 || mtf::plan_forced() || mtf::contraction_asked()) return false;
+  const int n = x->ndim;
+  if (n > mtf::kMaxTensorDims || h->ndim != n || y->ndim != n || !h->dims || !y->dims || (bias && (bias->ndim != 1 || !bias->dims))) return false;
+  auto is = [](const mtf_dim& a, const mtf_dim& b) { return a.name && b.name && a.size == b.size && strcmp(a.name, b.name) == 0; };
+  int64_t T = 1;
+  for (int i = 0; i + 1 < n; ++i) {
+    if (!is(x->dims[i], h->dims[i]) || !is(x->dims[i], y->dims[i])) return false;
+    T *= x->dims[i].size;
+    if (T <= 0 || T > 4096) return false;
+  }
+  if (!is(x->dims[n - 1], w->dims[0]) || !is(w->dims[1], v->dims[0]) || !is(w->dims[1], h->dims[n - 1]) || !is(v->dims[1], y->dims[n - 1]) || (bias && !is(bias->dims[0], w->dims[1]))) return false;
+  size[0] = T; size[1] = w->dims[0].size; size[2] = w->dims[1].size; size[3] = v->dims[1].size;
+  if (!mtf::ffn_small_pays(size[0], size[1], size[2], size[3], backward)) return false;
+  const uint8_t *lo[10], *hi[10];
+  int k = 0;
+  for (const mtf_tensor* p : t) {
+    if (!p) { lo[k] = hi[k] = nullptr; ++k; continue; }
+    if (p->dtype != MTF_F32 || !p->data) return false;
+    lo[k] = reinterpret_cast<const uint8_t*>(p->data);
+    hi[k] = lo[k] + numel(*p) * 4;
+    for (int i = 0; i < k; ++i)
+      if (k >= first_out && lo[k] < hi[i] && lo[i] < hi[k]) return false;
+    ++k;
+  }
+  return true;
+}
+
 // y_residual (NULL or a tensor with y's dims) is added to y in the second einsum's epilogue.
 mtf_status mtf::ffn_forward_impl(const mtf_layout_t* layout, const mtf_tensor* x, const mtf_tensor* w, const mtf_tensor* bias,
                                  const mtf_tensor* v, mtf_tensor* h_saved, mtf_tensor* y, const mtf_tensor* y_residual, void* workspace,
@@ -437,8 +478,18 @@ mtf_status mtf::ffn_forward_impl(const mtf_layout_t* layout, const mtf_tensor* x
   mtf_epilogue e1;
   e1.scale = 1.f; e1.relu = 1; e1.bias = bias; e1.relu_mask = nullptr; e1.residual = nullptr; e1.reduce_sum_out = nullptr;
   mtf_tensor in1[2] = {*x, *w};
-  if ((st = mtf_einsum(layout, nullptr, 2, in1, h_saved, &e1, workspace, workspace_bytes, stream)) != MTF_OK) return st;
   mtf_tensor in2[2] = {*h_saved, *v};
+  int64_t n[4];
+  if (!y_residual && ffn_small_shape(layout, x, w, v, h_saved, y, bias, {x, w, bias, v, h_saved, y}, 4, false, n)) {
+    // (the plans say whether the layout is legal)
+    const mtf_plan_t *P1 = nullptr, *P2 = nullptr;
+    if (cached_plan(layout, 2, in1, h_saved, &e1, &P1) == MTF_OK && cached_plan(layout, 2, in2, y, nullptr, &P2) == MTF_OK) {
+      (void)mtf::take_independent_hint();
+      return mtf::launch_ffn_small_forward(n[0], n[1], n[2], n[3], (const float*)x->data, (const float*)w->data, bias ? (const float*)bias->data : nullptr,
+                                           (const float*)v->data, (float*)h_saved->data, (float*)y->data, stream);
+    }
+  }
+  if ((st = mtf_einsum(layout, nullptr, 2, in1, h_saved, &e1, workspace, workspace_bytes, stream)) != MTF_OK) return st;
   mtf_epilogue e2;
   e2.scale = 1.f; e2.relu = 0; e2.bias = nullptr; e2.relu_mask = nullptr; e2.residual = y_residual; e2.reduce_sum_out = nullptr;
   return mtf_einsum(layout, nullptr, 2, in2, y, y_residual ? &e2 : nullptr, workspace, workspace_bytes, stream);
@@ -644,17 +695,30 @@ mtf_status mtf::ffn_backward_impl(const mtf_layout_t* layout, const mtf_tensor* 
   e1.scale = 1.f; e1.relu = 0; e1.bias = nullptr; e1.relu_mask = h_saved; e1.residual = nullptr;
   e1.reduce_sum_out = fuse_dbias ? dbias : nullptr;
   mtf_tensor in1[2] = {*dy, *v};
+  mtf_tensor in2[2] = {*h_saved, *dy};
+  mtf_tensor in3[2] = {*x, dhp};
+  mtf_tensor in4[2] = {dhp, *w};
+  int64_t n[4];
+  if (!dx_residual && same_dims(*x, *dx) && same_dims(*w, *dw) && same_dims(*v, *dv) &&
+      ffn_small_shape(layout, x, w, v, h_saved, dy, dbias, {x, w, v, h_saved, dy, &dhp, dx, dw, dbias, dv}, 5, true, n)) {
+    const mtf_plan_t* P = nullptr;
+    if (cached_plan(layout, 2, in1, &dhp, &e1, &P) == MTF_OK && cached_plan(layout, 2, in2, dv, nullptr, &P) == MTF_OK &&
+        cached_plan(layout, 2, in3, dw, nullptr, &P) == MTF_OK && cached_plan(layout, 2, in4, dx, nullptr, &P) == MTF_OK) {
+      (void)mtf::take_independent_hint();
+      st = mtf::launch_ffn_small_backward(n[0], n[1], n[2], n[3], (const float*)x->data, (const float*)w->data, (const float*)v->data, (const float*)h_saved->data,
+                                          (const float*)dy->data, (float*)dx->data, (float*)dw->data, dbias ? (float*)dbias->data : nullptr, (float*)dv->data,
+                                          mtf::tap_is_open() ? (float*)dhp.data : nullptr, stream);
+      return st != MTF_OK ? st : mtf::tap("dhp", dhp, stream);
+    }
+  }
   if ((st = mtf_einsum(layout, nullptr, 2, in1, &dhp, &e1, rest, rest_bytes, stream)) != MTF_OK) return st;
   if ((st = mtf::tap("dhp", dhp, stream)) != MTF_OK) return st;
   // dv = h^T . dy  and  dw = x^T . dhp  reduce out the token dims (Section 8.1)
-  mtf_tensor in2[2] = {*h_saved, *dy};
   mtf::hint_next_launch_independent();        // dv reads h and dy, which the dhp launch only reads, and writes dv
   if ((st = mtf_einsum(layout, nullptr, 2, in2, dv, nullptr, rest, rest_bytes, stream)) != MTF_OK) return st;
-  mtf_tensor in3[2] = {*x, dhp};
   if ((st = mtf_einsum(layout, nullptr, 2, in3, dw, nullptr, rest, rest_bytes, stream)) != MTF_OK) return st;
   if (dbias && !fuse_dbias && (st = mtf_reduce_sum(layout, &dhp, dbias, stream)) != MTF_OK) return st;
   // dx = dhp . w^T reduces out hidden (Section 8.2)
-  mtf_tensor in4[2] = {dhp, *w};
   mtf_epilogue e4;
   e4.scale = 1.f; e4.relu = 0; e4.bias = nullptr; e4.relu_mask = nullptr; e4.residual = dx_residual; e4.reduce_sum_out = nullptr;
   if (!(dbias && !fuse_dbias)) mtf::hint_next_launch_independent();      // dx reads dhp and w and writes dx; the dw launch before it reads x and dhp and writes dw
