@@ -790,8 +790,11 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   // (late_wait: this launch reads and writes nothing that the launch before it on the stream touches, so it
   // starts at once and fills the SMs that launch's last tiles leave idle; it waits for it before exiting
   // instead, so that whatever follows on the stream still sees every earlier launch complete.)
-  if (!a.late_wait) asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // Loading threads first work out their first tile: the launch's arguments are then at hand when the wait ends (1024 x 3072 x 4096 28.3 -> 27.0 us).
+  auto chain = [&]() {
+    if (!a.late_wait) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  };
 
   const int n_local = kPair ? a.block_n / 2 : a.block_n;       // N columns of B this CTA stages (wide: two runs of 128)
   const uint32_t b_bytes = (uint32_t)n_local * BK * 2;
@@ -801,9 +804,11 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     // A wait, the barrier's byte count and the copies of a k-block take one thread 560 - 680 cycles, however many stages the ring has; the
     // MMAs of a 256 x 256 tile's k-block take 512.  So two threads take turns: 8192 x 8192 x 1024 103.5 -> 97.5 us, 8192 x 32768 x 1024 415 -> 390,
     // 16384 x 2048 x 2048 101 -> 97.6 (launches apart; less where a stream of them runs into the power limit).
+    // What such a thread does between two copies counts where a k-block's MMAs take less than that: each walks only its own k-blocks and keeps the operands'
+    // maps, and 64 k-blocks of 256 x 128 tiles cost 20.0 -> 15.4 us (1024 x 1024 x 4096, both operands along M and N), two waves of them 35.9 -> 27.5.
     const int producer = warp == 0 ? 0 : warp - 1 - kEpilogueWarps;
     if (mtf::elect_one()) {
-      int stage = 0, turn = 0;
+      int stage = producer;
       uint32_t phase = 0;
       bool ok = true;
       SegIter it(a, work_first, work_step);
@@ -831,35 +836,39 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         ++dseq;
         return it.take(sg, (long long)t);
       };
-      while (ok && next_tile()) {
-        const int kb_first = sg.kb_begin, kb_count = sg.kb_count;
-        const Tile tl = decode_tile(a, sg.tile, kTileRows, a.block_n * CN);
+      bool more = next_tile();
+      Tile tl = decode_tile(a, more ? sg.tile : 0, kTileRows, a.block_n * CN);
+      const CUtensorMap *pa = &map_a, *pb = &map_b;
+      const uint32_t bytes = (kPair ? 2u : 1u) * (kAStageBytes + b_bytes);
+      chain();
+      int ahead = producer;      // k-blocks of the coming tile until this thread's next one
+      for (; more; more = ok && next_tile(), tl = decode_tile(a, more ? sg.tile : 0, kTileRows, a.block_n * CN)) {
+        const int kb_count = sg.kb_count;
         const int m0 = tl.m0 + pm * kPairRows + cta_rank * BM;
         const int n0 = tl.n0 + pn * a.block_n + cta_rank * n_local;
-        int term = kb_first / a.kb_term, kt = kb_first - term * a.kb_term;
-        for (int kb = 0; kb < kb_count; ++kb) {
-          if (drawn && drawer && !have_pending && kb == (kb_count > 4 ? kb_count - 4 : 0)) { pending = (unsigned)work_step + atomicAdd(a.sched, 1u); have_pending = true; }
-          // slices of the reduce group are walked in ascending order: k0 runs through slice 0's
-          // block of K, then slice 1's, ... (the blocks are contiguous in the global tensor); a
-          // multi-term launch then goes on with the next product's operands
+        // slices of the reduce group are walked in ascending order: k0 runs through slice 0's block of K, then slice 1's, ... (the
+        // blocks are contiguous in the global tensor); a multi-term launch then goes on with the next product's operands
+        int kb = ahead, kt = sg.kb_begin + ahead, term = 0;
+        auto operands = [&](int sel) {
+          pa = sel == 0 ? &map_a : &extra.m[2 * (sel - 1)];
+          pb = sel == 0 ? &map_b : &extra.m[2 * (sel - 1) + 1];
+        };
+        if (a.n_groups > 1) operands(sg.group);
+        else if (a.n_terms > 1) operands(0);
+        for (; kb < kb_count; kb += kProducers, kt += kProducers) {
+          if (drawn && drawer && !have_pending && kb >= kb_count - 5) { pending = (unsigned)work_step + atomicAdd(a.sched, 1u); have_pending = true; }
+          if (kt >= a.kb_term) {
+            do { kt -= a.kb_term; ++term; } while (kt >= a.kb_term);
+            operands(term);
+          }
           const int k0 = kt * BK;
-          const int sel = a.n_groups > 1 ? sg.group : term;          // operand pair: the problem of a grouped launch, else the term
-          const CUtensorMap* const pa = sel == 0 ? &map_a : &extra.m[2 * (sel - 1)];
-          const CUtensorMap* const pb = sel == 0 ? &map_b : &extra.m[2 * (sel - 1) + 1];
-          if (++kt == a.kb_term) { kt = 0; ++term; }
-          const bool mine = turn == producer;
-          if (++turn == kProducers) turn = 0;
-          const int at = stage;
-          const uint32_t at_phase = phase;
-          if (++stage == kStages) { stage = 0; phase ^= 1u; }
-          if (!mine) continue;
-          if (!(ok = mbar_wait(empty_bar(at), at_phase ^ 1u, 0x100 + at, abort_flag))) break;
+          if (!(ok = mbar_wait(empty_bar(stage), phase ^ 1u, 0x100 + stage, abort_flag))) break;
           // a pair's loads all count on the even CTA's barrier, which expects both CTAs' bytes
-          if (!kPair) mbar_expect_tx(full_bar(at), kAStageBytes + b_bytes);
-          else if (leader) mbar_expect_tx(full_bar(at), 2u * (kAStageBytes + b_bytes));
-          const uint32_t fb = kPair ? (full_bar(at) & 0xFEFFFFFFu) : full_bar(at);
-          const uint32_t sa = tiles_base + at * kStageBytes;
+          if (leader) mbar_expect_tx(full_bar(stage), bytes);
+          const uint32_t fb = kPair ? (full_bar(stage) & 0xFEFFFFFFu) : full_bar(stage);
+          const uint32_t sa = tiles_base + stage * kStageBytes;
           const uint32_t sb = sa + kAStageBytes;
+          if ((stage += kProducers) >= kStages) { stage -= kStages; phase ^= 1u; }
 #if defined(MTF_CLUSTER_SHARE)
           if (CN > 1) cluster_share_load_a(sa, pa, fb, pm, pn, CN, cta_rank, a.a_mn_major, BM / CN, m0, k0, tl.o[2], tl.o[1], tl.o[0]);
           else
@@ -886,13 +895,16 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
               }
             }
           } else if (a.b_mn_major) {
-            for (int j = 0; j < n_local / 64; ++j)
-              tma_load_5d<kPair>(sb + 8192 * j, pb, fb, n0 + 64 * j, k0, tl.o[2], tl.o[1], tl.o[0]);
+            for (int j = 0; j < n_local; j += 64)
+              tma_load_5d<kPair>(sb + 128 * j, pb, fb, n0 + j, k0, tl.o[2], tl.o[1], tl.o[0]);
           } else {
             tma_load_5d<kPair>(sb, pb, fb, k0, n0, tl.o[2], tl.o[1], tl.o[0]);
           }
         }
+        ahead = kb - kb_count;
       }
+    } else {
+      chain();
     }
   } else if (warp == 1) {
     // ------------------------------- MMA issuer (even CTA of a pair only) -------
@@ -908,6 +920,8 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
           if (i == pm || j == pn) empty_mask |= (uint16_t)(3u << (2 * (i * CN + j)));
       const uint32_t a_kstep = a.a_mn_major ? 2048u : 32u;   // bytes per 16 k-elements
       const uint32_t b_kstep = a.b_mn_major ? 2048u : 32u;
+      const uint64_t a_fix = make_smem_desc(0, a.a_mn_major), b_fix = make_smem_desc(0, a.b_mn_major);
+      chain();
       int stage = 0;
       uint32_t phase = 0;
       int iter = 0;
@@ -930,22 +944,24 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         for (int kb = 0; kb < kb_count; ++kb) {
           if (!(ok = mbar_wait(full_bar(stage), phase, 0x300 + stage, abort_flag))) break;
           tcgen05_fence_after();
-          const uint32_t sa = tiles_base + stage * kStageBytes;
+          const uint32_t sa = (tiles_base & 0x3FFFFu) + stage * kStageBytes;      // (an address' upper bits are the block's rank in its cluster)
           const uint32_t sb = sa + kAStageBytes;
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k) {
-            const uint64_t da = make_smem_desc(sa + k * a_kstep, a.a_mn_major);
-            const uint64_t db = make_smem_desc(sb + k * b_kstep, a.b_mn_major);
+            const uint64_t da = a_fix | ((sa + k * a_kstep) >> 4), db = b_fix | ((sb + k * b_kstep) >> 4);
             umma_bf16<kPair>(tmem_c, da, db, idesc, (kb | k) != 0);
-            if (kWide) umma_bf16<kPair>(tmem_c + 256u, da, make_smem_desc(sb + 16384u + k * b_kstep, a.b_mn_major), idesc, (kb | k) != 0);
+            if (kWide) umma_bf16<kPair>(tmem_c + 256u, da, db + (16384u >> 4), idesc, (kb | k) != 0);
           }
           umma_commit<kPair>(empty_bar(stage), empty_mask);   // frees the stage in every CTA that writes into this pair's tiles
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
         if (ok && !(iter == 0 && g_skip_first_commit)) umma_commit<kPair>(tfull_bar(acc), pair_mask);   // accumulator complete (in both CTAs of the pair)
       }
+    } else {
+      chain();
     }
   } else {
+    chain();
     // ------------------------------- epilogue -----------------------------------
     const EpiFlags f = epi_flags<EPI>(a);
     const int q = warp & 3;                        // TMEM lane quarter this warp may read
