@@ -97,6 +97,7 @@ struct TcArgs {
   long long outer_sC[3];
   int a_mn_major, b_mn_major;
   int block_n;
+  int b_box;               // columns of an N-contiguous B per copy: 64 (128-byte swizzle), or 32 (64-byte swizzle) where a CTA's half of the tile is no multiple of 64
   long long ldc;
   int k_sliced;            // walk K slice by slice (slice length is a multiple of BK)
   int reduce_mode;
@@ -479,10 +480,11 @@ __device__ __forceinline__ float ex2_approx(float x) {
 //   K-major  (rows of 64 K-elements = 128 B; 8-row groups 1024 B apart): LBO unused (1), SBO = 1024 B
 //   MN-major (rows of 64 M/N-elements = 128 B, one row per k; 64-wide column blocks 8 KB apart):
 //             LBO = 8192 B (next 64 M/N), SBO = 1024 B (next 8 k)
-__device__ __forceinline__ uint64_t make_smem_desc(uint32_t addr, int mn_major) {
-  const uint64_t lbo = mn_major ? (8192u >> 4) : 1u;
-  const uint64_t sbo = 1024u >> 4;
-  return (uint64_t)((addr & 0x3FFFF) >> 4) | (lbo << 16) | (sbo << 32) | (1ull << 46) | (2ull << 61);
+//   MN-major, 64-byte swizzle (rows of 32 M/N-elements = 64 B; 32-wide column blocks 4 KB apart): LBO = 4096 B, SBO = 512 B
+__device__ __forceinline__ uint64_t make_smem_desc(uint32_t addr, int mn_major, bool half = false) {
+  const uint64_t lbo = mn_major ? (half ? 4096u : 8192u) >> 4 : 1u;
+  const uint64_t sbo = (half ? 512u : 1024u) >> 4;
+  return (uint64_t)((addr & 0x3FFFF) >> 4) | (lbo << 16) | (sbo << 32) | (1ull << 46) | ((half ? 4ull : 2ull) << 61);
 }
 
 __device__ __forceinline__ float bf16_bits_to_float(uint32_t lo16) { return __uint_as_float(lo16 << 16); }
@@ -895,7 +897,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
               }
             }
           } else if (a.b_mn_major) {
-            for (int j = 0; j < n_local; j += 64)
+            for (int j = 0; j < n_local; j += a.b_box)
               tma_load_5d<kPair>(sb + 128 * j, pb, fb, n0 + j, k0, tl.o[2], tl.o[1], tl.o[0]);
           } else {
             tma_load_5d<kPair>(sb, pb, fb, k0, n0, tl.o[2], tl.o[1], tl.o[0]);
@@ -919,8 +921,9 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         for (int j = 0; j < CN; ++j)
           if (i == pm || j == pn) empty_mask |= (uint16_t)(3u << (2 * (i * CN + j)));
       const uint32_t a_kstep = a.a_mn_major ? 2048u : 32u;   // bytes per 16 k-elements
-      const uint32_t b_kstep = a.b_mn_major ? 2048u : 32u;
-      const uint64_t a_fix = make_smem_desc(0, a.a_mn_major), b_fix = make_smem_desc(0, a.b_mn_major);
+      const bool b_half = a.b_mn_major && a.b_box == 32;
+      const uint32_t b_kstep = a.b_mn_major ? (b_half ? 1024u : 2048u) : 32u;
+      const uint64_t a_fix = make_smem_desc(0, a.a_mn_major), b_fix = make_smem_desc(0, a.b_mn_major, b_half);
       chain();
       int stage = 0;
       uint32_t phase = 0;
@@ -1543,7 +1546,7 @@ EncodeTiledFn get_encode() {
 //   dim0 / dim1 : extents of the contiguous and of the strided dimension; ld = element stride of dim1
 //   box0 / box1 : box extents in elements (box0 * elem_bytes = 128)
 mtf_status make_map(CUtensorMap* map, const void* base, int elem_bytes, int64_t dim0, int64_t dim1, int64_t ld,
-                    int box0, int box1, const TcParams& t, const int64_t* outer_stride) {
+                    int box0, int box1, const TcParams& t, const int64_t* outer_stride) {      // (box0 elements: 128 or 64 bytes, which is then the swizzle)
   EncodeTiledFn enc = get_encode();
   if (!enc) return mtf::fail(MTF_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
   if (reinterpret_cast<uintptr_t>(base) & 15) return mtf::fail(MTF_ERR_INVALID_ARG, "tensor-core path needs 16-byte aligned tensors");
@@ -1570,7 +1573,7 @@ mtf_status make_map(CUtensorMap* map, const void* base, int elem_bytes, int64_t 
     }
   }
   CUresult r = mtf::in_context([&] { return enc(map, elem_bytes == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, const_cast<void*>(base),
-                   dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                   dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, box0 * elem_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE); });
   if (r != CUDA_SUCCESS)
     return mtf::fail(MTF_ERR_CUDA, "cuTensorMapEncodeTiled failed with %d (dims %llu %llu %llu %llu %llu, strides %llu %llu %llu %llu)", (int)r,
@@ -1791,6 +1794,58 @@ mtf_status debug_contraction(int bn, int split, int* ran_bn, int* ran_split) {
 int contraction_asked() { return g_asked_pick.split ? g_asked_pick.bn : 0; }
 void note_contraction(int columns, int split) { g_last_pick = {columns, split}; }
 
+// How long a launch of CTA pairs takes on 256 rows by bn columns, in microseconds: fits to 7459 drawn products (130 to 12000 rows, 136 to 8192 columns, K 64 to 8192,
+// every operand order, rows on and off 128-byte lines, whole and in slices, bf16 and f32 results; graphs of launches, operands in L2), which they miss by 10 % rms (512 columns
+// 6 %).  What a k-block costs is the larger of its MMAs, 2 bn cycles, and of the 128-byte requests that its copies make, 1.5 cycles each: more from rows off the lines, where a
+// line is shared, and from the 64-byte boxes of an N-contiguous B in 192 columns.
+// us on 256 columns inside the slices and on what is chosen:  1665 x 3080 x 776 in five slices, B K-contiguous 19.0 and 16.6 (192 across the slices);  1665 x 776 x
+// 3080 24.6 and 20.0 (128 across);  1024 x 3072 x 4096 27.0 and 22.6 (192);  1024 x 1024 x 4096 24.7 and 15.4 (128).
+static double tile_outer(const TcParams& t, int n_groups) {
+  double outer = n_groups;
+  for (int j = 0; j < t.n_outer; ++j) outer *= (double)t.outer_size[j];
+  return outer;
+}
+
+static double request_share(bool off_lines, double extra) { return off_lines ? 1.0 + extra : 1.0; }
+
+static double pair_us(const TcParams& t, double kb, double outer, int bn, bool flat) {
+  const int64_t sm = flat ? 1 : t.sm, sn = flat ? 1 : t.sn;
+  const double tiles = (double)((t.M / sm + 2 * BM - 1) / (2 * BM) * sm) * (double)((t.N / sn + bn - 1) / bn * sn) * outer, waves = std::ceil(tiles / (sm_count() / 2));
+  const double a = 128.0 * request_share(t.a_ld % 64 != 0, 0.42), b = bn / 2 * request_share(t.b_ld % 64 != 0, 0.42), wide = t.c_f32 ? 1.5 : 1.0;
+  if (bn == 512) return 2.35 + waves * (kb * std::max(1024.0, 1.5 * (a + b)) + 8960.0 * wide) / 1741.0;
+  const double main = kb * std::max(2.0 * bn, 1.5 * (a + b * (bn == 192 && t.b_mn_major ? 1.53 : 1.0))) + 4150.0, out = 11.0 * bn * wide;
+  return 1.85 + (main + out + (waves - 1.0) * std::max(main, out)) / 1787.0;
+}
+
+// Tiles of a launch of CTA pairs: 256 rows by bn columns (512: "wide"), inside the layout's slices or (flat) across their edges, which an output
+// element, one sum over all of K whoever owns it, does not notice.
+struct PairTiles { int bn; bool flat; double us; };
+
+// Wide tiles where they take less than two thirds of the waves and K hides their one accumulator's exposed epilogue.  They pull fewer bytes through L2, which counts where a
+// stream of launches runs into the power limit and not in one launch: 8192 x 1024 x 8192 108.9 us here and 123.0 with 256 columns, back to back for a quarter of a second;
+// 16384 x 2048 x 8192 with a residual 490 and 526; 2048 x 8192 x 16384 429 and 444; in graphs of a few launches nowhere better by more than 1 %.
+static bool widens(const TcParams& t, int n_terms, int n_groups) {
+  const double workers = sm_count() / 2, tiles = (double)((t.M / t.sm + 2 * BM - 1) / (2 * BM) * t.sm) * (double)(t.N / 256) * tile_outer(t, n_groups);
+  return t.K * n_terms >= 64 * BK && 3.0 * std::ceil(tiles / 2.0 / workers) < 2.0 * std::ceil(tiles / workers);
+}
+
+// free_tiles: the launch may leave 256 columns and the slices; may_widen: its epilogue allows 512 columns.  Narrower tiles pull more bytes per
+// multiply-add, so they have to be 3 % shorter by the estimate.
+static PairTiles pair_tiles(const TcParams& t, int n_terms, int n_groups, bool free_tiles, bool may_widen) {
+  const double kb = (double)((t.K + BK - 1) / BK) * n_terms, outer = tile_outer(t, n_groups);
+  if (may_widen && widens(t, n_terms, n_groups)) return {512, false, pair_us(t, kb, outer, 512, false)};
+  PairTiles best = {t.block_n, false, pair_us(t, kb, outer, t.block_n, false)};
+  if (free_tiles && t.block_n == 256 && t.reduce_mode != MTF_REDUCE_WORKSPACE && !t.balance) {
+    double least = best.us;
+    for (int bn = 256; bn >= 128; bn -= 64)
+      for (int flat = 0; flat <= (t.sm * t.sn > 1 ? 1 : 0); ++flat) {
+        const double us = pair_us(t, kb, outer, bn, flat != 0);
+        if (us * (bn < 256 ? 1.03 : 1.0) < least) { least = us * (bn < 256 ? 1.03 : 1.0); best = {bn, flat != 0, us}; }
+      }
+  }
+  return best;
+}
+
 // Which contractions run on 128-row tiles with K over a cluster, and how: the shorter of two estimates of a launch's time,
 // whose constants (microseconds) are fits to launches of 24 shapes from 128 x 1024 x 1024 to 4096 x 8192 x 1024 on each of
 // the eight variants and on gemm_tcgen05_kernel (B200, replayed back to back) when one thread loaded in either kernel.  Two load now, and a k-block costs
@@ -1808,18 +1863,19 @@ void note_contraction(int columns, int split) { g_last_pick = {columns, split}; 
 // rows off the lines a round of two CTAs an SM counts 1.2 times, more than one 1.3 times, and the persistent kernel 0.9 instead of
 // 0.95 times its own.  (When the factors came, 6 of 4400 drawn products then took more than 1.03 times their time there, at most 1.15 times; 88, up to
 // 1.5, without them; the mean gain was the same.)
-static ClusterPick cluster_rule(const TcParams& t, int n_terms, int n_groups, int most) {
+static ClusterPick cluster_rule(const TcParams& t, int n_terms, int n_groups, int most, bool may_widen) {
   ClusterPick best = {0, 0};
   if (!t.cluster_ok) return best;
   const double sms = sm_count();
   const double kb = (double)((t.K + BK - 1) / BK) * n_terms;
-  double outer = n_groups;
-  for (int j = 0; j < t.n_outer; ++j) outer *= (double)t.outer_size[j];
+  const double outer = tile_outer(t, n_groups);
   const int64_t rows = t.cta_pair ? 2 * BM : BM;
   const double tiles = (double)((t.M / t.sm + rows - 1) / rows * t.sm) * (double)((t.N / t.sn + t.block_n - 1) / t.block_n * t.sn) * outer;
   const double per_kb = t.cta_pair ? (t.block_n == 256 ? 0.36 : 0.24) : (t.block_n == 256 ? 0.45 : t.block_n == 128 ? 0.33 : 0.27);
   const bool on_lines = t.a_ld % 64 == 0 && t.b_ld % 64 == 0;
   double best_us = (on_lines ? 0.95 : 0.9) * (7.0 + std::ceil(tiles / std::floor(sms / (t.cta_pair ? 2 : 1))) * kb * per_kb);
+  // (what other tiles of the persistent kernel save there)
+  if (t.cta_pair) best_us *= std::min(1.0, pair_tiles(t, n_terms, n_groups, t.free_tiles, may_widen).us / pair_us(t, kb, outer, t.block_n, false));
   for (int bn = 64; bn <= 128; bn += 64) {
     const double ctas1 = (double)((t.M + BM - 1) / BM) * (double)((t.N + bn - 1) / bn) * outer;
     for (int split = 1; split <= most && split <= kb; split *= 2) {
@@ -1835,10 +1891,10 @@ static ClusterPick cluster_rule(const TcParams& t, int n_terms, int n_groups, in
   return best;
 }
 
-static ClusterPick cluster_pick(const TcParams& t, int n_terms, int n_groups) {
+static ClusterPick cluster_pick(const TcParams& t, int n_terms, int n_groups, bool may_widen) {
   if (!t.cluster_ok || (g_whole_sums && t.reduce_mode == MTF_REDUCE_WORKSPACE)) return {0, 0};
   if (g_asked_pick.split) return g_asked_pick.split <= (t.K + BK - 1) / BK * n_terms ? g_asked_pick : ClusterPick{0, 0};
-  return cluster_rule(t, n_terms, n_groups, g_whole_sums ? 1 : 8);
+  return cluster_rule(t, n_terms, n_groups, g_whole_sums ? 1 : 8, may_widen);
 }
 
 // Scratch for a fused reduce_sum whose column sums are finished in a fixed order: one fp32 row of N per 32-row group of the
@@ -1847,7 +1903,7 @@ size_t tc_rsum_partial_bytes(const TcParams& t) {
   const int rows = tc_tile_rows(t);
   int64_t outer = 1;
   for (int j = 0; j < t.n_outer; ++j) outer *= t.outer_size[j];
-  const int64_t groups = std::max(((t.M / t.sm + rows - 1) / rows) * (rows / 32) * t.sm, (t.M + BM - 1) / BM * cluster_rule(t, 1, 1, 8).split) * outer;
+  const int64_t groups = std::max(((t.M / t.sm + rows - 1) / rows) * (rows / 32) * t.sm, (t.M + BM - 1) / BM * cluster_rule(t, 1, 1, 8, false).split) * outer;
   return (size_t)groups * t.N * sizeof(float);
 }
 
@@ -1994,8 +2050,13 @@ mtf_status launch_tc(const mtf_plan_t& plan, const void* A, const void* B, void*
     if (reinterpret_cast<uintptr_t>(workspace) & 255) return fail(MTF_ERR_INVALID_ARG, "workspace must be 256-byte aligned");
   }
   g_last_pick = {0, 0};
+  // Wide tiles (256 x 512 per pair) for a plain epilogue, or with a residual as the only stage - the contractions whose result is added to a stream of the
+  // decoder layer - through the generic epilogue kind.
+  const bool plain_launch = scale == 1.f && !bias && !relu && !mask && !rsum && !row_softmax;
+  const bool wide_legal = t.cta_pair && t.block_n == 256 && t.reduce_mode != MTF_REDUCE_WORKSPACE && plain_launch && (!resid || n_terms == 1) && (t.N / t.sn) % 512 == 0;
+  const bool may_widen = wide_legal && t.wide_pref != 0;
   if (!row_softmax) {
-    const ClusterPick pick = g_last_pick = cluster_pick(t, n_terms, n_groups);
+    const ClusterPick pick = g_last_pick = cluster_pick(t, n_terms, n_groups, may_widen);
     if (pick.split)
       return launch_cluster(plan, pick, A, B, C, bias, dtBias, mask, dtMask, resid, dtRes, scale, relu, rsum, workspace, workspace_bytes, stream, n_terms,
                             extra_operands, n_groups, group_operands);
@@ -2016,9 +2077,6 @@ mtf_status launch_tc(const mtf_plan_t& plan, const void* A, const void* B, void*
   a.ldc = t.ldc;
   a.reduce_mode = (n_groups > 1 && t.reduce_mode == MTF_REDUCE_WORKSPACE) ? MTF_REDUCE_CHAINED : t.reduce_mode;     // a group has tiles enough: no fragments
   a.k_sliced = (t.sk > 1 && a.Ks % BK == 0) ? 1 : 0;
-  // Wide tiles (256 x 512 per pair) for long contractions with a plain epilogue: per tile about 1.5x
-  // the time of a 256 x 256 one (twice the MMAs at 3/4 of the L2 traffic each, epilogue exposed), so
-  // they win when they halve the number of waves.
   bool wide = false;
   // row_softmax == 5: a plain bf16 contraction that also leaves, per row and column part, the maximum and the sum of
   // exponentials of the stored values at the head of the workspace (float2 [rows][parts]; the caller combines them)
@@ -2037,23 +2095,21 @@ mtf_status launch_tc(const mtf_plan_t& plan, const void* A, const void* B, void*
       return fail(MTF_ERR_UNSUPPORTED, "row softmax in the epilogue needs a bf16 result whose rows fit one tile (N <= 256, or 512 with CTA pairs) and no other stage");
     wide = a.Ns == 512;
   }
-  // (wide tiles also with a residual as the only stage - the contractions whose result is added to a stream of the
-  //  decoder layer - through the generic epilogue kind)
-  const bool resid_only_epi = scale == 1.f && resid && !bias && !relu && !mask && !rsum && !row_softmax && n_terms == 1;
-  const bool wide_legal = t.cta_pair && t.block_n == 256 && t.reduce_mode != MTF_REDUCE_WORKSPACE && (plain_epi || resid_only_epi) && !row_lse && a.Ns % 512 == 0;
   if (t.wide_pref == 1 && !wide_legal)
     return fail(MTF_ERR_UNSUPPORTED, "wide tiles need CTA pairs, a plain or residual-only epilogue, no workspace reduction and an N slice that is a multiple of 512");
-  // Wide tiles where they take less than two thirds of the waves and K hides their epilogue.  474 drawn products that may run on either: 0.5 % from the better
-  // on average; of the 114 that run wide 32 take more than 1.03 times their time on narrow tiles (7936 x 2560 x 5120 worst: 191 us and 164), of the 360 others 6
-  // (at most 1.09 times).  Always narrow: 0.7 %, 46 products, at most 1.15 times.
-  if (wide_legal && t.wide_pref != 0) {
-    long long tiles = (long long)((a.Ms + 2 * BM - 1) / (2 * BM)) * (a.Ns / 256) * a.sm * a.sn;
-    for (int j = 0; j < t.n_outer; ++j) tiles *= t.outer_size[j];
-    const long long workers = sm_count() / 2;
-    const long long waves_narrow = (tiles + workers - 1) / workers, waves_wide = (tiles / 2 + workers - 1) / workers;
-    wide = t.wide_pref == 1 || (t.K * n_terms >= 64 * BK && 3 * waves_wide < 2 * waves_narrow);
+  if (t.cta_pair && !row_softmax && !row_lse) {
+#if defined(MTF_CLUSTER_SHARE)
+    const bool free_tiles = false;         // (its loads share 256-column tiles)
+#else
+    const bool free_tiles = t.free_tiles;
+#endif
+    const PairTiles pt = pair_tiles(t, n_terms, n_groups, free_tiles, may_widen);
+    wide = t.wide_pref == 1 || pt.bn == 512;
+    if (!wide) a.block_n = pt.bn;
+    if (pt.flat && !wide) { a.sm = a.sn = 1; a.Ms = a.M; a.Ns = a.N; }
   }
   if (wide) a.block_n = 512;
+  a.b_box = a.b_mn_major && t.cta_pair && a.block_n == 192 ? 32 : 64;
   // optional single-GPU build: clusters of CTA pairs that share operand tiles
   int cm = 1, cn = 1;
 #if defined(MTF_CLUSTER_SHARE)
@@ -2171,10 +2227,10 @@ mtf_status launch_tc(const mtf_plan_t& plan, const void* A, const void* B, void*
   mtf_status s;
   // operands: K-major = (K contiguous, M|N rows), box 64 x rows;  MN-major = (M|N contiguous, K rows), box 64 x 64
   // (a CTA of a sharing cluster loads 1/cn of its A rows and 1/cm of its B columns per box)
-  const int b_rows = (t.cta_pair ? t.block_n / 2 : t.block_n) / cm;
+  const int b_rows = (t.cta_pair ? (wide ? 256 : a.block_n) / 2 : t.block_n) / cm;
   s = t.a_mn_major ? make_map(&map_a, A, 2, t.M, t.K, t.a_ld, 64, BK, t, t.outer_sA) : make_map(&map_a, A, 2, t.K, t.M, t.a_ld, 64, BM / cn, t, t.outer_sA);
   if (s != MTF_OK) return s;
-  s = t.b_mn_major ? make_map(&map_b, B, 2, t.N, t.K, t.b_ld, 64, BK, t, t.outer_sB) : make_map(&map_b, B, 2, t.K, t.N, t.b_ld, 64, b_rows, t, t.outer_sB);
+  s = t.b_mn_major ? make_map(&map_b, B, 2, t.N, t.K, t.b_ld, a.b_box, BK, t, t.outer_sB) : make_map(&map_b, B, 2, t.K, t.N, t.b_ld, 64, b_rows, t, t.outer_sB);
   if (s != MTF_OK) return s;
   ExtraMaps extra;
   for (int i = 0; i < 4; ++i) extra.m[i] = i % 2 == 0 ? map_a : map_b;
@@ -2185,7 +2241,7 @@ mtf_status launch_tc(const mtf_plan_t& plan, const void* A, const void* B, void*
     if (!Ai || !Bi) return fail(MTF_ERR_INVALID_ARG, "multi-term contraction: NULL operand");
     s = t.a_mn_major ? make_map(&extra.m[2 * (i - 1)], Ai, 2, t.M, t.K, t.a_ld, 64, BK, t, t.outer_sA) : make_map(&extra.m[2 * (i - 1)], Ai, 2, t.K, t.M, t.a_ld, 64, BM / cn, t, t.outer_sA);
     if (s != MTF_OK) return s;
-    s = t.b_mn_major ? make_map(&extra.m[2 * (i - 1) + 1], Bi, 2, t.N, t.K, t.b_ld, 64, BK, t, t.outer_sB) : make_map(&extra.m[2 * (i - 1) + 1], Bi, 2, t.K, t.N, t.b_ld, 64, b_rows, t, t.outer_sB);
+    s = t.b_mn_major ? make_map(&extra.m[2 * (i - 1) + 1], Bi, 2, t.N, t.K, t.b_ld, a.b_box, BK, t, t.outer_sB) : make_map(&extra.m[2 * (i - 1) + 1], Bi, 2, t.K, t.N, t.b_ld, 64, b_rows, t, t.outer_sB);
     if (s != MTF_OK) return s;
   }
   // output: (N contiguous, M rows), boxes of 32 rows x 128 bytes for the staged stores
@@ -2200,7 +2256,7 @@ mtf_status launch_tc(const mtf_plan_t& plan, const void* A, const void* B, void*
     if (!Ag || !Bg || !Cg || (reinterpret_cast<uintptr_t>(Cg) & 15)) return fail(MTF_ERR_INVALID_ARG, "grouped launch: NULL or misaligned operand");
     s = t.a_mn_major ? make_map(&extra.m[2 * (g - 1)], Ag, 2, t.M, t.K, t.a_ld, 64, BK, t, t.outer_sA) : make_map(&extra.m[2 * (g - 1)], Ag, 2, t.K, t.M, t.a_ld, 64, BM / cn, t, t.outer_sA);
     if (s != MTF_OK) return s;
-    s = t.b_mn_major ? make_map(&extra.m[2 * (g - 1) + 1], Bg, 2, t.N, t.K, t.b_ld, 64, BK, t, t.outer_sB) : make_map(&extra.m[2 * (g - 1) + 1], Bg, 2, t.K, t.N, t.b_ld, 64, b_rows, t, t.outer_sB);
+    s = t.b_mn_major ? make_map(&extra.m[2 * (g - 1) + 1], Bg, 2, t.N, t.K, t.b_ld, a.b_box, BK, t, t.outer_sB) : make_map(&extra.m[2 * (g - 1) + 1], Bg, 2, t.K, t.N, t.b_ld, 64, b_rows, t, t.outer_sB);
     if (s != MTF_OK) return s;
     if ((s = make_map(&extra.c[g - 1], Cg, c_bytes, t.N, t.M, t.ldc, 128 / c_bytes, 32, t, t.outer_sC)) != MTF_OK) return s;
     a.C_group[g - 1] = Cg;

@@ -89,11 +89,14 @@ struct TcParams {
   int a_mn_major = 0, b_mn_major = 0;        // 0: K contiguous in smem rows, 1: M/N contiguous
   int64_t a_ld = 0, b_ld = 0;                // element stride of the non-contiguous one of (M|N, K)
   int64_t ldc = 0;                           // element stride of M in C (N is contiguous)
+  int c_f32 = 0;                             // f32 result
   int block_n = 256;
   int wide_pref = -1;                        // 256 x 512 pair tiles: -1 = launcher's wave heuristic, 0 = never, 1 = wherever the shape allows
   int balance = 0;                           // tiles leave a partly filled last wave: balanced k-range schedule (needs workspace)
   int cta_pair = 0;                          // two CTAs (a cluster) own a 256-row tile, tcgen05 cta_group::2
   int cluster_ok = 0;                        // no kernel or reduce mode was asked for: the launcher may take 128-row tiles with K over a cluster
+  int free_tiles = 0;                        // the launcher may choose the columns of a pair's tile and run tiles across slice edges: no sum is forced (the launch beside the attention core, whose
+                                             // sum is, wants few blocks) and no other kernel than the one with pairs
   int swapped = 0;                           // in[0] and in[1] exchanged so that N is contiguous in C
   int reduce_mode = MTF_REDUCE_NONE;
   int bias_along_m = 0;                      // bias varies with m (after a swap) instead of n
