@@ -58,7 +58,7 @@ bool dims_match(const std::vector<Dim>& want, const mtf_tensor& t) {
 
 mtf_status exec_plan(const mtf_plan_t* P, const mtf_tensor* in, mtf_tensor* out, const mtf_epilogue* epi,
                      void* workspace, size_t workspace_bytes, void* stream, int n_terms = 1, const void* const* extra_operands = nullptr,
-                     int row_softmax = 0, int n_groups = 1, const void* const* group_operands = nullptr) {
+                     int row_softmax = 0, int n_groups = 1, const void* const* group_operands = nullptr, bool f32_late = false, float* f32_bsum = nullptr) {
   if (!P || !in || !out) return fail(MTF_ERR_INVALID_ARG, "einsum exec: NULL argument");
   if (!dims_match(P->dimsA, in[0]) || (P->has_B && !dims_match(P->dimsB, in[1])) || !dims_match(P->dimsC, *out))
     return fail(MTF_ERR_SIZE_MISMATCH, "einsum exec: operand dims differ from the planned ones");
@@ -106,7 +106,9 @@ mtf_status exec_plan(const mtf_plan_t* P, const mtf_tensor* in, mtf_tensor* out,
     if (n_terms != 1 || row_softmax || n_groups != 1) return fail(MTF_ERR_UNSUPPORTED, "multi-term, grouped or fused-softmax contraction on the generic kernel");
     const int asked = mtf::contraction_asked();
     if (P->f32_ok && (P->f32_tiled || asked)) {
-      st = ((asked ? asked == 128 : P->f32_tensor_cores) ? mtf::launch_f32_tc : mtf::launch_f32)(P->f32, in[0].data, in[1].data, out->data, P->dtC, bias, P->epi.dtBias, mask, P->epi.dtMask, resid, P->epi.dtRes, scale, relu, rsum, stream);
+      st = (asked ? asked == 128 : P->f32_tensor_cores)
+               ? mtf::launch_f32_tc(P->f32, in[0].data, in[1].data, out->data, P->dtC, bias, P->epi.dtBias, mask, P->epi.dtMask, resid, P->epi.dtRes, scale, relu, rsum, stream, f32_late, f32_bsum)
+               : mtf::launch_f32(P->f32, in[0].data, in[1].data, out->data, P->dtC, bias, P->epi.dtBias, mask, P->epi.dtMask, resid, P->epi.dtRes, scale, relu, rsum, stream);
     } else {
       SimtParams s = P->simt;
       s.A = in[0].data;
@@ -709,6 +711,34 @@ mtf_status mtf::ffn_backward_impl(const mtf_layout_t* layout, const mtf_tensor* 
                                           (const float*)dy->data, (float*)dx->data, (float*)dw->data, dbias ? (float*)dbias->data : nullptr, (float*)dv->data,
                                           mtf::tap_is_open() ? (float*)dhp.data : nullptr, stream);
       return st != MTF_OK ? st : mtf::tap("dhp", dhp, stream);
+    }
+  }
+  // f32 on the tensor cores: dw = x^T . dhp reads every dhp, so its launch forms dbias too (no output to clear in front of dhp, nothing added to memory in
+  // an order that varies), and dv and dx start beside the launches before them, which they have nothing in common with.
+  {
+    const mtf_plan_t *P1 = nullptr, *P2 = nullptr, *P3 = nullptr, *P4 = nullptr, *Pd = nullptr;
+    mtf_epilogue ed = e1;
+    ed.reduce_sum_out = nullptr;
+    auto on_tc = [](const mtf_plan_t* P) { return P->kernel_kind != MTF_KERNEL_TCGEN05 && P->f32_ok && P->f32_tensor_cores; };
+    if (!dx_residual && fuse_dbias && layout && layout->bound_dim < 0 && !mtf::contraction_asked() && !mtf::tap_is_open() && x->dtype == MTF_F32 && h_saved->dtype == MTF_F32 &&
+        cached_plan(layout, 2, in1, &dhp, &e1, &P1) == MTF_OK && cached_plan(layout, 2, in1, &dhp, &ed, &Pd) == MTF_OK && cached_plan(layout, 2, in2, dv, nullptr, &P2) == MTF_OK &&
+        cached_plan(layout, 2, in3, dw, nullptr, &P3) == MTF_OK && cached_plan(layout, 2, in4, dx, nullptr, &P4) == MTF_OK && on_tc(Pd) && on_tc(P2) && on_tc(P3) && on_tc(P4) &&
+        mtf::f32_tc_sums_b(P3->f32, false) && dbias->data) {
+      // (an output over an operand of the launch before: one after the other, as launches without the hint run)
+      auto apart = [](const mtf_tensor& out, std::initializer_list<const mtf_tensor*> others) {
+        const uint8_t* const lo = reinterpret_cast<const uint8_t*>(out.data);
+        for (const mtf_tensor* o : others) {
+          const uint8_t* const q = reinterpret_cast<const uint8_t*>(o->data);
+          if (lo < q + numel(*o) * elem_bytes(o->dtype) && q < lo + numel(out) * elem_bytes(out.dtype)) return false;
+        }
+        return true;
+      };
+      const bool dv_beside = apart(*dv, {dy, v, h_saved, &dhp}), dx_beside = apart(*dx, {x, &dhp, dw, dbias});
+      (void)mtf::take_independent_hint();
+      if ((st = exec_plan(Pd, in1, &dhp, &ed, rest, rest_bytes, stream)) != MTF_OK) return st;
+      if ((st = exec_plan(P2, in2, dv, nullptr, rest, rest_bytes, stream, 1, nullptr, 0, 1, nullptr, dv_beside)) != MTF_OK) return st;
+      if ((st = exec_plan(P3, in3, dw, nullptr, rest, rest_bytes, stream, 1, nullptr, 0, 1, nullptr, false, reinterpret_cast<float*>(dbias->data))) != MTF_OK) return st;
+      return exec_plan(P4, in4, dx, nullptr, rest, rest_bytes, stream, 1, nullptr, 0, 1, nullptr, dx_beside);
     }
   }
   if ((st = mtf_einsum(layout, nullptr, 2, in1, &dhp, &e1, rest, rest_bytes, stream)) != MTF_OK) return st;

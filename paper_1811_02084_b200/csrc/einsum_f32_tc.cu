@@ -60,6 +60,8 @@ struct F32TcArgs {
   const void* mask;
   const void* resid;
   float* rsum;
+  float* bsum;                      // not NULL: the sums over k of B's columns (of the blocks with the first rows)
+  int late_wait;                    // this launch touches nothing that the launch before it touches: it waits for that one at its end
   int c_bf16, bias_bf16, mask_bf16, resid_bf16, relu;
   int rsum_mode;                    // 0: added to the zeroed output; 1: one block has all rows; 2: one cluster has
   float scale;
@@ -351,7 +353,7 @@ __global__ void __launch_bounds__(kThreads, 1) einsum_f32_tc_kernel(const __grid
   fence_after();
   const uint32_t tmem = tmem_slot;
   // the launch before this one on the stream may have written the operands; the next one may set itself up
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (!a.late_wait) asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   const int row = (warp & 3) * 32 + lane, col = (warp >> 2) * 16;       // a row of the tile, 16 of its columns
@@ -416,6 +418,11 @@ __global__ void __launch_bounds__(kThreads, 1) einsum_f32_tc_kernel(const __grid
   pa.load(s0, K, a.vecA, ra[0]);
   pb.load(s0, K, a.vecB, rb[0]);
   if (s0 + 1 < s1) { pa.load(s0 + 1, K, a.vecA, ra[1]); pb.load(s0 + 1, K, a.vecB, rb[1]); }
+  // (a thread's values of B are the same four columns at every k.  Both operands along M and N, as in the weight gradients, has this code; a variant of its own
+  // for the one launch that wants it cost that launch 1.7 us of instruction fetches, and in the other orders it cost the loop 1 %)
+  constexpr bool kSumsB = !kAlongA && !kAlongB;
+  const bool sums_b = kSumsB && a.bsum && mt == 0;
+  float4 b_sum = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 1
   for (int s = s0; s < s1; s += 2) {
 #pragma unroll
@@ -425,6 +432,14 @@ __global__ void __launch_bounds__(kThreads, 1) einsum_f32_tc_kernel(const __grid
       uint8_t* const sa = ring + (uint32_t)u * kStage;           // (free: the stage two back is complete, add_up waited for it)
       pa.template store<kPieceA>(sa, ra[u]);
       pb.template store<kPieceB>(sa + 3 * kPieceA, rb[u]);
+      if (kSumsB && sums_b) {
+        static_assert(Pieces<kTN, kAlongB>::kN % 2 == 0, "pairs");
+#pragma unroll
+        for (int i = 0; i < Pieces<kTN, kAlongB>::kN; i += 2) {
+          const float4 p = rb[u][i], q = rb[u][i + 1];
+          b_sum.x += p.x + q.x; b_sum.y += p.y + q.y; b_sum.z += p.z + q.z; b_sum.w += p.w + q.w;
+        }
+      }
       if (c + 2 < s1) { pa.load(c + 2, K, a.vecA, ra[u]); pb.load(c + 2, K, a.vecB, rb[u]); }
       if (c > s0) add_up(c - 1);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -520,21 +535,28 @@ __global__ void __launch_bounds__(kThreads, 1) einsum_f32_tc_kernel(const __grid
       }
     }
   }
-  if (a.rsum) {                                     // fused reduce_sum: the 32 threads of a column piece, in a fixed order
+  // fused reduce_sum (over the rows of C), or the sums over k of B's columns: the 32 threads of a column piece, in a fixed order; the cluster's
+  // parts in ascending order
+  if (a.rsum || sums_b) {
+    float* const to = sums_b ? a.bsum : a.rsum;
+    const int mode = sums_b ? (a.split > 1 ? 2 : 1) : a.rsum_mode;
+    const float4 mine4 = sums_b ? b_sum : col_sum;
     const uint32_t cs = base + 32768u;              // (past the tile: the rest of the cluster may still read it)
-    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(cs + (uint32_t)(tid >> 4) * 256u + (uint32_t)c4 * 4u), "f"(col_sum.x), "f"(col_sum.y), "f"(col_sum.z),
-                 "f"(col_sum.w) : "memory");
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(cs + (uint32_t)(tid >> 4) * 256u + (uint32_t)c4 * 4u), "f"(mine4.x), "f"(mine4.y), "f"(mine4.z),
+                 "f"(mine4.w) : "memory");
     __syncthreads();
     float x = 0.f;
     if (tid < kTN) {
+      float x4[4] = {0.f, 0.f, 0.f, 0.f};           // (four runs of eight: fewer roundings on the way)
 #pragma unroll 8
       for (int i = 0; i < kThreads / 16; ++i) {
         float y;
         asm volatile("ld.shared.f32 %0, [%1];" : "=f"(y) : "r"(cs + (uint32_t)i * 256u + (uint32_t)tid * 4u) : "memory");
-        x += y;
+        x4[i & 3] += y;
       }
+      x = (x4[0] + x4[1]) + (x4[2] + x4[3]);
     }
-    if (a.rsum_mode == 2) {
+    if (mode == 2) {
       if (tid < kTN) col_part[tid] = x;
       cluster_sync();
       if (part == 0 && tid < kTN && n0 + tid < N) {
@@ -545,11 +567,11 @@ __global__ void __launch_bounds__(kThreads, 1) einsum_f32_tc_kernel(const __grid
                        : "=f"(y) : "r"(s_u32(&col_part[tid])), "r"(q) : "memory");
           x += y;
         }
-        a.rsum[n0 + tid] = x;
+        to[n0 + tid] = x;
       }
     } else if (tid < kTN && n0 + tid < N) {
-      if (a.rsum_mode == 1) a.rsum[n0 + tid] = x;
-      else atomicAdd(a.rsum + n0 + tid, x);
+      if (mode == 1) to[n0 + tid] = x;
+      else atomicAdd(to + n0 + tid, x);
     }
   }
   __syncwarp();
@@ -557,6 +579,7 @@ __global__ void __launch_bounds__(kThreads, 1) einsum_f32_tc_kernel(const __grid
     for (int i = 0; i < 2000; ++i) __nanosleep(1000);      // failure path: MMAs in flight land before the resources go away
   if (a.split > 1) cluster_sync();                  // the cluster may still read this block's part
   else __syncthreads();
+  if (a.late_wait) asm volatile("griddepcontrol.wait;" ::: "memory");
   if (warp == 0) {
     __syncwarp();
     fence_after();
@@ -594,6 +617,8 @@ bool f32_tensor_cores_pay(const F32Params& p) {
   return (split > 1 ? 0.5 : 0.0) + rounds * ((p.n_outer ? 4.0 : 3.8) + 1.5 * (double)part) < f32_tile_us(p);
 }
 
+bool f32_tc_sums_b(const F32Params& p, bool other_sums) { return !other_sums && !p.swapped && !p.n_outer && p.sAk != 1 && p.sBn == 1 && p.sBk != 1; }
+
 template <bool kAlongA, bool kAlongB>
 static mtf_status launch_orders(const F32TcArgs& a, int64_t blocks, cudaStream_t st) {
   // the opt-in to the shared memory is a property of a device
@@ -617,12 +642,14 @@ static mtf_status launch_orders(const F32TcArgs& a, int64_t blocks, cudaStream_t
 }
 
 mtf_status launch_f32_tc(const F32Params& p, const void* A, const void* B, void* C, int dtC, const void* bias, int dtBias, const void* mask, int dtMask,
-                         const void* resid, int dtRes, float scale, int relu, float* rsum, void* stream) {
+                         const void* resid, int dtRes, float scale, int relu, float* rsum, void* stream, bool late, float* bsum) {
   F32TcArgs a;
   a.p = p;
   if (p.swapped) std::swap(A, B);
   a.A = reinterpret_cast<const float*>(A); a.B = reinterpret_cast<const float*>(B);
   a.C = C; a.bias = bias; a.mask = mask; a.resid = resid; a.rsum = rsum;
+  a.bsum = bsum; a.late_wait = late ? 1 : 0;
+  if (bsum && !f32_tc_sums_b(p, rsum != nullptr)) return fail(MTF_ERR_UNSUPPORTED, "f32 product: column sums of B need operands contiguous along M and N, no batch and no other column sums");
   a.c_bf16 = dtC == MTF_BF16; a.bias_bf16 = dtBias == MTF_BF16; a.mask_bf16 = dtMask == MTF_BF16; a.resid_bf16 = dtRes == MTF_BF16;
   a.relu = relu; a.scale = scale;
   auto vec = [&](const void* base, int64_t s_mn, int64_t s_k, const int64_t* outer) {

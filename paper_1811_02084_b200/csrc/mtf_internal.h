@@ -201,8 +201,10 @@ double f32_tile_us(const F32Params& p);
 bool f32_tensor_cores_pay(const F32Params& p);
 mtf_status launch_f32(const F32Params& p, const void* A, const void* B, void* C, int dtC, const void* bias, int dtBias, const void* mask, int dtMask,
                       const void* resid, int dtRes, float scale, int relu, float* rsum, void* stream);
+bool f32_tc_sums_b(const F32Params& p, bool other_sums);      // whether launch_f32_tc can take a bsum
+// late: the launch touches nothing that the launch before it on the stream touches (which waits at its own start); bsum (NULL: none): sums over k of B's columns
 mtf_status launch_f32_tc(const F32Params& p, const void* A, const void* B, void* C, int dtC, const void* bias, int dtBias, const void* mask, int dtMask,
-                         const void* resid, int dtRes, float scale, int relu, float* rsum, void* stream);
+                         const void* resid, int dtRes, float scale, int relu, float* rsum, void* stream, bool late = false, float* bsum = nullptr);
 mtf_status launch_tc(const mtf_plan_t& plan, const void* A, const void* B, void* C, const void* bias, int dtBias,
                      const void* mask, int dtMask, const void* resid, int dtRes, float scale, int relu, float* rsum,
                      void* workspace, size_t workspace_bytes, void* stream, int n_terms = 1,

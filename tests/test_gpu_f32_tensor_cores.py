@@ -201,3 +201,37 @@ def test_pieces_are_chosen_by_size(mtf):  # noqa: F811
         x, y, o = torch.randn(m, k, device="cuda"), torch.randn(k, n, device="cuda"), torch.empty(m, n, device="cuda")
         mtf.mtf_einsum(layout(mtf, *ONE), None, [mtf.named(x, ["i", "k"]), mtf.named(y, ["k", "j"])], mtf.named(o, ["i", "j"]))
         assert mtf.mtf_debug_contraction()[0] == ran, (m, n, k)
+
+
+@pytest.mark.parametrize("tokens,d_in,hidden,d_out", [(1024, 256, 1024, 256), (264, 260, 1028, 260), (1000, 72, 2052, 100), (2048, 40, 1000, 40)])
+def test_feed_forward_backward_in_pieces(tokens, d_in, hidden, d_out):
+    """dbias comes from the launch of dw, dv and dx run beside the launches before them: every output against 64 bits from what the launch read, the same bits
+    from run to run, and launch by launch where dx lies over x."""
+    import torch
+    import paper_1811_02084_b200 as mtf
+    g = torch.Generator(device="cuda").manual_seed(3)
+    r = lambda *s: torch.randn(*s, generator=g, device="cuda")  # noqa: E731
+    t = {"x": r(tokens, d_in), "w": r(d_in, hidden) * d_in ** -0.5, "v": r(hidden, d_out) * hidden ** -0.5, "h": r(tokens, hidden).relu(), "dy": r(tokens, d_out)}
+    dims = {"x": "td", "w": "df", "v": "fe", "h": "tf", "dy": "te", "dx": "td", "dw": "df", "dbias": "f", "dv": "fe"}
+    lay = mtf.mtf_layout(mtf.mtf_mesh_create([("p", 1)]), [])
+
+    def run(over_x):
+        o = {"dw": torch.empty(d_in, hidden, device="cuda"), "dbias": torch.empty(hidden, device="cuda"), "dv": torch.empty(hidden, d_out, device="cuda")}
+        x = t["x"].clone()
+        o["dx"] = x if over_x else torch.empty_like(x)
+        for k in ("dw", "dbias", "dv"):
+            o[k].fill_(float("nan"))
+        n = {k: mtf.named(v, list(dims[k])) for k, v in {**t, **o, "x": x}.items()}
+        ws = torch.empty(mtf.mtf_ffn_workspace_bytes(lay, n["x"], n["w"]), dtype=torch.uint8, device="cuda")
+        mtf.mtf_ffn_backward(lay, n["x"], n["w"], n["v"], n["h"], n["dy"], n["dx"], n["dw"], n["dbias"], n["dv"], ws)
+        mtf.mtf_device_status()
+        return o
+
+    first, again, over = run(False), run(False), run(True)
+    d = {k: v.double() for k, v in t.items()}
+    dhp = (d["dy"] @ d["v"].t()) * (d["h"] > 0)
+    ref = {"dv": d["h"].t() @ d["dy"], "dw": d["x"].t() @ dhp, "dx": dhp @ d["w"].t(), "dbias": dhp.sum(0)}
+    for k, want in ref.items():
+        # (2-norm; sums of up to 2052 terms: the kernel's own error is 1.2e-7 at K = 2048, dhp's rounding 3e-8 more)
+        assert (first[k].double() - want).norm() <= 1e-6 * want.norm(), k
+        assert torch.equal(first[k], again[k]) and torch.equal(first[k], over[k]), k
