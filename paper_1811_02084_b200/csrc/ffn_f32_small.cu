@@ -247,15 +247,16 @@ mtf_status launch(void (*kernel)(SmallArgs), std::once_flag* once, cudaError_t* 
 
 namespace mtf {
 
-// Whether a direction runs here, or as one launch per einsum: up to 2^18 (forward) or 2^20 multiply-adds a product, fewer where much of w and v has to be
-// copied.  us, forward / backward, here and launch by launch (tokens x widths x hidden units; graphs of ten passes):
-//   8 x 64 x 256     6.7 / 7.8   9.0 / 17.1      64 x 40 x 72     7.2 / 10.4   9.7 / 19.4      4 x 128 x 512    8.8 / 12.1   9.6 / 19.7
-//   16 x 64 x 512    9.6 / 12.0  9.4 / 17.4      64 x 64 x 256   11.1 / 18.4   9.8 / 21.2      8 x 256 x 512   14.6 / 21.2  10.1 / 19.2
-//   1 x 256 x 512   11.4 / 17.3  9.9 / 19.0      32 x 128 x 512  15.5 / 23.4  10.4 / 19.3      1 x 48 x 2048    9.9 / 14.5  13.9 / 21.0
+// Whether a direction runs here, or as one launch per einsum: forward up to 3 x 2^17 multiply-adds a product; backward up to 2^20, where the products over at most 32 tokens
+// are no work for the tensor cores, else as many as forward; fewer where much of w and v has to be copied.  us, here and launch by launch (graphs of ten passes):
+//   tokens x width x hidden   8 x 64 x 256  16 x 64 x 512  4 x 128 x 512  64 x 40 x 72  128 x 40 x 72  48 x 64 x 256  16 x 128 x 512  8 x 128 x 1024  1 x 48 x 2048
+//   forward                     6.5   9.1      9.6   9.6      8.8   9.8     7.0  10.0     10.1  10.3     9.5   9.8      12.8  10.3     14.1  11.8       9.9  13.8
+//   backward                    7.6  17.0     12.1  17.5     12.3  19.5    10.4  13.7     14.3  15.1    15.8  14.1      18.0  19.0     20.9  20.6      14.6  21.2
 bool ffn_small_pays(int64_t T, int64_t D, int64_t F, int64_t E, bool backward) {
   if (T <= 0 || D <= 0 || F <= 0 || E <= 0 || T > 4096 || D > 8192 || F > 65536 || E > 8192) return false;
   const int64_t weights = F * std::max(D, E), work = T * weights;
-  if (backward ? work > (weights > 65536 ? 1 << 19 : 1 << 20) || weights > 131072 : work > 1 << 18 || weights > 65536) return false;
+  const int64_t most = !backward || T > 32 ? 3 << 17 : weights > 65536 ? 1 << 19 : 1 << 20;
+  if (work > most || weights > (backward ? 131072 : 65536)) return false;
   return smem_bytes(T, D, F, E, backward) <= kMaxSmem;
 }
 
