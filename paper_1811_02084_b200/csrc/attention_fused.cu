@@ -49,7 +49,6 @@ struct AttArgs {
   int B, H, L;
   int causal;
   float scale;
-  __nv_bfloat16* o;              // [B, L, H, 64]
   long long units;               // B * H
 };
 
@@ -148,7 +147,7 @@ __device__ __forceinline__ int live_chunks(const AttArgs& a, int qt) { return a.
 
 __global__ void __launch_bounds__(kThreads, 1)
 attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
-                     const __grid_constant__ CUtensorMap map_p, const AttArgs a) {
+                     const __grid_constant__ CUtensorMap map_p, const __grid_constant__ CUtensorMap map_o, const AttArgs a) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = s_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -443,7 +442,11 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
           ++pu;
         }
         ok = __all_sync(0xffffffffu, ok);
-        // the part-0 warps read O (64 columns, accumulated over the first chunk's columns) and write it out
+        // The part-0 warps read O (64 columns, accumulated over the first chunk's columns), hand the tensor memory to the next tile's logits at once, and
+        // write O through the box of their last chunk (its MMAs have retired) by TMA.  Stores from registers, 16 bytes of 32 rows an instruction, in front of the
+        // hand-over cost 1000 of the 7500 cycles of a tile of 256 positions: 2048 pairs of 256 126 -> 121 us, 256 pairs of 512 69 and 69.  (What holds those: exponentials 4700
+        // cycles of the special-function unit, then 4200 in which the shared-memory port moves the weights three times - stored by the warps, read by the MMAs and by the
+        // TMA store - and 2000 until O is complete.  Logits of all columns but O's first 64 issued before O is read: 69.2 and 123 us.)
         if (part == 0 && ok) {
           ok = wait_all(7, (uint32_t)tile_seq & 1u, 0x923);
           fence_after();
@@ -452,18 +455,20 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             tmem_ld32(taddr, r0);
             tmem_ld32(taddr + 32u, r1);
             tmem_ld_wait();
-            uint4* dst = reinterpret_cast<uint4*>(a.o + (((long long)b * L + row) * a.H + h) * 64);
-#pragma unroll
-            for (int qq = 0; qq < 4; ++qq)
-              dst[qq] = make_uint4(pack2(__uint_as_float(r0[qq * 8]), __uint_as_float(r0[qq * 8 + 1])), pack2(__uint_as_float(r0[qq * 8 + 2]), __uint_as_float(r0[qq * 8 + 3])),
-                                   pack2(__uint_as_float(r0[qq * 8 + 4]), __uint_as_float(r0[qq * 8 + 5])), pack2(__uint_as_float(r0[qq * 8 + 6]), __uint_as_float(r0[qq * 8 + 7])));
-#pragma unroll
-            for (int qq = 0; qq < 4; ++qq)
-              dst[4 + qq] = make_uint4(pack2(__uint_as_float(r1[qq * 8]), __uint_as_float(r1[qq * 8 + 1])), pack2(__uint_as_float(r1[qq * 8 + 2]), __uint_as_float(r1[qq * 8 + 3])),
-                                       pack2(__uint_as_float(r1[qq * 8 + 4]), __uint_as_float(r1[qq * 8 + 5])), pack2(__uint_as_float(r1[qq * 8 + 6]), __uint_as_float(r1[qq * 8 + 7])));
             fence_before();
+            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");      // the chunk's store has read the box
             __syncwarp();
             if (lane == 0) mb_arrive(bar(8));
+#pragma unroll
+            for (int qq = 0; qq < 4; ++qq) {
+              sts_v4(rowaddr + ((((uint32_t)qq) ^ swz) << 4), pack2(__uint_as_float(r0[qq * 8]), __uint_as_float(r0[qq * 8 + 1])), pack2(__uint_as_float(r0[qq * 8 + 2]), __uint_as_float(r0[qq * 8 + 3])),
+                     pack2(__uint_as_float(r0[qq * 8 + 4]), __uint_as_float(r0[qq * 8 + 5])), pack2(__uint_as_float(r0[qq * 8 + 6]), __uint_as_float(r0[qq * 8 + 7])));
+              sts_v4(rowaddr + ((((uint32_t)(4 + qq)) ^ swz) << 4), pack2(__uint_as_float(r1[qq * 8]), __uint_as_float(r1[qq * 8 + 1])), pack2(__uint_as_float(r1[qq * 8 + 2]), __uint_as_float(r1[qq * 8 + 3])),
+                     pack2(__uint_as_float(r1[qq * 8 + 4]), __uint_as_float(r1[qq * 8 + 5])), pack2(__uint_as_float(r1[qq * 8 + 6]), __uint_as_float(r1[qq * 8 + 7])));
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) tma_store_4d(&map_o, box, 0, row0, h, b);
           }
         }
       }
@@ -526,16 +531,15 @@ mtf_status launch_attention_fwd_fused(const void* q, const void* kk, const void*
   for (const void* p : {q, kk, vv, (const void*)weights, (const void*)o})
     if (!p || (reinterpret_cast<uintptr_t>(p) & 15)) return fail(MTF_ERR_INVALID_ARG, "fused attention: NULL or misaligned tensor");
   if (B * H <= 0) return MTF_OK;
-  CUtensorMap mq, mk, mv, mp;
+  CUtensorMap mq, mk, mv, mp, mo;
   const int64_t qd[4] = {64, L, H, B}, qs[3] = {H * 64, 64, L * H * 64};
   const int64_t pd[4] = {L, L, H, B}, ps[3] = {L, L * L, H * L * L};
   mtf_status st;
   if ((st = map4(&mq, q, qd, qs, 64, 128)) != MTF_OK || (st = map4(&mk, kk, qd, qs, 64, 128)) != MTF_OK || (st = map4(&mv, vv, qd, qs, 64, 64)) != MTF_OK ||
-      (st = map4(&mp, weights, pd, ps, 64, 32)) != MTF_OK)
+      (st = map4(&mp, weights, pd, ps, 64, 32)) != MTF_OK || (st = map4(&mo, o, qd, qs, 64, 32)) != MTF_OK)
     return st;
   AttArgs a;
   a.B = (int)B; a.H = (int)H; a.L = (int)L; a.causal = causal ? 1 : 0; a.scale = scale;
-  a.o = reinterpret_cast<__nv_bfloat16*>(o);
   a.units = B * H;
   const size_t smem = 1024 + kQBytes + (size_t)L * 256 + kPBufs * kPBufBytes + 4096 + 2 * kSoftmaxWarps * 32 * 4 + 24 * 8 + 64;
   cudaError_t e = cudaFuncSetAttribute(attention_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -547,7 +551,7 @@ mtf_status launch_attention_fwd_fused(const void* q, const void* kk, const void*
   const long long grid = std::min<long long>(a.units * (L / 128), device_sm_count());
   cfg.gridDim = dim3((unsigned)grid, 1, 1); cfg.blockDim = dim3(kThreads, 1, 1); cfg.dynamicSmemBytes = smem; cfg.stream = (cudaStream_t)stream;
   cfg.attrs = at; cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, attention_fwd_kernel, mq, mk, mv, mp, a);
+  e = cudaLaunchKernelEx(&cfg, attention_fwd_kernel, mq, mk, mv, mp, mo, a);
   if (e != cudaSuccess) return fail(MTF_ERR_CUDA, "attention_fwd_kernel: %s", cudaGetErrorString(e));
   count_launch();
   return MTF_OK;
