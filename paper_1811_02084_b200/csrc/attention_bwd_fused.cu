@@ -18,19 +18,24 @@
 // block j (128 keys, outer loop), query block i (128 queries), and the steps are walked twice.  Pass 0 forms the row
 // terms: D[l] = sum_m dP[l, m] P[l, m] = sum_v do[l, v] O[l, v] with O = P vv, so the MMA thread alone accumulates the
 // unrounded O_i = sum_j P_ij vv_j in fp32 in the tensor-memory columns that hold dq_i afterwards, and when the pass ends
-// every warp multiplies its rows of O with its rows of do (read from global memory).  Pass 1 computes dP (four MMAs per
+// the warps multiply their rows of O with their rows of do (read from global memory).  Pass 1 computes dP (four MMAs per
 // step) and everything else.  The second read of a tile of P comes from L2 or HBM.
 // Tensor memory (512 columns):
 //   [0, 256)    pass 0: O of the (up to) four query blocks; pass 1: dq of the same blocks, accumulated over j
 //   [256, 320)  dkk of key block j, [320, 384) dvv of key block j, accumulated over i
 //   [384, 512)  dP of the current step (rows of at most 256: dq ends at column 128 and [128, 256) is a second dP buffer)
-// Warp roles (320 threads):
+// Warp roles (576 threads):
 //   warp 0     TMA producer: V_j (both passes) and K_j (pass 1) per key block; the 128 x 128 tile of P per step, q_i and do_i
 //              per step of pass 1 (rings of three)
 //   warp 1     MMA issuer:   pass 0: O_i += P_ij vv_j; pass 1: dP and dvv += P^T do of the NEXT step as soon as this step's dP
 //                            has been read out of tensor memory, then this step's dkk += dS^T q, dq_i += dS kk_j
-//   warps 2-9  two per tensor-memory lane quarter (each owns 64 of the step's 128 key columns): the row terms, dS from dP
+//   warps 2-17 four per tensor-memory lane quarter (each owns 32 of the step's 128 key columns): the row terms, dS from dP
 //              and P, and the read-out of finished accumulators to HBM
+// Bound: the chain of hand-overs.  Sixteen warps and not eight: a step's dS is the longest link that the warps have (2300 cycles, 1250 with sixteen), and the rows that
+// leave or enter through registers cross 32 lines an instruction whatever its width, so they move 32 bytes at a time, each query block's row terms are formed by one part and
+// not by both, and accumulators are handed back before their rows are stored.  256 pairs of 512 positions 114.6 -> 111.5 us, 2048 pairs of 256 causal positions 235 -> 200.
+// Of a pair's cycles there pass 0 takes 29 %, waiting for the last MMAs of a key block (pair) and reading dkk, dvv (dq) out 31 %: at 512 positions tensor memory has no room for a
+// second set of their columns.
 // Every mbarrier wait is bounded; on expiry a code is recorded in the status word, a CTA-wide abort flag is
 // raised, the remaining waits return at once and all roles leave through the teardown.
 #include <cuda.h>
@@ -45,7 +50,7 @@
 
 namespace {
 
-constexpr int kCompWarps = 8;
+constexpr int kCompWarps = 16;
 constexpr int kThreads = 64 + 32 * kCompWarps;
 constexpr uint32_t kBox = 128 * 64 * 2;           // one 128-row x 64-column bf16 box (128-byte rows, 128B swizzle)
 constexpr int kMaxL = 512;
@@ -59,7 +64,7 @@ constexpr size_t kSmemBytes = 1024 + kOffBars + kNumBars * 8 + 64;
 constexpr uint32_t kColDK = 256, kColDV = 320, kColDP = 384;
 
 enum { B_K_FULL = 0, B_K_EMPTY, B_V_FULL, B_V_EMPTY, B_DP_FULL /*2*/, B_DP_EMPTY = 6 /*2*/, B_DKV_FULL = 8, B_DKV_EMPTY, B_DQ_FULL, B_DQ_EMPTY, B_D_SYNC /*O of a pair complete*/,
-       B_QDO_FULL = 13 /*3*/, B_QDO_EMPTY = 16 /*3*/, B_P_FULL = 19 /*3*/, B_P_EMPTY = 22 /*3*/, B_PV_DONE = 25 /*3*/, B_DS_FULL = 28 /*3*/ };
+       B_QDO_FULL = 13 /*3*/, B_QDO_EMPTY = 16 /*3*/, B_P_FULL = 19 /*3*/, B_P_EMPTY = 22 /*3*/, B_PV_DONE = 25 /*3*/, B_DS_FULL = 28 /*3*/, B_D_READY = 31 /*the row terms of a pair stand in tensor memory*/ };
 
 __device__ int g_attb_status = 0;
 
@@ -136,6 +141,22 @@ __device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t* r) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_ld1(uint32_t taddr, uint32_t& v) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(v) : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tmem_st1(uint32_t taddr, uint32_t v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(taddr), "r"(v) : "memory");
+  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+// 32 bytes at a 32-byte aligned address
+__device__ __forceinline__ void ld_v8(const void* p, uint32_t* v) {
+  asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "l"(p) : "memory");
+}
+__device__ __forceinline__ void st_v8(void* p, const uint32_t* v) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+               ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // Shared-memory matrix descriptor of a 128B-swizzled tile whose rows are 128 bytes (64 bf16):
 //   K-major  (a row holds 64 k-elements of one m/n index; 8-row groups 1024 bytes apart)
@@ -239,6 +260,7 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     mb_init(bar(B_DP_EMPTY), kCompWarps); mb_init(bar(B_DP_EMPTY + 1), kCompWarps);
     for (int i = 0; i < kRing; ++i) mb_init(bar(B_DS_FULL + i), kCompWarps);
     mb_init(bar(B_DKV_EMPTY), kCompWarps);
+    mb_init(bar(B_D_READY), kCompWarps);
     mb_init(bar(B_DQ_EMPTY), kCompWarps);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -412,23 +434,21 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   } else {
     // ------------------------------- dS and read-out warps ----------------------
     const int q = warp & 3;                        // tensor-memory lane quarter this warp may access
-    const int half = (warp - 2) >> 2;              // which 64 of the step's 128 key columns
+    const int part = (warp - 2) >> 2;              // which 32 of the step's 128 key columns
     const int row_l = q * 32 + lane;               // row inside a 128-row block
     const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16);
     const uint32_t sw = (uint32_t)(row_l & 7);
     auto wait_all = [&](int b, uint32_t parity, int code) -> bool {      // all lanes wait
       return __all_sync(0xffffffffu, mb_wait(bar(b), parity, code, abort_flag));
     };
-    auto store_row = [&](__nv_bfloat16* dst, const uint32_t* r0, const uint32_t* r1, float s) {      // 64 fp32 -> one 128-byte row
-      uint4* d4 = reinterpret_cast<uint4*>(dst);
+    auto store_half_row = [&](__nv_bfloat16* dst, const uint32_t* r, float s) {      // 32 fp32 -> 64 bytes of a row (32 bytes an instruction: all of a sector)
 #pragma unroll
-      for (int g = 0; g < 4; ++g)
-        d4[g] = make_uint4(pack2(__uint_as_float(r0[g * 8]) * s, __uint_as_float(r0[g * 8 + 1]) * s), pack2(__uint_as_float(r0[g * 8 + 2]) * s, __uint_as_float(r0[g * 8 + 3]) * s),
-                           pack2(__uint_as_float(r0[g * 8 + 4]) * s, __uint_as_float(r0[g * 8 + 5]) * s), pack2(__uint_as_float(r0[g * 8 + 6]) * s, __uint_as_float(r0[g * 8 + 7]) * s));
+      for (int g = 0; g < 2; ++g) {
+        uint32_t w[8];
 #pragma unroll
-      for (int g = 0; g < 4; ++g)
-        d4[4 + g] = make_uint4(pack2(__uint_as_float(r1[g * 8]) * s, __uint_as_float(r1[g * 8 + 1]) * s), pack2(__uint_as_float(r1[g * 8 + 2]) * s, __uint_as_float(r1[g * 8 + 3]) * s),
-                               pack2(__uint_as_float(r1[g * 8 + 4]) * s, __uint_as_float(r1[g * 8 + 5]) * s), pack2(__uint_as_float(r1[g * 8 + 6]) * s, __uint_as_float(r1[g * 8 + 7]) * s));
+        for (int e = 0; e < 8; ++e) w[e] = pack2(__uint_as_float(r[g * 16 + 2 * e]) * s, __uint_as_float(r[g * 16 + 2 * e + 1]) * s);
+        st_v8(dst + g * 16, w);
+      }
     };
     StepIter it;
     it.init((int)blockIdx.x, (int)gridDim.x, a.units, a.H, nb, a.causal);
@@ -438,33 +458,40 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       const int b = it.b, h = it.h;
       const int slot = it.slot;
       const uint32_t par = it.par;
-      uint32_t r0[32], r1[32];
+      uint32_t r0[32];
       if (it.pass == 0) {
-        // pass 0 belongs to the MMA thread (O_i = sum_j P_ij vv_j in fp32, in the columns of dq_i).  When it ends, every warp
-        // forms the row terms of its rows for all query blocks: D[l] = sum_v do[l, v] O[l, v], which equals sum_m dP[l, m] P[l, m]
-        // with the unrounded dP.  (Both warps of a lane quarter do this for the same rows: cheaper than an exchange.)
+        // pass 0 belongs to the MMA thread (O_i = sum_j P_ij vv_j in fp32, in the columns of dq_i).  When it ends, the warps form the row terms of their
+        // rows: D[l] = sum_v do[l, v] O[l, v], which equals sum_m dP[l, m] P[l, m] with the unrounded dP.  Part i takes query block i and leaves D
+        // in the first column of O_i, where the other three warps of the lane quarter find it.
         if (it.last_of_pass0()) {
           if (!(ok = wait_all(B_D_SYNC, (uint32_t)it.unit_seq & 1u, 0xC06))) break;
           fence_after();
-          for (int i2 = 0; i2 < nb; ++i2) {
-            tmem_ld32(taddr + (uint32_t)i2 * 64u, r0);
-            tmem_ld32(taddr + (uint32_t)i2 * 64u + 32u, r1);
-            const uint4* drow = reinterpret_cast<const uint4*>(a.dout + (((long long)b * L + i2 * 128 + row_l) * a.H + h) * 64);
-            uint4 dv4[8];
-#pragma unroll
-            for (int pc = 0; pc < 8; ++pc) dv4[pc] = __ldg(drow + pc);
-            tmem_ld_wait();
+          if (part < nb) {
+            const __nv_bfloat16* const drow = a.dout + (((long long)b * L + part * 128 + row_l) * a.H + h) * 64;
+            uint32_t dv[16];
             float d = 0.f;
 #pragma unroll
-            for (int pc = 0; pc < 8; ++pc) {
-              const uint32_t* rr = pc < 4 ? r0 + pc * 8 : r1 + (pc - 4) * 8;
-              d = fmaf(bf_lo(dv4[pc].x), __uint_as_float(rr[0]), d); d = fmaf(bf_hi(dv4[pc].x), __uint_as_float(rr[1]), d);
-              d = fmaf(bf_lo(dv4[pc].y), __uint_as_float(rr[2]), d); d = fmaf(bf_hi(dv4[pc].y), __uint_as_float(rr[3]), d);
-              d = fmaf(bf_lo(dv4[pc].z), __uint_as_float(rr[4]), d); d = fmaf(bf_hi(dv4[pc].z), __uint_as_float(rr[5]), d);
-              d = fmaf(bf_lo(dv4[pc].w), __uint_as_float(rr[6]), d); d = fmaf(bf_hi(dv4[pc].w), __uint_as_float(rr[7]), d);
+            for (int hh = 0; hh < 2; ++hh) {
+              ld_v8(drow + hh * 32, dv);
+              ld_v8(drow + hh * 32 + 16, dv + 8);
+              tmem_ld32(taddr + (uint32_t)part * 64u + (uint32_t)hh * 32u, r0);
+              tmem_ld_wait();
+#pragma unroll
+              for (int e = 0; e < 16; ++e) { d = fmaf(bf_lo(dv[e]), __uint_as_float(r0[2 * e]), d); d = fmaf(bf_hi(dv[e]), __uint_as_float(r0[2 * e + 1]), d); }
             }
-            if (i2 == 0) D0 = d; else if (i2 == 1) D1 = d; else if (i2 == 2) D2 = d; else D3 = d;
+            tmem_st1(taddr + (uint32_t)part * 64u, __float_as_uint(d));
           }
+          fence_before();
+          __syncwarp();
+          if (lane == 0) mb_arrive(bar(B_D_READY));
+          if (!(ok = wait_all(B_D_READY, (uint32_t)it.unit_seq & 1u, 0xC07))) break;
+          fence_after();
+          uint32_t d4[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+          for (int i2 = 0; i2 < 4; ++i2)
+            if (i2 < nb) tmem_ld1(taddr + (uint32_t)i2 * 64u, d4[i2]);
+          tmem_ld_wait();
+          D0 = __uint_as_float(d4[0]); D1 = __uint_as_float(d4[1]); D2 = __uint_as_float(d4[2]); D3 = __uint_as_float(d4[3]);
           fence_before();
         }
         it.advance();
@@ -473,19 +500,22 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       if (!(ok = wait_all(B_DP_FULL + it.dp_buf(), (uint32_t)it.dp_use() & 1u, 0xC01))) break;
       fence_after();
       if (!(ok = wait_all(B_P_FULL + slot, par, 0xC02))) break;
-      tmem_ld32(taddr + it.dp_col() + (uint32_t)half * 64u, r0);
-      tmem_ld32(taddr + it.dp_col() + (uint32_t)half * 64u + 32u, r1);
+      tmem_ld32(taddr + it.dp_col() + (uint32_t)part * 32u, r0);
+      // this thread's four pieces of the tile of P
+      const uint32_t prow = sP + (uint32_t)slot * 2u * kBox + (uint32_t)(part >> 1) * kBox + (uint32_t)row_l * 128u;
+      auto piece = [&](int pc) { return prow + ((((uint32_t)(part & 1) * 4u + (uint32_t)pc) ^ sw) << 4); };
+      uint4 out[4];
+#pragma unroll
+      for (int pc = 0; pc < 4; ++pc) out[pc] = lds_v4(piece(pc));
       tmem_ld_wait();
       fence_before();
       __syncwarp();
       if (lane == 0) mb_arrive(bar(B_DP_EMPTY + it.dp_buf()));            // dP is in registers: the buffer's next dP may overwrite it
       const float Dr = it.i == 0 ? D0 : (it.i == 1 ? D1 : (it.i == 2 ? D2 : D3));
-      const uint32_t prow = sP + (uint32_t)slot * 2u * kBox + (uint32_t)half * kBox + (uint32_t)row_l * 128u;
-      uint4 out[8];
 #pragma unroll
-      for (int pc = 0; pc < 8; ++pc) {
-        const uint4 pv = lds_v4(prow + ((((uint32_t)pc) ^ sw) << 4));
-        const uint32_t* rr = pc < 4 ? r0 + pc * 8 : r1 + (pc - 4) * 8;
+      for (int pc = 0; pc < 4; ++pc) {
+        const uint4 pv = out[pc];
+        const uint32_t* rr = r0 + pc * 8;
         out[pc] = make_uint4(pack2(bf_lo(pv.x) * (__uint_as_float(rr[0]) - Dr), bf_hi(pv.x) * (__uint_as_float(rr[1]) - Dr)),
                              pack2(bf_lo(pv.y) * (__uint_as_float(rr[2]) - Dr), bf_hi(pv.y) * (__uint_as_float(rr[3]) - Dr)),
                              pack2(bf_lo(pv.z) * (__uint_as_float(rr[4]) - Dr), bf_hi(pv.z) * (__uint_as_float(rr[5]) - Dr)),
@@ -495,42 +525,41 @@ attention_bwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       // dS goes where this tile of P stands: its last reader, the dvv MMAs of this step, must have run
       if (!(ok = wait_all(B_PV_DONE + s1slot, it.s1par, 0xC03))) break;
       if (a.ds_dump) {      // (testing: the bf16 values the two contractions below consume)
-        uint4* dd = reinterpret_cast<uint4*>(a.ds_dump + ((((long long)b * a.H + h) * L + it.i * 128 + row_l) * L + it.j * 128 + half * 64));
+        uint4* dd = reinterpret_cast<uint4*>(a.ds_dump + ((((long long)b * a.H + h) * L + it.i * 128 + row_l) * L + it.j * 128 + part * 32));
 #pragma unroll
-        for (int pc = 0; pc < 8; ++pc) dd[pc] = out[pc];
+        for (int pc = 0; pc < 4; ++pc) dd[pc] = out[pc];
       }
-      const uint32_t drow = prow;
 #pragma unroll
-      for (int pc = 0; pc < 8; ++pc) sts_v4(drow + ((((uint32_t)pc) ^ sw) << 4), out[pc].x, out[pc].y, out[pc].z, out[pc].w);
+      for (int pc = 0; pc < 4; ++pc) sts_v4(piece(pc), out[pc].x, out[pc].y, out[pc].z, out[pc].w);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) mb_arrive(bar(B_DS_FULL + s1slot));
       if (it.last_i()) {
-        // key block j is complete: dkk (scaled) leaves through the warps of column half 0, dvv through those of half 1
+        // key block j is complete: dkk (scaled) leaves through the warps of parts 0 and 1, dvv through those of 2 and 3; the columns are free once they are in registers
         if (!(ok = wait_all(B_DKV_FULL, (uint32_t)it.k_seq & 1u, 0xC04))) break;
         fence_after();
-        tmem_ld32(taddr + (half == 0 ? kColDK : kColDV), r0);
-        tmem_ld32(taddr + (half == 0 ? kColDK : kColDV) + 32u, r1);
+        tmem_ld32(taddr + (part < 2 ? kColDK : kColDV) + (uint32_t)(part & 1) * 32u, r0);
         tmem_ld_wait();
-        const long long off = (((long long)b * L + it.j * 128 + row_l) * a.H + h) * 64;
-        store_row((half == 0 ? a.dk : a.dv) + off, r0, r1, half == 0 ? a.scale : 1.f);
         fence_before();
         __syncwarp();
         if (lane == 0) mb_arrive(bar(B_DKV_EMPTY));
+        const long long off = (((long long)b * L + it.j * 128 + row_l) * a.H + h) * 64 + (part & 1) * 32;
+        store_half_row((part < 2 ? a.dk : a.dv) + off, r0, part < 2 ? a.scale : 1.f);
       }
       if (it.last_of_unit()) {
         if (!(ok = wait_all(B_DQ_FULL, (uint32_t)it.unit_seq & 1u, 0xC05))) break;
         fence_after();
-        for (int i2 = half; i2 < nb; i2 += 2) {
-          tmem_ld32(taddr + (uint32_t)i2 * 64u, r0);
-          tmem_ld32(taddr + (uint32_t)i2 * 64u + 32u, r1);
+        for (int n = part; n < 2 * nb; n += 4) {          // halves of query blocks' rows
+          tmem_ld32(taddr + (uint32_t)n * 32u, r0);
           tmem_ld_wait();
-          const long long off = (((long long)b * L + i2 * 128 + row_l) * a.H + h) * 64;
-          store_row(a.dq + off, r0, r1, a.scale);
+          if (n + 4 >= 2 * nb) {
+            fence_before();
+            __syncwarp();
+            if (lane == 0) mb_arrive(bar(B_DQ_EMPTY));
+          }
+          store_half_row(a.dq + (((long long)b * L + (n >> 1) * 128 + row_l) * a.H + h) * 64 + (n & 1) * 32, r0, a.scale);
         }
-        fence_before();
-        __syncwarp();
-        if (lane == 0) mb_arrive(bar(B_DQ_EMPTY));
+        if (part >= 2 * nb && lane == 0) mb_arrive(bar(B_DQ_EMPTY));
       }
       it.advance();
     }
@@ -590,6 +619,8 @@ mtf_status launch_attention_bwd_fused(const void* q, const void* kk, const void*
   if (!attention_bwd_fused_supported(L, 64, 64)) return fail(MTF_ERR_UNSUPPORTED, "fused attention backward: length %lld", (long long)L);
   for (const void* p : {q, kk, vv, weights, dout, (const void*)dq, (const void*)dkk, (const void*)dvv})
     if (!p || (reinterpret_cast<uintptr_t>(p) & 15)) return fail(MTF_ERR_INVALID_ARG, "fused attention backward: NULL or misaligned tensor");
+  for (const void* p : {dout, (const void*)dq, (const void*)dkk, (const void*)dvv})      // (the block's own scratch: read and written 32 bytes at a time)
+    if (reinterpret_cast<uintptr_t>(p) & 31) return fail(MTF_ERR_INVALID_ARG, "fused attention backward: misaligned scratch");
   if (B * H <= 0) return MTF_OK;
   if (B * H > 0x3fffffff) return fail(MTF_ERR_UNSUPPORTED, "fused attention backward: %lld pairs", (long long)(B * H));
   CUtensorMap mq, mk, mv, md, mp;
