@@ -1978,6 +1978,8 @@ static mtf_status launch_cluster(const mtf_plan_t& plan, ClusterPick pick, const
       if (zs != MTF_OK) return zs;
     }
   }
+  a.c_wide = !a.c_bf16 && t.ldc % 8 == 0;
+  for (int j = 0; j < t.n_outer; ++j) a.c_wide = a.c_wide && t.outer_sC[j] % 8 == 0;
   CUtensorMap map_a, map_b;
   ExtraMaps extra;
   auto maps = [&](const void* Ap, const void* Bp, CUtensorMap* ma, CUtensorMap* mb) {
@@ -2000,6 +2002,7 @@ static mtf_status launch_cluster(const mtf_plan_t& plan, ClusterPick pick, const
       if (!a.C[i] || (reinterpret_cast<uintptr_t>(a.C[i]) & 15)) return fail(MTF_ERR_INVALID_ARG, "grouped launch: NULL or misaligned output");
     }
   }
+  for (const void* c : a.C) a.c_wide = a.c_wide && !(reinterpret_cast<uintptr_t>(c) & 31);
   const bool stages = bias || relu || mask || resid || rsum;
 #define MTF_CL(BN, S) (stages ? launch_cluster_variant<BN, S, true>(map_a, map_b, extra, a, ctas, st) : launch_cluster_variant<BN, S, false>(map_a, map_b, extra, a, ctas, st))
   if (pick.bn == 64) s = pick.split == 8 ? MTF_CL(64, 8) : pick.split == 4 ? MTF_CL(64, 4) : pick.split == 2 ? MTF_CL(64, 2) : MTF_CL(64, 1);

@@ -190,3 +190,26 @@ def test_which_products_it_takes(mtf, a, b, out, dtype, cluster):
     mtf.mtf_einsum(layout(mtf, *ONE), None, [mtf.named(x, list(s)) for x, s in zip(t, sizes)], mtf.named(c, ["i", "j"]))
     mtf.mtf_device_status()
     assert (mtf.mtf_debug_contraction()[1] > 0) == cluster
+
+
+@pytest.mark.parametrize("n", [8, 64, 68, 72, 136, 200])
+@pytest.mark.parametrize("shift", [0, 4])
+@pytest.mark.parametrize("columns,split", [(64, 1), (64, 4), (128, 1), (128, 2)])
+def test_f32_rows_on_and_off_32_bytes(mtf, n, shift, columns, split):
+    """f32 results are stored 32 bytes at a time where every row starts on 32 bytes, else 16: row lengths of either kind, outputs that start on 16 bytes only."""
+    import torch
+    m, k = 200, 264
+    g = torch.Generator(device="cuda").manual_seed(2)
+    x, y = torch.randn(m, k, generator=g, device="cuda").bfloat16(), torch.randn(n, k, generator=g, device="cuda").bfloat16()      # (B along K: any n)
+    room = torch.full((m * n + 16,), 7.0, device="cuda")
+    out = room[shift:shift + m * n].view(m, n)
+    mtf.mtf_debug_contraction(columns, split)
+    try:
+        mtf.mtf_einsum(layout(mtf, *ONE), None, [mtf.named(x, ["i", "k"]), mtf.named(y, ["j", "k"])], mtf.named(out, ["i", "j"]))
+    finally:
+        assert mtf.mtf_debug_contraction(0, 0) == (columns, split)
+    mtf.mtf_device_status()
+    ref = x.double() @ y.double().t()
+    # f32 sums of k products, of which the accumulator drops at most 2^-23 of the running sum each
+    assert ((out.double() - ref).abs() / ref.abs().clamp_min(k ** 0.5)).max() <= k * 2.0 ** -23
+    assert (room[:shift] == 7.0).all() and (room[shift + m * n:] == 7.0).all()
