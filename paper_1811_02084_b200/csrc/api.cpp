@@ -741,11 +741,19 @@ mtf_status mtf::ffn_backward_impl(const mtf_layout_t* layout, const mtf_tensor* 
       return exec_plan(P4, in4, dx, nullptr, rest, rest_bytes, stream, 1, nullptr, 0, 1, nullptr, dx_beside);
     }
   }
-  if ((st = mtf_einsum(layout, nullptr, 2, in1, &dhp, &e1, rest, rest_bytes, stream)) != MTF_OK) return st;
-  if ((st = mtf::tap("dhp", dhp, stream)) != MTF_OK) return st;
+  // the small launch that finishes dbias comes behind dv, which then starts beside dhp itself (dv must not want the workspace, where the partial sums are)
+  const mtf_plan_t* Pv = nullptr;
+  const bool late_sums = fuse_dbias && layout && layout->bound_dim < 0 && cached_plan(layout, 2, in2, dv, nullptr, &Pv) == MTF_OK && Pv->kernel_kind == MTF_KERNEL_TCGEN05 &&
+                         Pv->reduce_mode != MTF_REDUCE_WORKSPACE && !Pv->tc.balance;
+  mtf::defer_column_sums(late_sums);
+  st = mtf_einsum(layout, nullptr, 2, in1, &dhp, &e1, rest, rest_bytes, stream);
+  if (st == MTF_OK) st = mtf::tap("dhp", dhp, stream);
   // dv = h^T . dy  and  dw = x^T . dhp  reduce out the token dims (Section 8.1)
   mtf::hint_next_launch_independent();        // dv reads h and dy, which the dhp launch only reads, and writes dv
-  if ((st = mtf_einsum(layout, nullptr, 2, in2, dv, nullptr, rest, rest_bytes, stream)) != MTF_OK) return st;
+  if (st == MTF_OK) st = mtf_einsum(layout, nullptr, 2, in2, dv, nullptr, rest, rest_bytes, stream);
+  (void)mtf::take_independent_hint();
+  const mtf_status fs = mtf::finish_deferred_column_sums();
+  if (st != MTF_OK || (st = fs) != MTF_OK) return st;
   if ((st = mtf_einsum(layout, nullptr, 2, in3, dw, nullptr, rest, rest_bytes, stream)) != MTF_OK) return st;
   if (dbias && !fuse_dbias && (st = mtf_reduce_sum(layout, &dhp, dbias, stream)) != MTF_OK) return st;
   // dx = dhp . w^T reduces out hidden (Section 8.2)

@@ -1907,6 +1907,20 @@ size_t tc_rsum_partial_bytes(const TcParams& t) {
   return (size_t)groups * t.N * sizeof(float);
 }
 
+// The launch that finishes a contraction's column sums, behind it or (defer_column_sums) where the caller puts it.
+static thread_local struct { bool asked; const float* partial; int groups, n; float* out; void* stream; } g_deferred = {false, nullptr, 0, 0, nullptr, nullptr};
+void defer_column_sums(bool on) { g_deferred.asked = on; g_deferred.partial = nullptr; }
+static mtf_status finish_column_sums(const float* partial, int groups, int n, float* out, void* stream) {
+  if (!g_deferred.asked) return launch_colsum_finalize(partial, groups, 1, n, out, nullptr, stream);
+  g_deferred = {false, partial, groups, n, out, stream};
+  return MTF_OK;
+}
+mtf_status finish_deferred_column_sums() {
+  const auto d = g_deferred;
+  defer_column_sums(false);
+  return d.partial ? launch_colsum_finalize(d.partial, d.groups, 1, d.n, d.out, nullptr, d.stream) : MTF_OK;
+}
+
 template <int BN, int kSplit, bool kEpi>
 static mtf_status launch_cluster_variant(const CUtensorMap& map_a, const CUtensorMap& map_b, const ExtraMaps& extra, const ClusterArgs& a, long long ctas, cudaStream_t st) {
   static std::once_flag once[kMaxDevices];           // the shared-memory opt-in is a property of a device
@@ -2009,7 +2023,7 @@ static mtf_status launch_cluster(const mtf_plan_t& plan, ClusterPick pick, const
   else s = pick.split == 8 ? MTF_CL(128, 8) : pick.split == 4 ? MTF_CL(128, 4) : pick.split == 2 ? MTF_CL(128, 2) : MTF_CL(128, 1);
 #undef MTF_CL
   if (s != MTF_OK || !a.rsum_partial) return s;
-  return launch_colsum_finalize(a.rsum_partial, (int)groups, 1, (int)t.N, rsum, nullptr, stream);
+  return finish_column_sums(a.rsum_partial, (int)groups, (int)t.N, rsum, stream);
 }
 
 // Two independent sums over queries of one shape, each with a scale of its own: dkk = s dS^T q and dvv = P^T do (the plan is
@@ -2304,7 +2318,7 @@ mtf_status launch_tc(const mtf_plan_t& plan, const void* A, const void* B, void*
   count_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(MTF_ERR_CUDA, "gemm_tcgen05_kernel: %s", cudaGetErrorString(e));
-  if (a.rsum_partial) return launch_colsum_finalize(a.rsum_partial, (int)rsum_groups, 1, (int)t.N, rsum, nullptr, stream);
+  if (a.rsum_partial) return finish_column_sums(a.rsum_partial, (int)rsum_groups, (int)t.N, rsum, stream);
   return MTF_OK;
 }
 

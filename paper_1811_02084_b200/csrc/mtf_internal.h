@@ -216,6 +216,10 @@ mtf_status launch_tc(const mtf_plan_t& plan, const void* A, const void* B, void*
 // Hint for the next tensor-core launch of this thread: it neither reads nor writes anything the launch
 // before it on the same stream touches (set by the block compositions, consumed by the launch).
 void hint_next_launch_independent();
+// While asked for (this thread), the next contraction with column sums leaves their partial rows in the workspace; finish_deferred_column_sums launches what
+// finishes them (nothing, where the contraction did without).  The workspace must not be used in between.
+void defer_column_sums(bool on);
+mtf_status finish_deferred_column_sums();
 // Sets the reduce mode that plans made on this thread are forced to (-1: the planner's choice); returns the old one.
 int swap_force_reduce(int mode);
 bool take_independent_hint();
