@@ -1874,8 +1874,7 @@ static ClusterPick cluster_rule(const TcParams& t, int n_terms, int n_groups, in
   const double per_kb = t.cta_pair ? (t.block_n == 256 ? 0.36 : 0.24) : (t.block_n == 256 ? 0.45 : t.block_n == 128 ? 0.33 : 0.27);
   const bool on_lines = t.a_ld % 64 == 0 && t.b_ld % 64 == 0;
   double best_us = (on_lines ? 0.95 : 0.9) * (7.0 + std::ceil(tiles / std::floor(sms / (t.cta_pair ? 2 : 1))) * kb * per_kb);
-  // (what other tiles of the persistent kernel save there)
-  if (t.cta_pair) best_us *= std::min(1.0, pair_tiles(t, n_terms, n_groups, t.free_tiles, may_widen).us / pair_us(t, kb, outer, t.block_n, false));
+  const double persistent_us = best_us;
   for (int bn = 64; bn <= 128; bn += 64) {
     const double ctas1 = (double)((t.M + BM - 1) / BM) * (double)((t.N + bn - 1) / bn) * outer;
     for (int split = 1; split <= most && split <= kb; split *= 2) {
@@ -1888,6 +1887,12 @@ static ClusterPick cluster_rule(const TcParams& t, int n_terms, int n_groups, in
       if (us < best_us) { best_us = us; best = {bn, split}; }
     }
   }
+  // Other tiles than 256 columns may make the persistent kernel the shorter one again: by its own estimate, with 15 % to spare, and not for launches under 18 us, which
+  // in a chain of short ones do better in the kernel that leaves room for the next (669 x 2112 x 1952: the feed-forward block 77 us there and 92 here, 3 x 200 to 5 x 48 tokens 6 to 11 %;
+  // 1665 x 776 x 3080 24.4 and 20.0).
+  if (best.split && t.cta_pair && best_us > 18.0 &&
+      1.15 * persistent_us * pair_tiles(t, n_terms, n_groups, t.free_tiles, may_widen).us / pair_us(t, kb, outer, t.block_n, false) < best_us)
+    best = {0, 0};
   return best;
 }
 
