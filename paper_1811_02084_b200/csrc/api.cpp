@@ -442,7 +442,7 @@ mtf_status mtf_ffn_forward(const mtf_layout_t* layout, const mtf_tensor* x, cons
 // ranks, no output that lies over an operand or another output (launch by launch that is well defined).  `t`: operands, then outputs from `first_out`.
 static bool ffn_small_shape(const mtf_layout_t* layout, const mtf_tensor* x, const mtf_tensor* w, const mtf_tensor* v, const mtf_tensor* h, const mtf_tensor* y,
                             const mtf_tensor* bias, std::initializer_list<const mtf_tensor*> t, int first_out, bool backward, int64_t* size) {
-  if (!layout || layout->bound_dim >= 0 || mtf::plan_forced() || mtf::contraction_asked()) return false;
+  if (x->dtype != MTF_F32 || !layout || layout->bound_dim >= 0 || mtf::plan_forced() || mtf::contraction_asked()) return false;
   const int n = x->ndim;
   if (n > mtf::kMaxTensorDims || h->ndim != n || y->ndim != n || !h->dims || !y->dims || (bias && (bias->ndim != 1 || !bias->dims))) return false;
   auto is = [](const mtf_dim& a, const mtf_dim& b) { return a.name && b.name && a.size == b.size && strcmp(a.name, b.name) == 0; };
@@ -701,7 +701,7 @@ mtf_status mtf::ffn_backward_impl(const mtf_layout_t* layout, const mtf_tensor* 
   mtf_tensor in3[2] = {*x, dhp};
   mtf_tensor in4[2] = {dhp, *w};
   int64_t n[4];
-  if (!dx_residual && same_dims(*x, *dx) && same_dims(*w, *dw) && same_dims(*v, *dv) &&
+  if (x->dtype == MTF_F32 && !dx_residual && same_dims(*x, *dx) && same_dims(*w, *dw) && same_dims(*v, *dv) &&
       ffn_small_shape(layout, x, w, v, h_saved, dy, dbias, {x, w, v, h_saved, dy, &dhp, dx, dw, dbias, dv}, 5, true, n)) {
     const mtf_plan_t* P = nullptr;
     if (cached_plan(layout, 2, in1, &dhp, &e1, &P) == MTF_OK && cached_plan(layout, 2, in2, dv, nullptr, &P) == MTF_OK &&
