@@ -131,8 +131,9 @@ __device__ __forceinline__ void product(int M, int N, int K, const float* A, int
   __syncthreads();                                // (the next product may use `red`)
 }
 
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// (aligned barriers take whole warps; a product in one part ends in a loop that lanes leave at different turns, and nothing else brings them together)
+__device__ __forceinline__ void cluster_arrive() { __syncwarp(); asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { __syncwarp(); asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 // out[i] = the sum over the cluster's blocks of part[i], each block an eighth of the elements
 __device__ __forceinline__ void add_blocks(const double* part, int n, int rank, float* out) {
@@ -179,7 +180,6 @@ __global__ void __cluster_dims__(kBlocks, 1, 1) __launch_bounds__(kThreads, 1) f
   cluster_arrive();
   cluster_wait();
   add_blocks(part, a.T * a.E, rank, a.y);
-  __syncwarp();
   cluster_arrive();                               // (the cluster may still read this block's part)
   cluster_wait();
 }
@@ -206,7 +206,6 @@ __global__ void __cluster_dims__(kBlocks, 1, 1) __launch_bounds__(kThreads, 1) f
   });
   __syncthreads();
   product<true>(a.T, a.D, n, dhp, lf, w, 1, sw, red, [&](int t, int d, double s) { part[t * a.D + d] = s; });
-  __syncwarp();
   cluster_arrive();                               // (the results that are this block's alone while the others get there)
   product<false>(n, a.E, a.T, h, lf, dy, le, 1, red, [&](int f, int e, double s) { a.dv[(long long)(f0 + f) * a.E + e] = (float)s; });
   product<false>(a.D, n, a.T, x, ld, dhp, lf, 1, red, [&](int d, int f, double s) { a.dw[(long long)d * a.F + f0 + f] = (float)s; });
@@ -216,10 +215,8 @@ __global__ void __cluster_dims__(kBlocks, 1, 1) __launch_bounds__(kThreads, 1) f
       for (int t = 0; t < a.T; ++t) s += (double)dhp[t * lf + f];
       a.dbias[f0 + f] = (float)s;
     }
-  __syncwarp();
   cluster_wait();
   add_blocks(part, a.T * a.D, rank, a.dx);
-  __syncwarp();
   cluster_arrive();
   cluster_wait();
 }
