@@ -263,7 +263,9 @@ mtf_status mtf_ffn_forward(const mtf_layout_t* layout, const mtf_tensor* x, cons
 /* Backward (Section 8.1: parameter gradients are einsums that reduce out the token dims; Section
  * 8.2: the gradient on x reduces out hidden):
  *   dhp = (dy . v^T) * [h_saved > 0];  dv = h^T . dy;  dw = x^T . dhp;  dbias = sum_tokens dhp;
- *   dx = dhp . w^T.   dbias may be NULL.  dhp lives in the workspace. */
+ *   dx = dhp . w^T.   dbias may be NULL.  dhp lives in the workspace.
+ * The products run in this order.  An output may lie over an operand that its own product and those behind
+ * it do not read (dv over v, dx over x); those that then share memory do not run beside each other. */
 mtf_status mtf_ffn_backward(const mtf_layout_t* layout, const mtf_tensor* x, const mtf_tensor* w,
                             const mtf_tensor* v, const mtf_tensor* h_saved, const mtf_tensor* dy,
                             mtf_tensor* dx, mtf_tensor* dw, mtf_tensor* dbias, mtf_tensor* dv,

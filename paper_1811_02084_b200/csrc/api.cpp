@@ -2,7 +2,6 @@
 // numerical step runs in the CUDA kernels; this file only validates, plans and launches.
 #include <algorithm>
 #include <cstring>
-#include <initializer_list>
 
 #include "mtf_internal.h"
 
@@ -580,6 +579,23 @@ mtf_status mtf::einsum_terms(const mtf_layout_t* layout, int n_terms, const mtf_
 }
 
 void mtf::hint_next_launch_independent() { g_next_independent = true; }
+
+// Blocks hint a launch only where this holds: tensors that share memory (dv over v, dx over x) are in order launch by launch, and stay so.
+bool mtf::may_run_beside(std::initializer_list<const mtf_tensor*> writes, std::initializer_list<const mtf_tensor*> reads, std::initializer_list<const mtf_tensor*> writes_before,
+                         std::initializer_list<const mtf_tensor*> reads_before) {
+  auto known = [](const mtf_tensor* t) { return t->ndim >= 0 && t->ndim <= mtf::kMaxTensorDims && (t->dims || !t->ndim); };
+  auto apart = [&](std::initializer_list<const mtf_tensor*> some, std::initializer_list<const mtf_tensor*> others) {
+    for (const mtf_tensor* a : some)
+      for (const mtf_tensor* b : others) {
+        if (!a || !b || !a->data || !b->data) continue;
+        if (!known(a) || !known(b)) return false;
+        const uint8_t *const p = reinterpret_cast<const uint8_t*>(a->data), *const q = reinterpret_cast<const uint8_t*>(b->data);
+        if (p < q + numel(*b) * elem_bytes(b->dtype) && q < p + numel(*a) * elem_bytes(a->dtype)) return false;
+      }
+    return true;
+  };
+  return apart(writes, writes_before) && apart(writes, reads_before) && apart(reads, writes_before);
+}
 int mtf::swap_force_reduce(int mode) { const int was = g_force_reduce; g_force_reduce = mode; return was; }
 bool mtf::plan_forced() { return g_force_kernel >= 0 || g_force_reduce >= 0; }
 bool mtf::take_independent_hint() {
@@ -713,8 +729,11 @@ mtf_status mtf::ffn_backward_impl(const mtf_layout_t* layout, const mtf_tensor* 
       return st != MTF_OK ? st : mtf::tap("dhp", dhp, stream);
     }
   }
+  // dv reads h and dy, which the dhp launch only reads, and dx reads dhp and w, of which the dw launch before it reads dhp
+  const bool dv_beside = mtf::may_run_beside({dv}, {h_saved, dy}, {&dhp, fuse_dbias ? dbias : nullptr}, {dy, v, h_saved});
+  const bool dx_beside = mtf::may_run_beside({dx}, {&dhp, w, dx_residual}, {dw, fuse_dbias ? dbias : nullptr}, {x, &dhp});
   // f32 on the tensor cores: dw = x^T . dhp reads every dhp, so its launch forms dbias too (no output to clear in front of dhp, nothing added to memory in
-  // an order that varies), and dv and dx start beside the launches before them, which they have nothing in common with.
+  // an order that varies), and dv and dx start beside the launches before them.
   {
     const mtf_plan_t *P1 = nullptr, *P2 = nullptr, *P3 = nullptr, *P4 = nullptr, *Pd = nullptr;
     mtf_epilogue ed = e1;
@@ -724,16 +743,6 @@ mtf_status mtf::ffn_backward_impl(const mtf_layout_t* layout, const mtf_tensor* 
         cached_plan(layout, 2, in1, &dhp, &e1, &P1) == MTF_OK && cached_plan(layout, 2, in1, &dhp, &ed, &Pd) == MTF_OK && cached_plan(layout, 2, in2, dv, nullptr, &P2) == MTF_OK &&
         cached_plan(layout, 2, in3, dw, nullptr, &P3) == MTF_OK && cached_plan(layout, 2, in4, dx, nullptr, &P4) == MTF_OK && on_tc(Pd) && on_tc(P2) && on_tc(P3) && on_tc(P4) &&
         mtf::f32_tc_sums_b(P3->f32, false) && dbias->data) {
-      // (an output over an operand of the launch before: one after the other, as launches without the hint run)
-      auto apart = [](const mtf_tensor& out, std::initializer_list<const mtf_tensor*> others) {
-        const uint8_t* const lo = reinterpret_cast<const uint8_t*>(out.data);
-        for (const mtf_tensor* o : others) {
-          const uint8_t* const q = reinterpret_cast<const uint8_t*>(o->data);
-          if (lo < q + numel(*o) * elem_bytes(o->dtype) && q < lo + numel(out) * elem_bytes(out.dtype)) return false;
-        }
-        return true;
-      };
-      const bool dv_beside = apart(*dv, {dy, v, h_saved, &dhp}), dx_beside = apart(*dx, {x, &dhp, dw, dbias});
       (void)mtf::take_independent_hint();
       if ((st = exec_plan(Pd, in1, &dhp, &ed, rest, rest_bytes, stream)) != MTF_OK) return st;
       if ((st = exec_plan(P2, in2, dv, nullptr, rest, rest_bytes, stream, 1, nullptr, 0, 1, nullptr, dv_beside)) != MTF_OK) return st;
@@ -743,13 +752,13 @@ mtf_status mtf::ffn_backward_impl(const mtf_layout_t* layout, const mtf_tensor* 
   }
   // the small launch that finishes dbias comes behind dv, which then starts beside dhp itself (dv must not want the workspace, where the partial sums are)
   const mtf_plan_t* Pv = nullptr;
-  const bool late_sums = fuse_dbias && layout && layout->bound_dim < 0 && cached_plan(layout, 2, in2, dv, nullptr, &Pv) == MTF_OK && Pv->kernel_kind == MTF_KERNEL_TCGEN05 &&
-                         Pv->reduce_mode != MTF_REDUCE_WORKSPACE && !Pv->tc.balance;
+  const bool late_sums = fuse_dbias && dv_beside && layout && layout->bound_dim < 0 && cached_plan(layout, 2, in2, dv, nullptr, &Pv) == MTF_OK &&
+                         Pv->kernel_kind == MTF_KERNEL_TCGEN05 && Pv->reduce_mode != MTF_REDUCE_WORKSPACE && !Pv->tc.balance;
   mtf::defer_column_sums(late_sums);
   st = mtf_einsum(layout, nullptr, 2, in1, &dhp, &e1, rest, rest_bytes, stream);
   if (st == MTF_OK) st = mtf::tap("dhp", dhp, stream);
   // dv = h^T . dy  and  dw = x^T . dhp  reduce out the token dims (Section 8.1)
-  mtf::hint_next_launch_independent();        // dv reads h and dy, which the dhp launch only reads, and writes dv
+  if (dv_beside) mtf::hint_next_launch_independent();
   if (st == MTF_OK) st = mtf_einsum(layout, nullptr, 2, in2, dv, nullptr, rest, rest_bytes, stream);
   (void)mtf::take_independent_hint();
   const mtf_status fs = mtf::finish_deferred_column_sums();
@@ -759,7 +768,7 @@ mtf_status mtf::ffn_backward_impl(const mtf_layout_t* layout, const mtf_tensor* 
   // dx = dhp . w^T reduces out hidden (Section 8.2)
   mtf_epilogue e4;
   e4.scale = 1.f; e4.relu = 0; e4.bias = nullptr; e4.relu_mask = nullptr; e4.residual = dx_residual; e4.reduce_sum_out = nullptr;
-  if (!(dbias && !fuse_dbias)) mtf::hint_next_launch_independent();      // dx reads dhp and w and writes dx; the dw launch before it reads x and dhp and writes dw
+  if (dx_beside && !(dbias && !fuse_dbias)) mtf::hint_next_launch_independent();
   return mtf_einsum(layout, nullptr, 2, in4, dx, dx_residual ? &e4 : nullptr, rest, rest_bytes, stream);
 }
 

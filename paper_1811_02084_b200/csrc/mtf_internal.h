@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cstdint>
+#include <initializer_list>
 #include <map>
 #include <memory>
 #include <mutex>
@@ -216,6 +217,10 @@ mtf_status launch_tc(const mtf_plan_t& plan, const void* A, const void* B, void*
 // Hint for the next tensor-core launch of this thread: it neither reads nor writes anything the launch
 // before it on the same stream touches (set by the block compositions, consumed by the launch).
 void hint_next_launch_independent();
+// Whether a launch with these outputs and operands touches nothing that the launch before it touches, other than reading what that one reads (NULL tensors
+// touch nothing).
+bool may_run_beside(std::initializer_list<const mtf_tensor*> writes, std::initializer_list<const mtf_tensor*> reads, std::initializer_list<const mtf_tensor*> writes_before,
+                    std::initializer_list<const mtf_tensor*> reads_before);
 // While asked for (this thread), the next contraction with column sums leaves their partial rows in the workspace; finish_deferred_column_sums launches what
 // finishes them (nothing, where the contraction did without).  The workspace must not be used in between.
 void defer_column_sums(bool on);
