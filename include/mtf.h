@@ -338,7 +338,9 @@ mtf_status mtf_attention_forward(const mtf_layout_t* layout, const mtf_tensor* x
  * causal: a hint, never needed for the result (causal weights hold exact zeros where m > l and those
  * zeros give zero gradients): non-zero promises that `weights` came from a causal forward call, and the
  * one-launch backward core then skips the key blocks that lie wholly right of the diagonal.  A non-zero
- * hint on weights that are not causal gives wrong gradients. */
+ * hint on weights that are not causal gives wrong gradients.
+ * dwq, dwk and dwv, then dx, come behind everything that reads q, kk, vv, weights, o and dy, and dx behind what
+ * reads x: outputs may lie over those (dx over x). */
 mtf_status mtf_attention_backward(const mtf_layout_t* layout, const mtf_tensor* x, const mtf_tensor* wq,
                                   const mtf_tensor* wk, const mtf_tensor* wv, const mtf_tensor* wo, int32_t causal,
                                   const mtf_tensor* q,

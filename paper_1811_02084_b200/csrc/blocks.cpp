@@ -390,6 +390,7 @@ mtf_status mtf_attention_backward(const mtf_layout_t* layout, const mtf_tensor* 
   // accumulators: no cleared counters in front of it); otherwise it goes first.  Behind the core by rows, 3 x 200 positions, 8 heads of
   // 64: the block 48.1 -> 43.8 us; 4 x 1024, 8 heads of 128, whose core fills the chip: 205.7 and 206.4.
   const bool dwo_late = core_ok || rows_ok;
+  const bool dwo_beside = mtf::may_run_beside({dwo}, {o, dy}, {}, {q, kk, vv, weights});       // (the core writes scratch)
   if (!dwo_late && (st = ein(layout, *o, *dy, dwo, nullptr, rest, rest_bytes, stream)) != MTF_OK) return st;
   if ((st = ein(layout, *dy, *wo, &dob.t, nullptr, rest, rest_bytes, stream)) != MTF_OK) return st;
   if ((st = mtf::tap("do", dob.t, stream)) != MTF_OK) return st;
@@ -405,7 +406,7 @@ mtf_status mtf_attention_backward(const mtf_layout_t* layout, const mtf_tensor* 
       core_done = true;
       if (dwo_late) {
         const int was = mtf::swap_force_reduce(MTF_REDUCE_CHAINED);
-        mtf::hint_next_launch_independent();
+        if (dwo_beside) mtf::hint_next_launch_independent();
         st = ein(layout, *o, *dy, dwo, nullptr, rest, rest_bytes, stream);
         mtf::swap_force_reduce(was);
         if (st != MTF_OK) return st;
@@ -419,7 +420,7 @@ mtf_status mtf_attention_backward(const mtf_layout_t* layout, const mtf_tensor* 
     st = mtf::launch_attention_rows(true, dob.t.data, kk->data, vv->data, weights->data, dlg.t.data, dq.t.data, s.b.size, s.h.size, s.l.size, s.k.size, (float)s.scale,
                                     causal ? 1 : 0, mtf::tap_is_open() ? 1 : 0, stream);
     if (st != MTF_OK || (st = mtf::tap("dlogits", dlg.t, stream)) != MTF_OK) return st;
-    mtf::hint_next_launch_independent();
+    if (dwo_beside) mtf::hint_next_launch_independent();
     if ((st = ein(layout, *o, *dy, dwo, nullptr, rest, rest_bytes, stream)) != MTF_OK) return st;
     if ((st = mtf::attention_kv(layout, &dlg.t, q, &dkk.t, (float)s.scale, weights, &dob.t, &dvv.t, causal ? 1 : 0, stream)) != MTF_OK) return st;
     core_done = true;
@@ -466,7 +467,7 @@ mtf_status mtf_attention_backward(const mtf_layout_t* layout, const mtf_tensor* 
     const mtf_tensor terms[3][2] = {{dq.t, *wq}, {dkk.t, *wk}, {dvv.t, *wv}};
     // (it reads what the weight-gradient launch before it only reads and writes dx: an independent launch, whose tiles
     //  start on the SMs that launch's few tiles leave idle)
-    mtf::hint_next_launch_independent();
+    if (mtf::may_run_beside({dx}, {wq, wk, wv, dx_residual}, {dwq, dwk, dwv}, {x})) mtf::hint_next_launch_independent();
     st = mtf::einsum_terms(layout, 3, terms, dx, dx_residual ? &er : nullptr, rest, rest_bytes, stream);
     (void)mtf::take_independent_hint();
     if (st == MTF_OK) return mtf::rank_wait(layout, stream);

@@ -70,3 +70,45 @@ def test_a_later_product_reads_what_an_earlier_one_wrote(mtf):  # noqa: F811
     dhp = (t["dy"].double() @ t["v"].double().t()) * (t["h"] > 0)
     ref = dhp @ got["dw"].double().t()
     assert (got["dx"].double() - ref).norm() <= 1e-6 * ref.norm()
+
+
+# rows of 512 (one-launch core), of 200 (core by rows) and of 136 with heads of 32 (launch by launch)
+@pytest.mark.parametrize("B,L,M,H,K", [(8, 512, 1024, 16, 64), (3, 200, 512, 8, 64), (2, 136, 256, 4, 32)])
+@pytest.mark.parametrize("over", [{"dx": "x"}, {"dwk": "kk"}, {"dx": "x", "dwv": "weights"}, {"dx": "dy"}])
+def test_attention_backward(mtf, B, L, M, H, K, over):  # noqa: F811
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(4)
+    words, f32 = ["batch", "length", "d_model"], torch.float32
+    shapes = {"x": ((B, L, M), words), "dy": ((B, L, M), words), "y": ((B, L, M), words), "wo": ((H, K, M), ["heads", "d_v", "d_model"]),
+              "weights": ((B, H, L, L), ["batch", "heads", "length", "memory_length"])}
+    shapes |= {w: ((M, H, K), ["d_model", "heads", "d_v" if w == "wv" else "d_k"]) for w in ("wq", "wk", "wv")}
+    shapes |= {a: ((B, L, H, K), ["batch", "length" if a in ("q", "o") else "memory_length", "heads", "d_v" if a in ("vv", "o") else "d_k"]) for a in ("q", "kk", "vv", "o")}
+    first = {k: (torch.randn(*s, generator=g, device="cuda") * (M ** -0.5 if k[0] == "w" and k != "weights" else 1.0)).bfloat16() for k, (s, _) in shapes.items()}
+    lay = layout(mtf, [("all", 1)], [])
+    named = {k: mtf.named(first[k], shapes[k][1]) for k in shapes}
+    ws = torch.empty(mtf.mtf_attention_workspace_bytes(lay, named["x"], named["wq"], named["wv"]), dtype=torch.uint8, device="cuda")
+    mtf.mtf_attention_forward(lay, *[named[k] for k in ("x", "wq", "wk", "wv", "wo")], False, None, *[named[k] for k in ("q", "kk", "vv", "weights", "o", "y")], ws)
+
+    def backward(over):
+        t = dict(first)
+        out = {"dx": ("x", torch.bfloat16), "dwq": ("wq", f32), "dwk": ("wk", f32), "dwv": ("wv", f32), "dwo": ("wo", f32)}
+        for k, (like, dt) in out.items():
+            size = first[like].numel() * (2 if dt == torch.bfloat16 else 4)
+            if k in over:
+                src = first[over[k]]
+                buf = torch.empty(max(size, src.numel() * 2), dtype=torch.uint8, device="cuda")
+                t[over[k]] = buf[:src.numel() * 2].view(torch.bfloat16).view(src.shape)
+                t[over[k]].copy_(src)
+                t[k] = buf[:size].view(dt).view(first[like].shape)
+            else:
+                t[k] = torch.full(first[like].shape, float("nan"), dtype=dt, device="cuda")
+        n = {k: mtf.named(v, shapes[out[k][0] if k in out else k][1]) for k, v in t.items()}
+        mtf.mtf_attention_backward(lay, *[n[k] for k in ("x", "wq", "wk", "wv", "wo", "q", "kk", "vv", "weights", "o", "dy")], None,
+                                   *[n[k] for k in ("dx", "dwq", "dwk", "dwv", "dwo")], ws)
+        mtf.mtf_device_status()
+        return {k: t[k].clone() for k in out}
+
+    want = backward({})
+    for _ in range(3):
+        got = backward(over)
+        assert all(torch.equal(got[k], want[k]) for k in want)
