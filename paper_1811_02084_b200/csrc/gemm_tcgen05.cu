@@ -1817,6 +1817,16 @@ static double pair_us(const TcParams& t, double kb, double outer, int bn, bool f
   return 1.85 + (main + out + (waves - 1.0) * std::max(main, out)) / 1787.0;
 }
 
+// Whether a launch of CTA pairs may leave 256 columns and the layout's slices (the optional build's loads share 256-column tiles).
+static bool tiles_are_free(const TcParams& t) {
+#if defined(MTF_CLUSTER_SHARE)
+  (void)t;
+  return false;
+#else
+  return t.free_tiles && t.block_n == 256 && t.reduce_mode != MTF_REDUCE_WORKSPACE && !t.balance;
+#endif
+}
+
 // Tiles of a launch of CTA pairs: 256 rows by bn columns (512: "wide"), inside the layout's slices or (flat) across their edges, which an output
 // element, one sum over all of K whoever owns it, does not notice.
 struct PairTiles { int bn; bool flat; double us; };
@@ -1829,13 +1839,13 @@ static bool widens(const TcParams& t, int n_terms, int n_groups) {
   return t.K * n_terms >= 64 * BK && 3.0 * std::ceil(tiles / 2.0 / workers) < 2.0 * std::ceil(tiles / workers);
 }
 
-// free_tiles: the launch may leave 256 columns and the slices; may_widen: its epilogue allows 512 columns.  Narrower tiles pull more bytes per
-// multiply-add, so they have to be 3 % shorter by the estimate.
-static PairTiles pair_tiles(const TcParams& t, int n_terms, int n_groups, bool free_tiles, bool may_widen) {
+// may_widen: the launch's epilogue allows 512 columns.  Narrower tiles pull more bytes per multiply-add, so they have to be 3 % shorter by the
+// estimate.
+static PairTiles pair_tiles(const TcParams& t, int n_terms, int n_groups, bool may_widen) {
   const double kb = (double)((t.K + BK - 1) / BK) * n_terms, outer = tile_outer(t, n_groups);
   if (may_widen && widens(t, n_terms, n_groups)) return {512, false, pair_us(t, kb, outer, 512, false)};
   PairTiles best = {t.block_n, false, pair_us(t, kb, outer, t.block_n, false)};
-  if (free_tiles && t.block_n == 256 && t.reduce_mode != MTF_REDUCE_WORKSPACE && !t.balance) {
+  if (tiles_are_free(t)) {
     double least = best.us;
     for (int bn = 256; bn >= 128; bn -= 64)
       for (int flat = 0; flat <= (t.sm * t.sn > 1 ? 1 : 0); ++flat) {
@@ -1891,7 +1901,7 @@ static ClusterPick cluster_rule(const TcParams& t, int n_terms, int n_groups, in
   // in a chain of short ones do better in the kernel that leaves room for the next (669 x 2112 x 1952: the feed-forward block 77 us there and 92 here, 3 x 200 to 5 x 48 tokens 6 to 11 %;
   // 1665 x 776 x 3080 24.4 and 20.0).
   if (best.split && t.cta_pair && best_us > 18.0 &&
-      1.15 * persistent_us * pair_tiles(t, n_terms, n_groups, t.free_tiles, may_widen).us / pair_us(t, kb, outer, t.block_n, false) < best_us)
+      1.15 * persistent_us * pair_tiles(t, n_terms, n_groups, may_widen).us / pair_us(t, kb, outer, t.block_n, false) < best_us)
     best = {0, 0};
   return best;
 }
@@ -2122,12 +2132,7 @@ mtf_status launch_tc(const mtf_plan_t& plan, const void* A, const void* B, void*
   if (t.wide_pref == 1 && !wide_legal)
     return fail(MTF_ERR_UNSUPPORTED, "wide tiles need CTA pairs, a plain or residual-only epilogue, no workspace reduction and an N slice that is a multiple of 512");
   if (t.cta_pair && !row_softmax && !row_lse) {
-#if defined(MTF_CLUSTER_SHARE)
-    const bool free_tiles = false;         // (its loads share 256-column tiles)
-#else
-    const bool free_tiles = t.free_tiles;
-#endif
-    const PairTiles pt = pair_tiles(t, n_terms, n_groups, free_tiles, may_widen);
+    const PairTiles pt = pair_tiles(t, n_terms, n_groups, may_widen);
     wide = t.wide_pref == 1 || pt.bn == 512;
     if (!wide) a.block_n = pt.bn;
     if (pt.flat && !wide) { a.sm = a.sn = 1; a.Ms = a.M; a.Ns = a.N; }

@@ -50,3 +50,27 @@ def test_parity_suite_on_the_opt_in_library():
            os.path.join(ROOT, "tests", "test_gpu_einsum.py"), os.path.join(ROOT, "tests", "test_gpu_ffn.py")]
     proc = subprocess.run(cmd, cwd=ROOT, env=env, capture_output=True, text=True, timeout=900)
     assert proc.returncode == 0, proc.stdout[-3000:] + proc.stderr[-2000:]
+
+
+@pytest.mark.gpu
+def test_products_stay_on_the_kernel_that_the_opt_in_library_runs_fastest():
+    """The default library takes this product from the 128-row kernel for the sake of narrower tiles on CTA pairs; the opt-in one has no such tiles."""
+    import torch
+    if not os.path.exists(os.path.join(ROOT, "paper_1811_02084_b200", "libmtf_b200_mc.so")) or torch.cuda.device_count() != 1:
+        pytest.skip("the optional single-GPU library is not built, or this process sees more than one GPU")
+    code = """
+import torch, paper_1811_02084_b200 as mtf
+lay = mtf.mtf_layout(mtf.mtf_mesh_create([("p", 5)]), [("i", "p")])
+a, b, c = (torch.zeros(*s, dtype=torch.bfloat16, device="cuda") for s in ((1665, 3080), (3080, 776), (1665, 776)))
+mtf.mtf_einsum(lay, None, [mtf.named(a, ["i", "k"]), mtf.named(b, ["k", "j"])], mtf.named(c, ["i", "j"]), None, None)
+mtf.mtf_device_status()
+print(*mtf.mtf_debug_contraction())
+"""
+    ran = {}
+    for share in ("0", "1"):
+        env = dict(os.environ, MTF_CLUSTER_SHARE=share)
+        env.pop("WORLD_SIZE", None)
+        proc = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=env, capture_output=True, text=True, timeout=300)
+        assert proc.returncode == 0, proc.stderr[-2000:]
+        ran[share] = [int(n) for n in proc.stdout.split()]
+    assert ran["0"] == [0, 0] and ran["1"][0] > 0, ran
