@@ -503,6 +503,11 @@ mtf_status mtf_debug_wait_test(int64_t limit_cycles, int32_t withhold_one_signal
  * the tensor cores, in bf16 pieces of the values (128 rows a tile).  ran_columns, ran_split (may be NULL): what this
  * thread's last contraction before the call ran on; 0, 0 if on the persistent or the generic kernel. */
 mtf_status mtf_debug_contraction(int32_t columns, int32_t split, int32_t* ran_columns, int32_t* ran_split);
+/* Testing hook: contractions launched afterwards by this thread on CTA pairs, where the launcher may choose their tiles (slices of more
+ * than 128 rows and columns, no forced or workspace reduction, no row softmax or row statistics), run on 256 rows by `columns` (128, 192
+ * or 256) columns, inside the layout's slices or, with across != 0, across their edges; 0 gives the choice back to the library.
+ * ran_columns, ran_across (may be NULL): the tiles of this thread's last contraction before the call; 0, 0 if not on CTA pairs. */
+mtf_status mtf_debug_pair_tiles(int32_t columns, int32_t across, int32_t* ran_columns, int32_t* ran_across);
 /* Number of kernels this library has launched from this process (all threads). */
 int64_t mtf_launch_count(void);
 

@@ -157,6 +157,7 @@ def _load():
                               POINTER(mtf_tensor), vp, c_size_t, vp],
         "mtf_debug_wait_test": [c_int64, c_int32],
         "mtf_debug_contraction": [c_int32, c_int32, POINTER(c_int32), POINTER(c_int32)],
+        "mtf_debug_pair_tiles": [c_int32, c_int32, POINTER(c_int32), POINTER(c_int32)],
         "mtf_stage_tap_begin": [vp, c_size_t],
         "mtf_stage_tap_end": [POINTER(c_int32)],
         "mtf_stage_tap_entry": [c_int32, POINTER(c_char_p), POINTER(c_size_t), POINTER(c_size_t)],
@@ -661,6 +662,13 @@ def mtf_debug_contraction(columns: int = 0, split: int = 0) -> tuple[int, int]:
     bn, sp = c_int32(), c_int32()
     _check(_lib.mtf_debug_contraction(int(columns), int(split), byref(bn), byref(sp)))
     return bn.value, sp.value
+
+
+def mtf_debug_pair_tiles(columns: int = 0, across: bool = False) -> tuple[int, bool]:
+    """Testing hook: see mtf_debug_pair_tiles in include/mtf.h.  Returns what the last contraction ran on."""
+    bn, flat = c_int32(), c_int32()
+    _check(_lib.mtf_debug_pair_tiles(int(columns), 1 if across else 0, byref(bn), byref(flat)))
+    return bn.value, flat.value != 0
 
 
 def mtf_debug_wait_test(limit_cycles: int = 0, withhold_one_signal: bool = False) -> None:

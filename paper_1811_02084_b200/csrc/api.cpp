@@ -18,6 +18,7 @@ mtf_status read_bad_index(int* seen);
 mtf_status read_row_status(int* code);
 mtf_status debug_wait_test(long long limit_cycles, int skip_first_commit);
 mtf_status debug_contraction(int bn, int split, int* ran_bn, int* ran_split);
+mtf_status debug_pair_tiles(int bn, int across, int* ran_bn, int* ran_across);
 mtf_status read_attention_status(int* code);
 mtf_status launch_permute_copy(const void* src, void* dst, int elem_bytes, int ndim, const int64_t* sizes, const int64_t* sstr, const int64_t* dstr, void* stream);
 mtf_status read_attention_bwd_status(int* code);
@@ -818,6 +819,10 @@ int64_t mtf_launch_count(void) { return mtf::launch_count(); }
 
 mtf_status mtf_debug_contraction(int32_t columns, int32_t split, int32_t* ran_columns, int32_t* ran_split) {
   return mtf::debug_contraction(columns, split, ran_columns, ran_split);
+}
+
+mtf_status mtf_debug_pair_tiles(int32_t columns, int32_t across, int32_t* ran_columns, int32_t* ran_across) {
+  return mtf::debug_pair_tiles(columns, across, ran_columns, ran_across);
 }
 
 mtf_status mtf_debug_wait_test(int64_t limit_cycles, int32_t withhold_one_signal) { return mtf::debug_wait_test(limit_cycles, withhold_one_signal); }

@@ -1798,8 +1798,8 @@ void note_contraction(int columns, int split) { g_last_pick = {columns, split}; 
 // every operand order, rows on and off 128-byte lines, whole and in slices, bf16 and f32 results; graphs of launches, operands in L2), which they miss by 10 % rms (512 columns
 // 6 %).  What a k-block costs is the larger of its MMAs, 2 bn cycles, and of the 128-byte requests that its copies make, 1.5 cycles each: more from rows off the lines, where a
 // line is shared, and from the 64-byte boxes of an N-contiguous B in 192 columns.
-// us on 256 columns inside the slices and on what is chosen:  1665 x 3080 x 776 in five slices, B K-contiguous 19.0 and 16.6 (192 across the slices);  1665 x 776 x
-// 3080 24.6 and 20.0 (128 across);  1024 x 3072 x 4096 27.0 and 22.6 (192);  1024 x 1024 x 4096 24.7 and 15.4 (128).
+// us on 256 columns inside the slices and on what is chosen:  1665 x 3080 x 776 in five slices, B K-contiguous 19.0 and 16.7 (192 across the slices; inside 22.1);
+// 1665 x 776 x 3080 24.8 and 20.6 (128; one wave either way, across 20.2);  1024 x 3072 x 4096 26.4 and 21.6 (192);  1024 x 1024 x 4096 24.1 and 15.3 (128).
 static double tile_outer(const TcParams& t, int n_groups) {
   double outer = n_groups;
   for (int j = 0; j < t.n_outer; ++j) outer *= (double)t.outer_size[j];
@@ -1830,6 +1830,16 @@ static bool tiles_are_free(const TcParams& t) {
 // Tiles of a launch of CTA pairs: 256 rows by bn columns (512: "wide"), inside the layout's slices or (flat) across their edges, which an output
 // element, one sum over all of K whoever owns it, does not notice.
 struct PairTiles { int bn; bool flat; double us; };
+
+// Testing hook (mtf_debug_pair_tiles): the tiles asked for on this thread, and those of its last contraction.
+static thread_local PairTiles g_asked_tiles = {0, false, 0.0}, g_last_tiles = {0, false, 0.0};
+mtf_status debug_pair_tiles(int bn, int across, int* ran_bn, int* ran_across) {
+  if (bn && bn != 128 && bn != 192 && bn != 256) return fail(MTF_ERR_INVALID_ARG, "debug_pair_tiles: 128, 192 or 256 columns (0: the library's choice)");
+  g_asked_tiles = {bn, bn && across, 0.0};
+  if (ran_bn) *ran_bn = g_last_tiles.bn;
+  if (ran_across) *ran_across = g_last_tiles.flat ? 1 : 0;
+  return MTF_OK;
+}
 
 // Wide tiles where they take less than two thirds of the waves and K hides their one accumulator's exposed epilogue.  They pull fewer bytes through L2, which counts where a
 // stream of launches runs into the power limit and not in one launch: 8192 x 1024 x 8192 108.9 us here and 123.0 with 256 columns, back to back for a quarter of a second;
@@ -1899,7 +1909,7 @@ static ClusterPick cluster_rule(const TcParams& t, int n_terms, int n_groups, in
   }
   // Other tiles than 256 columns may make the persistent kernel the shorter one again: by its own estimate, with 15 % to spare, and not for launches under 18 us, which
   // in a chain of short ones do better in the kernel that leaves room for the next (669 x 2112 x 1952: the feed-forward block 77 us there and 92 here, 3 x 200 to 5 x 48 tokens 6 to 11 %;
-  // 1665 x 776 x 3080 24.4 and 20.0).
+  // 1665 x 776 x 3080 24.8 and 20.6).
   if (best.split && t.cta_pair && best_us > 18.0 &&
       1.15 * persistent_us * pair_tiles(t, n_terms, n_groups, may_widen).us / pair_us(t, kb, outer, t.block_n, false) < best_us)
     best = {0, 0};
@@ -2084,6 +2094,7 @@ mtf_status launch_tc(const mtf_plan_t& plan, const void* A, const void* B, void*
     if (reinterpret_cast<uintptr_t>(workspace) & 255) return fail(MTF_ERR_INVALID_ARG, "workspace must be 256-byte aligned");
   }
   g_last_pick = {0, 0};
+  g_last_tiles = {0, false, 0.0};
   // Wide tiles (256 x 512 per pair) for a plain epilogue, or with a residual as the only stage - the contractions whose result is added to a stream of the
   // decoder layer - through the generic epilogue kind.
   const bool plain_launch = scale == 1.f && !bias && !relu && !mask && !rsum && !row_softmax;
@@ -2132,12 +2143,14 @@ mtf_status launch_tc(const mtf_plan_t& plan, const void* A, const void* B, void*
   if (t.wide_pref == 1 && !wide_legal)
     return fail(MTF_ERR_UNSUPPORTED, "wide tiles need CTA pairs, a plain or residual-only epilogue, no workspace reduction and an N slice that is a multiple of 512");
   if (t.cta_pair && !row_softmax && !row_lse) {
-    const PairTiles pt = pair_tiles(t, n_terms, n_groups, may_widen);
+    PairTiles pt = pair_tiles(t, n_terms, n_groups, may_widen);
+    if (g_asked_tiles.bn && tiles_are_free(t)) pt = {g_asked_tiles.bn, g_asked_tiles.flat && t.sm * t.sn > 1, 0.0};
     wide = t.wide_pref == 1 || pt.bn == 512;
     if (!wide) a.block_n = pt.bn;
     if (pt.flat && !wide) { a.sm = a.sn = 1; a.Ms = a.M; a.Ns = a.N; }
   }
   if (wide) a.block_n = 512;
+  if (t.cta_pair) g_last_tiles = {a.block_n, a.sm * a.sn < t.sm * t.sn, 0.0};
   a.b_box = a.b_mn_major && t.cta_pair && a.block_n == 192 ? 32 : 64;
   // optional single-GPU build: clusters of CTA pairs that share operand tiles
   int cm = 1, cn = 1;
