@@ -113,6 +113,21 @@ def test_the_tiles_that_are_asked_for(mtf, m, n, k, sm, sn, order, stage, column
         assert ((sums.double() - ref.sum(0)).abs() / (m * k) ** 0.5).max() <= 1e-4
 
 
+def test_what_may_not_choose_keeps_256_columns(mtf):  # noqa: F811
+    """A forced reduce mode leaves the tiles alone, whatever is asked for."""
+    import torch
+    lay = layout(mtf, [("p", 2)], [("k", "p")])
+    a, b, c = (torch.randn(*s, device="cuda").bfloat16() for s in ((512, 256), (256, 512), (512, 512)))
+    mtf.mtf_plan_force(1, 1)
+    mtf.mtf_debug_pair_tiles(128)
+    try:
+        mtf.mtf_einsum(lay, None, [mtf.named(a, ["i", "k"]), mtf.named(b, ["k", "j"])], mtf.named(c, ["i", "j"]), None, None)
+    finally:
+        mtf.mtf_plan_force(-1, -1)
+        ran = mtf.mtf_debug_pair_tiles(0)
+    assert ran == (256, False)
+
+
 # (sizes of the ragged feed-forward block and of the first test; columns and whether tiles cross the slices)
 @pytest.mark.parametrize("b,m,n,k,slices,order,want", [(1, 2048, 2048, 512, 1, "ik,kj", (256, False)), (9, 512, 768, 320, 1, "ik,kj", (192, False)), (9, 512, 768, 320, 1, "ik,jk", (192, False)),
                                                        (1, 512, 512, 256, 1, "ik,kj", (128, False)), (1, 1665, 3080, 776, 5, "ik,jk", (192, True)), (1, 1640, 1280, 2048, 5, "ik,kj", (128, True)), (1, 1640, 2560, 512, 5, "ik,jk", (256, True))])
