@@ -6,12 +6,15 @@
 // them (y, dx) is the Allreduce, taken through distributed shared memory in block order.
 //
 // All operands are copied to shared memory at once (4-byte asynchronous copies: any alignment, one wait).  Products run from there: a thread
-// owns four rows by two columns, sums eight terms in f32 and the eights in f64, K over several threads where outputs are few; their parts and the blocks'
-// parts are added in f64 too, and every result is rounded once, so that no sum is less exact than one on the matrix kernels (2-norm error against 64
-// bits, the largest of the outputs' at 8 tokens, 64 x 256: 7.6e-8 here and there, 64 tokens 7.6e-8 and 1.2e-7).
+// owns four rows by two columns, sums four terms in f32 and the fours in f64, K over several threads where outputs are few; their parts and the blocks'
+// parts are added in f64 too, and every result is rounded once, so that no sum is less exact than one on the matrix kernels.  2-norm errors against 64 bits
+// in 1e-8, launch by launch | in eights | in fours:
+//   8 tokens, 64 x 256    h 5.6 | 6.0 | 4.8   y 8.2 | 7.8 | 6.4   dx 7.7 | 7.7 | 6.2   dw 6.6 | 7.3 | 6.4   dv 7.0 | 7.3 | 6.4
+//   64 tokens, 40 x 72    h 5.1 | 5.9 | 4.7   y 7.0 | 7.6 | 6.2   dx 6.6 | 7.7 | 6.3   dw 6.2 | 7.7 | 6.3   dv 6.6 | 7.7 | 6.2
 //
 // Bound: latency (launch, one round of loads, two barriers of the cluster) and, towards the limits below, the copies and the shared-memory reads of eight
-// SMs.  The block at 8 tokens, 64 x 256, forward and backward: 28.5 -> 15.1 us (launch by launch six dependent launches of 4 - 5 us).
+// SMs.  The block at 8 tokens, 64 x 256, forward and backward: 28.5 -> 15.5 us (launch by launch six dependent launches of 4 - 5 us; sums of eight
+// terms in f32 instead of four 15.1).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -60,7 +63,7 @@ __device__ __forceinline__ void product(int M, int N, int K, const float* A, int
   if (tasks == 0) return;
   int parts = 1;
   while (2 * parts * tasks <= kThreads && K >= 16 * parts) parts *= 2;
-  const int len = ((K + parts - 1) / parts + 7) / 8 * 8;
+  const int len = ((K + parts - 1) / parts + 3) / 4 * 4;
   const int part = parts > 1 ? (int)threadIdx.x / tasks : 0;
   for (int task = (int)threadIdx.x - part * tasks; task < tasks && part < parts; task += kThreads) {
     const int m0 = task / nh * 4, n0 = task % nh, n1 = n0 + nh;
@@ -70,29 +73,28 @@ __device__ __forceinline__ void product(int M, int N, int K, const float* A, int
     const float* b0 = B + n0 * sBn + k * sBk;
     const float* b1 = B + min(n1, N - 1) * sBn + k * sBk;
     double acc[4][2] = {};
-    for (; k < k1; k += 8) {
+#pragma unroll 1                                  // (short code: it is fetched cold; unrolled twice 4 % of the launch)
+    for (; k < k1; k += 4) {
       float s[4][2] = {};
-      if (k + 8 <= k1) {
+      if (k + 4 <= k1) {                         // four 16-byte reads of A, which every lane of a row shares
+        float f[4][4];
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {            // four k: four 16-byte reads of A, which every lane of a row shares
-          float f[4][4];
+        for (int i = 0; i < 4; ++i) {
+          const float4 q = *reinterpret_cast<const float4*>(a + i * lda);
+          const float r[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float4 q = *reinterpret_cast<const float4*>(a + i * lda);
-            const float r[4] = {q.x, q.y, q.z, q.w};
+          for (int t = 0; t < 4; ++t) (kAlongK ? f[i][t] : f[t][i]) = r[t];      // f[row][k]
+        }
+        a += kAlongK ? 4 : 4 * lda;
 #pragma unroll
-            for (int t = 0; t < 4; ++t) (kAlongK ? f[i][t] : f[t][i]) = r[t];      // f[row][k]
-          }
-          a += kAlongK ? 4 : 4 * lda;
+        for (int t = 0; t < 4; ++t) {
+          const float p = *b0, q = *b1;
+          b0 += sBk; b1 += sBk;
 #pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            const float p = *b0, q = *b1;
-            b0 += sBk; b1 += sBk;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) { s[i][0] = fmaf(f[i][t], p, s[i][0]); s[i][1] = fmaf(f[i][t], q, s[i][1]); }
-          }
+          for (int i = 0; i < 4; ++i) { s[i][0] = fmaf(f[i][t], p, s[i][0]); s[i][1] = fmaf(f[i][t], q, s[i][1]); }
         }
       } else {
+#pragma unroll 1
         for (int t = k; t < k1; ++t) {
           const float p = *b0, q = *b1;
           b0 += sBk; b1 += sBk;
@@ -124,9 +126,9 @@ __device__ __forceinline__ void product(int M, int N, int K, const float* A, int
   for (int i = (int)threadIdx.x; i < 8 * tasks; i += kThreads) {
     const int j = i / tasks, task = i - j * tasks, m = task / nh * 4 + j / 2, n = task % nh + (j & 1) * nh;
     if (m >= M || n >= N) continue;
-    double s = red[i];
-    for (int q = 1; q < parts; ++q) s += red[q * 8 * tasks + i];
-    out(m, n, s);
+    double s = 0.0, s1 = 0.0;                     // (parts is a power of two above one: two chains)
+    for (int q = 0; q < parts; q += 2) { s += red[q * 8 * tasks + i]; s1 += red[(q + 1) * 8 * tasks + i]; }
+    out(m, n, s + s1);
   }
   __syncthreads();                                // (the next product may use `red`)
 }
@@ -247,8 +249,10 @@ namespace mtf {
 // Whether a direction runs here, or as one launch per einsum: forward up to 3 x 2^17 multiply-adds a product; backward up to 2^20, where the products over at most 32 tokens
 // are no work for the tensor cores, else as many as forward; fewer where much of w and v has to be copied.  us, here and launch by launch (graphs of ten passes):
 //   tokens x width x hidden   8 x 64 x 256  16 x 64 x 512  4 x 128 x 512  64 x 40 x 72  128 x 40 x 72  48 x 64 x 256  16 x 128 x 512  8 x 128 x 1024  1 x 48 x 2048
-//   forward                     6.5   9.1      9.6   9.6      8.8   9.8     7.0  10.0     10.1  10.3     9.5   9.8      12.8  10.3     14.1  11.8       9.9  13.8
-//   backward                    7.6  17.0     12.1  17.5     12.3  19.5    10.4  13.7     14.3  15.1    15.8  14.1      18.0  19.0     20.9  20.6      14.6  21.2
+//   forward                     6.6   9.3      9.5   9.8      8.7  10.2     7.1  10.2     9.8  10.7    10.1  10.2      13.3  10.5     14.2  11.5       9.8  14.1
+//   backward                    8.6  17.6     12.9  18.1     12.2  19.9    10.9  14.7    14.9  15.3    17.6  14.7      19.4  19.3     22.4  20.2      14.6  21.5
+// The forward limit of 65536 weights is a cautious one: with up to 8 tokens the launch is the shorter one up to 131072 (2 x 40 x 3000 11.5 and 17.0, 4 x 48 x 2048
+// 10.3 and 14.0, 8 x 48 x 2048 12.8 and 14.2), which runs launch by launch.
 bool ffn_small_pays(int64_t T, int64_t D, int64_t F, int64_t E, bool backward) {
   if (T <= 0 || D <= 0 || F <= 0 || E <= 0 || T > 4096 || D > 8192 || F > 65536 || E > 8192) return false;
   const int64_t weights = F * std::max(D, E), work = T * weights;
