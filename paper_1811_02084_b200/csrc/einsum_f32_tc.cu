@@ -18,7 +18,7 @@
 // more for a small product.)
 // Bound: a stage takes 1.3 us (2500 cycles) and no unit is full in it: issue slots 53 %, shared memory's wavefronts 41 %, tensor pipe 28 % of the
 // active cycles (2048 x 2048 x 1024).  Its steps follow one another: split and store, wait for the stage before, read its accumulators, barrier, issue; the
-// tensor core idles from that wait to the issue, since a second set of a1 b1 blocks would need 640 of 512 columns.  A small product is the chain of
+// tensor core idles from that wait to the issue, since a second set of a stage's a1 b1 blocks would need 640 of 512 columns (two sets of half a stage 384: not written).  A small product is the chain of
 // launch, first loads, one stage and stores (4.5 us).
 // Measured against plain FP32 arithmetic on the 64 x 64 tiles of einsum_f32.cu: 1024 x 1024 x 256 22.2 -> 9.5 us, 1024 x 256 x 1024 23.3 ->
 // 11.2, 2048^3 503 -> 170, 128^3 6.1 -> 5.2, 8 x 256 x 64 4.8 -> 4.5; error against 64 bits (2-norm, normal values) 1.5e-7 -> 6.4e-8 at K = 256,
