@@ -13,7 +13,7 @@
 //   64 tokens, 40 x 72    h 5.1 | 5.9 | 4.7   y 7.0 | 7.6 | 6.2   dx 6.6 | 7.7 | 6.3   dw 6.2 | 7.7 | 6.3   dv 6.6 | 7.7 | 6.2
 //
 // Bound: latency (launch, one round of loads, two barriers of the cluster) and, towards the limits below, the copies and the shared-memory reads of eight
-// SMs.  The block at 8 tokens, 64 x 256, forward and backward: 28.5 -> 15.5 us (launch by launch six dependent launches of 4 - 5 us; sums of eight
+// SMs.  The block at 8 tokens, 64 x 256, forward and backward: 28.5 -> 15.3 us (launch by launch six dependent launches of 4 - 5 us; sums of eight
 // terms in f32 instead of four 15.1).
 #include <cuda_runtime.h>
 
@@ -127,6 +127,7 @@ __device__ __forceinline__ void product(int M, int N, int K, const float* A, int
     const int j = i / tasks, task = i - j * tasks, m = task / nh * 4 + j / 2, n = task % nh + (j & 1) * nh;
     if (m >= M || n >= N) continue;
     double s = 0.0, s1 = 0.0;                     // (parts is a power of two above one: two chains)
+#pragma unroll 1                                  // (as above: 1 %)
     for (int q = 0; q < parts; q += 2) { s += red[q * 8 * tasks + i]; s1 += red[(q + 1) * 8 * tasks + i]; }
     out(m, n, s + s1);
   }
@@ -249,10 +250,10 @@ namespace mtf {
 // Whether a direction runs here, or as one launch per einsum: forward up to 3 x 2^17 multiply-adds a product; backward up to 2^20, where the products over at most 32 tokens
 // are no work for the tensor cores, else as many as forward; fewer where much of w and v has to be copied.  us, here and launch by launch (graphs of ten passes):
 //   tokens x width x hidden   8 x 64 x 256  16 x 64 x 512  4 x 128 x 512  64 x 40 x 72  128 x 40 x 72  48 x 64 x 256  16 x 128 x 512  8 x 128 x 1024  1 x 48 x 2048
-//   forward                     6.6   9.3      9.5   9.8      8.7  10.2     7.1  10.2     9.8  10.7    10.1  10.2      13.3  10.5     14.2  11.5       9.8  14.1
-//   backward                    8.6  17.6     12.9  18.1     12.2  19.9    10.9  14.7    14.9  15.3    17.6  14.7      19.4  19.3     22.4  20.2      14.6  21.5
-// The forward limit of 65536 weights is a cautious one: with up to 8 tokens the launch is the shorter one up to 131072 (2 x 40 x 3000 11.5 and 17.0, 4 x 48 x 2048
-// 10.3 and 14.0, 8 x 48 x 2048 12.8 and 14.2), which runs launch by launch.
+//   forward                     6.6   9.2      9.1   9.4      8.8   9.8     6.9   9.7     9.6  10.2     9.9   9.9      13.0  10.2     14.1  11.4       9.7  14.1
+//   backward                    8.6  17.0     12.6  17.6     12.0  19.4    10.7  14.3    14.5  15.1    16.9  14.4      18.9  18.8     22.1  20.1      14.7  21.5
+// The forward limit of 65536 weights is a cautious one: with up to 8 tokens the launch is the shorter one up to 131072 (2 x 40 x 3000 11.4 and 17.3, 4 x 48 x 2048
+// 9.9 and 13.9, 8 x 48 x 2048 12.5 and 14.2), which runs launch by launch.
 bool ffn_small_pays(int64_t T, int64_t D, int64_t F, int64_t E, bool backward) {
   if (T <= 0 || D <= 0 || F <= 0 || E <= 0 || T > 4096 || D > 8192 || F > 65536 || E > 8192) return false;
   const int64_t weights = F * std::max(D, E), work = T * weights;
