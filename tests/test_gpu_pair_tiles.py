@@ -1,5 +1,6 @@
 """The tiles that CTA pairs may take beside 256 columns inside a slice: 192 columns (an N-contiguous B in 32-column boxes) and 128, and tiles across the edges of
-slices.  Sizes at which the launcher's estimate takes each, whole and ragged, with every operand order and fused stage, against 64-bit sums."""
+slices, whole and ragged, with every operand order and fused stage, against 64-bit sums.  The first test leaves the tiles to the launcher's estimate, the others
+ask for each by name or look at what the estimate took."""
 import pytest
 
 from test_gpu_einsum import layout, mtf  # noqa: F401
